@@ -202,6 +202,18 @@ static int bwd_impl(const void* q, const void* k, const void* v, const void* la_
     if (sizeof(T) == 2 ? !(tc_supported(dk, dv) || recurrence_supported(dk, dv)) : !recurrence_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
     if (empty) return VIG_OK;
     const long long units = (long long)B * H;
+    if constexpr (sizeof(T) == 2) {
+        if (grad_supported(units, L, dk, dv) && kernel_preference() != VIG_TEST_KERNEL_SIMT) {
+            const size_t need = grad_scratch_bytes(units, L, dk, dv);
+            void* ws = nullptr;
+            if (need > 0 && pool_alloc(&ws, need, stream) != cudaSuccess) return VIG_ERR_CUDA;
+            if (launch_bigla_grad((const T*)q, (const T*)k, (const T*)v, (const T*)la_f, (const T*)la_b, (const T*)d_out, (T*)dq, (T*)dk_out,
+                                  (T*)dv_out, (T*)dla_f, (T*)dla_b, ws, units, L, dk, dv, stream) != cudaSuccess)
+                st = VIG_ERR_CUDA;
+            if (need > 0 && cudaFreeAsync(ws, stream) != cudaSuccess && st == VIG_OK) st = VIG_ERR_CUDA;
+            return st;
+        }
+    }
     const size_t gate_bytes = ((size_t)units * L * dk * sizeof(T) + 255) / 256 * 256;
     char* scratch = nullptr;
     const size_t walk_bytes = bwd_scratch_bytes(units, L, dk, dv);

@@ -1,0 +1,116 @@
+// Warp-level tensor-core pieces (mma.sync, fragments in registers) and the swizzled shared-memory tiles they read.
+//
+// Fragment conventions (lane = 4 g + c, g = 0 .. 7, c = 0 .. 3), for D[16 x 8] += A[16 x 16] B[16 x 8]:
+//   A: a0 (row g, k 2c, 2c+1), a1 (row g + 8, same k), a2 (row g, k 2c + 8, 2c + 9), a3 (row g + 8, k 2c + 8, 2c + 9)
+//   B: b0 (k 2c, 2c+1; column g), b1 (k 2c + 8, 2c + 9; column g)
+//   D: d0, d1 (row g, columns 2c, 2c+1), d2, d3 (row g + 8, same columns)
+// so the D fragment of one product, packed to bf16, is the A fragment of the next.
+#pragma once
+#include <cuda_bf16.h>
+
+#include "ptx.cuh"
+
+namespace vig {
+namespace wmma16 {
+
+constexpr float kLog2e = 1.4426950408889634f;
+
+__device__ __forceinline__ void mma_k16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(b0));
+}
+// D = A B
+__device__ __forceinline__ void mma_k16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+// D = A B + (lo, hi) in the even, odd columns of every row.
+__device__ __forceinline__ void mma_k16_from(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1, float lo,
+                                             float hi) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%10,%11};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(lo), "f"(hi));
+}
+// Transpose of the 8 x 8 matrix of bf16 of which a warp holds one row per four lanes.
+__device__ __forceinline__ uint32_t movmatrix(uint32_t x) {
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t mul_bf16x2(uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+    return d;
+}
+
+__device__ __forceinline__ void ldsm(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm_trans(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+// A [rows][RB bytes] bf16 tile in shared memory under the TMA swizzle of span RB, seen by one lane of an ldmatrix /
+// stmatrix of four 8 x 8 matrices: rows row0 .. row0 + 15, 16-byte column pieces 2 n and 2 n + 1.  The operands of an mma
+// are consecutive registers, so the order of the four matrices is chosen for the use (moves otherwise cost as many
+// instructions as the products):
+//   load        as A operand: a0 .. a3 of K step n
+//   load_b      as B operand with the tile's rows as columns: rows 0-7 take (r[0], r[1]), rows 8-15 (r[2], r[3])
+//   load_trans  as B operand that contracts over the rows: columns of piece 2n take (r[0], r[1]), of piece 2n + 1 (r[2], r[3])
+//   (with off_b and a transposing load: A operand with the tile's columns as rows, a0 .. a3)
+template <int RB>
+struct Tile {
+    uint32_t off[RB / 32], off_b[RB / 32];   // this lane's row of the sixteen and its swizzled piece, per n, in either order
+    __device__ __forceinline__ explicit Tile(int lane) {
+        auto at = [](int r, int h, int n) {
+            const uint32_t sw = RB == 128 ? (uint32_t)((h ^ (r & 7)) << 4) : (uint32_t)((h ^ ((r >> 1) & 3)) << 4);
+            return (uint32_t)r * RB + (sw ^ (uint32_t)(n << 5));
+        };
+#pragma unroll
+        for (int n = 0; n < RB / 32; ++n) {
+            off[n] = at(lane & 15, lane >> 4, n);
+            off_b[n] = at((lane & 7) + ((lane >> 4) << 3), (lane >> 3) & 1, n);
+        }
+    }
+    __device__ __forceinline__ uint32_t at(uint32_t tile, int row0, int n) const { return tile + (uint32_t)row0 * RB + off[n]; }
+    __device__ __forceinline__ void load(uint32_t tile, int row0, int n, uint32_t (&r)[4]) const { ldsm(at(tile, row0, n), r); }
+    __device__ __forceinline__ void load_b(uint32_t tile, int row0, int n, uint32_t (&r)[4]) const { ldsm(tile + (uint32_t)row0 * RB + off_b[n], r); }
+    __device__ __forceinline__ void load_trans(uint32_t tile, int row0, int n, uint32_t (&r)[4]) const { ldsm_trans(at(tile, row0, n), r); }
+    __device__ __forceinline__ void store(uint32_t tile, int row0, int n, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3) const {
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(at(tile, row0, n)), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
+                     : "memory");
+    }
+};
+
+// A fragment (a0 = a3) of the diagonal 8 x 8 blocks of the lower triangle of ones, with or without the diagonal; a1 of the
+// 16 x 16 triangle is kOnes, a2 zero.
+__device__ __forceinline__ uint32_t triangle(int g, int c, bool diagonal) {
+    const int lim = diagonal ? g : g - 1;
+    return (2 * c <= lim ? 0x3F80u : 0u) | (2 * c + 1 <= lim ? 0x3F800000u : 0u);
+}
+constexpr uint32_t kOnes = 0x3F803F80u;
+
+// x = hi + lo with two bf16 each: sixteen significant bits of an fp32 value as two tensor-core operands.
+__device__ __forceinline__ void split_bf16(f32x2 x, uint32_t& hi, uint32_t& lo) {
+    float x0, x1;
+    unpack2(x, x0, x1);
+    hi = pack_bf16(x0, x1);
+    unpack2(ffma2(pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pack2(-1.f, -1.f), x), x0, x1);
+    lo = pack_bf16(x0, x1);
+}
+
+}  // namespace wmma16
+}  // namespace vig

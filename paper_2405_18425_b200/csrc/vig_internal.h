@@ -79,6 +79,14 @@ template <typename T>
 cudaError_t launch_bigla_bwd(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, const T* d_out, T* dq, T* dk_out, T* dla_f,
                              T* dla_b, float* scratch, long long units, int L, int dk, int dv, cudaStream_t stream);
 
+// ---- the whole gradient of the bf16 forward pass on the tensor cores (head sizes of the paper's models, 16 tokens or more) ----
+bool grad_supported(long long units, int L, int dk, int dv);
+size_t grad_scratch_bytes(long long units, int L, int dk, int dv);   // 0: the call uses no scratch
+cudaError_t launch_bigla_grad(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v, const __nv_bfloat16* la_f,
+                              const __nv_bfloat16* la_b, const __nv_bfloat16* d_out, __nv_bfloat16* dq, __nv_bfloat16* dk_out,
+                              __nv_bfloat16* dv_out, __nv_bfloat16* dla_f, __nv_bfloat16* dla_b, void* scratch, long long units, int L, int dk,
+                              int dv, cudaStream_t stream);
+
 // Launch with programmatic stream serialization: the kernel's prologue (everything before its pdl_wait) may overlap
 // the tail of the kernel before it in the stream.
 template <typename... KArgs, typename... Args>

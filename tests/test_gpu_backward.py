@@ -155,3 +155,28 @@ def test_gradient_is_bitwise_reproducible(B, H, L, dk, dv):
             first = got
         for a, b in zip(first, got):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("dk,dv", [(16, 32), (24, 48), (32, 64), (32, 48)])
+@pytest.mark.parametrize("L", [16, 31, 32, 112, 127, 128, 129, 143, 144, 145, 208, 223, 224, 225, 256, 288, 289, 577])
+def test_bf16_gradient_chunk_edges(oracle, dk, dv, L):
+    """The tensor-core gradient at the edges of its tiles (16 tokens), of one chunk (128), of a pair of chunks (224) and of
+    the chunks of longer sequences (96)."""
+    cfg, x = random_problem(4500 + L, 2, 3, L, dk, dv, "bf16", gate_mean=0.5)
+    got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
+    _check(got, ref, "bf16")
+
+
+@pytest.mark.parametrize("L", [60, 100, 200, 400])
+@pytest.mark.parametrize("direction", ["g_fwd", "g_bwd"])
+def test_bf16_gradient_out_of_range_unit_per_form(oracle, L, direction):
+    """One unit with closed gates (log alpha = -40 over three tokens) in each form of the tensor-core gradient - one chunk,
+    a pair, chunks through scratch: that unit alone takes the recurrence, and every gradient meets the bar."""
+    cfg, x = random_problem(4600 + L, 2, 2, L, 24, 48, "bf16", gate_mean=1.0)
+    g = synth.stored_to_f64(x[direction], "bf16").copy()
+    g[1, 0, 20:23] = -640.0
+    x[direction] = synth.store(g, "bf16")
+    vig.vig_test_take_fallback_count()
+    got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
+    assert vig.vig_test_take_fallback_count() == 1
+    _check(got, ref, "bf16")
