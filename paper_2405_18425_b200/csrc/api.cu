@@ -139,9 +139,9 @@ static int fwd_bf16_impl(const void* q, const void* k, const void* v, const void
         }
         return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
     }
-    if (!recurrence_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
+    if (!scan_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
     if (empty) return VIG_OK;
-    cudaError_t e = launch_recurrence<bf>(q_, k_, v_, f_, b_, (bf*)out, units, L, dk, dv, stream);
+    cudaError_t e = launch_scan_fwd<bf>(q_, k_, v_, f_, b_, (bf*)out, units, L, dk, dv, false, stream);
     return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
 }
 
@@ -161,7 +161,7 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     if ((o_local != nullptr) != (z2d != nullptr)) return VIG_ERR_NULL_POINTER;
     if (o_local && (!aligned16(o_local) || !aligned16(z2d))) return VIG_ERR_MISALIGNED;
     if (!(tau > 0.f) || !std::isfinite(tau)) return VIG_ERR_BAD_DIM;
-    if (!tc_supported(dk, dv) && !recurrence_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
+    if (!tc_supported(dk, dv) && !scan_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
     if (empty) return VIG_OK;
     const long long units = (long long)B * H;
     using bf = __nv_bfloat16;
@@ -185,11 +185,9 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     return st;
 }
 
-static int fwd_f32_impl(const void* q, const void* k, const void* v, const void* la_f, const void* la_b, void* out,
-                        int B, int H, int L, int dk, int dv, cudaStream_t stream);
-
-// Gradient of the forward pass (Eq. 6) for d_out = dLoss/d_out.  Three steps in the stream: the gates shifted by one
-// token, the forward pass on (k, q, d_out) with them (= dv), the two recurrence walks for dq, dk and the gate gradients.
+// Gradient of the forward pass (Eq. 6) for d_out = dLoss/d_out.  The bf16 head sizes of the tensor-core kernels: one call
+// of those, from sixteen tokens on.  Everything else: the forward pass on (k, q, d_out) with the gates moved by one token
+// (= dv), then the recurrence walks for dq, dk and the gate gradients.
 template <typename T>
 static int bwd_impl(const void* q, const void* k, const void* v, const void* la_f, const void* la_b, const void* d_out, void* dq,
                     void* dk_out, void* dv_out, void* dla_f, void* dla_b, int B, int H, int L, int dk, int dv, cudaStream_t stream) {
@@ -199,36 +197,41 @@ static int bwd_impl(const void* q, const void* k, const void* v, const void* la_
     if (!dq || !dk_out || !dv_out || !dla_f || !dla_b) return VIG_ERR_NULL_POINTER;
     if (!aligned16(dq) || !aligned16(dk_out) || !aligned16(dv_out) || !aligned16(dla_f) || !aligned16(dla_b)) return VIG_ERR_MISALIGNED;
     if (!bwd_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
-    if (sizeof(T) == 2 ? !(tc_supported(dk, dv) || recurrence_supported(dk, dv)) : !recurrence_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
     if (empty) return VIG_OK;
     const long long units = (long long)B * H;
+    const T *q_ = (const T*)q, *k_ = (const T*)k, *v_ = (const T*)v, *f_ = (const T*)la_f, *b_ = (const T*)la_b, *g_ = (const T*)d_out;
+    bool tc = false;   // dv on the tensor-core forward kernel (bf16, fewer than sixteen tokens)
     if constexpr (sizeof(T) == 2) {
-        if (grad_supported(units, L, dk, dv) && kernel_preference() != VIG_TEST_KERNEL_SIMT) {
+        tc = tc_supported(dk, dv) && kernel_preference() != VIG_TEST_KERNEL_SIMT;
+        if (tc && grad_supported(units, L, dk, dv)) {
             const size_t need = grad_scratch_bytes(units, L, dk, dv);
             void* ws = nullptr;
             if (need > 0 && pool_alloc(&ws, need, stream) != cudaSuccess) return VIG_ERR_CUDA;
-            if (launch_bigla_grad((const T*)q, (const T*)k, (const T*)v, (const T*)la_f, (const T*)la_b, (const T*)d_out, (T*)dq, (T*)dk_out,
-                                  (T*)dv_out, (T*)dla_f, (T*)dla_b, ws, units, L, dk, dv, stream) != cudaSuccess)
+            if (launch_bigla_grad(q_, k_, v_, f_, b_, g_, (T*)dq, (T*)dk_out, (T*)dv_out, (T*)dla_f, (T*)dla_b, ws, units, L, dk, dv, stream) !=
+                cudaSuccess)
                 st = VIG_ERR_CUDA;
             if (need > 0 && cudaFreeAsync(ws, stream) != cudaSuccess && st == VIG_OK) st = VIG_ERR_CUDA;
             return st;
         }
     }
-    const size_t gate_bytes = ((size_t)units * L * dk * sizeof(T) + 255) / 256 * 256;
-    char* scratch = nullptr;
+    const size_t gate_bytes = tc ? ((size_t)units * L * dk * sizeof(T) + 255) / 256 * 256 : 0;
     const size_t walk_bytes = bwd_scratch_bytes(units, L, dk, dv);
     if (walk_bytes == 0) return VIG_ERR_CUDA;
+    char* scratch = nullptr;
     if (pool_alloc((void**)&scratch, 2 * gate_bytes + walk_bytes, stream) != cudaSuccess) return VIG_ERR_CUDA;
-    T *sf = (T*)scratch, *sb = (T*)(scratch + gate_bytes);
-    if (launch_shift_gates<T>((const T*)la_f, (const T*)la_b, sf, sb, units, L, dk, stream) != cudaSuccess) st = VIG_ERR_CUDA;
-    if (st == VIG_OK) {
-        if constexpr (sizeof(T) == 2) st = fwd_bf16_impl(k, q, d_out, sf, sb, dv_out, B, H, L, dk, dv, nullptr, 0, true, stream);
-        else st = fwd_f32_impl(k, q, d_out, sf, sb, dv_out, B, H, L, dk, dv, stream);
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(T) == 2) {
+        if (tc) {
+            T *sf = (T*)scratch, *sb = (T*)(scratch + gate_bytes);
+            e = launch_shift_gates<T>(f_, b_, sf, sb, units, L, dk, stream);
+            if (e == cudaSuccess) st = fwd_bf16_impl(k, q, d_out, sf, sb, dv_out, B, H, L, dk, dv, nullptr, 0, true, stream);
+        }
     }
-    if (st == VIG_OK && launch_bigla_bwd<T>((const T*)q, (const T*)k, (const T*)v, (const T*)la_f, (const T*)la_b, (const T*)d_out, (T*)dq,
-                                            (T*)dk_out, (T*)dla_f, (T*)dla_b, (float*)(scratch + 2 * gate_bytes), units, L, dk, dv,
-                                            stream) != cudaSuccess)
-        st = VIG_ERR_CUDA;
+    if (!tc) e = launch_scan_fwd<T>(k_, q_, g_, f_, b_, (T*)dv_out, units, L, dk, dv, true, stream);
+    if (e == cudaSuccess && st == VIG_OK)
+        e = launch_bigla_bwd<T>(q_, k_, v_, f_, b_, g_, (T*)dq, (T*)dk_out, (T*)dla_f, (T*)dla_b, (float*)(scratch + 2 * gate_bytes), units, L, dk, dv,
+                                stream);
+    if (e != cudaSuccess) st = VIG_ERR_CUDA;
     if (cudaFreeAsync(scratch, stream) != cudaSuccess && st == VIG_OK) st = VIG_ERR_CUDA;
     return st;
 }
@@ -257,10 +260,10 @@ static int fwd_f32_impl(const void* q, const void* k, const void* v, const void*
     bool empty;
     int st = check_fwd_args(q, k, v, la_f, la_b, out, B, H, L, dk, dv, &empty);
     if (st != VIG_OK) return st;
-    if (!recurrence_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
+    if (!scan_supported(dk, dv)) return VIG_ERR_UNSUPPORTED;
     if (empty) return VIG_OK;
-    cudaError_t e = launch_recurrence<float>((const float*)q, (const float*)k, (const float*)v, (const float*)la_f,
-                                             (const float*)la_b, (float*)out, (long long)B * H, L, dk, dv, stream);
+    cudaError_t e = launch_scan_fwd<float>((const float*)q, (const float*)k, (const float*)v, (const float*)la_f,
+                                           (const float*)la_b, (float*)out, (long long)B * H, L, dk, dv, false, stream);
     return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
 }
 
@@ -429,7 +432,7 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
     if (!q || !k || !v || !g_fwd || !g_bwd || !out) return VIG_ERR_NULL_POINTER;
     if (B < 0 || H < 0 || L < 0 || dk < 1 || dv < 1 || !(tau > 0.f) || !std::isfinite(tau)) return VIG_ERR_BAD_DIM;
     if (dtype != VIG_DTYPE_F32 && dtype != VIG_DTYPE_BF16) return VIG_ERR_UNSUPPORTED;
-    if (dtype == VIG_DTYPE_F32 ? !recurrence_supported(dk, dv) : !(tc_supported(dk, dv) || recurrence_supported(dk, dv)))
+    if (dtype == VIG_DTYPE_F32 ? !scan_supported(dk, dv) : !(tc_supported(dk, dv) || scan_supported(dk, dv)))
         return VIG_ERR_UNSUPPORTED;
     if ((long long)B * H > 0x7fffffffLL) return VIG_ERR_UNSUPPORTED;
     if (B == 0 || H == 0 || L == 0) return VIG_OK;

@@ -12,12 +12,13 @@
 // (element-wise) and E<_t likewise:   dlog alpha>_t = sum_{m >= t} E>_m,   dlog alpha<_t = sum_{m <= t} E<_m
 // = - sum_{m > t} E<_m  (each direction is unchanged by q -> q / c, k -> c k per key dimension, so sum_m E_m = 0).
 //
-// One block per unit walks the sequence twice.  The ascending walk carries S> and Z< and leaves dq>_t, dk<_t in fp32
+// A block walks one segment of one unit twice.  The ascending walk carries S> and Z< and leaves dq>_t, dk<_t in fp32
 // scratch; the descending walk carries S< and Z>, reads them back and finishes all four outputs, the gate gradients as
 // running sums in walking order.  Thread (i, cg) keeps columns [cg CN, cg CN + CN) of row i of both dk x dv matrices in
 // registers; the sums over the value dimension are finished over the two or four lanes of a row by shuffles.  Inputs and
 // outputs pass through shared memory sixteen tokens at a time: asynchronous copies (cp.async) bring the next sixteen
 // tokens in while the block works on these, where a token's row is a whole number of 16-byte pieces.
+// Few units and long sequences only (see the plan below); everything else walks its segments within one block.
 #include <atomic>
 #include <cstring>
 
@@ -35,11 +36,11 @@ template <typename T>
 struct BwdArgs {
     const T *q, *k, *v, *la_f, *la_b, *g;
     T *dq, *dkey, *dla_f, *dla_b;
-    float* scratch;   // [units][L][dk][2] fp32: (dq>, dk<) between the two walks (then the local gate sums of a segmented call)
-    // Segmented call (few units, long sequences): a block walks one segment of seg_len tokens.  states: [units][nseg][4]
+    float* scratch;   // [units][L][dk][2] fp32: (dq>, dk<) between the two walks, then the segment's own gate sums
+    // states: [units][nseg][4]
     // [dk][CG CN] fp32 - S>, Z<, S<, Z> of a segment run from zero, replaced by the states entering the segment; decay:
     // [units][nseg][4][dk] - the products of the gates over the segment; totals: [units][nseg][2][dk] - the segment's sums of
-    // E> and E<.  All NULL / nseg = 1 for the call that walks whole units.
+    // E> and E<.
     float *states, *decay, *totals;
     long long units;
     int L, dk, dv, nseg, seg_len;
@@ -81,22 +82,16 @@ __device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src)
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem_dst)), "l"(gmem_src) : "memory");
 }
 
-// Block shapes known at compile time are held to 85 registers (768 threads per SM: six blocks of 128).
-constexpr int bwd_max_threads(int rows, int cg) { return rows > 0 ? rows * cg : 512; }
-constexpr int bwd_min_blocks(int rows, int cg) { return rows > 0 ? 768 / (rows * cg) : 1; }
-
-// CG: threads (adjacent lanes) per state row, 2 or 4.  CN: columns of the state per thread (a multiple of 4).  ROWS: state
-// rows of the block (threads / CG) when known at compile time - every shared-memory offset is then an immediate - or 0
-// for any block size.
-// SUMMARY: the first launch of a segmented call - the four states of every segment run from zero and the products of their
+// CG: threads (adjacent lanes) per state row, 2 or 4.  CN: columns of the state per thread (a multiple of 4).
+// SUMMARY: the first launch of a call - the four states of every segment run from zero and the products of their
 // gates (state updates only, nothing else is read or written).
-template <typename T, int CN, int ROWS, int CG, bool SUMMARY>
-__global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS, CG)) bigla_bwd_kernel(BwdArgs<T> a) {
+template <typename T, int CN, int CG, bool SUMMARY>
+__global__ void __launch_bounds__(512) bigla_bwd_kernel(BwdArgs<T> a) {
     constexpr int kBwdCG = CG;
     static_assert(CN % 4 == 0, "columns per thread come in 16-byte pieces");
     extern __shared__ __align__(16) float bw_smem[];
-    const int tid = threadIdx.x, nt = ROWS ? ROWS * kBwdCG : blockDim.x;
-    const int rows = ROWS ? ROWS : nt / kBwdCG;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int rows = nt / kBwdCG;
     constexpr int cols = kBwdCG * (CN + 4);   // a token's row of v / d_out: CG groups of CN (+ 4 unused) floats
     const int i = tid / kBwdCG, cg = tid % kBwdCG;
     const int L = a.L, dk = a.dk, dv = a.dv;
@@ -112,18 +107,11 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
     T* raw_v = raw_z + kBwdTT * dk;
     T* raw_g = raw_v + kBwdTT * dv;
     float2* raw_x = reinterpret_cast<float2*>(raw_g + kBwdTT * dv);
-    // The instances for the paper's head sizes (bf16, dv = CG CN exactly, whole 16-byte rows) read v and d_out in the walk
-    // straight from the landing zone, as bf16: half the shared-memory traffic of the walk, which is what bounds it.  The
-    // landing zone of v and d_out then has a second buffer (in place of the fp32 staging of the two).
-    constexpr bool kVG16 = ROWS != 0 && sizeof(T) == 2;
-    T* raw_v1 = reinterpret_cast<T*>(vs);
-    T* raw_g1 = raw_v1 + kBwdTT * dv;
     // Rows of whole 16-byte pieces: the next sixteen tokens are copied asynchronously while these are worked on.
     const bool ahead = (dk * sizeof(T)) % 16 == 0 && (dv * sizeof(T)) % 16 == 0;
     for (size_t x = tid; x < bwd_stage_floats(rows, CN, CG); x += nt) bw_smem[x] = 0.f;   // the padding stays zero
     __syncthreads();
     const int st_r = tid % rows, st_t = tid / rows;   // staging: thread = one key dimension of every fourth token
-    const bool segmented = a.states != nullptr;
 
     for (long long w = blockIdx.x; w < a.units * a.nseg; w += gridDim.x) {
         const long long unit = w / a.nseg;
@@ -141,7 +129,7 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
             float run_f = 0.f, run_b = 0.f;   // running sums of E> and E< (descending walk)
             float prod_s = 1.f, prod_z = 1.f;   // SUMMARY: products of the gates of S and of Z over the segment
             const size_t st_base = ((size_t)w * 4 + (walk == 0 ? 0 : 2)) * dk;   // kinds: S> 0, Z< 1, S< 2, Z> 3
-            if (!SUMMARY && segmented && i < dk) {   // the states that enter this segment
+            if (!SUMMARY && i < dk) {   // the states that enter this segment
                 const float* ps = a.states + (st_base + i) * (CG * CN) + cg * CN;
                 const float* pz = ps + (size_t)dk * (CG * CN);
 #pragma unroll
@@ -168,8 +156,8 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                 }
                 const char* gv = reinterpret_cast<const char*>(a.v + ov + (size_t)t0 * dv);
                 const char* gg = reinterpret_cast<const char*>(a.g + ov + (size_t)t0 * dv);
-                char* dv_ = reinterpret_cast<char*>(kVG16 && (cc & 1) ? raw_v1 : raw_v);
-                char* dg_ = reinterpret_cast<char*>(kVG16 && (cc & 1) ? raw_g1 : raw_g);
+                char* dv_ = reinterpret_cast<char*>(raw_v);
+                char* dg_ = reinterpret_cast<char*>(raw_g);
                 for (int x = tid; x < pv; x += nt) {
                     cp_async16(dv_ + 16 * x, gv + 16 * x);
                     cp_async16(dg_ + 16 * x, gg + 16 * x);
@@ -225,7 +213,7 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                         xo[1] = xb;
                     }
                 }
-                for (int x = tid; x < (kVG16 ? 0 : nv * qv); x += nt) {   // (kVG16: v and d_out stay where they landed)
+                for (int x = tid; x < nv * qv; x += nt) {
                     const int tt = x / qv, j0 = (x - tt * qv) * 4;
                     const int at = tt * cols + (j0 / CN) * (CN + 4) + j0 % CN;
                     float f[4];
@@ -258,23 +246,15 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                     float4* op = rowd + (walk == 0 ? 0 : nv - 1) * rows + i;   // the record is replaced by the results (the lanes of a
                                                                                 // row read it in the same instruction, before this lane writes)
                     const int first = walk == 0 ? 0 : nv - 1;
-                    // this thread's columns of v and d_out, token by token: fp32 staging, or (kVG16) the bf16 rows as they landed
-                    const char* vp = kVG16 ? reinterpret_cast<const char*>(((cc & 1) ? raw_v1 : raw_v) + first * dv + cg * CN)
-                                           : reinterpret_cast<const char*>(vs + first * cols + cg * (CN + 4));
-                    const char* gp = kVG16 ? reinterpret_cast<const char*>(((cc & 1) ? raw_g1 : raw_g) + first * dv + cg * CN)
-                                           : reinterpret_cast<const char*>(gs + first * cols + cg * (CN + 4));
-                    const int srow = step * rows, scol = step * (kVG16 ? dv * 2 : cols * 4);   // bytes per token
+                    // this thread's columns of v and d_out, token by token
+                    const char* vp = reinterpret_cast<const char*>(vs + first * cols + cg * (CN + 4));
+                    const char* gp = reinterpret_cast<const char*>(gs + first * cols + cg * (CN + 4));
+                    const int srow = step * rows, scol = step * cols * 4;   // scol: bytes per token
                     // four columns (two fp32 pairs) number c4 of the row at p
                     auto quad = [&](const char* p, int c4, f32x2& lo, f32x2& hi) {
-                        if constexpr (kVG16) {
-                            const uint2 wv = reinterpret_cast<const uint2*>(p)[c4];   // a bf16 is the upper half of its fp32
-                            lo = pack2(__uint_as_float(wv.x << 16), __uint_as_float(wv.x & 0xffff0000u));
-                            hi = pack2(__uint_as_float(wv.y << 16), __uint_as_float(wv.y & 0xffff0000u));
-                        } else {
-                            const ulonglong2 q2 = reinterpret_cast<const ulonglong2*>(p)[c4];
-                            lo = q2.x;
-                            hi = q2.y;
-                        }
+                        const ulonglong2 q2 = reinterpret_cast<const ulonglong2*>(p)[c4];
+                        lo = q2.x;
+                        hi = q2.y;
                     };
 #pragma unroll 4
                     for (int n = 0; n < nv; ++n, rp += srow, xp += srow, op += srow, vp += scol, gp += scol) {
@@ -353,14 +333,9 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                         } else {
                             store4(a.dq + ok + gi, o[0]);
                             store4(a.dkey + ok + gi, o[1]);
-                            if (segmented) {   // the gate sums of this segment alone, in fp32 over the consumed pairs
-                                float4* so = reinterpret_cast<float4*>(sc + gi);
-                                so[0] = make_float4(o[2][0], o[3][0], o[2][1], o[3][1]);
-                                so[1] = make_float4(o[2][2], o[3][2], o[2][3], o[3][3]);
-                            } else {
-                                store4(a.dla_f + ok + gi, o[2]);
-                                store4(a.dla_b + ok + gi, o[3]);
-                            }
+                            float4* so = reinterpret_cast<float4*>(sc + gi);   // the gate sums of this segment alone, in fp32 over the consumed pairs
+                            so[0] = make_float4(o[2][0], o[3][0], o[2][1], o[3][1]);
+                            so[1] = make_float4(o[2][2], o[3][2], o[2][3], o[3][3]);
                         }
                     }
                 } else if (st_r < dk) {
@@ -372,12 +347,7 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                         } else {
                             rec_store(a.dq + ok + gi, o4.x);
                             rec_store(a.dkey + ok + gi, o4.y);
-                            if (segmented) {
-                                sc[gi] = make_float2(o4.z, o4.w);
-                            } else {
-                                rec_store(a.dla_f + ok + gi, o4.z);
-                                rec_store(a.dla_b + ok + gi, o4.w);
-                            }
+                            sc[gi] = make_float2(o4.z, o4.w);
                         }
                     }
                 }
@@ -395,7 +365,7 @@ __global__ void __launch_bounds__(bwd_max_threads(ROWS, CG), bwd_min_blocks(ROWS
                     a.decay[st_base + dk + i] = prod_z;
                 }
             }
-            if (!SUMMARY && segmented && walk == 1 && cg == 0 && i < dk) {
+            if (!SUMMARY && walk == 1 && cg == 0 && i < dk) {
                 a.totals[((size_t)w * 2) * dk + i] = run_f;
                 a.totals[((size_t)w * 2 + 1) * dk + i] = run_b;
             }
@@ -471,7 +441,7 @@ __global__ void __launch_bounds__(256) shift_gates_kernel(const V* __restrict__ 
     }
 }
 
-template <typename T, int CN, int ROWS, int CG, bool SUMMARY>
+template <typename T, int CN, int CG, bool SUMMARY>
 cudaError_t launch_bwd_kernel(const BwdArgs<T>& a, int threads, int sms, cudaStream_t stream) {
     const size_t smem = bwd_smem_bytes(threads / CG, CN, CG, a.dk, a.dv, sizeof(T));
     static std::atomic<bool> configured[64];
@@ -480,24 +450,23 @@ cudaError_t launch_bwd_kernel(const BwdArgs<T>& a, int threads, int sms, cudaStr
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!configured[dev].load(std::memory_order_acquire)) {
-        if ((e = cudaFuncSetAttribute(bigla_bwd_kernel<T, CN, ROWS, CG, SUMMARY>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) !=
+        if ((e = cudaFuncSetAttribute(bigla_bwd_kernel<T, CN, CG, SUMMARY>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)) !=
             cudaSuccess)
             return e;
         configured[dev].store(true, std::memory_order_release);
     }
     const long long work = a.units * a.nseg;
     long long grid = work < 32LL * sms ? work : 32LL * sms;
-    bigla_bwd_kernel<T, CN, ROWS, CG, SUMMARY><<<(unsigned)grid, threads, smem, stream>>>(a);
+    bigla_bwd_kernel<T, CN, CG, SUMMARY><<<(unsigned)grid, threads, smem, stream>>>(a);
     count_launch();
     return cudaGetLastError();
 }
 
-// The walks of a call: one launch over whole units, or - segmented - the segments' own states, the fold that turns them
-// into the states entering each segment, the walks proper from those states, and the gate gradients put together.
-template <typename T, int CN, int ROWS, int CG>
+// The walks of a call: the segments' own states, the fold that turns them into the states entering each segment, the walks
+// proper from those states, and the gate gradients put together.
+template <typename T, int CN, int CG>
 cudaError_t launch_bwd_t(const BwdArgs<T>& a, int threads, int sms, cudaStream_t stream) {
-    if (a.nseg == 1) return launch_bwd_kernel<T, CN, ROWS, CG, false>(a, threads, sms, stream);
-    cudaError_t e = launch_bwd_kernel<T, CN, ROWS, CG, true>(a, threads, sms, stream);
+    cudaError_t e = launch_bwd_kernel<T, CN, CG, true>(a, threads, sms, stream);
     if (e != cudaSuccess) return e;
     const int cols = CG * CN;
     const long long n = a.units * a.dk * (cols / 4);
@@ -506,7 +475,7 @@ cudaError_t launch_bwd_t(const BwdArgs<T>& a, int threads, int sms, cudaStream_t
     bwd_fold_kernel<<<(unsigned)blocks, 256, 0, stream>>>(a.states, a.decay, a.units, a.nseg, a.dk, cols);
     count_launch();
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = launch_bwd_kernel<T, CN, ROWS, CG, false>(a, threads, sms, stream)) != cudaSuccess) return e;
+    if ((e = launch_bwd_kernel<T, CN, CG, false>(a, threads, sms, stream)) != cudaSuccess) return e;
     bwd_finish_kernel<T><<<(unsigned)(a.units * a.nseg), 256, 2 * a.dk * sizeof(float), stream>>>(
         reinterpret_cast<const float2*>(a.scratch), a.totals, a.dla_f, a.dla_b, a.L, a.dk, a.nseg, a.seg_len);
     count_launch();
@@ -524,15 +493,16 @@ int bwd_cn(int dv, int cg) {   // columns per thread: the instantiated size that
     return cn <= 8 ? 8 : (cn <= 12 ? 12 : (cn <= 16 ? 16 : (cn <= 24 ? 24 : 32)));
 }
 
-// Few units and long sequences: the sequence is cut into segments so that about five blocks per SM walk at once (a lone
-// block per SM needs about 550 cycles per token).  Segments are multiples of the staging group and at least 64 tokens.
-void bwd_plan(long long units, int L, int sms, int* nseg, int* seg_len) {
+// Segments in blocks of their own (nseg > 1), where the walks within one block per unit and eight key dimensions would
+// leave most of the chip idle: few units and long sequences (12 units of 784 tokens, fp32: 157 us a call against 210, 16
+// units of 4096 tokens 672 against 1187; at 196 tokens the walks within a block take 45 us against 100).  About five blocks per SM (a lone block per SM needs about 550
+// cycles per token); segments are multiples of the staging group and at least 64 tokens.
+void bwd_plan(long long units, int L, int dk, int sms, int* nseg, int* seg_len) {
     *nseg = 1;
     *seg_len = L > 0 ? L : 1;
-    if (units >= 2LL * sms || L < 128) return;
+    if (L < 512 || units * ((dk + 7) / 8) * 8 >= 4LL * sms) return;
     long long want = (5LL * sms + units - 1) / units;
     if (want > L / 64) want = L / 64;
-    if (want < 2) return;
     const int len = (int)(((L + want - 1) / want + kBwdTT - 1) / kBwdTT * kBwdTT);
     *seg_len = len;
     *nseg = (L + len - 1) / len;
@@ -565,7 +535,7 @@ static void bwd_scratch_layout(long long units, int L, int dk, int dv, int nseg,
 size_t bwd_scratch_bytes(long long units, int L, int dk, int dv) {
     int sms = 0, nseg, seg_len;
     if (sm_count_of_device(&sms) != cudaSuccess) return 0;
-    bwd_plan(units, L, sms, &nseg, &seg_len);
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
     size_t p, st, de, to;
     bwd_scratch_layout(units, L, dk, dv, nseg, &p, &st, &de, &to);
     return (p + st + de + to) * sizeof(float);
@@ -592,22 +562,18 @@ cudaError_t launch_bigla_bwd(const T* q, const T* k, const T* v, const T* la_f, 
     int sms = 0, nseg, seg_len;
     cudaError_t e = sm_count_of_device(&sms);
     if (e != cudaSuccess) return e;
-    bwd_plan(units, L, sms, &nseg, &seg_len);
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
+    if (nseg == 1) return launch_scan_bwd<T>(q, k, v, la_f, la_b, d_out, dq, dk_out, dla_f, dla_b, scratch, units, L, dk, dv, stream);
     size_t p, st, de, to;
     bwd_scratch_layout(units, L, dk, dv, nseg, &p, &st, &de, &to);
     BwdArgs<T> a{q, k, v, la_f, la_b, d_out, dq, dk_out, dla_f, dla_b, scratch,
-                 nseg > 1 ? scratch + p : nullptr, nseg > 1 ? scratch + p + st : nullptr, nseg > 1 ? scratch + p + st + de : nullptr,
+                 scratch + p, scratch + p + st, scratch + p + st + de,
                  units, L, dk, dv, nseg, seg_len};
-    const int cg = bwd_cg(dv), threads = bwd_threads(dk, cg), cn = bwd_cn(dv, cg), rows = threads / cg;
-#define VIG_BWD_CASE(CN_, ROWS_, CG_) \
-    if (cn == CN_ && cg == CG_ && (ROWS_ == 0 || (dk == ROWS_ && dv == CG_ * CN_))) return launch_bwd_t<T, CN_, ROWS_, CG_>(a, threads, sms, stream);
-    if constexpr (sizeof(T) == 2) {   // the head sizes of the paper's models: block shape known at compile time
-        VIG_BWD_CASE(8, 16, 4) VIG_BWD_CASE(8, 24, 4) VIG_BWD_CASE(8, 32, 4)        // dv = 32; dk = 16, 24, 32
-        VIG_BWD_CASE(12, 16, 4) VIG_BWD_CASE(12, 24, 4) VIG_BWD_CASE(12, 32, 4)     // dv = 48
-        VIG_BWD_CASE(16, 16, 4) VIG_BWD_CASE(16, 24, 4) VIG_BWD_CASE(16, 32, 4)     // dv = 64
-    }
-    VIG_BWD_CASE(8, 0, 2) VIG_BWD_CASE(12, 0, 2) VIG_BWD_CASE(16, 0, 2)             // dv < 32
-    VIG_BWD_CASE(8, 0, 4) VIG_BWD_CASE(12, 0, 4) VIG_BWD_CASE(16, 0, 4) VIG_BWD_CASE(24, 0, 4) VIG_BWD_CASE(32, 0, 4)
+    const int cg = bwd_cg(dv), threads = bwd_threads(dk, cg), cn = bwd_cn(dv, cg);
+#define VIG_BWD_CASE(CN_, CG_) \
+    if (cn == CN_ && cg == CG_) return launch_bwd_t<T, CN_, CG_>(a, threads, sms, stream);
+    VIG_BWD_CASE(8, 2) VIG_BWD_CASE(12, 2) VIG_BWD_CASE(16, 2)             // dv < 32
+    VIG_BWD_CASE(8, 4) VIG_BWD_CASE(12, 4) VIG_BWD_CASE(16, 4) VIG_BWD_CASE(24, 4) VIG_BWD_CASE(32, 4)
 #undef VIG_BWD_CASE
     return cudaErrorInvalidValue;
 }

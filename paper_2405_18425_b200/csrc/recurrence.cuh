@@ -35,6 +35,32 @@ __device__ __forceinline__ float rec_to_float(__nv_bfloat16 x) { return __bfloat
 __device__ __forceinline__ void rec_store(float* p, float x) { *p = x; }
 __device__ __forceinline__ void rec_store(__nv_bfloat16* p, float x) { *p = __float2bfloat16_rn(x); }
 
+// Four consecutive elements of a row in registers, as loaded; the first n of them exist, the others read as zero.  VEC: rows
+// are whole pieces, one load.
+template <typename T, bool VEC>
+struct Piece {
+    T e[4];
+    __device__ __forceinline__ void load(const T* p, int n) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x) e[x] = x < n ? p[x] : T(0.f);
+    }
+    __device__ __forceinline__ float4 get() const { return make_float4(rec_to_float(e[0]), rec_to_float(e[1]), rec_to_float(e[2]), rec_to_float(e[3])); }
+};
+template <>
+struct Piece<float, true> {
+    float4 e;
+    __device__ __forceinline__ void load(const float* p, int n) { e = n > 0 ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f); }
+    __device__ __forceinline__ float4 get() const { return e; }
+};
+template <>
+struct Piece<__nv_bfloat16, true> {
+    uint2 e;
+    __device__ __forceinline__ void load(const __nv_bfloat16* p, int n) { e = n > 0 ? *reinterpret_cast<const uint2*>(p) : make_uint2(0u, 0u); }
+    __device__ __forceinline__ float4 get() const {   // a bf16 is the upper half of its fp32
+        return make_float4(__uint_as_float(e.x << 16), __uint_as_float(e.x & 0xffff0000u), __uint_as_float(e.y << 16), __uint_as_float(e.y & 0xffff0000u));
+    }
+};
+
 // All threads of the block must call this (it uses __syncthreads).  q, k, la_f, la_b: [L, dk];
 // v, out: [L, dv] of this unit (global or shared memory); ws: rec_plan(...).smem_floats floats of
 // shared memory.  The forward pass stores o> in `out` (rounded to T), the backward pass turns it

@@ -17,11 +17,18 @@ int* device_status_ptr();            // device address of the status word of the
 int take_expire_next_wait();         // test hook: 1 once after vig_test_expire_next_wait(), else 0
 void count_launch(unsigned n = 1);   // bumps the process-wide launch counter
 
-// ---- fp32 SIMT recurrence (Eq. 6 evaluated step by step), any dk <= 128, dv <= 256 ----
-bool recurrence_supported(int dk, int dv);
+// ---- Eq. 6 step by step in fp32 on the CUDA cores, any dk <= 128, dv <= 256.  adjoint: with the gates of the two directions
+// exchanged and moved by one token, so that on (k, q, d_out) the result is the gradient with respect to v:
+//   dv_r = 1/2 sum_{t >= r} (k_r * prod_{m = r+1..t} alpha>_m . q_t) g_t + 1/2 sum_{t <= r} (k_r * prod_{m = t..r-1} alpha<_m . q_t) g_t ----
+bool scan_supported(int dk, int dv);
 template <typename T>
-cudaError_t launch_recurrence(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, T* out,
-                              long long units, int L, int dk, int dv, cudaStream_t stream);
+cudaError_t launch_scan_fwd(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, T* out, long long units, int L, int dk, int dv,
+                            bool adjoint, cudaStream_t stream);
+// Its gradient with respect to q, k and the log gates, segments of a sequence walked side by side within a block; scratch:
+// [units][L][dk] pairs of floats.
+template <typename T>
+cudaError_t launch_scan_bwd(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, const T* d_out, T* dq, T* dk_out, T* dla_f, T* dla_b,
+                            void* scratch, long long units, int L, int dk, int dv, cudaStream_t stream);
 
 // ---- gate preparation ----
 template <typename T>
@@ -69,8 +76,9 @@ cudaError_t launch_bigla_umma_long(const __nv_bfloat16* q, const __nv_bfloat16* 
                                    const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out,
                                    long long units, int L, int dk, int dv, void* ws, cudaStream_t stream);
 
-// ---- gradient of the forward pass with respect to q, k and the log gates (fp32 recurrences on the CUDA cores); the
-// gradient with respect to v is the forward pass on (k, q, d_out) with the gates from launch_shift_gates ----
+// ---- gradient of the forward pass with respect to q, k and the log gates (fp32 recurrences on the CUDA cores):
+// launch_scan_bwd, or walks over segments in several launches.  The gates of dv's forward pass on (k, q, d_out), moved by
+// one token: launch_shift_gates ----
 bool bwd_supported(int dk, int dv);
 size_t bwd_scratch_bytes(long long units, int L, int dk, int dv);   // 0: the device could not be queried
 template <typename T>

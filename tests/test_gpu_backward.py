@@ -180,3 +180,22 @@ def test_bf16_gradient_out_of_range_unit_per_form(oracle, L, direction):
     got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
     assert vig.vig_test_take_fallback_count() == 1
     _check(got, ref, "bf16")
+
+
+@pytest.mark.parametrize("units,L", [(1, 1), (2, 5), (1, 9), (3, 63), (48, 196), (700, 37), (1, 511), (1, 512), (2, 1030)])
+@pytest.mark.parametrize("dk,dv", [(32, 64), (24, 48), (13, 31), (70, 100)])
+def test_f32_walks_in_segments(oracle, units, L, dk, dv):
+    """fp32 forward and gradient where the walks change form: one segment, a ragged last one, eight of them, units enough to
+    walk whole sequences, segments in blocks of their own (512 tokens and more); rows of whole pieces and odd ones."""
+    if units * L * dk > 40000 * 32:
+        dk, dv = min(dk, 32), min(dv, 64)
+    cfg, x = random_problem(4700 + L, units, 1, L, dk, dv, "f32", gate_mean=0.5)
+    got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
+    _check(got, ref, "f32")
+    la = [oracle_log_alpha(oracle, x[n], "f32", cfg.tau) for n in ("g_fwd", "g_bwd")]
+    d = [to_device(a, "f32") for a in (x["q"], x["k"], x["v"], *la)]
+    out = torch.full_like(d[2], float("nan"))
+    vig.vig_bigla_fwd_f32(*d, out)
+    torch.cuda.synchronize()
+    f = lambda a: synth.stored_to_f64(a, "f32")
+    assert rel_err(device_to_f64(out, "f32"), oracle.bigla_fwd(f(x["q"]), f(x["k"]), f(x["v"]), f(la[0]), f(la[1]), nthreads=4)) <= TOL["f32"]
