@@ -302,8 +302,8 @@ static int gate_prep_bwd_impl(const void* g_f, const void* g_b, const void* d_f,
     return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
 }
 
-// ---- host-buffer path: per device, two copy streams and the events that order them with the caller's stream -------
-constexpr int kHostSlices = 4;
+// ---- host-buffer path: per device, the copy streams and the events that order them with the caller's stream -------
+constexpr int kHostSlices = 3;
 struct HostPath {
     std::mutex mu;
     cudaStream_t s_in = nullptr, s_out = nullptr;
@@ -448,40 +448,71 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
     if (pool_alloc((void**)&base, 4 * nk + 2 * nv, stream) != cudaSuccess) return VIG_ERR_CUDA;
     char *dq = base, *dk_ = base + nk, *dgf = base + 2 * nk, *dgb = base + 3 * nk, *dv_ = base + 4 * nk,
          *dout = base + 4 * nk + nv;
-    // Slices of whole units: the copy of slice i + 1 to the device, the kernels of slice i and the copy of slice i - 1
-    // back run at the same time (the host link carries both directions at once).  A slice offset must keep the 16-byte
-    // alignment of the device pointers: unit sizes are multiples of 16 bytes whenever dk and dv are multiples of
-    // 8 (bf16) or 4 (fp32); otherwise the call runs as one slice.
-    int nsl = (unit_k % 16 == 0 && unit_v % 16 == 0 && units * (4 * unit_k + 2 * unit_v) >= (4u << 20)) ? kHostSlices : 1;
-    if (nsl > units) nsl = (int)units;
-    int st = VIG_OK;
-    bool ok = cudaEventRecord(hp->ev_start, stream) == cudaSuccess &&
-              cudaStreamWaitEvent(hp->s_in, hp->ev_start, 0) == cudaSuccess &&
-              cudaStreamWaitEvent(hp->s_out, hp->ev_start, 0) == cudaSuccess;
-    for (int i = 0; ok && i < nsl && st == VIG_OK; ++i) {
-        const long long u0 = units * i / nsl, u1 = units * (i + 1) / nsl, nu = u1 - u0;
-        const size_t ok_ = (size_t)u0 * unit_k, ov = (size_t)u0 * unit_v;
-        ok = cudaMemcpyAsync(dgf + ok_, (const char*)g_fwd + ok_, nu * unit_k, cudaMemcpyHostToDevice, hp->s_in) == cudaSuccess &&
-             cudaMemcpyAsync(dgb + ok_, (const char*)g_bwd + ok_, nu * unit_k, cudaMemcpyHostToDevice, hp->s_in) == cudaSuccess &&
-             cudaMemcpyAsync(dq + ok_, (const char*)q + ok_, nu * unit_k, cudaMemcpyHostToDevice, hp->s_in) == cudaSuccess &&
-             cudaMemcpyAsync(dk_ + ok_, (const char*)k + ok_, nu * unit_k, cudaMemcpyHostToDevice, hp->s_in) == cudaSuccess &&
-             cudaMemcpyAsync(dv_ + ov, (const char*)v + ov, nu * unit_v, cudaMemcpyHostToDevice, hp->s_in) == cudaSuccess &&
-             cudaEventRecord(hp->ev_in[i], hp->s_in) == cudaSuccess && cudaStreamWaitEvent(stream, hp->ev_in[i], 0) == cudaSuccess;
-        if (!ok) break;
+    auto kernels = [&](size_t ok_, size_t ov, int nu) {
         if (dtype == VIG_DTYPE_F32) {
-            st = vig_gate_prep_f32(dgf + ok_, dgb + ok_, dgf + ok_, dgb + ok_, (int)nu, 1, L, dk, tau, stream_);
-            if (st == VIG_OK) st = vig_bigla_fwd_f32(dq + ok_, dk_ + ok_, dv_ + ov, dgf + ok_, dgb + ok_, dout + ov, (int)nu, 1, L, dk, dv, stream_);
-        } else {
-            st = vig_bigla_fwd_gates_bf16(dq + ok_, dk_ + ok_, dv_ + ov, dgf + ok_, dgb + ok_, dout + ov, (int)nu, 1, L, dk, dv, tau, stream_);
+            const int r = vig_gate_prep_f32(dgf + ok_, dgb + ok_, dgf + ok_, dgb + ok_, nu, 1, L, dk, tau, stream_);
+            return r != VIG_OK ? r : vig_bigla_fwd_f32(dq + ok_, dk_ + ok_, dv_ + ov, dgf + ok_, dgb + ok_, dout + ov, nu, 1, L, dk, dv, stream_);
         }
-        if (st != VIG_OK) break;
-        ok = cudaEventRecord(hp->ev_k[i], stream) == cudaSuccess && cudaStreamWaitEvent(hp->s_out, hp->ev_k[i], 0) == cudaSuccess &&
-             cudaMemcpyAsync((char*)out + ov, dout + ov, nu * unit_v, cudaMemcpyDeviceToHost, hp->s_out) == cudaSuccess;
+        return vig_bigla_fwd_gates_bf16(dq + ok_, dk_ + ok_, dv_ + ov, dgf + ok_, dgb + ok_, dout + ov, nu, 1, L, dk, dv, tau, stream_);
+    };
+    // A unit's bytes are multiples of 16 whenever dk and dv are multiples of 8 (bf16) or 4 (fp32).
+    const size_t in_bytes = units * (4 * unit_k + unit_v), out_bytes = units * unit_v;
+    const bool whole = unit_k % 16 == 0 && unit_v % 16 == 0;
+    // The way back by a kernel, beside the copies to the device; the way in by a kernel as well where the fixed cost of five
+    // engine copies (20 us more) outweighs the engine's higher rate (7 %).  Pageable memory takes the engines.
+    const bool out_kernel = whole && host_copy_usable(out, out_bytes);
+    const bool in_kernel = out_kernel && in_bytes <= (8u << 20) && host_copy_usable(q, 16) && host_copy_usable(k, 16) && host_copy_usable(v, 16) &&
+                           host_copy_usable(g_fwd, 16) && host_copy_usable(g_bwd, 16);
+    auto copy_in = [&](size_t ok_, size_t ov, size_t nbk, size_t nbv, cudaStream_t s) {
+        const HostCopy c[5] = {{(const char*)g_fwd + ok_, dgf + ok_, nbk},
+                               {(const char*)g_bwd + ok_, dgb + ok_, nbk},
+                               {(const char*)q + ok_, dq + ok_, nbk},
+                               {(const char*)k + ok_, dk_ + ok_, nbk},
+                               {(const char*)v + ov, dv_ + ov, nbv}};
+        if (in_kernel) return launch_host_copy(c, 5, 32, s) == cudaSuccess;
+        bool good = true;
+        for (const HostCopy& x : c) good = good && cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
+        return good;
+    };
+    // Slices of whole units: while slice i + 1 travels to the device, the kernels of slice i run and slice i - 1 travels back.
+    // The way in bounds the call (55 GB/s), and what comes after the last copy in is pure addition, so each slice is about
+    // 0.35 of the one before: just enough for its way in to cover the way back of that one (a third of the bytes).  More
+    // slices only pay for larger results.  Small results, and unit sizes that would misalign a slice, go through the caller's
+    // stream in one piece.
+    int nsl = out_bytes >= (8u << 20) ? 3 : (out_bytes >= (1u << 20) ? 2 : 1);
+    if (!whole || units < 8) nsl = 1;
+    auto copy_out = [&](size_t ov, size_t nbv, cudaStream_t s) {
+        const HostCopy c = {dout + ov, (char*)out + ov, nbv};
+        return out_kernel ? launch_host_copy(&c, 1, nsl > 1 ? 2 : 32, s) == cudaSuccess : cudaMemcpyAsync(c.dst, c.src, nbv, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+    };
+    int st = VIG_OK;
+    bool ok = true;
+    if (nsl == 1) {
+        ok = copy_in(0, 0, units * unit_k, units * unit_v, stream);
+        if (ok) st = kernels(0, 0, (int)units);
+        if (ok && st == VIG_OK) ok = copy_out(0, units * unit_v, stream);
+    } else {
+        ok = cudaEventRecord(hp->ev_start, stream) == cudaSuccess && cudaStreamWaitEvent(hp->s_in, hp->ev_start, 0) == cudaSuccess &&
+             cudaStreamWaitEvent(hp->s_out, hp->ev_start, 0) == cudaSuccess;
+        long long u0 = 0;
+        for (int i = 0; ok && i < nsl && st == VIG_OK; ++i) {
+            const long long rest = units - u0;
+            const long long nu = i + 1 == nsl ? rest : (long long)(rest * (nsl - i == 3 ? 0.68 : 0.74));   // 1 : 0.35 : 0.12, 1 : 0.35
+            const size_t ok_ = (size_t)u0 * unit_k, ov = (size_t)u0 * unit_v;
+            ok = copy_in(ok_, ov, nu * unit_k, nu * unit_v, hp->s_in) && cudaEventRecord(hp->ev_in[i], hp->s_in) == cudaSuccess &&
+                 cudaStreamWaitEvent(stream, hp->ev_in[i], 0) == cudaSuccess;
+            if (!ok) break;
+            st = kernels(ok_, ov, (int)nu);
+            if (st != VIG_OK) break;
+            ok = cudaEventRecord(hp->ev_k[i], stream) == cudaSuccess && cudaStreamWaitEvent(hp->s_out, hp->ev_k[i], 0) == cudaSuccess &&
+                 copy_out(ov, nu * unit_v, hp->s_out);
+            u0 += nu;
+        }
+        // the caller's stream takes over again once both copy streams have drained (also after an error, so that the buffer
+        // is not freed under a copy in flight)
+        ok = (cudaEventRecord(hp->ev_done_in, hp->s_in) == cudaSuccess) & (cudaEventRecord(hp->ev_done_out, hp->s_out) == cudaSuccess) &
+             (cudaStreamWaitEvent(stream, hp->ev_done_in, 0) == cudaSuccess) & (cudaStreamWaitEvent(stream, hp->ev_done_out, 0) == cudaSuccess) & ok;
     }
-    // the caller's stream takes over again once both copy streams have drained (also after an error, so that the
-    // buffer is not freed under a copy in flight)
-    ok = (cudaEventRecord(hp->ev_done_in, hp->s_in) == cudaSuccess) & (cudaEventRecord(hp->ev_done_out, hp->s_out) == cudaSuccess) &
-         (cudaStreamWaitEvent(stream, hp->ev_done_in, 0) == cudaSuccess) & (cudaStreamWaitEvent(stream, hp->ev_done_out, 0) == cudaSuccess) & ok;
     if (!ok && st == VIG_OK) st = VIG_ERR_CUDA;
     if (cudaFreeAsync(base, stream) != cudaSuccess && st == VIG_OK) st = VIG_ERR_CUDA;
     if (cudaStreamSynchronize(stream) != cudaSuccess && st == VIG_OK) st = VIG_ERR_CUDA;

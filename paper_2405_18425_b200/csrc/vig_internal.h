@@ -95,6 +95,16 @@ cudaError_t launch_bigla_grad(const __nv_bfloat16* q, const __nv_bfloat16* k, co
                               __nv_bfloat16* dv_out, __nv_bfloat16* dla_f, __nv_bfloat16* dla_b, void* scratch, long long units, int L, int dk,
                               int dv, cudaStream_t stream);
 
+// ---- copies between pinned host memory and the device by a kernel ----
+constexpr int kHostCopies = 5;   // per launch
+struct HostCopy {
+    const void* src;
+    void* dst;
+    size_t bytes;   // a multiple of 16; both addresses 16-byte aligned
+};
+bool host_copy_usable(const void* host, size_t bytes);   // pinned and mapped, aligned
+cudaError_t launch_host_copy(const HostCopy* copies, int n, int max_blocks, cudaStream_t stream);
+
 // Launch with programmatic stream serialization: the kernel's prologue (everything before its pdl_wait) may overlap
 // the tail of the kernel before it in the stream.
 template <typename... KArgs, typename... Args>
