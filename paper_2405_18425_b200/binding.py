@@ -89,7 +89,11 @@ def status_string(status: int) -> str:
 
 def _stream(stream) -> int:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the handle itself: torch.cuda.current_stream() builds a Stream object on every call (4.7 us against 0.2 us, of the
+        # 15 us a forward call took on the host)
+        if not torch.cuda.is_initialized():
+            torch.cuda.init()
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

@@ -20,8 +20,14 @@ int kernel_preference() { return g_kernel_pref.load(std::memory_order_relaxed); 
 void count_launch(unsigned n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
 int* device_status_ptr() {
-    int* p = nullptr;
-    if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_device_status) != cudaSuccess) return nullptr;
+    static std::atomic<int*> of_device[64];   // looked up once per device: every launch passes it on
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    int* p = of_device[dev].load(std::memory_order_relaxed);
+    if (!p) {
+        if (cudaGetSymbolAddress(reinterpret_cast<void**>(&p), g_device_status) != cudaSuccess) return nullptr;
+        of_device[dev].store(p, std::memory_order_relaxed);
+    }
     return p;
 }
 

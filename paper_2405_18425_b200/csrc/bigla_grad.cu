@@ -97,21 +97,6 @@ __device__ __forceinline__ void st_async1(uint32_t addr, uint32_t v, uint32_t ba
 }
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }   // orders no memory accesses
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-// Lane c of a group of four holds words (c, 0 .. 3); afterwards words (0 .. 3, c).
-__device__ __forceinline__ void transpose4(uint32_t (&x)[4], int c) {
-#pragma unroll
-    for (int p = 0; p < 4; p += 2) {
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, (c & 1) ? x[p] : x[p + 1], 1);
-        if (c & 1) x[p] = y;
-        else x[p + 1] = y;
-    }
-#pragma unroll
-    for (int p = 0; p < 2; ++p) {
-        const uint32_t y = __shfl_xor_sync(0xffffffffu, (c & 2) ? x[p] : x[p + 2], 2);
-        if (c & 2) x[p] = y;
-        else x[p + 2] = y;
-    }
-}
 
 // Sixteen bits of two words: an fp32 kept in two bf16 buffers.
 __device__ __forceinline__ void put_halves(__nv_bfloat16* hi, __nv_bfloat16* lo, float x) {
@@ -442,95 +427,76 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         return;
     }
 
-    // What a 16 x 16 tile of scores on the diagonal keeps: columns up to the row (the left side) or from it on.
-    auto mask = [&](float (&d0)[4], float (&d1)[4], bool left) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int row = g + 8 * (e >> 1), col = 2 * c + (e & 1);
-            if (left ? col > row : col < row) d0[e] = 0.f;
-            if (left ? col + 8 > row : col + 8 < row) d1[e] = 0.f;
-        }
-    };
-    // Every sum below is taken over steps: first the tiles up to the warp's own (the left side), then its own again and the
-    // tiles after it (the right side), nT + 1 steps by one copy of the code - unrolled, the passes overflow the instruction
-    // cache -, the scores of a step computed one step ahead of the product that takes them.
+    const DiagonalMask dmask(g, c);
+    // Every sum below runs over the tiles up to the warp's own (the left side) and from it on (the right side): a loop, the
+    // two halves of the diagonal tile, a loop, so that no loop carries the masks or a change of operands (as one loop over
+    // nT + 1 steps with both inside, the moves and selects of a step were as many as its products: 43 M warp instructions
+    // at 768 units of 196 tokens, 32 x 64, against 37 M).
 
     // ---- dq, dk: the scores D = g v^T (this warp's tokens as queries), then D^T (as keys), split, times the scaled operands ----
     float sum[2][2][NP][4];   // [dq, dk][left, right side], not yet scaled
     if (live) {
         uint32_t ra[MV][4];
-        float acc[NP][4], d0[4], d1[4], n0[4], n1[4];
-        auto own_rows = [&](uint32_t tile) {
-#pragma unroll
-            for (int m = 0; m < MV; ++m) tvv.load(tile, 16 * wt, m, ra[m]);
-        };
-        auto scores = [&](uint32_t tile, float (&s0)[4], float (&s1)[4]) {
+        // scores of this warp's rows against a tile of rows, split, times that tile's operand pair; keep: 0 all scores, 1 left, 2 right
+        auto tile = [&](uint32_t s_tile, uint32_t o_tile, float (&acc)[NP][4], int keep) {
+            float d0[4], d1[4];
 #pragma unroll
             for (int m = 0; m < MV; ++m) {
                 uint32_t r[4];
-                tvv.load_b(tile, 0, m, r);
+                tvv.load_b(s_tile, 0, m, r);
                 if (m == 0) {
-                    mma_k16_zero(s0, ra[0], r[0], r[1]);
-                    mma_k16_zero(s1, ra[0], r[2], r[3]);
+                    mma_k16_zero(d0, ra[0], r[0], r[1]);
+                    mma_k16_zero(d1, ra[0], r[2], r[3]);
                 } else {
-                    mma_k16(s0, ra[m], r[0], r[1]);
-                    mma_k16(s1, ra[m], r[2], r[3]);
+                    mma_k16(d0, ra[m], r[0], r[1]);
+                    mma_k16(d1, ra[m], r[2], r[3]);
                 }
             }
+            uint32_t ah[4], al[4];
+            split_bf16(pack2(d0[0], d0[1]), ah[0], al[0]);
+            split_bf16(pack2(d0[2], d0[3]), ah[1], al[1]);
+            split_bf16(pack2(d1[0], d1[1]), ah[2], al[2]);
+            split_bf16(pack2(d1[2], d1[3]), ah[3], al[3]);
+            if (keep) {
+                dmask.apply(ah, keep == 1);
+                dmask.apply(al, keep == 1);
+            }
+#pragma unroll
+            for (int m = 0; m < MP; ++m) {
+                uint32_t h[4], l[4];
+                t64.load_trans(o_tile, 0, m, h);
+                t64.load_trans(o_tile + lay.op_bytes, 0, m, l);
+                mma_k16(acc[2 * m], ah, h[0], h[1]);
+                if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], ah, h[2], h[3]);
+                mma_k16(acc[2 * m], al, h[0], h[1]);
+                if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], al, h[2], h[3]);
+                mma_k16(acc[2 * m], ah, l[0], l[1]);
+                if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], ah, l[2], l[3]);
+            }
         };
-        auto keep = [&](float (&to)[NP][4]) {
-#pragma unroll
-            for (int j = 0; j < NP; ++j)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    to[j][e] = acc[j][e];
-                    acc[j][e] = 0.f;
-                }
-        };
-#pragma unroll
-        for (int j = 0; j < NP; ++j)
-#pragma unroll
-            for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
 #pragma unroll
         for (int pass = 0; pass < 2; ++pass) {
             // dq: g rows against v tiles, k~> left, k~< right;  dk: v rows against g tiles, q~< left, q~> right
-            own_rows(pass == 0 ? tg : tv);
+#pragma unroll
+            for (int m = 0; m < MV; ++m) tvv.load(pass == 0 ? tg : tv, 16 * wt, m, ra[m]);
+#pragma unroll
+            for (int side = 0; side < 2; ++side)
+#pragma unroll
+                for (int j = 0; j < NP; ++j)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) sum[pass][side][j][e] = 0.f;
             uint32_t s_tile = pass == 0 ? tv : tg, o_tile = op(pass == 0 ? kKf : kQb);
-            scores(s_tile, d0, d1);
 #pragma unroll 1
-            for (int s = 0; s <= nT; ++s) {
-                if (s != wt) s_tile += 16 * RV;
-                if (s < nT) scores(s_tile, n0, n1);
-                if (s == wt || s == wt + 1) mask(d0, d1, s == wt);
-                uint32_t ah[4], al[4];
-                split_bf16(pack2(d0[0], d0[1]), ah[0], al[0]);
-                split_bf16(pack2(d0[2], d0[3]), ah[1], al[1]);
-                split_bf16(pack2(d1[0], d1[1]), ah[2], al[2]);
-                split_bf16(pack2(d1[2], d1[3]), ah[3], al[3]);
-#pragma unroll
-                for (int m = 0; m < MP; ++m) {
-                    uint32_t h[4], l[4];
-                    t64.load_trans(o_tile, 0, m, h);
-                    t64.load_trans(o_tile + lay.op_bytes, 0, m, l);
-                    mma_k16(acc[2 * m], ah, h[0], h[1]);
-                    if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], ah, h[2], h[3]);
-                    mma_k16(acc[2 * m], al, h[0], h[1]);
-                    if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], al, h[2], h[3]);
-                    mma_k16(acc[2 * m], ah, l[0], l[1]);
-                    if (2 * m + 1 < NP) mma_k16(acc[2 * m + 1 < NP ? 2 * m + 1 : 0], ah, l[2], l[3]);
-                }
+            for (int j = 0; j < wt; ++j, s_tile += 16 * RV, o_tile += 1024) tile(s_tile, o_tile, sum[pass][0], 0);
+            tile(s_tile, o_tile, sum[pass][0], 1);
+            o_tile = op(pass == 0 ? kKb : kQf) + wt * 1024;
+            tile(s_tile, o_tile, sum[pass][1], 2);
+#pragma unroll 1
+            for (int j = wt + 1; j < nT; ++j) {
+                s_tile += 16 * RV;
                 o_tile += 1024;
-                if (s == wt) {
-                    keep(sum[pass][0]);
-                    o_tile = op(pass == 0 ? kKb : kQf) + wt * 1024;
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    d0[e] = n0[e];
-                    d1[e] = n1[e];
-                }
+                tile(s_tile, o_tile, sum[pass][1], 0);
             }
-            keep(sum[pass][1]);
         }
     }
 
@@ -656,42 +622,29 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         for (int e = 0; e < 4; ++e) o[n][e] = 0.f;
     if (live) {
         uint32_t kk[MP][4];
-        float d0[4], d1[4], n0[4], n1[4];
-        auto key_scores = [&](uint32_t tile, float (&s0)[4], float (&s1)[4]) {
-#pragma unroll
-            for (int m = 0; m < MP; ++m) {
-                uint32_t r[4];
-                t64.load_b(tile, 0, m, r);
-                if (m == 0) {
-                    mma_k16_zero(s0, kk[0], r[0], r[1]);
-                    mma_k16_zero(s1, kk[0], r[2], r[3]);
-                } else if (2 * m + 1 < NP) {
-                    mma_k16(s0, kk[m], r[0], r[1]);
-                    mma_k16(s1, kk[m], r[2], r[3]);
-                } else {
-                    mma_k8(s0, kk[m][0], kk[m][1], r[0]);
-                    mma_k8(s1, kk[m][0], kk[m][1], r[2]);
-                }
-            }
-        };
         auto own_keys = [&](int which) {
 #pragma unroll
             for (int m = 0; m < MP; ++m) t64.load(op(which), 16 * wt, m, kk[m]);
         };
-        own_keys(kKb);
-        uint32_t q_tile = op(kQb), g_tile = tg;
-        key_scores(q_tile, d0, d1);
-#pragma unroll 1
-        for (int s = 0; s <= nT; ++s) {
-            if (s == wt) {   // from here on the right side: the next step is the warp's own tile once more
-                own_keys(kKf);
-                q_tile = op(kQf) + wt * 1024;
-            } else {
-                q_tile += 1024;
+        auto tile = [&](uint32_t q_tile, uint32_t g_tile, int keep) {
+            float d0[4], d1[4];
+#pragma unroll
+            for (int m = 0; m < MP; ++m) {
+                uint32_t r[4];
+                t64.load_b(q_tile, 0, m, r);
+                if (m == 0) {
+                    mma_k16_zero(d0, kk[0], r[0], r[1]);
+                    mma_k16_zero(d1, kk[0], r[2], r[3]);
+                } else if (2 * m + 1 < NP) {
+                    mma_k16(d0, kk[m], r[0], r[1]);
+                    mma_k16(d1, kk[m], r[2], r[3]);
+                } else {
+                    mma_k8(d0, kk[m][0], kk[m][1], r[0]);
+                    mma_k8(d1, kk[m][0], kk[m][1], r[2]);
+                }
             }
-            if (s < nT) key_scores(q_tile, n0, n1);
-            if (s == wt || s == wt + 1) mask(d0, d1, s == wt);
-            const uint32_t p[4] = {pack_bf16(d0[0], d0[1]), pack_bf16(d0[2], d0[3]), pack_bf16(d1[0], d1[1]), pack_bf16(d1[2], d1[3])};
+            uint32_t p[4] = {pack_bf16(d0[0], d0[1]), pack_bf16(d0[2], d0[3]), pack_bf16(d1[0], d1[1]), pack_bf16(d1[2], d1[3])};
+            if (keep) dmask.apply(p, keep == 1);
 #pragma unroll
             for (int n2 = 0; n2 < MV; ++n2) {
                 uint32_t r[4];
@@ -699,12 +652,20 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 mma_k16(o[2 * n2], p, r[0], r[1]);
                 mma_k16(o[2 * n2 + 1], p, r[2], r[3]);
             }
-            if (s != wt) g_tile += 16 * RV;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                d0[e] = n0[e];
-                d1[e] = n1[e];
-            }
+        };
+        own_keys(kKb);
+        uint32_t q_tile = op(kQb), g_tile = tg;
+#pragma unroll 1
+        for (int j = 0; j < wt; ++j, q_tile += 1024, g_tile += 16 * RV) tile(q_tile, g_tile, 0);
+        tile(q_tile, g_tile, 1);
+        own_keys(kKf);
+        q_tile = op(kQf) + wt * 1024;
+        tile(q_tile, g_tile, 2);
+#pragma unroll 1
+        for (int j = wt + 1; j < nT; ++j) {
+            q_tile += 1024;
+            g_tile += 16 * RV;
+            tile(q_tile, g_tile, 0);
         }
         if (MODE != kSingle) {   // dv from the border states, one bf16 per operand
 #pragma unroll 1

@@ -103,6 +103,88 @@ __device__ __forceinline__ uint32_t triangle(int g, int c, bool diagonal) {
 }
 constexpr uint32_t kOnes = 0x3F803F80u;
 
+// A 16 x 16 tile of scores on the diagonal, packed as A operand (p[0]: rows g, columns 2c, 2c+1; p[1]: rows g + 8; p[2], p[3]:
+// columns + 8): left keeps the columns up to the row, else those from the row on.
+struct DiagonalMask {
+    uint32_t l, r;
+    __device__ __forceinline__ DiagonalMask(int g, int c) {
+        l = (2 * c <= g ? 0xFFFFu : 0u) | (2 * c + 1 <= g ? 0xFFFF0000u : 0u);
+        r = (2 * c >= g ? 0xFFFFu : 0u) | (2 * c + 1 >= g ? 0xFFFF0000u : 0u);
+    }
+    __device__ __forceinline__ void apply(uint32_t (&p)[4], bool left) const {
+        p[0] &= left ? l : r;
+        p[3] &= left ? l : r;
+        if (left) p[2] = 0u;
+        else p[1] = 0u;
+    }
+};
+
+// 1 / x for two packed positive, normal bf16 values without the special-function unit and without leaving the packed
+// format: a bit-level first guess per half (one 32-bit subtraction: neither half borrows) and one Newton step r (2 - x r) in
+// bf16x2 arithmetic.  Relative error at most 0.63 % (root mean square 0.27 %, the same as rounding an exact reciprocal to
+// bf16 after a first guess of this kind); the result only scales bf16 operands, whose own rounding unit is 0.39 %, and it
+// is the reciprocal of the very factor the other operand is scaled by.
+__device__ __forceinline__ uint32_t rcp_bf16x2(uint32_t x) {
+    const uint32_t r0 = 0x7EF27EF2u - x;
+    const __nv_bfloat162 xb = *reinterpret_cast<const __nv_bfloat162*>(&x), rb = *reinterpret_cast<const __nv_bfloat162*>(&r0);
+    const __nv_bfloat162 r1 = __hmul2(rb, __hfma2(__hneg2(xb), rb, __float2bfloat162_rn(2.0f)));
+    return *reinterpret_cast<const uint32_t*>(&r1);
+}
+
+// log2 alpha = logsigmoid(g) / (tau ln 2) (Eq. 5 line 1, in base 2 so that the operand scaling needs no further
+// multiplication) of two gate logits, evaluated in fp32 as (min(g, 0) log2(e) - log2(1 + e)) / tau with e = e^{-|g|} in (0, 1]
+// from the special-function unit and log2(1 + e) = e p(e), p of degree three (absolute error 1e-4, i.e. 7e-5 / tau in log
+// alpha: below the bf16 rounding that follows), on the FMA pipe, two values per instruction.
+__device__ __forceinline__ uint32_t log2_alpha_pair(uint32_t g, float inv_tau) {
+    const uint32_t a = g | 0x80008000u;   // -|g|
+    uint32_t m;                           // min(g, 0)
+    asm("min.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(g), "r"(0u));
+    float y0, y1;
+    unpack2(fmul2(pack2(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u)), pack2(kLog2e, kLog2e)), y0, y1);
+    const f32x2 e = pack2(ex2(y0), ex2(y1));
+    f32x2 p = pack2(-0.08476800471544266f, -0.08476800471544266f);
+    p = ffma2(p, e, pack2(0.3255951702594757f, 0.3255951702594757f));
+    p = ffma2(p, e, pack2(-0.6799444556236267f, -0.6799444556236267f));
+    p = ffma2(p, e, pack2(1.4390150308609009f, 1.4390150308609009f));
+    const float c_lin = kLog2e * inv_tau;
+    const f32x2 lin = fmul2(pack2(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u)), pack2(c_lin, c_lin));
+    unpack2(ffma2(fmul2(p, e), pack2(-inv_tau, -inv_tau), lin), y0, y1);
+    return pack_bf16(y0, y1);
+}
+
+// This lane's pairs of key dimensions of a row of DK bf16, straight from global memory.  Which dimensions pair j of lane c
+// holds only has to be the same in both operands of a contraction; it is chosen so that a warp reads its rows in whole
+// pieces, contiguous across the four lanes of a row:
+//   DK = 32: dims 8c + 2j, +1;   DK = 24: dims 4c + 2j, +1 (j = 0, 1) and 16 + 2c, +1 (j = 2);   DK = 16: dims 4c + 2j, +1
+template <int DK>
+__device__ __forceinline__ void load_pairs(const __nv_bfloat16* row, int c, uint32_t (&r)[DK / 8]) {
+    const char* p = reinterpret_cast<const char*>(row);
+    if constexpr (DK == 32) {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(p + 16 * c));
+        r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
+    } else {
+        const uint2 x = __ldg(reinterpret_cast<const uint2*>(p + 8 * c));
+        r[0] = x.x; r[1] = x.y;
+        if constexpr (DK == 24) r[2] = __ldg(reinterpret_cast<const uint32_t*>(p + 32 + 4 * c));
+    }
+}
+
+// Lane c of a group of four holds words (c, 0 .. 3); afterwards words (0 .. 3, c).
+__device__ __forceinline__ void transpose4(uint32_t (&x)[4], int c) {
+#pragma unroll
+    for (int p = 0; p < 4; p += 2) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, (c & 1) ? x[p] : x[p + 1], 1);
+        if (c & 1) x[p] = y;
+        else x[p + 1] = y;
+    }
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, (c & 2) ? x[p] : x[p + 2], 2);
+        if (c & 2) x[p] = y;
+        else x[p + 2] = y;
+    }
+}
+
 // x = hi + lo with two bf16 each: sixteen significant bits of an fp32 value as two tensor-core operands.
 __device__ __forceinline__ void split_bf16(f32x2 x, uint32_t& hi, uint32_t& lo) {
     float x0, x1;
