@@ -1,0 +1,441 @@
+// bf16 BiGLA forward for units of at most 256 tokens: one block per (batch, head) unit, one warp per 16 tokens, every
+// product a chain of 16 x 16 tiles whose scores stay in registers (mma.sync).
+//
+// With b_t the inclusive prefix sum of log alpha> and x_t the exclusive prefix sum of log alpha< (the backward decay from t
+// to s > t is exp(x_s - x_t): the gates t .. s-1), both from the start of a chunk of 128 tokens, Eq. 6 is, per chunk,
+//     q~> = q e^{b} / 2,  k~> = k e^{-b},  q~< = q e^{-x} / 2,  k~< = k e^{x}
+//     out_t = sum_{s <= t} (q~>_t k~>_s) v_s + sum_{s >= t} (q~<_t k~<_s) v_s + q~ S
+// with S the state the other chunk of the unit hands over (k~>^T v of chunk 0 forward, k~<^T v of chunk 1 backward, either
+// times the whole decay of chunk 0).
+//
+// A warp reads its rows of q, k and the gates straight into fragment order, takes their prefix sums as products with a
+// 16 x 16 triangle of ones (fp32 accumulation of bf16 values: exact up to fp32 addition), leaves k~ in shared memory and
+// keeps q~ in registers; v comes by one TMA load.  Then it runs over the tiles of its chunk: scores, packed to bf16 as the A
+// operand of the product with v.  Two block barriers (gate totals, k~) and one mbarrier (states) order the warps.
+//
+// What bounds it: with one block per SM the latency of that chain (4.5 us at 100 tokens, 6.5 us at 196), with more of them
+// instruction issue (about 1600 warp instructions per warp at 196 tokens, 32 x 64), so registers are held to what lets two
+// blocks of thirteen or sixteen warps, or three of eight, share an SM.  Against the tcgen05 form (two 128-row chunk
+// pipelines per block, whose hand-overs between tensor-core batches bound it): 148 units of 49 tokens 3.1 us to 6.2, 768 of
+// 128 tokens 14.9 to 24.5 (24 x 48), 1536 of 196 tokens 53.6 to 61.9 (24 x 48); mma_preferred holds the shapes it loses.
+#include <cuda.h>
+
+#include <atomic>
+
+#include "mma.cuh"
+#include "recurrence.cuh"
+#include "tma_host.h"
+#include "vig_internal.h"
+
+namespace vig {
+namespace {
+
+using namespace wmma16;
+
+constexpr float kGateRange = 60.f;    // largest decay of a chunk, as -log, that the factorised tiles take
+
+struct MArgs {
+    const __nv_bfloat16 *q, *k, *v, *la_f, *la_b;   // GATES: la_f / la_b hold the gate logits
+    __nv_bfloat16* out;
+    int L, units;
+    int* dev_status;
+    float inv_tau;
+    int ahead;         // the unit this many blocks on is pulled into L2
+    int expire_wait;   // test hook: every block lets one bounded wait, on an mbarrier nothing completes, run out
+};
+
+// Shared memory: v [rows][RV], k~> and k~< [rows][64 B], the two states [DV][64 B], gate totals [tile][2][32] fp32.
+template <int DV>
+struct MLayout {
+    static constexpr uint32_t kVRow = DV == 32 ? 64 : 128, kState = DV * 64;
+    uint32_t kf, kb, st, totals, bar, total;
+    __host__ __device__ explicit MLayout(int tiles) {
+        const uint32_t rows = tiles * 16u;
+        kf = rows * kVRow;
+        kb = kf + rows * 64;
+        st = kb + rows * 64;
+        totals = st + (tiles > 8 ? 2 * kState : 0);
+        bar = totals + tiles * 256u;
+        total = bar + 64;
+    }
+};
+
+template <int DK, int DV, bool GATES, int MAXT>
+__global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const MArgs args) {
+    constexpr int NP = DK / 8, MP = (NP + 1) / 2;   // 8-column tiles of the key dimensions, pairs of them
+    constexpr int NV = DV / 8, MV = DV / 16;        // ... of the value dimensions
+    constexpr int RV = MLayout<DV>::kVRow;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int g = lane >> 2, c = lane & 3;
+    const int L = args.L, unit = blockIdx.x, T = (L + 15) >> 4;
+    const bool live = w < T;                          // (blocks have two warps at least: the in-kernel recurrence needs them)
+    const int ch = MAXT > 8 ? w >> 3 : 0, c0 = 8 * ch;   // this warp's chunk and its first tile
+    const MLayout<DV> lay(T);
+    const uint32_t base = smem_u32(smem), tv = base, tkf = base + lay.kf, tkb = base + lay.kb, tst = base + lay.st, bar = base + lay.bar;
+    float* totals = reinterpret_cast<float*>(smem + lay.totals);
+    volatile int* slow = reinterpret_cast<volatile int*>(smem + lay.bar + 32);
+
+    pdl_launch_dependents();
+    if (tid == 0) {
+        mbar_init(bar, 1);
+        mbar_init(bar + 8, 2 * MV);   // one arrival per piece of the states
+        mbar_init(bar + 16, 1);       // never completed: only the test hook waits on it
+        *slow = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    pdl_wait();
+    if (tid == 0) {
+        mbar_expect_tx(bar, (uint32_t)T * 16 * RV);
+        tma_load_3d(tv, &tm_v, 0, 0, unit, bar);   // rows >= L and columns >= DV arrive as zeros
+    }
+
+    // ---- this warp's 16 rows (g and g + 8) in fragment order: pair j of lane c ----
+    uint32_t qr[2][NP], kr[2][NP], af[2][NP], ab[2][NP];
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int row = w * 16 + 8 * r + g;
+        if (row < L) {
+            const size_t at = ((size_t)unit * L + row) * DK;
+            load_pairs<DK>(args.la_f + at, c, af[r]);
+            load_pairs<DK>(args.la_b + at, c, ab[r]);
+            load_pairs<DK>(args.k + at, c, kr[r]);
+            load_pairs<DK>(args.q + at, c, qr[r]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {   // rows past the end: q = k = 0 and no decay (GATES: a logit of 100, log alpha = 0)
+                qr[r][j] = kr[r][j] = 0u;
+                af[r][j] = ab[r][j] = GATES ? 0x42C842C8u : 0u;
+            }
+        }
+    }
+    if (tid == 0 && unit + args.ahead < args.units) {   // a block that starts when one of these is done finds its unit in L2
+        const size_t at = (size_t)(unit + args.ahead) * L;
+        prefetch_l2(args.la_f + at * DK, (uint32_t)L * DK * 2);
+        prefetch_l2(args.la_b + at * DK, (uint32_t)L * DK * 2);
+        prefetch_l2(args.k + at * DK, (uint32_t)L * DK * 2);
+        prefetch_l2(args.q + at * DK, (uint32_t)L * DK * 2);
+        prefetch_l2(args.v + at * DV, (uint32_t)L * DV * 2);
+    }
+    // ---- gate totals of the tile; the gates turned, as B operands of products over the tokens ----
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            if (GATES) {
+                af[r][j] = log2_alpha_pair(af[r][j], args.inv_tau);
+                ab[r][j] = log2_alpha_pair(ab[r][j], args.inv_tau);
+            }
+            af[r][j] = movmatrix(af[r][j]);
+            ab[r][j] = movmatrix(ab[r][j]);
+        }
+        float tf[4], tb[4];
+        mma_k16_from(tf, kOnes, kOnes, kOnes, kOnes, af[0][j], af[1][j], 0.f, 0.f);
+        mma_k16_from(tb, kOnes, kOnes, kOnes, kOnes, ab[0][j], ab[1][j], 0.f, 0.f);
+        if (g == 0 && live) {
+            *reinterpret_cast<float2*>(totals + (w * 2) * 32 + 8 * j + 2 * c) = make_float2(tf[0], tf[1]);
+            *reinterpret_cast<float2*>(totals + (w * 2 + 1) * 32 + 8 * j + 2 * c) = make_float2(tb[0], tb[1]);
+        }
+    }
+    __syncthreads();
+    // sums over tiles [from, to) of one direction
+    auto sum_totals = [&](int dir, int from, int to, f32x2 (&s)[NP]) {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) s[j] = 0ull;   // (+0, +0)
+        const float* p = totals + (from * 2 + dir) * 32 + 2 * c;
+#pragma unroll 1
+        for (int x = from; x < to; ++x, p += 64)
+#pragma unroll
+            for (int j = 0; j < NP; ++j) s[j] = fadd2(s[j], *reinterpret_cast<const f32x2*>(p + 8 * j));
+    };
+    if (w == T - 1 && lane < DK) {   // range check: the decay of each chunk per key dim and direction
+#pragma unroll
+        for (int h = 0; h < (MAXT > 8 ? 2 : 1); ++h)
+#pragma unroll
+            for (int d = 0; d < 2; ++d) {
+                float s = 0.f;
+                for (int x = 8 * h; x < min(T, 8 * h + 8); ++x) s += totals[(x * 2 + d) * 32 + lane];
+                if (!(s >= -kGateRange * (GATES ? kLog2e : 1.f))) *slow = 1;
+            }
+    }
+    // ---- prefix sums from the start of the chunk and scaled operands: k~ to shared memory, q~ in registers ----
+    uint32_t qf[MP][4], qb[MP][4];
+    if (live) {
+        const uint32_t tri_i = triangle(g, c, true), tri_x = triangle(g, c, false);
+        const Tile<64> t64(lane);
+        f32x2 cf[NP], cb[NP];
+        sum_totals(0, c0, w, cf);
+        sum_totals(1, c0, w, cb);
+#pragma unroll
+        for (int m = 0; m < MP; ++m) {
+            uint32_t kfw[4], kbw[4];
+#pragma unroll
+            for (int jj = 0; jj < 2; ++jj) {
+                const int j = 2 * m + jj;
+                if (j < NP) {
+                    float b[4], x[4], f0, f1, e0, e1;
+                    unpack2(cf[j], f0, f1);
+                    unpack2(cb[j], e0, e1);
+                    mma_k16_from(b, tri_i, kOnes, 0u, tri_i, af[0][j], af[1][j], f0, f1);
+                    mma_k16_from(x, tri_x, kOnes, 0u, tri_x, ab[0][j], ab[1][j], e0, e1);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        float b0 = b[2 * r], b1 = b[2 * r + 1], x0 = x[2 * r], x1 = x[2 * r + 1];
+                        if constexpr (!GATES) {   // natural logarithms in
+                            unpack2(fmul2(pack2(b0, b1), pack2(kLog2e, kLog2e)), b0, b1);
+                            unpack2(fmul2(pack2(x0, x1), pack2(kLog2e, kLog2e)), x0, x1);
+                        }
+                        // the decaying factors on the special-function unit, the growing ones as their packed reciprocals
+                        const uint32_t ef = pack_bf16(ex2(b0), ex2(b1)), eb = pack_bf16(ex2(x0), ex2(x1));
+                        const uint32_t hq = mul_bf16x2(qr[r][j], 0x3F003F00u);   // the 1/2 of the result: exact
+                        kfw[2 * jj + r] = mul_bf16x2(kr[r][j], rcp_bf16x2(ef));
+                        kbw[2 * jj + r] = mul_bf16x2(kr[r][j], eb);
+                        qf[m][2 * jj + r] = mul_bf16x2(hq, ef);
+                        qb[m][2 * jj + r] = mul_bf16x2(hq, rcp_bf16x2(eb));
+                    }
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) kfw[2 + r] = kbw[2 + r] = qf[m][2 + r] = qb[m][2 + r] = 0u;
+                }
+            }
+            t64.store(tkf, 16 * w, m, kfw[0], kfw[1], kfw[2], kfw[3]);
+            t64.store(tkb, 16 * w, m, kbw[0], kbw[1], kbw[2], kbw[3]);
+        }
+    }
+    bool ok = true;
+    if (args.expire_wait && tid == 0) ok = mbar_wait_bounded(bar + 16, 0, 64);   // test hook: this wait cannot succeed
+    ok = mbar_wait_bounded(bar, 0) && ok;
+    if (!__syncthreads_and(ok)) {   // a load that never lands: report it and leave, all threads together, nothing stored
+        if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
+        return;
+    }
+    if (*slow) {   // gates beyond the range of the factorised tiles: Eq. 6 step by step, over the dead tiles
+        if (tid == 0) atomicAdd(args.dev_status + 1, 1);
+        __syncthreads();
+        const size_t okk = (size_t)unit * L * DK, ov = (size_t)unit * L * DV;
+        recurrence_unit<__nv_bfloat16>(args.q + okk, args.k + okk, args.v + ov, args.la_f + okk, args.la_b + okk, args.out + ov, L, DK, DV,
+                                       reinterpret_cast<float*>(smem), args.inv_tau);
+        return;
+    }
+    if (!live) return;
+    const Tile<64> t64(lane);
+    const Tile<RV> tvv(lane);
+
+    // ---- the states the chunks hand each other, transposed: rows of v times k~ over the tokens, 16 value columns a job; the
+    // last warps first: theirs is the shorter chunk ----
+    if (MAXT > 8 && T > 8) {
+        for (int job = T - 1 - w; job < 2 * MV; job += T) {
+            const int dir = job & 1, mt = job >> 1;   // dir 0: chunk 0 -> 1 (forward);  dir 1: chunk 1 -> 0
+            const int t0 = dir == 0 ? 0 : 8, t1 = dir == 0 ? 8 : T;
+            float u[2 * MP][4];
+#pragma unroll
+            for (int j = 0; j < 2 * MP; ++j)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) u[j][e] = 0.f;
+            uint32_t left = tv + t0 * 16 * RV + (tvv.off_b[0] ^ (uint32_t)(mt << 5));   // (the piece bits of an offset are its swizzle alone)
+            uint32_t right = (dir == 0 ? tkf : tkb) + t0 * 1024;
+#pragma unroll 2
+            for (int t = t0; t < t1; ++t, left += 16 * RV, right += 1024) {
+                uint32_t va[4];
+                ldsm_trans(left, va);
+#pragma unroll
+                for (int m = 0; m < MP; ++m) {
+                    uint32_t h[4];
+                    t64.load_trans(right, 0, m, h);
+                    mma_k16(u[2 * m], va, h[0], h[1]);
+                    if (2 * m + 1 < NP) mma_k16(u[2 * m + 1], va, h[2], h[3]);
+                }
+            }
+            f32x2 dec[NP];
+            sum_totals(dir, 0, 8, dec);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {   // times chunk 0's decay: of what it leaves behind (forward), of what it takes in (backward)
+                float d0, d1;
+                unpack2(GATES ? dec[j] : fmul2(dec[j], pack2(kLog2e, kLog2e)), d0, d1);
+                d0 = ex2(d0);
+                d1 = ex2(d1);
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const int n = 16 * mt + 8 * r + g;
+                    *reinterpret_cast<uint32_t*>(smem + lay.st + dir * MLayout<DV>::kState + n * 64 + ((j ^ ((n >> 1) & 3)) << 4) + 4 * c) =
+                        pack_bf16(u[j][2 * r] * d0, u[j][2 * r + 1] * d1);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar + 8);
+        }
+    }
+
+    // ---- this warp's rows against the tiles of its chunk: forward products up to the diagonal tile, backward ones from it on
+    // (loops without the masks and the change of operands in them: those cost as many instructions as the products) ----
+    float o[NV][4];
+#pragma unroll
+    for (int n = 0; n < NV; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[n][e] = 0.f;
+    const DiagonalMask dmask(g, c);
+    const int nT = min(T - c0, 8), mine = w - c0;
+    // one tile of keys: scores with q~ (in qq), keep: 0 all of them, 1 columns up to the row, 2 columns from the row on
+    auto tile = [&](const uint32_t (&qq)[MP][4], uint32_t kt, uint32_t vt, int keep) {
+        float d0[4], d1[4];
+#pragma unroll
+        for (int m = 0; m < MP; ++m) {
+            uint32_t r[4];
+            t64.load_b(kt, 0, m, r);
+            if (m == 0) {
+                mma_k16_zero(d0, qq[0], r[0], r[1]);
+                mma_k16_zero(d1, qq[0], r[2], r[3]);
+            } else if (2 * m + 1 < NP) {
+                mma_k16(d0, qq[m], r[0], r[1]);
+                mma_k16(d1, qq[m], r[2], r[3]);
+            } else {
+                mma_k8(d0, qq[m][0], qq[m][1], r[0]);
+                mma_k8(d1, qq[m][0], qq[m][1], r[2]);
+            }
+        }
+        uint32_t p[4] = {pack_bf16(d0[0], d0[1]), pack_bf16(d0[2], d0[3]), pack_bf16(d1[0], d1[1]), pack_bf16(d1[2], d1[3])};
+        if (keep) dmask.apply(p, keep == 1);
+#pragma unroll
+        for (int n2 = 0; n2 < MV; ++n2) {
+            uint32_t r[4];
+            tvv.load_trans(vt, 0, n2, r);
+            mma_k16(o[2 * n2], p, r[0], r[1]);
+            mma_k16(o[2 * n2 + 1], p, r[2], r[3]);
+        }
+    };
+    {
+        uint32_t kt = tkf + (uint32_t)c0 * 1024, vt = tv + (uint32_t)c0 * 16 * RV;
+#pragma unroll 1
+        for (int j = 0; j < mine; ++j, kt += 1024, vt += 16 * RV) tile(qf, kt, vt, 0);
+        tile(qf, kt, vt, 1);
+        kt += tkb - tkf;
+        tile(qb, kt, vt, 2);
+#pragma unroll 1
+        for (int j = mine + 1; j < nT; ++j) {
+            kt += 1024;
+            vt += 16 * RV;
+            tile(qb, kt, vt, 0);
+        }
+    }
+    if (MAXT > 8 && T > 8) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar + 8, 0))) {   // (never expected: the warps of this block are all running)
+            if (lane == 0) atomicOr(args.dev_status, kDevStatusTimeout);
+            return;
+        }
+        auto state = [&](const uint32_t (&qq)[MP][4], uint32_t st) {
+#pragma unroll
+            for (int n2 = 0; n2 < MV; ++n2) {
+#pragma unroll
+                for (int m = 0; m < MP; ++m) {
+                    uint32_t r[4];
+                    t64.load_b(st, 16 * n2, m, r);
+                    if (2 * m + 1 < NP) {
+                        mma_k16(o[2 * n2], qq[m], r[0], r[1]);
+                        mma_k16(o[2 * n2 + 1], qq[m], r[2], r[3]);
+                    } else {
+                        mma_k8(o[2 * n2], qq[m][0], qq[m][1], r[0]);
+                        mma_k8(o[2 * n2 + 1], qq[m][0], qq[m][1], r[2]);
+                    }
+                }
+            }
+        };
+        if (ch == 0) state(qb, tst + MLayout<DV>::kState);
+        else state(qf, tst);
+    }
+    // ---- out: four 8-column tiles at a time turned so that a lane holds sixteen bytes of a row ----
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int row = 16 * w + 8 * r + g;
+        __nv_bfloat16* op = args.out + ((size_t)unit * L + row) * DV;
+#pragma unroll
+        for (int n4 = 0; n4 < NV; n4 += 4) {
+            uint32_t x[4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) x[n] = n4 + n < NV ? pack_bf16(o[n4 + n < NV ? n4 + n : 0][2 * r], o[n4 + n < NV ? n4 + n : 0][2 * r + 1]) : 0u;
+            transpose4(x, c);
+            if (row < L && n4 + c < NV) *reinterpret_cast<uint4*>(op + 8 * (n4 + c)) = make_uint4(x[0], x[1], x[2], x[3]);
+        }
+    }
+}
+
+template <int DK, int DV, bool GATES, int MAXT>
+cudaError_t launch_mma_t(MArgs a, int T, long long units, cudaStream_t stream) {
+    CUtensorMap tv;
+    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
+    const int threads = (T < 2 ? 2 : T) * 32;
+    const size_t tiles = MLayout<DV>(T).total, rec = (size_t)rec_plan(threads, DK, DV).smem_floats * 4;
+    static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    int sms = sms_of[dev].load(std::memory_order_acquire);
+    if (sms == 0) {
+        if ((e = cudaFuncSetAttribute(bigla_mma_kernel<DK, DV, GATES, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(bigla_mma_kernel<DK, DV, GATES, MAXT>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+            return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        sms_of[dev].store(sms, std::memory_order_release);
+    }
+    a.ahead = 2 * sms;
+    const cudaError_t le = launch_pdl(bigla_mma_kernel<DK, DV, GATES, MAXT>, dim3((unsigned)units), dim3(threads), tiles > rec ? tiles : rec, stream, tv, a);
+    count_launch();
+    return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+// Registers per thread follow from the longest unit an instance takes.
+template <int DK, int DV, bool GATES>
+cudaError_t launch_mma(const MArgs& a, long long units, cudaStream_t stream) {
+    const int T = (a.L + 15) / 16;
+    if (T <= 8) return launch_mma_t<DK, DV, GATES, 8>(a, T, units, stream);
+    if (T <= 13) return launch_mma_t<DK, DV, GATES, 13>(a, T, units, stream);
+    return launch_mma_t<DK, DV, GATES, 16>(a, T, units, stream);
+}
+
+}  // namespace
+
+// Where this form is the faster one, as units per SM up to which it is (measured against the tcgen05 form for head sizes of
+// 512 to 2048 state elements, 128 to 256 tokens, 16 to 1536 units).  Up to 128 tokens always, by 1.0 to 3 times.  With a
+// second chunk its work per token grows with the state while the other form's hand-overs cost the same, and above 208
+// tokens two blocks per SM leave 64 registers a thread: the larger the state, the fewer units it takes before the other
+// form, which has its latency hidden by then, catches up.  Gates prepared in the kernel cost this form less.
+bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
+    constexpr int kAlways = 1 << 20;
+    const int state = dk * dv;
+    int waves = kAlways;
+    if (L > 208) {
+        if (state > 1536) waves = 0;
+        else if (state > 1152) waves = 1;
+        else if (state > 768) waves = gates ? (dk == 32 ? 3 : kAlways) : 2;
+    } else if (L > 128) {
+        if (state > 1536) waves = 1;
+        else if (state > 1152) waves = gates ? 4 : 3;
+    }
+    if (waves == kAlways) return true;
+    static std::atomic<int> sms_of[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    int sms = sms_of[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+        sms_of[dev].store(sms, std::memory_order_relaxed);
+    }
+    return units <= (long long)waves * sms;
+}
+
+cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                             const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
+                             int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
+    MArgs a{q, k, v, la_f, la_b, out, L, (int)units, device_status_ptr(), gate_tau > 0.f ? 1.f / gate_tau : 0.f, 0, take_expire_next_wait()};
+    if (!a.dev_status) return cudaErrorUnknown;
+#define VIG_CASE(DK_, DV_) \
+    if (dk == DK_ && dv == DV_) return gate_tau > 0.f ? launch_mma<DK_, DV_, true>(a, units, stream) : launch_mma<DK_, DV_, false>(a, units, stream);
+    VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
+    VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
+    VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)
+#undef VIG_CASE
+    return cudaErrorNotSupported;
+}
+
+}  // namespace vig

@@ -54,6 +54,13 @@ cudaError_t launch_bigla_umma(const __nv_bfloat16* q, const __nv_bfloat16* k, co
                               const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out,
                               long long units, int L, int dk, int dv, float gate_tau, cudaStream_t stream);
 
+// The same on the warp-level tensor-core instructions, a block per unit, a warp per 16 tokens; mma_preferred: the shapes
+// (of those of umma_supported) it is the faster of the two for.
+bool mma_preferred(long long units, int L, int dk, int dv, bool gates);
+cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                             const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out,
+                             long long units, int L, int dk, int dv, float gate_tau, cudaStream_t stream);
+
 // ---- Eq. 7 around the mixer: depth-wise 3 x 3 convolution (channels last) and the 2-D gate blend ----
 bool dwconv_supported(int C, size_t elem);
 template <typename T>
