@@ -58,16 +58,35 @@ static bool use_segments(long long units, int L, int dk, int dv) {
     return units * nseg <= 2LL * sms;
 }
 
+static bool use_mma_chunks(long long units, int L, int dk, int dv, bool gates) {
+    return kernel_preference() == VIG_TEST_KERNEL_AUTO && !umma_supported(dk, dv, L) && mma_chunks_supported(units, L, dk, dv) &&
+           mma_chunks_preferred(units, L, dk, dv, gates);
+}
+
+// Scratch of the tcgen05 forms.
+static size_t umma_workspace_bytes(long long units, int L, int dk, int dv) {
+    return use_segments(units, L, dk, dv) ? umma_seg_workspace_bytes(units, L) : umma_long_workspace_bytes(units, L, dk, dv);
+}
+
 size_t tc_workspace_bytes(long long units, int L, int dk, int dv) {
     if (umma_supported(dk, dv, L)) return 0;   // one thread block covers a unit
-    if (use_segments(units, L, dk, dv)) return umma_seg_workspace_bytes(units, L);
-    return umma_long_workspace_bytes(units, L, dk, dv);
+    return use_mma_chunks(units, L, dk, dv, false) ? mma_chunks_workspace_bytes(units, L, dk, dv) : umma_workspace_bytes(units, L, dk, dv);
+}
+
+// The least a caller's scratch has to hold.
+size_t tc_least_workspace_bytes(long long units, int L, int dk, int dv) {
+    const size_t fast = tc_workspace_bytes(units, L, dk, dv);
+    if (fast == 0) return 0;
+    const size_t other = umma_workspace_bytes(units, L, dk, dv);
+    return other < fast ? other : fast;
 }
 
 cudaError_t launch_bigla_tc(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                             const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
-                            int L, int dk, int dv, void* ws, cudaStream_t stream) {
+                            int L, int dk, int dv, void* ws, size_t ws_bytes, cudaStream_t stream) {
     if (umma_supported(dk, dv, L)) return launch_bigla_umma(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, stream);
+    if (use_mma_chunks(units, L, dk, dv, false) && ws_bytes >= mma_chunks_workspace_bytes(units, L, dk, dv))
+        return launch_bigla_mma_chunks(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, ws, stream);
     if (use_segments(units, L, dk, dv)) return launch_bigla_umma_seg(q, k, v, la_f, la_b, out, units, L, dk, dv, ws, stream);
     return launch_bigla_umma_long(q, k, v, la_f, la_b, out, units, L, dk, dv, ws, stream);
 }
@@ -132,14 +151,14 @@ static int fwd_bf16_impl(const void* q, const void* k, const void* v, const void
     if (tc_supported(dk, dv) && kernel_preference() != VIG_TEST_KERNEL_SIMT) {
         const size_t need = tc_workspace_bytes(units, L, dk, dv);
         if (!own_ws && need > 0) {
-            if (!ws || ws_bytes < need || (reinterpret_cast<uintptr_t>(ws) & 255u)) return VIG_ERR_WORKSPACE;
+            if (!ws || ws_bytes < tc_least_workspace_bytes(units, L, dk, dv) || (reinterpret_cast<uintptr_t>(ws) & 255u)) return VIG_ERR_WORKSPACE;
         }
         if (empty) return VIG_OK;
         void* scratch = ws;
         if (own_ws && need > 0) {
             if (pool_alloc(&scratch, need, stream) != cudaSuccess) return VIG_ERR_CUDA;
         }
-        cudaError_t e = launch_bigla_tc(q_, k_, v_, f_, b_, (bf*)out, units, L, dk, dv, scratch, stream);
+        cudaError_t e = launch_bigla_tc(q_, k_, v_, f_, b_, (bf*)out, units, L, dk, dv, scratch, own_ws ? need : ws_bytes, stream);
         if (own_ws && need > 0) {
             if (cudaFreeAsync(scratch, stream) != cudaSuccess) return VIG_ERR_CUDA;
         }
@@ -151,8 +170,8 @@ static int fwd_bf16_impl(const void* q, const void* k, const void* v, const void
     return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
 }
 
-// Forward pass from the gate logits (Eq. 5 line 1 + Eq. 6).  Units of at most 256 tokens on the tensor-core shapes:
-// one kernel that prepares log alpha on chip.  Everything else: gate preparation into scratch of the stream, then the
+// Forward pass from the gate logits (Eq. 5 line 1 + Eq. 6).  Tensor-core shapes: log alpha is prepared on chip.  Everything
+// else: gate preparation into scratch of the stream, then the
 // ordinary forward pass.
 // o_local != NULL: followed by the 2-D gate blend of Eq. 7 lines 3-4 as an element-wise launch over `out` (programmatic
 // dependent launch: its set-up overlaps the forward kernel's tail, and it finds `out` in L2).  The blend inside the forward
@@ -174,6 +193,16 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     if (tc_supported(dk, dv) && umma_supported(dk, dv, L) && kernel_preference() == VIG_TEST_KERNEL_AUTO) {
         cudaError_t e = launch_bigla_umma((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out,
                                           units, L, dk, dv, tau, stream);
+        if (e == cudaSuccess && o_local)
+            e = launch_gate_blend<bf>((const bf*)o_local, (const bf*)z2d, (const bf*)out, (bf*)out, (long long)units * L * dv, stream);
+        return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
+    }
+    if (tc_supported(dk, dv) && use_mma_chunks(units, L, dk, dv, true)) {
+        void* ws = nullptr;
+        if (pool_alloc(&ws, mma_chunks_workspace_bytes(units, L, dk, dv), stream) != cudaSuccess) return VIG_ERR_CUDA;
+        cudaError_t e = launch_bigla_mma_chunks((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out, units, L, dk, dv, tau,
+                                                ws, stream);
+        if (cudaFreeAsync(ws, stream) != cudaSuccess) return VIG_ERR_CUDA;
         if (e == cudaSuccess && o_local)
             e = launch_gate_blend<bf>((const bf*)o_local, (const bf*)z2d, (const bf*)out, (bf*)out, (long long)units * L * dv, stream);
         return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;

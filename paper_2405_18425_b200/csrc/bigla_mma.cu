@@ -1,5 +1,7 @@
-// bf16 BiGLA forward for units of at most 256 tokens: one block per (batch, head) unit, one warp per 16 tokens, every
-// product a chain of 16 x 16 tiles whose scores stay in registers (mma.sync).
+// bf16 BiGLA forward on the warp-level tensor-core instructions (mma.sync): one warp per 16 tokens, every product a chain of
+// 16 x 16 tiles whose scores stay in registers.  Units of at most 256 tokens are one block each; longer sequences are cut
+// into chunks of up to 128 tokens, one block each, in three launches: the state every chunk adds in either direction, a
+// fold over the chunks, the chunks themselves from the states that enter them.
 //
 // With b_t the inclusive prefix sum of log alpha> and x_t the exclusive prefix sum of log alpha< (the backward decay from t
 // to s > t is exp(x_s - x_t): the gates t .. s-1), both from the start of a chunk of 128 tokens, Eq. 6 is, per chunk,
@@ -32,15 +34,25 @@ namespace {
 
 using namespace wmma16;
 
+#pragma nv_diag_suppress 128   // the summary instances return half way: the loops behind that are not reachable in them
+
+enum { kUnit = 0, kSummary = 1, kMain = 2 };
+constexpr int kChunkTiles = 8;        // 16-token tiles of a chunk at most
 constexpr float kGateRange = 60.f;    // largest decay of a chunk, as -log, that the factorised tiles take
 
 struct MArgs {
     const __nv_bfloat16 *q, *k, *v, *la_f, *la_b;   // GATES: la_f / la_b hold the gate logits
     __nv_bfloat16* out;
-    int L, units;
+    int L;
+    long long blocks;  // units (kUnit) or units x chunks
+    int nch, tiles;    // chunks per unit, tiles per chunk (long sequences)
+    float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
+    uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
+    float* ends;       // [unit][chunk][2][32]: sums of log alpha over the chunk
+    int* flags;        // [unit][chunk]: gates out of range
     int* dev_status;
     float inv_tau;
-    int ahead;         // the unit this many blocks on is pulled into L2
+    int ahead;         // the block this many further on has its inputs pulled into L2
     int expire_wait;   // test hook: every block lets one bounded wait, on an mbarrier nothing completes, run out
 };
 
@@ -49,29 +61,35 @@ template <int DV>
 struct MLayout {
     static constexpr uint32_t kVRow = DV == 32 ? 64 : 128, kState = DV * 64;
     uint32_t kf, kb, st, totals, bar, total;
-    __host__ __device__ explicit MLayout(int tiles) {
+    __host__ __device__ MLayout(int tiles, bool states) {
         const uint32_t rows = tiles * 16u;
         kf = rows * kVRow;
         kb = kf + rows * 64;
         st = kb + rows * 64;
-        totals = st + (tiles > 8 ? 2 * kState : 0);
+        totals = st + (states ? 2 * kState : 0);
         bar = totals + tiles * 256u;
         total = bar + 64;
     }
 };
 
-template <int DK, int DV, bool GATES, int MAXT>
+template <int DK, int DV, bool GATES, int MAXT, int MODE>
 __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const MArgs args) {
     constexpr int NP = DK / 8, MP = (NP + 1) / 2;   // 8-column tiles of the key dimensions, pairs of them
     constexpr int NV = DV / 8, MV = DV / 16;        // ... of the value dimensions
     constexpr int RV = MLayout<DV>::kVRow;
+    constexpr uint32_t kState = MLayout<DV>::kState;
+    constexpr bool kTwo = MODE == kUnit && MAXT > 8;   // units of two chunks
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int g = lane >> 2, c = lane & 3;
-    const int L = args.L, unit = blockIdx.x, T = (L + 15) >> 4;
+    const int L = args.L, nch = MODE == kUnit ? 1 : args.nch;
+    const int chunk = MODE == kUnit ? 0 : (int)(blockIdx.x % (unsigned)nch);
+    const size_t unit = MODE == kUnit ? blockIdx.x : blockIdx.x / (unsigned)nch;
+    const int Tall = (L + 15) >> 4, tiles = MODE == kUnit ? Tall : args.tiles;
+    const int tok0 = chunk * tiles * 16, T = min(tiles, Tall - chunk * tiles);   // this block's first token and its tiles
     const bool live = w < T;                          // (blocks have two warps at least: the in-kernel recurrence needs them)
-    const int ch = MAXT > 8 ? w >> 3 : 0, c0 = 8 * ch;   // this warp's chunk and its first tile
-    const MLayout<DV> lay(T);
+    const int ch = kTwo ? w >> 3 : 0, c0 = 8 * ch;    // this warp's chunk and its first tile
+    const MLayout<DV> lay(tiles, kTwo ? Tall > 8 : MODE == kMain);
     const uint32_t base = smem_u32(smem), tv = base, tkf = base + lay.kf, tkb = base + lay.kb, tst = base + lay.st, bar = base + lay.bar;
     float* totals = reinterpret_cast<float*>(smem + lay.totals);
     volatile int* slow = reinterpret_cast<volatile int*>(smem + lay.bar + 32);
@@ -79,28 +97,32 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
     pdl_launch_dependents();
     if (tid == 0) {
         mbar_init(bar, 1);
-        mbar_init(bar + 8, 2 * MV);   // one arrival per piece of the states
+        mbar_init(bar + 8, MODE == kMain ? 1 : 2 * MV);   // the states: one bulk copy, or one arrival per piece formed here
         mbar_init(bar + 16, 1);       // never completed: only the test hook waits on it
         *slow = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();
     if (tid == 0) {
-        mbar_expect_tx(bar, (uint32_t)T * 16 * RV);
-        tma_load_3d(tv, &tm_v, 0, 0, unit, bar);   // rows >= L and columns >= DV arrive as zeros
+        mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
+        tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
+        if (MODE == kMain) {
+            mbar_expect_tx(bar + 8, 2 * kState);
+            bulk_load(tst, args.img + (size_t)blockIdx.x * 2 * kState, 2 * kState, bar + 8);
+        }
     }
 
     // ---- this warp's 16 rows (g and g + 8) in fragment order: pair j of lane c ----
     uint32_t qr[2][NP], kr[2][NP], af[2][NP], ab[2][NP];
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int row = w * 16 + 8 * r + g;
-        if (row < L) {
-            const size_t at = ((size_t)unit * L + row) * DK;
+        const int row = tok0 + w * 16 + 8 * r + g;
+        if (live && row < L) {
+            const size_t at = (unit * L + row) * DK;
             load_pairs<DK>(args.la_f + at, c, af[r]);
             load_pairs<DK>(args.la_b + at, c, ab[r]);
             load_pairs<DK>(args.k + at, c, kr[r]);
-            load_pairs<DK>(args.q + at, c, qr[r]);
+            if (MODE != kSummary) load_pairs<DK>(args.q + at, c, qr[r]);
         } else {
 #pragma unroll
             for (int j = 0; j < NP; ++j) {   // rows past the end: q = k = 0 and no decay (GATES: a logit of 100, log alpha = 0)
@@ -109,13 +131,18 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
             }
         }
     }
-    if (tid == 0 && unit + args.ahead < args.units) {   // a block that starts when one of these is done finds its unit in L2
-        const size_t at = (size_t)(unit + args.ahead) * L;
-        prefetch_l2(args.la_f + at * DK, (uint32_t)L * DK * 2);
-        prefetch_l2(args.la_b + at * DK, (uint32_t)L * DK * 2);
-        prefetch_l2(args.k + at * DK, (uint32_t)L * DK * 2);
-        prefetch_l2(args.q + at * DK, (uint32_t)L * DK * 2);
-        prefetch_l2(args.v + at * DV, (uint32_t)L * DV * 2);
+    if (tid == 0 && blockIdx.x + (long long)args.ahead < args.blocks) {   // a block that starts when one of these is done finds its inputs in L2
+        const size_t next = blockIdx.x + (size_t)args.ahead;
+        const int nr = MODE == kUnit ? 0 : (int)(next % (unsigned)nch) * tiles * 16;
+        const size_t at = (MODE == kUnit ? next : next / (unsigned)nch) * L + nr;
+        const uint32_t n = min(tiles * 16, L - nr);
+        if (MODE != kMain) {   // (the summary launch has just read everything but q)
+            prefetch_l2(args.la_f + at * DK, n * DK * 2);
+            prefetch_l2(args.la_b + at * DK, n * DK * 2);
+            prefetch_l2(args.k + at * DK, n * DK * 2);
+            prefetch_l2(args.v + at * DV, n * DV * 2);
+        }
+        if (MODE != kSummary) prefetch_l2(args.q + at * DK, n * DK * 2);
     }
     // ---- gate totals of the tile; the gates turned, as B operands of products over the tokens ----
 #pragma unroll
@@ -150,7 +177,7 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
     };
     if (w == T - 1 && lane < DK) {   // range check: the decay of each chunk per key dim and direction
 #pragma unroll
-        for (int h = 0; h < (MAXT > 8 ? 2 : 1); ++h)
+        for (int h = 0; h < (kTwo ? 2 : 1); ++h)
 #pragma unroll
             for (int d = 0; d < 2; ++d) {
                 float s = 0.f;
@@ -187,11 +214,13 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
                         }
                         // the decaying factors on the special-function unit, the growing ones as their packed reciprocals
                         const uint32_t ef = pack_bf16(ex2(b0), ex2(b1)), eb = pack_bf16(ex2(x0), ex2(x1));
-                        const uint32_t hq = mul_bf16x2(qr[r][j], 0x3F003F00u);   // the 1/2 of the result: exact
                         kfw[2 * jj + r] = mul_bf16x2(kr[r][j], rcp_bf16x2(ef));
                         kbw[2 * jj + r] = mul_bf16x2(kr[r][j], eb);
-                        qf[m][2 * jj + r] = mul_bf16x2(hq, ef);
-                        qb[m][2 * jj + r] = mul_bf16x2(hq, rcp_bf16x2(eb));
+                        if (MODE != kSummary) {
+                            const uint32_t hq = mul_bf16x2(qr[r][j], 0x3F003F00u);   // the 1/2 of the result: exact
+                            qf[m][2 * jj + r] = mul_bf16x2(hq, ef);
+                            qb[m][2 * jj + r] = mul_bf16x2(hq, rcp_bf16x2(eb));
+                        }
                     }
                 } else {
 #pragma unroll
@@ -207,12 +236,27 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
     ok = mbar_wait_bounded(bar, 0) && ok;
     if (!__syncthreads_and(ok)) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
+        if (MODE == kMain) mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
         return;
     }
-    if (*slow) {   // gates beyond the range of the factorised tiles: Eq. 6 step by step, over the dead tiles
+    if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
+        float s = 0.f;
+        for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
+        args.ends[(size_t)blockIdx.x * 64 + tid] = s;
+        if (tid == 0) args.flags[blockIdx.x] = *slow;
+    }
+    bool redo = MODE == kUnit && *slow;
+    if (MODE == kMain) {
+        int any = 0;
+        for (int x = tid; x < nch; x += blockDim.x) any |= args.flags[unit * nch + x];
+        redo = __syncthreads_or(any);
+        if (redo) mbar_wait_bounded(bar + 8, 0);
+    }
+    if (redo) {   // gates beyond the range of the factorised tiles: Eq. 6 step by step, over the dead tiles, by one block of the unit
+        if (chunk != 0) return;
         if (tid == 0) atomicAdd(args.dev_status + 1, 1);
         __syncthreads();
-        const size_t okk = (size_t)unit * L * DK, ov = (size_t)unit * L * DV;
+        const size_t okk = unit * L * DK, ov = unit * L * DV;
         recurrence_unit<__nv_bfloat16>(args.q + okk, args.k + okk, args.v + ov, args.la_f + okk, args.la_b + okk, args.out + ov, L, DK, DV,
                                        reinterpret_cast<float*>(smem), args.inv_tau);
         return;
@@ -223,10 +267,10 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
 
     // ---- the states the chunks hand each other, transposed: rows of v times k~ over the tokens, 16 value columns a job; the
     // last warps first: theirs is the shorter chunk ----
-    if (MAXT > 8 && T > 8) {
+    if (MODE == kSummary || (kTwo && T > 8)) {
         for (int job = T - 1 - w; job < 2 * MV; job += T) {
-            const int dir = job & 1, mt = job >> 1;   // dir 0: chunk 0 -> 1 (forward);  dir 1: chunk 1 -> 0
-            const int t0 = dir == 0 ? 0 : 8, t1 = dir == 0 ? 8 : T;
+            const int dir = job & 1, mt = job >> 1;   // two chunks: dir 0: chunk 0 -> 1 (forward), dir 1: chunk 1 -> 0
+            const int t0 = MODE == kSummary || dir == 0 ? 0 : 8, t1 = kTwo && dir == 0 ? 8 : T;
             float u[2 * MP][4];
 #pragma unroll
             for (int j = 0; j < 2 * MP; ++j)
@@ -247,23 +291,29 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
                 }
             }
             f32x2 dec[NP];
-            sum_totals(dir, 0, 8, dec);
+            sum_totals(dir, 0, min(T, 8), dec);
 #pragma unroll
-            for (int j = 0; j < NP; ++j) {   // times chunk 0's decay: of what it leaves behind (forward), of what it takes in (backward)
+            for (int j = 0; j < NP; ++j) {
+                // two chunks: times chunk 0's decay, of what it leaves behind (forward), of what it takes in (backward); long
+                // sequences: the forward state alone decays to the chunk's end
                 float d0, d1;
                 unpack2(GATES ? dec[j] : fmul2(dec[j], pack2(kLog2e, kLog2e)), d0, d1);
-                d0 = ex2(d0);
-                d1 = ex2(d1);
+                d0 = MODE == kSummary && dir == 1 ? 1.f : ex2(d0);
+                d1 = MODE == kSummary && dir == 1 ? 1.f : ex2(d1);
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int n = 16 * mt + 8 * r + g;
-                    *reinterpret_cast<uint32_t*>(smem + lay.st + dir * MLayout<DV>::kState + n * 64 + ((j ^ ((n >> 1) & 3)) << 4) + 4 * c) =
-                        pack_bf16(u[j][2 * r] * d0, u[j][2 * r + 1] * d1);
+                    const float u0 = u[j][2 * r] * d0, u1 = u[j][2 * r + 1] * d1;
+                    if (MODE == kSummary)
+                        *reinterpret_cast<float2*>(args.u + (((size_t)blockIdx.x * 2 + dir) * DV + n) * DK + 8 * j + 2 * c) = make_float2(u0, u1);
+                    else
+                        *reinterpret_cast<uint32_t*>(smem + lay.st + dir * kState + n * 64 + ((j ^ ((n >> 1) & 3)) << 4) + 4 * c) = pack_bf16(u0, u1);
                 }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar + 8);
+            if (kTwo && lane == 0) mbar_arrive(bar + 8);
         }
+        if (MODE == kSummary) return;
     }
 
     // ---- this warp's rows against the tiles of its chunk: forward products up to the diagonal tile, backward ones from it on
@@ -317,8 +367,8 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
             tile(qb, kt, vt, 0);
         }
     }
-    if (MAXT > 8 && T > 8) {
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar + 8, 0))) {   // (never expected: the warps of this block are all running)
+    if (MODE == kMain || (kTwo && T > 8)) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar + 8, 0))) {   // (never expected where the warps of this block form the states)
             if (lane == 0) atomicOr(args.dev_status, kDevStatusTimeout);
             return;
         }
@@ -339,14 +389,20 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
                 }
             }
         };
-        if (ch == 0) state(qb, tst + MLayout<DV>::kState);
-        else state(qf, tst);
+        if (MODE == kMain) {   // (the first chunk's S> and the last one's S< are zero)
+            if (chunk > 0) state(qf, tst);
+            if (chunk + 1 < nch) state(qb, tst + kState);
+        } else if (ch == 0) {
+            state(qb, tst + kState);
+        } else {
+            state(qf, tst);
+        }
     }
     // ---- out: four 8-column tiles at a time turned so that a lane holds sixteen bytes of a row ----
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-        const int row = 16 * w + 8 * r + g;
-        __nv_bfloat16* op = args.out + ((size_t)unit * L + row) * DV;
+        const int row = tok0 + 16 * w + 8 * r + g;
+        __nv_bfloat16* op = args.out + (unit * L + row) * DV;
 #pragma unroll
         for (int n4 = 0; n4 < NV; n4 += 4) {
             uint32_t x[4];
@@ -358,12 +414,67 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
     }
 }
 
-template <int DK, int DV, bool GATES, int MAXT>
-cudaError_t launch_mma_t(MArgs a, int T, long long units, cudaStream_t stream) {
-    CUtensorMap tv;
-    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
-    const int threads = (T < 2 ? 2 : T) * 32;
-    const size_t tiles = MLayout<DV>(T).total, rec = (size_t)rec_plan(threads, DK, DV).smem_floats * 4;
+// Second launch of a long call: the states that enter every chunk from what the chunks add, S> ascending, in(c + 1) =
+// d>(c) in(c) + own(c), S< descending, in(c - 1) = d<(c) in(c) + own(c), stored times d<(c), the decay from the chunk's end to
+// its start.  A thread takes a pair of key dimensions of one value column over a run of chunks, eight loads in flight; GROUPS
+// runs of a sequence are taken side by side, first for what each adds and by how much it decays, then from the carry of the
+// runs before it (128 chunks as one run: 17.7 us).
+template <int DK, int DV, int GROUPS>
+__global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a, float scale) {
+    constexpr int P = DK / 2, kBatch = 8, kItems = 256 / GROUPS;
+    constexpr uint32_t kState = MLayout<DV>::kState;
+    __shared__ float2 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
+    const size_t unit = blockIdx.x;
+    const int dir = blockIdx.y, item = threadIdx.x % kItems, grp = threadIdx.x / kItems;
+    const int x = blockIdx.z * kItems + item, nch = a.nch;
+    const int run = (nch + GROUPS - 1) / GROUPS, i0 = min(nch, grp * run), i1 = min(nch, i0 + run);   // in walking order
+    const bool in = x < P * DV;
+    const int p = in ? x % P : 0, n = in ? x / P : 0;
+    pdl_launch_dependents();
+    pdl_wait();
+    float2 carry = make_float2(0.f, 0.f), decay = make_float2(1.f, 1.f);
+    auto walk = [&](bool emit) {
+        for (int b0 = i0; b0 < i1; b0 += kBatch) {
+            float2 own[kBatch], e[kBatch];
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+                if (b0 + b < i1) {
+                    const size_t ch = unit * nch + (dir == 0 ? b0 + b : nch - 1 - (b0 + b));
+                    own[b] = *reinterpret_cast<const float2*>(a.u + ((ch * 2 + dir) * DV + n) * DK + 2 * p);
+                    e[b] = *reinterpret_cast<const float2*>(a.ends + ch * 64 + dir * 32 + 2 * p);
+                }
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b)
+                if (b0 + b < i1) {
+                    const size_t ch = unit * nch + (dir == 0 ? b0 + b : nch - 1 - (b0 + b));
+                    const float2 d = make_float2(ex2(e[b].x * scale), ex2(e[b].y * scale));
+                    if (emit) {
+                        const uint32_t off = n * 64 + (((p >> 2) ^ ((n >> 1) & 3)) << 4) + 4 * (p & 3);
+                        *reinterpret_cast<uint32_t*>(a.img + (ch * 2 + dir) * kState + off) =
+                            dir == 0 ? pack_bf16(carry.x, carry.y) : pack_bf16(carry.x * d.x, carry.y * d.y);
+                    } else {
+                        decay = make_float2(decay.x * d.x, decay.y * d.y);
+                    }
+                    carry = make_float2(fmaf(d.x, carry.x, own[b].x), fmaf(d.y, carry.y, own[b].y));
+                }
+        }
+    };
+    if (GROUPS > 1) {
+        if (in) walk(false);
+        s_state[grp][item] = carry;
+        s_decay[grp][item] = decay;
+        __syncthreads();
+        carry = make_float2(0.f, 0.f);
+        for (int y = 0; y < grp; ++y)
+            carry = make_float2(fmaf(s_decay[y][item].x, carry.x, s_state[y][item].x), fmaf(s_decay[y][item].y, carry.y, s_state[y][item].y));
+    }
+    if (in) walk(true);
+}
+
+template <int DK, int DV, bool GATES, int MAXT, int MODE>
+cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t stream) {
+    const int threads = (tiles < 2 ? 2 : tiles) * 32;
+    const size_t smem = MLayout<DV>(tiles, MODE == kMain || (MODE == kUnit && tiles > 8)).total, rec = (size_t)rec_plan(threads, DK, DV).smem_floats * 4;
     static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -371,26 +482,64 @@ cudaError_t launch_mma_t(MArgs a, int T, long long units, cudaStream_t stream) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     int sms = sms_of[dev].load(std::memory_order_acquire);
     if (sms == 0) {
-        if ((e = cudaFuncSetAttribute(bigla_mma_kernel<DK, DV, GATES, MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(bigla_mma_kernel<DK, DV, GATES, MAXT>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
-            return e;
+        auto kernel = bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
-    a.ahead = 2 * sms;
-    const cudaError_t le = launch_pdl(bigla_mma_kernel<DK, DV, GATES, MAXT>, dim3((unsigned)units), dim3(threads), tiles > rec ? tiles : rec, stream, tv, a);
+    a.ahead = (MAXT <= 8 ? 3 : 2) * sms;
+    const cudaError_t le = launch_pdl(bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>, dim3((unsigned)a.blocks), dim3(threads), smem > rec ? smem : rec, stream, tv, a);
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
 }
 
 // Registers per thread follow from the longest unit an instance takes.
 template <int DK, int DV, bool GATES>
-cudaError_t launch_mma(const MArgs& a, long long units, cudaStream_t stream) {
+cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
     const int T = (a.L + 15) / 16;
-    if (T <= 8) return launch_mma_t<DK, DV, GATES, 8>(a, T, units, stream);
-    if (T <= 13) return launch_mma_t<DK, DV, GATES, 13>(a, T, units, stream);
-    return launch_mma_t<DK, DV, GATES, 16>(a, T, units, stream);
+    CUtensorMap tv;
+    if (!make_map(&tv, a.v, a.blocks, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
+    if (T <= 8) return launch_mma_t<DK, DV, GATES, 8, kUnit>(a, tv, T, stream);
+    if (T <= 13) return launch_mma_t<DK, DV, GATES, 13, kUnit>(a, tv, T, stream);
+    return launch_mma_t<DK, DV, GATES, 16, kUnit>(a, tv, T, stream);
+}
+
+// Sequences of any length: chunks of equal numbers of tiles.
+struct ChunkPlan {
+    int nch, tiles;
+    size_t u, img, ends, flags, total;   // byte offsets in the scratch
+};
+ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
+    ChunkPlan p;
+    const int T = (L + 15) / 16;
+    p.nch = (T + kChunkTiles - 1) / kChunkTiles;
+    p.tiles = (T + p.nch - 1) / p.nch;
+    p.nch = (T + p.tiles - 1) / p.tiles;
+    const size_t n = (size_t)units * p.nch;
+    p.u = 0;
+    p.img = n * 2 * dk * dv * 4;
+    p.ends = p.img + n * 2 * dv * 64;
+    p.flags = p.ends + n * 64 * 4;
+    p.total = (p.flags + n * 4 + 255) / 256 * 256;
+    return p;
+}
+
+template <int DK, int DV, bool GATES>
+cudaError_t launch_chunks(const MArgs& a, long long units, cudaStream_t stream) {
+    CUtensorMap tv;
+    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
+    cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
+    if (e != cudaSuccess) return e;
+    constexpr int kGroups = 8, kWork = DK / 2 * DV;
+    const float scale = GATES ? 1.f : kLog2e;
+    if (a.nch > 8)
+        e = launch_pdl(mma_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 2, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0, stream, a, scale);
+    else
+        e = launch_pdl(mma_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 2, (kWork + 255) / 256), dim3(256), 0, stream, a, scale);
+    count_launch();
+    if (e != cudaSuccess) return e;
+    return launch_mma_t<DK, DV, GATES, 8, kMain>(a, tv, a.tiles, stream);
 }
 
 }  // namespace
@@ -427,10 +576,49 @@ bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
 cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                              const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                              int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
-    MArgs a{q, k, v, la_f, la_b, out, L, (int)units, device_status_ptr(), gate_tau > 0.f ? 1.f / gate_tau : 0.f, 0, take_expire_next_wait()};
+    MArgs a{};
+    a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
+    a.L = L; a.blocks = units;
+    a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
+    a.expire_wait = take_expire_next_wait();
+    a.dev_status = device_status_ptr();
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_) \
-    if (dk == DK_ && dv == DV_) return gate_tau > 0.f ? launch_mma<DK_, DV_, true>(a, units, stream) : launch_mma<DK_, DV_, false>(a, units, stream);
+    if (dk == DK_ && dv == DV_) return gate_tau > 0.f ? launch_mma<DK_, DV_, true>(a, stream) : launch_mma<DK_, DV_, false>(a, stream);
+    VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
+    VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
+    VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)
+#undef VIG_CASE
+    return cudaErrorNotSupported;
+}
+
+#ifndef VIG_CH_RULE
+#define VIG_CH_RULE true
+#endif
+bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) { return VIG_CH_RULE; }
+
+bool mma_chunks_supported(long long units, int L, int dk, int dv) { return units * chunk_plan(units, L, dk, dv).nch <= 0x7fffffffLL; }
+
+size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv) { return chunk_plan(units, L, dk, dv).total; }
+
+cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                                    const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
+                                    int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream) {
+    const ChunkPlan p = chunk_plan(units, L, dk, dv);
+    char* b = static_cast<char*>(ws);
+    MArgs a{};
+    a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
+    a.L = L; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
+    a.u = reinterpret_cast<float*>(b + p.u);
+    a.img = reinterpret_cast<uint8_t*>(b + p.img);
+    a.ends = reinterpret_cast<float*>(b + p.ends);
+    a.flags = reinterpret_cast<int*>(b + p.flags);
+    a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
+    a.dev_status = device_status_ptr();
+    if (!a.dev_status) return cudaErrorUnknown;
+#define VIG_CASE(DK_, DV_)        \
+    if (dk == DK_ && dv == DV_) \
+        return gate_tau > 0.f ? launch_chunks<DK_, DV_, true>(a, units, stream) : launch_chunks<DK_, DV_, false>(a, units, stream);
     VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
     VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
     VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)

@@ -51,7 +51,7 @@ extern "C" int vig_bigla_fwd_static_bf16(const void* q, const void* k, const voi
         if (reinterpret_cast<uintptr_t>(p) & 15u) return VIG_ERR_MISALIGNED;
     if (!tc_supported(dk, dv) || (long long)B * H > 0x7fffffffLL) return VIG_ERR_UNSUPPORTED;
     const long long units = (long long)B * H;
-    const size_t need = tc_workspace_bytes(units, L, dk, dv);
+    const size_t need = tc_least_workspace_bytes(units, L, dk, dv);
     if (need > (size_t)VIG_STATIC_SCRATCH_BYTES) return VIG_ERR_WORKSPACE;   // beyond the fixed scratch: use the _ws form
     if (B == 0 || H == 0 || L == 0) return VIG_OK;
     void* scratch = nullptr;
@@ -59,7 +59,7 @@ extern "C" int vig_bigla_fwd_static_bf16(const void* q, const void* k, const voi
     // Nothing in the scratch has to survive from call to call, and nothing in it has to start at zero: every word
     // a launch reads to form the result was written earlier in the same call.
     cudaError_t e = launch_bigla_tc((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)log_alpha_fwd,
-                                     (const bf*)log_alpha_bwd, (bf*)out, units, L, dk, dv, scratch,
+                                     (const bf*)log_alpha_bwd, (bf*)out, units, L, dk, dv, scratch, (size_t)VIG_STATIC_SCRATCH_BYTES,
                                      (cudaStream_t)stream);
     return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
 }

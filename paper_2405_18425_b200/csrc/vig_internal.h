@@ -43,9 +43,11 @@ cudaError_t launch_gate_prep_bwd(const T* g_f, const T* g_b, const T* d_f, const
 bool tc_supported(int dk, int dv);
 // Scratch bytes the tensor-core path needs for this shape; 0 if no launch of it uses scratch.
 size_t tc_workspace_bytes(long long units, int L, int dk, int dv);
+size_t tc_least_workspace_bytes(long long units, int L, int dk, int dv);   // what the form that needs least takes
+// ws_bytes: what there is of it; a form that needs less is taken where the fastest one does not fit.
 cudaError_t launch_bigla_tc(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                             const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out,
-                            long long units, int L, int dk, int dv, void* ws, cudaStream_t stream);
+                            long long units, int L, int dk, int dv, void* ws, size_t ws_bytes, cudaStream_t stream);
 
 // ---- bf16 tcgen05 / TMEM path (units of at most 256 tokens) ----
 bool umma_supported(int dk, int dv, int L);
@@ -60,6 +62,15 @@ bool mma_preferred(long long units, int L, int dk, int dv, bool gates);
 cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                              const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out,
                              long long units, int L, int dk, int dv, float gate_tau, cudaStream_t stream);
+
+// Longer sequences on the same instructions: chunks of up to 128 tokens, states through scratch (three launches), the gates
+// prepared on the way as well.  mma_chunks_preferred: the shapes it is the faster form for.
+bool mma_chunks_supported(long long units, int L, int dk, int dv);
+bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates);
+size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv);
+cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                                    const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
+                                    int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream);
 
 // ---- Eq. 7 around the mixer: depth-wise 3 x 3 convolution (channels last) and the 2-D gate blend ----
 bool dwconv_supported(int C, size_t elem);
