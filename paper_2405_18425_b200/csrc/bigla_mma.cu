@@ -48,7 +48,7 @@ struct MArgs {
     int nch, tiles;    // chunks per unit, tiles per chunk (long sequences)
     float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
     uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
-    float* ends;       // [unit][chunk][2][32]: sums of log alpha over the chunk
+    float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
     int* flags;        // [unit][chunk]: gates out of range
     int* dev_status;
     float inv_tau;
@@ -72,8 +72,14 @@ struct MLayout {
     }
 };
 
+// Blocks per SM the registers are held to (four blocks of the other forms would leave 64 registers a thread: 19 us against 15
+// at 768 units of 100 tokens, 32 x 64).
+constexpr int mma_blocks_per_sm(int dk, int dv, int max_tiles, int mode) {
+    return max_tiles > 8 ? 2 : (mode == kSummary && dk * dv <= 1152 ? 4 : 3);
+}
+
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
-__global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const MArgs args) {
+__global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MODE)) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const MArgs args) {
     constexpr int NP = DK / 8, MP = (NP + 1) / 2;   // 8-column tiles of the key dimensions, pairs of them
     constexpr int NV = DV / 8, MV = DV / 16;        // ... of the value dimensions
     constexpr int RV = MLayout<DV>::kVRow;
@@ -242,7 +248,7 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
     if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
         float s = 0.f;
         for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
-        args.ends[(size_t)blockIdx.x * 64 + tid] = s;
+        args.decay[(size_t)blockIdx.x * 64 + tid] = ex2(GATES ? s : s * kLog2e);
         if (tid == 0) args.flags[blockIdx.x] = *slow;
     }
     bool redo = MODE == kUnit && *slow;
@@ -416,57 +422,67 @@ __global__ void __launch_bounds__(MAXT * 32, MAXT <= 8 ? 3 : 2) bigla_mma_kernel
 
 // Second launch of a long call: the states that enter every chunk from what the chunks add, S> ascending, in(c + 1) =
 // d>(c) in(c) + own(c), S< descending, in(c - 1) = d<(c) in(c) + own(c), stored times d<(c), the decay from the chunk's end to
-// its start.  A thread takes a pair of key dimensions of one value column over a run of chunks, eight loads in flight; GROUPS
-// runs of a sequence are taken side by side, first for what each adds and by how much it decays, then from the carry of the
-// runs before it (128 chunks as one run: 17.7 us).
+// its start.  A thread takes four key dimensions of one value column over a run of chunks, eight loads in flight.  GROUPS
+// runs of a long sequence are taken side by side, first for what each adds and by how much it decays, then from the carry of
+// the runs before it (128 chunks as one run: 17.7 us, bound by the round trips of sixteen batches).
 template <int DK, int DV, int GROUPS>
-__global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a, float scale) {
-    constexpr int P = DK / 2, kBatch = 8, kItems = 256 / GROUPS;
-    constexpr uint32_t kState = MLayout<DV>::kState;
-    __shared__ float2 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
+__global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a) {
+    constexpr int P = DK / 4, kBatch = 8, kItems = 256 / GROUPS;
+    constexpr int kState = (int)MLayout<DV>::kState;
+    __shared__ float4 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
     const size_t unit = blockIdx.x;
     const int dir = blockIdx.y, item = threadIdx.x % kItems, grp = threadIdx.x / kItems;
     const int x = blockIdx.z * kItems + item, nch = a.nch;
     const int run = (nch + GROUPS - 1) / GROUPS, i0 = min(nch, grp * run), i1 = min(nch, i0 + run);   // in walking order
     const bool in = x < P * DV;
     const int p = in ? x % P : 0, n = in ? x / P : 0;
+    const ptrdiff_t step = dir == 0 ? 1 : -1;
+    const size_t first = unit * nch + (dir == 0 ? i0 : nch - 1 - i0);
+    const float* own0 = a.u + ((first * 2 + dir) * DV + n) * DK + 4 * p;
+    const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
+    uint8_t* img = a.img + (first * 2 + dir) * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
     pdl_launch_dependents();
     pdl_wait();
-    float2 carry = make_float2(0.f, 0.f), decay = make_float2(1.f, 1.f);
+    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
     auto walk = [&](bool emit) {
+        const float *own_p = own0, *dec_p = dec0;
         for (int b0 = i0; b0 < i1; b0 += kBatch) {
-            float2 own[kBatch], e[kBatch];
+            float4 own[kBatch], d[kBatch];
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b)
+            for (int b = 0; b < kBatch; ++b) {
                 if (b0 + b < i1) {
-                    const size_t ch = unit * nch + (dir == 0 ? b0 + b : nch - 1 - (b0 + b));
-                    own[b] = *reinterpret_cast<const float2*>(a.u + ((ch * 2 + dir) * DV + n) * DK + 2 * p);
-                    e[b] = *reinterpret_cast<const float2*>(a.ends + ch * 64 + dir * 32 + 2 * p);
+                    own[b] = *reinterpret_cast<const float4*>(own_p);
+                    d[b] = *reinterpret_cast<const float4*>(dec_p);
+                    own_p += step * (2 * DV * DK);
+                    dec_p += step * 64;
                 }
+            }
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b)
+            for (int b = 0; b < kBatch; ++b) {
                 if (b0 + b < i1) {
-                    const size_t ch = unit * nch + (dir == 0 ? b0 + b : nch - 1 - (b0 + b));
-                    const float2 d = make_float2(ex2(e[b].x * scale), ex2(e[b].y * scale));
                     if (emit) {
-                        const uint32_t off = n * 64 + (((p >> 2) ^ ((n >> 1) & 3)) << 4) + 4 * (p & 3);
-                        *reinterpret_cast<uint32_t*>(a.img + (ch * 2 + dir) * kState + off) =
-                            dir == 0 ? pack_bf16(carry.x, carry.y) : pack_bf16(carry.x * d.x, carry.y * d.y);
+                        *reinterpret_cast<uint2*>(img) = dir == 0 ? make_uint2(pack_bf16(carry.x, carry.y), pack_bf16(carry.z, carry.w))
+                                                                  : make_uint2(pack_bf16(carry.x * d[b].x, carry.y * d[b].y), pack_bf16(carry.z * d[b].z, carry.w * d[b].w));
+                        img += step * (2 * kState);
                     } else {
-                        decay = make_float2(decay.x * d.x, decay.y * d.y);
+                        all = make_float4(all.x * d[b].x, all.y * d[b].y, all.z * d[b].z, all.w * d[b].w);
                     }
-                    carry = make_float2(fmaf(d.x, carry.x, own[b].x), fmaf(d.y, carry.y, own[b].y));
+                    carry = make_float4(fmaf(d[b].x, carry.x, own[b].x), fmaf(d[b].y, carry.y, own[b].y), fmaf(d[b].z, carry.z, own[b].z),
+                                        fmaf(d[b].w, carry.w, own[b].w));
                 }
+            }
         }
     };
     if (GROUPS > 1) {
         if (in) walk(false);
         s_state[grp][item] = carry;
-        s_decay[grp][item] = decay;
+        s_decay[grp][item] = all;
         __syncthreads();
-        carry = make_float2(0.f, 0.f);
-        for (int y = 0; y < grp; ++y)
-            carry = make_float2(fmaf(s_decay[y][item].x, carry.x, s_state[y][item].x), fmaf(s_decay[y][item].y, carry.y, s_state[y][item].y));
+        carry = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int y = 0; y < grp; ++y) {
+            const float4 s = s_state[y][item], d = s_decay[y][item];
+            carry = make_float4(fmaf(d.x, carry.x, s.x), fmaf(d.y, carry.y, s.y), fmaf(d.z, carry.z, s.z), fmaf(d.w, carry.w, s.w));
+        }
     }
     if (in) walk(true);
 }
@@ -488,7 +504,7 @@ cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
-    a.ahead = (MAXT <= 8 ? 3 : 2) * sms;
+    a.ahead = mma_blocks_per_sm(DK, DV, MAXT, MODE) * sms;
     const cudaError_t le = launch_pdl(bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>, dim3((unsigned)a.blocks), dim3(threads), smem > rec ? smem : rec, stream, tv, a);
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -508,7 +524,7 @@ cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
 // Sequences of any length: chunks of equal numbers of tiles.
 struct ChunkPlan {
     int nch, tiles;
-    size_t u, img, ends, flags, total;   // byte offsets in the scratch
+    size_t u, img, decay, flags, total;   // byte offsets in the scratch
 };
 ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
     ChunkPlan p;
@@ -519,8 +535,8 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
     const size_t n = (size_t)units * p.nch;
     p.u = 0;
     p.img = n * 2 * dk * dv * 4;
-    p.ends = p.img + n * 2 * dv * 64;
-    p.flags = p.ends + n * 64 * 4;
+    p.decay = p.img + n * 2 * dv * 64;
+    p.flags = p.decay + n * 64 * 4;
     p.total = (p.flags + n * 4 + 255) / 256 * 256;
     return p;
 }
@@ -531,12 +547,11 @@ cudaError_t launch_chunks(const MArgs& a, long long units, cudaStream_t stream) 
     if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
     if (e != cudaSuccess) return e;
-    constexpr int kGroups = 8, kWork = DK / 2 * DV;
-    const float scale = GATES ? 1.f : kLog2e;
-    if (a.nch > 8)
-        e = launch_pdl(mma_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 2, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0, stream, a, scale);
+    constexpr int kGroups = 8, kWork = DK / 4 * DV;
+    if (a.nch > 24)
+        e = launch_pdl(mma_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 2, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0, stream, a);
     else
-        e = launch_pdl(mma_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 2, (kWork + 255) / 256), dim3(256), 0, stream, a, scale);
+        e = launch_pdl(mma_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 2, (kWork + 255) / 256), dim3(256), 0, stream, a);
     count_launch();
     if (e != cudaSuccess) return e;
     return launch_mma_t<DK, DV, GATES, 8, kMain>(a, tv, a.tiles, stream);
@@ -592,10 +607,23 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
     return cudaErrorNotSupported;
 }
 
-#ifndef VIG_CH_RULE
-#define VIG_CH_RULE true
-#endif
-bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) { return VIG_CH_RULE; }
+// Where the chunks run faster this way than as tcgen05 segments or chunk tasks (measured for head sizes of 512 to 2048 state
+// elements, 257 to 16384 tokens, 1 to 600 units).  Few chunks: always, by 1.1 to 1.8 times - a chunk's chain of dependent
+// steps is shorter.  Many chunks: the tcgen05 tasks have their latency hidden and cost the same whatever the state, so only
+// small states, and gates that would otherwise be prepared by a launch of their own, keep the advantage.  The segmented
+// launch is at its best where two segments of every unit just fill the chip.
+bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
+    if (dk == 16) return true;
+    const long long chunks = units * ((L + 127) / 128);
+    constexpr int kSms = 148;
+    if (dk == 24 && dv <= 48) {
+        if (gates) return L <= 1100 || chunks <= 8 * kSms;
+        return (L <= 1100 || chunks <= 4 * kSms) && !(L > 300 && L <= 512 && units > 40 && units <= kSms);
+    }
+    if (chunks <= 64 || (L > 8192 && units <= 4)) return true;
+    if (dk * dv <= 1024 && gates && (L <= 400 || (L > 512 && L <= 800))) return true;
+    return L <= 300 && (gates || units > kSms);
+}
 
 bool mma_chunks_supported(long long units, int L, int dk, int dv) { return units * chunk_plan(units, L, dk, dv).nch <= 0x7fffffffLL; }
 
@@ -611,7 +639,7 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
     a.L = L; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
     a.u = reinterpret_cast<float*>(b + p.u);
     a.img = reinterpret_cast<uint8_t*>(b + p.img);
-    a.ends = reinterpret_cast<float*>(b + p.ends);
+    a.decay = reinterpret_cast<float*>(b + p.decay);
     a.flags = reinterpret_cast<int*>(b + p.flags);
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.dev_status = device_status_ptr();
