@@ -51,7 +51,7 @@ struct GArgs {
     int L, nch, tiles;      // tokens, chunks per unit, tiles per chunk
     float* u;               // [unit][chunk][kind][DV][DK] fp32: the chunks' own states (kinds S>, Z<, S<, Z>)
     uint8_t* img;           // [unit][chunk][kind][hi, lo][DV][64 B]: the states entering a chunk, as shared-memory tiles
-    float* ends;            // [unit][chunk][2][32]: sums of log alpha>, log alpha< over the chunk
+    float* decay;           // [unit][chunk][2][32]: products of alpha>, alpha< over the chunk
     int* flags;             // [unit][chunk]: gates out of range
     long long chunks;       // of the call
     int ahead;              // the chunk this many blocks on is pulled into L2
@@ -405,7 +405,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
         if (MODE == kSummary) {
             for (int x = tid; x < 64; x += nw * 32)
-                if ((x & 31) < DK) a.ends[(unit * nch + chunk) * 64 + x] = ends[x];
+                if ((x & 31) < DK) a.decay[(unit * nch + chunk) * 64 + x] = ex2(ends[x] * kLog2e);
             if (tid == 0) a.flags[unit * nch + chunk] = state_word[0];
             return;
         }
@@ -827,45 +827,73 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
 }
 
 // Second launch of a long call: the states entering every chunk, from the chunks' own: S> and Z< ascending, in(c + 1) =
-// d(c) in(c) + own(c); S< and Z> descending, in(c - 1) = d(c) in(c) + own(c).  One block per (unit, kind), one thread per
-// pair of key dimensions of one value column; the loads of eight chunks are in flight together.
-template <int DK, int DV>
+// d(c) in(c) + own(c); S< and Z> descending, in(c - 1) = d(c) in(c) + own(c).  A thread takes four key dimensions of one value
+// column over a run of chunks, eight loads in flight; GROUPS runs of a long sequence are taken side by side, first for what
+// each adds and by how much it decays, then from the carry of the runs before it.
+template <int DK, int DV, int GROUPS>
 __global__ void __launch_bounds__(256) grad_fold_kernel(const GArgs a) {
-    constexpr int P = DK / 2, kBatch = 8;
-    constexpr uint32_t kState = GLayout<DV>::kState;
+    constexpr int P = DK / 4, kBatch = 8, kItems = 256 / GROUPS;
+    constexpr int kState = (int)GLayout<DV>::kState;
+    __shared__ float4 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
     const size_t unit = blockIdx.x;
     const int kind = blockIdx.y, dir = (kind == 0 || kind == 3) ? 0 : 1;   // S>, Z> decay by log alpha>
     const bool up = kind < 2;
+    const int item = threadIdx.x % kItems, grp = threadIdx.x / kItems, x = blockIdx.z * kItems + item, nch = a.nch;
+    const int run = (nch + GROUPS - 1) / GROUPS, i0 = min(nch, grp * run), i1 = min(nch, i0 + run);   // in walking order
+    const bool in = x < P * DV;
+    const int p = in ? x % P : 0, n = in ? x / P : 0;
+    const ptrdiff_t step = up ? 1 : -1;
+    const size_t first = unit * nch + (up ? i0 : nch - 1 - i0);
+    const float* own0 = a.u + ((first * 4 + kind) * DV + n) * DK + 4 * p;
+    const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
+    uint8_t* img = a.img + (first * 4 + kind) * 2 * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
     pdl_launch_dependents();
     pdl_wait();
-    const int x = blockIdx.z * 256 + threadIdx.x;
-    if (x >= P * DV) return;
-    const int p = x % P, n = x / P;
-    float2 carry = make_float2(0.f, 0.f);
-    const uint32_t off = n * 64 + (((p >> 2) ^ ((n >> 1) & 3)) << 4) + 4 * (p & 3);
-    for (int c0 = 0; c0 < a.nch; c0 += kBatch) {
-        float2 own[kBatch], e[kBatch];
+    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
+    auto walk = [&](bool emit) {
+        const float *own_p = own0, *dec_p = dec0;
+        for (int b0 = i0; b0 < i1; b0 += kBatch) {
+            float4 own[kBatch], d[kBatch];
 #pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            if (c0 + b < a.nch) {
-                const int ch = up ? c0 + b : a.nch - 1 - (c0 + b);
-                own[b] = *reinterpret_cast<const float2*>(a.u + (((unit * a.nch + ch) * 4 + kind) * DV + n) * DK + 2 * p);
-                e[b] = *reinterpret_cast<const float2*>(a.ends + (unit * a.nch + ch) * 64 + dir * 32 + 2 * p);
+            for (int b = 0; b < kBatch; ++b) {
+                if (b0 + b < i1) {
+                    own[b] = *reinterpret_cast<const float4*>(own_p);
+                    d[b] = *reinterpret_cast<const float4*>(dec_p);
+                    own_p += step * (4 * DV * DK);
+                    dec_p += step * 64;
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < kBatch; ++b) {
+                if (b0 + b < i1) {
+                    if (emit) {
+                        uint2 hi, lo;
+                        split_bf16(pack2(carry.x, carry.y), hi.x, lo.x);
+                        split_bf16(pack2(carry.z, carry.w), hi.y, lo.y);
+                        *reinterpret_cast<uint2*>(img) = hi;
+                        *reinterpret_cast<uint2*>(img + kState) = lo;
+                        img += step * (8 * kState);
+                    } else {
+                        all = make_float4(all.x * d[b].x, all.y * d[b].y, all.z * d[b].z, all.w * d[b].w);
+                    }
+                    carry = make_float4(fmaf(d[b].x, carry.x, own[b].x), fmaf(d[b].y, carry.y, own[b].y), fmaf(d[b].z, carry.z, own[b].z),
+                                        fmaf(d[b].w, carry.w, own[b].w));
+                }
             }
         }
-#pragma unroll
-        for (int b = 0; b < kBatch; ++b) {
-            if (c0 + b < a.nch) {
-                const int ch = up ? c0 + b : a.nch - 1 - (c0 + b);
-                uint32_t hi, lo;
-                split_bf16(pack2(carry.x, carry.y), hi, lo);
-                uint8_t* q = a.img + ((unit * a.nch + ch) * 4 + kind) * 2 * kState + off;
-                *reinterpret_cast<uint32_t*>(q) = hi;
-                *reinterpret_cast<uint32_t*>(q + kState) = lo;
-                carry = make_float2(fmaf(ex2(e[b].x * kLog2e), carry.x, own[b].x), fmaf(ex2(e[b].y * kLog2e), carry.y, own[b].y));
-            }
+    };
+    if (GROUPS > 1) {
+        if (in) walk(false);
+        s_state[grp][item] = carry;
+        s_decay[grp][item] = all;
+        __syncthreads();
+        carry = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int y = 0; y < grp; ++y) {
+            const float4 s = s_state[y][item], d = s_decay[y][item];
+            carry = make_float4(fmaf(d.x, carry.x, s.x), fmaf(d.y, carry.y, s.y), fmaf(d.z, carry.z, s.z), fmaf(d.w, carry.w, s.w));
         }
     }
+    if (in) walk(true);
 }
 
 // How a sequence is cut: one chunk of up to eight tiles, two of up to seven, else chunks of six.
@@ -879,7 +907,7 @@ GPlan grad_plan(int L) {
     return {kMain, max_tiles(kMain), (T + max_tiles(kMain) - 1) / max_tiles(kMain)};
 }
 struct GScratch {
-    size_t u, img, ends, flags, total;   // byte offsets
+    size_t u, img, decay, flags, total;   // byte offsets
 };
 GScratch grad_scratch(const GPlan& p, long long units, int dk, int dv) {
     GScratch s{};
@@ -887,8 +915,8 @@ GScratch grad_scratch(const GPlan& p, long long units, int dk, int dv) {
     const size_t n = (size_t)units * p.nch;
     s.u = 0;
     s.img = n * 4 * dk * dv * 4;
-    s.ends = s.img + n * 8 * dv * 64;
-    s.flags = s.ends + n * 64 * 4;
+    s.decay = s.img + n * 8 * dv * 64;
+    s.flags = s.decay + n * 64 * 4;
     s.total = (s.flags + n * 4 + 255) / 256 * 256;
     return s;
 }
@@ -950,7 +978,12 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
         e = launch_grad(bigla_grad_kernel<DK, DV, kSummary>, grid, threads(kSummary), GLayout<DV>(p.tiles, kSummary).total, false, stream, tq, tk, tf, tb, tv, tg, a);
         if (e == cudaSuccess) {
             count_launch();
-            e = launch_pdl(grad_fold_kernel<DK, DV>, dim3((unsigned)units, 4, (DK / 2 * DV + 255) / 256), dim3(256), 0, stream, a);
+            constexpr int kGroups = 8, kWork = DK / 4 * DV;
+            if (p.nch > 24)
+                e = launch_pdl(grad_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 4, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0,
+                               stream, a);
+            else
+                e = launch_pdl(grad_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 4, (kWork + 255) / 256), dim3(256), 0, stream, a);
         }
         if (e == cudaSuccess)
             e = launch_grad(bigla_grad_kernel<DK, DV, kMain>, grid, threads(kMain), GLayout<DV>(p.tiles, kMain).total, false, stream, tq, tk, tf, tb, tv, tg, a);
@@ -975,7 +1008,7 @@ cudaError_t launch_bigla_grad(const __nv_bfloat16* q, const __nv_bfloat16* k, co
     const GScratch s = grad_scratch(p, units, dk, dv);
     char* b = static_cast<char*>(scratch);
     GArgs a{q, k, v, la_f, la_b, d_out, dq, dk_out, dv_out, dla_f, dla_b, L, p.nch, p.tiles,
-            reinterpret_cast<float*>(b + s.u), reinterpret_cast<uint8_t*>(b + s.img), reinterpret_cast<float*>(b + s.ends),
+            reinterpret_cast<float*>(b + s.u), reinterpret_cast<uint8_t*>(b + s.img), reinterpret_cast<float*>(b + s.decay),
             reinterpret_cast<int*>(b + s.flags), units * p.nch, 0, device_status_ptr()};
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_) \
