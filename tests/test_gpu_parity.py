@@ -446,6 +446,24 @@ def test_fused_gates_small_and_ragged(oracle, dk, dv, L):
     assert rel_err(got, ref) <= TOL["bf16"]
 
 
+@pytest.mark.parametrize("dk,dv", [(16, 48), (24, 32), (24, 64), (32, 48)])
+@pytest.mark.parametrize("L", [15, 112, 128, 129, 208, 209, 256, 257, 384, 385, 1025, 3201])
+def test_warp_tile_forward_edges(oracle, dk, dv, L):
+    """Few units, so that every shape takes the kernels of one warp per 16 tokens: the edges of their tiles, of the instances
+    for 8, 13 and 16 tiles, of two chunks, of many (the fold in one run and in eight), both entry points.  Beyond 256 tokens
+    one unit leaves the range of the factorised tiles, so that its chunks go through the recurrence beside ordinary units."""
+    cfg, x = random_problem(2600 + L, 1, 3, L, dk, dv, "bf16", gate_mean=1.0)
+    if L > 256:
+        for name in ("g_fwd", "g_bwd"):
+            g = synth.stored_to_f64(x[name], "bf16").copy()
+            g[0, 1, L // 2] = -2000.0
+            x[name] = synth.store(g, "bf16")
+    for run in (_run_fused, _run_unfused):
+        got, ref = run(oracle, cfg, x)
+        for h in range(3):
+            assert rel_err(got[:, h], ref[:, h]) <= TOL["bf16"]
+
+
 @pytest.mark.parametrize("tau", [1.0, 3.0, 16.0, 64.0])
 def test_fused_gates_temperature_and_extreme_logits(oracle, tau):
     """tau = 1 makes the gates steep (padded columns must not trip the range check), tau = 64 nearly open; logits
