@@ -59,12 +59,12 @@ typedef enum vig_dtype { VIG_DTYPE_F32 = 0, VIG_DTYPE_BF16 = 1 } vig_dtype;
  * q, k, log_alpha_fwd, log_alpha_bwd: [B,H,L,dk];  v, out: [B,H,L,dv].
  *
  * bf16: dk in {16, 24, 32} with dv in {32, 48, 64} run on the tensor-core kernels; any other
- *       dk <= 128, dv <= 256 runs on the fp32 SIMT recurrence kernel (slow, same result
+ *       dk <= 128, dv <= 256 runs as fp32 walks on the CUDA cores (slower, same result
  *       contract).  Tensor-core operands are bf16 with fp32 accumulation; states that cross
  *       a 128-token chunk are rounded to bf16 as tensor-core operands.  A unit whose gates decay
  *       by more than e^-60 inside one chunk of 128 tokens is computed by an in-kernel fp32
  *       recurrence (Eq. 6 step by step) instead of the factorised tiles.
- * f32:  dk <= 128, dv <= 256; fp32 SIMT recurrence, meant for validation-sized inputs.
+ * f32:  dk <= 128, dv <= 256; fp32 walks on the CUDA cores, a sequence cut into segments that run side by side.
  * Sequences of at most 256 tokens run in one launch with a unit per thread block and use no scratch.
  * Longer ones are cut into 256-token segments (one launch; the blocks of a unit exchange segment
  * summaries through scratch) or into 128-token chunk tasks (three launches; chunk summaries and
@@ -192,15 +192,14 @@ int vig_bigla_fwd_blend_bf16(const void* q, const void* k, const void* v,
  * (gradients with respect to the LOG gates as passed to the forward call; a caller that feeds gate logits g chains
  * them through vig_gate_prep_bwd_* below).  All device pointers of the call's element type, contiguous,
  * 16-byte aligned; inputs are not written; outputs must not overlap inputs or one another.
- * How: dv is the forward pass itself on (k, q, d_out) with the gates moved by one token (the tensor-core kernels for
- * the bf16 head sizes they cover); dq, dk and the gate gradients come from two fp32 walks over the sequence per unit
- * on the CUDA cores (states in registers), with the gate gradients as running sums of q * dq - k * dk per direction.
- * Calls with few units and long sequences (fewer than two units per SM, 128 tokens or more) cut every sequence into
- * segments that are walked in parallel: a first launch finds what each segment adds to the four states, a fold carries
- * the states across segments, the walks start from them, and a last launch adds the later segments' sums to the gate
- * gradients (vig_t-like 1024 x 1024 inputs, 32 units of 4096 tokens: 2.19 ms -> 0.55 ms).
- * Scratch (the moved gates, 8 L dk bytes per unit of partial results, the segments' states) comes from the library's
- * pool, stream-ordered.
+ * How: bf16 with the forward pass's tensor-core head sizes and 16 tokens or more runs wholly on the tensor cores, chunk by
+ * chunk: one launch up to 224 tokens, three (the chunks' own states, a fold over the chunks, the chunks) beyond.  Operands
+ * of dq, dk and the gate gradients are taken as two bf16 each, so they carry about sixteen significant bits before the
+ * rounding to bf16; dv takes one bf16 per operand like the forward pass.  A unit whose gates decay by more than e^-60
+ * inside one chunk is computed by an in-kernel fp32 recurrence.  Everything else takes fp32 walks over the sequence on the
+ * CUDA cores: dv as the forward walk on (k, q, d_out) with the gates moved by one token, dq and dk from the four states,
+ * the gate gradients as running sums of q * dq - k * dk per direction; sequences are walked in segments side by side.
+ * Scratch (the chunks' or segments' states, partial results) comes from the library's pool, stream-ordered.
  * Head sizes: dk <= 128, dv <= 128, and whatever the forward entry point of the same type takes.
  * Errors: NULL_POINTER, BAD_DIM, MISALIGNED, UNSUPPORTED, CUDA. */
 int vig_bigla_bwd_bf16(const void* q, const void* k, const void* v,
