@@ -36,6 +36,9 @@ bool tc_supported(int dk, int dv) {
     return (dk == 16 || dk == 24 || dk == 32) && (dv == 32 || dv == 48 || dv == 64);
 }
 
+static thread_local long long t_batch_units = 0;   // units of the host call whose slices this thread is launching
+long long form_units(long long units) { return t_batch_units > units ? t_batch_units : units; }
+
 // Sequences of more than 256 tokens.  One launch with a block per 256-token segment reads every input once, but the
 // blocks of a unit stall together while they exchange their summaries, and every block reads every other segment's
 // summary: measured against the three chunk-task launches it wins for two segments, and for up to eight when all
@@ -55,7 +58,7 @@ static bool use_segments(long long units, int L, int dk, int dv) {
         if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
         sms_cached.store(sms, std::memory_order_relaxed);
     }
-    return units * nseg <= 2LL * sms;
+    return form_units(units) * nseg <= 2LL * sms;
 }
 
 static bool use_mma_chunks(long long units, int L, int dk, int dv, bool gates) {
@@ -483,6 +486,10 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
     if (pool_alloc((void**)&base, 4 * nk + 2 * nv, stream) != cudaSuccess) return VIG_ERR_CUDA;
     char *dq = base, *dk_ = base + nk, *dgf = base + 2 * nk, *dgb = base + 3 * nk, *dv_ = base + 4 * nk,
          *dout = base + 4 * nk + nv;
+    struct Batch {   // while slices of this call are launched
+        explicit Batch(long long n) { t_batch_units = n; }
+        ~Batch() { t_batch_units = 0; }
+    } batch(units);
     auto kernels = [&](size_t ok_, size_t ov, int nu) {
         if (dtype == VIG_DTYPE_F32) {
             const int r = vig_gate_prep_f32(dgf + ok_, dgb + ok_, dgf + ok_, dgb + ok_, nu, 1, L, dk, tau, stream_);

@@ -585,7 +585,7 @@ bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
         sms_of[dev].store(sms, std::memory_order_relaxed);
     }
-    return units <= (long long)waves * sms;
+    return form_units(units) <= (long long)waves * sms;
 }
 
 cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
@@ -614,6 +614,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
 // launch is at its best where two segments of every unit just fill the chip.
 bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
     if (dk == 16) return true;
+    units = form_units(units);
     const long long chunks = units * ((L + 127) / 128);
     constexpr int kSms = 148;
     if (dk == 24 && dv <= 48) {

@@ -244,7 +244,8 @@ cudaError_t launch_scan_t(ScanArgs<T> a, long long units, cudaStream_t stream) {
     // Segments: about sixteen warps per SM over the whole call (what hides a token's chain of dependent operations), in
     // whole groups of TG tokens.
     const int slabs = (a.dv + kCols - 1) / kCols;
-    long long want = (16LL * sms + units * slabs - 1) / (units * slabs);
+    const long long n = form_units(units) * slabs;
+    long long want = (16LL * sms + n - 1) / n;
     if (want > kMaxWarps) want = kMaxWarps;
     a.seg_len = (int)(((a.L + want - 1) / want + TG - 1) / TG * TG);
     const int nw = (a.L + a.seg_len - 1) / a.seg_len;

@@ -39,6 +39,10 @@ template <typename T>
 cudaError_t launch_gate_prep_bwd(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n, float tau,
                                  cudaStream_t stream);
 
+// The number of units by which a form is chosen where that depends on it: the call's own, or, for the slices of a host call,
+// that of the whole batch, so that a slice has the bits of a device call on the batch.
+long long form_units(long long units);
+
 // ---- bf16 tensor-core path: dispatch over the tcgen05 kernels (defined with the entry points) ----
 bool tc_supported(int dk, int dv);
 // Scratch bytes the tensor-core path needs for this shape; 0 if no launch of it uses scratch.
