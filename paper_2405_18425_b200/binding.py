@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libvig_bigla.so: argument marshalling only.
+"""Thin binding of libvig_bigla.so: argument marshalling only, for the device entry points in a native module
+(csrc/binding_call.cpp), else by ctypes.
 
 Every function mirrors the C entry point of the same name (include/vig_bigla.h), takes torch
 tensors for device buffers (numpy arrays or torch CPU tensors for the host entry point), passes
@@ -20,6 +21,8 @@ VIG_DTYPE_F32 = 0
 VIG_DTYPE_BF16 = 1
 
 _lib = None
+_addr = {}    # of the entry points called through the native module
+_call = None  # its call()
 
 
 class VigError(RuntimeError):
@@ -30,7 +33,7 @@ class VigError(RuntimeError):
 
 def load() -> ctypes.CDLL:
     """Loads the CUDA library (built in-tree by paper_2405_18425_b200.build).  Raises if it is missing."""
-    global _lib
+    global _lib, _call
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise ImportError(
@@ -79,6 +82,15 @@ def load() -> ctypes.CDLL:
         lib.vig_test_expire_next_wait.restype = None
         lib.vig_kernel_launch_count.argtypes = []
         lib.vig_kernel_launch_count.restype = ctypes.c_ulonglong
+        try:
+            from . import _binding_call
+        except ImportError as e:
+            raise ImportError(f"the binding's native module is missing: build it with `python -m paper_2405_18425_b200.build` ({e})") from e
+        for name in ("vig_bigla_fwd", "vig_bigla_fwd_bf16", "vig_bigla_fwd_f32", "vig_bigla_fwd_static_bf16", "vig_gate_prep_bf16",
+                     "vig_gate_prep_f32", "vig_bigla_fwd_gates_bf16", "vig_bigla_fwd_blend_bf16", "vig_dwconv3x3_bf16", "vig_dwconv3x3_f32",
+                     "vig_bigla_bwd_bf16", "vig_bigla_bwd_f32", "vig_gate_prep_bwd_bf16", "vig_gate_prep_bwd_f32"):
+            _addr[name] = ctypes.cast(getattr(lib, name), vp).value
+        _call = _binding_call.call
         _lib = lib
     return _lib
 
@@ -113,36 +125,33 @@ def _dev(*tensors):
             raise ValueError("device entry points take contiguous CUDA tensors")
 
 
+def _device_call(name, v, tau, stream, *tensors, same_dtype=False):
+    """Calls a device entry point: sizes from the first tensor and, unless v is -1, the last dimension of tensor v."""
+    if _lib is None:
+        load()
+    status = _call(_addr[name], None if stream is None else _stream(stream), v, same_dtype, tau, *tensors)
+    if status != VIG_OK:
+        raise VigError(status, name)
+
+
 def vig_bigla_fwd_bf16(q, k, v, log_alpha_fwd, log_alpha_bwd, out, stream=None):
-    _dev(q, k, v, log_alpha_fwd, log_alpha_bwd, out)
-    _check(load().vig_bigla_fwd_bf16(q.data_ptr(), k.data_ptr(), v.data_ptr(), log_alpha_fwd.data_ptr(),
-                                     log_alpha_bwd.data_ptr(), out.data_ptr(), *_dims(q, v), _stream(stream)),
-           "vig_bigla_fwd_bf16")
+    _device_call("vig_bigla_fwd_bf16", 2, None, stream, q, k, v, log_alpha_fwd, log_alpha_bwd, out)
     return out
 
 
 def vig_bigla_fwd(q, k, v, log_alpha_fwd, log_alpha_bwd, out, stream=None):
-    _dev(q, k, v, log_alpha_fwd, log_alpha_bwd, out)
-    _check(load().vig_bigla_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), log_alpha_fwd.data_ptr(),
-                                log_alpha_bwd.data_ptr(), out.data_ptr(), *_dims(q, v), _stream(stream)),
-           "vig_bigla_fwd")
+    _device_call("vig_bigla_fwd", 2, None, stream, q, k, v, log_alpha_fwd, log_alpha_bwd, out)
     return out
 
 
 def vig_bigla_fwd_f32(q, k, v, log_alpha_fwd, log_alpha_bwd, out, stream=None):
-    _dev(q, k, v, log_alpha_fwd, log_alpha_bwd, out)
-    _check(load().vig_bigla_fwd_f32(q.data_ptr(), k.data_ptr(), v.data_ptr(), log_alpha_fwd.data_ptr(),
-                                    log_alpha_bwd.data_ptr(), out.data_ptr(), *_dims(q, v), _stream(stream)),
-           "vig_bigla_fwd_f32")
+    _device_call("vig_bigla_fwd_f32", 2, None, stream, q, k, v, log_alpha_fwd, log_alpha_bwd, out)
     return out
 
 
 def vig_bigla_fwd_static_bf16(q, k, v, log_alpha_fwd, log_alpha_bwd, out, stream=None):
     """The forward pass with the library's fixed built-in scratch: allocates nothing (see the header)."""
-    _dev(q, k, v, log_alpha_fwd, log_alpha_bwd, out)
-    _check(load().vig_bigla_fwd_static_bf16(q.data_ptr(), k.data_ptr(), v.data_ptr(), log_alpha_fwd.data_ptr(),
-                                            log_alpha_bwd.data_ptr(), out.data_ptr(), *_dims(q, v),
-                                            _stream(stream)), "vig_bigla_fwd_static_bf16")
+    _device_call("vig_bigla_fwd_static_bf16", 2, None, stream, q, k, v, log_alpha_fwd, log_alpha_bwd, out)
     return out
 
 
@@ -161,10 +170,7 @@ def vig_bigla_fwd_ws_bf16(q, k, v, log_alpha_fwd, log_alpha_bwd, out, ws, stream
 
 
 def _gate_prep(fn_name, g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd, tau, stream):
-    _dev(g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd)
-    B, H, L, dk = g_fwd.shape
-    _check(getattr(load(), fn_name)(g_fwd.data_ptr(), g_bwd.data_ptr(), log_alpha_fwd.data_ptr(),
-                                    log_alpha_bwd.data_ptr(), B, H, L, dk, float(tau), _stream(stream)), fn_name)
+    _device_call(fn_name, -1, tau, stream, g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd)
     return log_alpha_fwd, log_alpha_bwd
 
 
@@ -178,19 +184,13 @@ def vig_gate_prep_f32(g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd, tau=16.0, stre
 
 def vig_bigla_fwd_gates_bf16(q, k, v, g_fwd, g_bwd, out, tau=16.0, stream=None):
     """Forward pass from the gate logits: log alpha = logsigmoid(g) / tau is prepared inside the call."""
-    _dev(q, k, v, g_fwd, g_bwd, out)
-    _check(load().vig_bigla_fwd_gates_bf16(q.data_ptr(), k.data_ptr(), v.data_ptr(), g_fwd.data_ptr(), g_bwd.data_ptr(),
-                                           out.data_ptr(), *_dims(q, v), float(tau), _stream(stream)),
-           "vig_bigla_fwd_gates_bf16")
+    _device_call("vig_bigla_fwd_gates_bf16", 2, tau, stream, q, k, v, g_fwd, g_bwd, out)
     return out
 
 
 def vig_bigla_fwd_blend_bf16(q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out, tau=16.0, stream=None):
     """Forward pass from the gate logits with the 2-D gate blend of Eq. 7 in the same call."""
-    _dev(q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out)
-    _check(load().vig_bigla_fwd_blend_bf16(q.data_ptr(), k.data_ptr(), v.data_ptr(), g_fwd.data_ptr(), g_bwd.data_ptr(),
-                                           o_local.data_ptr(), gate2d_logits.data_ptr(), out.data_ptr(), *_dims(q, v),
-                                           float(tau), _stream(stream)), "vig_bigla_fwd_blend_bf16")
+    _device_call("vig_bigla_fwd_blend_bf16", 2, tau, stream, q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out)
     return out
 
 
@@ -204,32 +204,20 @@ def _by_dtype(t, stem):
 
 def vig_bigla_bwd(q, k, v, log_alpha_fwd, log_alpha_bwd, d_out, dq, dk, dv, dlog_alpha_fwd, dlog_alpha_bwd, stream=None):
     """Gradient of the forward pass (Eq. 6) for d_out = dLoss/d_out; writes and returns the five gradient tensors."""
-    ts = (q, k, v, log_alpha_fwd, log_alpha_bwd, d_out, dq, dk, dv, dlog_alpha_fwd, dlog_alpha_bwd)
-    _dev(*ts)
-    name = _by_dtype(q, "vig_bigla_bwd")
-    if any(t.dtype != q.dtype for t in ts):
-        raise ValueError("all tensors of one call share a dtype")
-    _check(getattr(load(), name)(*(t.data_ptr() for t in ts), *_dims(q, v), _stream(stream)), name)
+    _device_call(_by_dtype(q, "vig_bigla_bwd"), 2, None, stream, q, k, v, log_alpha_fwd, log_alpha_bwd, d_out, dq, dk, dv, dlog_alpha_fwd,
+                 dlog_alpha_bwd, same_dtype=True)
     return dq, dk, dv, dlog_alpha_fwd, dlog_alpha_bwd
 
 
 def vig_gate_prep_bwd(g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd, tau=16.0, stream=None):
     """Gradient through the gate preparation: dg = dlog_alpha * sigmoid(-g) / tau, both directions."""
-    ts = (g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd)
-    _dev(*ts)
-    name = _by_dtype(g_fwd, "vig_gate_prep_bwd")
-    B, H, L, dk = g_fwd.shape
-    _check(getattr(load(), name)(*(t.data_ptr() for t in ts), B, H, L, dk, float(tau), _stream(stream)), name)
+    _device_call(_by_dtype(g_fwd, "vig_gate_prep_bwd"), -1, tau, stream, g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd)
     return dg_fwd, dg_bwd
 
 
 def vig_dwconv3x3(x, w, bias, out, stream=None):
     """Depth-wise 3x3 convolution (Eq. 7 line 1); x, out: [B, Hh, Ww, C]; w: [C, 3, 3]; bias: [C] or None."""
-    _dev(x, w, out)
-    name = _by_dtype(x, "vig_dwconv3x3")
-    B, Hh, Ww, C = x.shape
-    _check(getattr(load(), name)(x.data_ptr(), w.data_ptr(), bias.data_ptr() if bias is not None else None, out.data_ptr(),
-                                 B, Hh, Ww, C, _stream(stream)), name)
+    _device_call(_by_dtype(x, "vig_dwconv3x3"), -1, None, stream, x, w, bias, out)
     return out
 
 

@@ -1,4 +1,5 @@
-"""Builds libvig_bigla.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Builds libvig_bigla.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and _binding_call.so, the native
+half of the Python binding, with the host compiler against torch's headers.
 
     python -m paper_2405_18425_b200.build [--force] [--verbose]
 """
@@ -8,11 +9,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libvig_bigla.so")
+BINDING_SRC = os.path.join(CSRC, "binding_call.cpp")
+BINDING_LIB = os.path.join(PKG, "_binding_call.so")
 BUILD_DIR = os.path.join(PKG, "_build")
 
 NVCC_FLAGS = [
@@ -37,10 +41,34 @@ def is_stale() -> bool:
     return any(os.path.getmtime(p) > t for p in _deps())
 
 
+def _binding_command(out: str):
+    import torch
+    root = os.path.dirname(torch.__file__)
+    lib = os.path.join(root, "lib")
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+            *(x for i in inc for x in ("-isystem", i)), BINDING_SRC, "-o", out, "-L" + lib, "-Wl,-rpath," + lib,
+            "-ltorch_python", "-ltorch_cpu", "-lc10_cuda", "-lc10"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ and link the shared library.  Returns its path."""
-    if not force and not is_stale():
-        return LIB
+    """Compile every .cu under csrc/ and link the shared library, and the binding's module.  Returns the library's path."""
+    binding_stale = force or not os.path.exists(BINDING_LIB) or os.path.getmtime(BINDING_LIB) < os.path.getmtime(BINDING_SRC)
+    lib_stale = force or is_stale()
+    tmp = BINDING_LIB + f".tmp{os.getpid()}"
+    binding = subprocess.Popen(_binding_command(tmp)) if binding_stale else None
+    if lib_stale:
+        _build_library(verbose)
+    if binding is not None:
+        if binding.wait() != 0:
+            raise RuntimeError("building the binding's module failed")
+        os.replace(tmp, BINDING_LIB)
+    return LIB
+
+
+def _build_library(verbose: bool) -> None:
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(BUILD_DIR, exist_ok=True)
     inc = ["-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -63,7 +91,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
     tmp = LIB + f".tmp{os.getpid()}"
     subprocess.check_call([nvcc, "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
     os.replace(tmp, LIB)
-    return LIB
 
 
 if __name__ == "__main__":
