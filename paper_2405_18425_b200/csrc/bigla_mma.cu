@@ -156,8 +156,8 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
             if (GATES) {
-                af[r][j] = log2_alpha_pair(af[r][j], args.inv_tau);
-                ab[r][j] = log2_alpha_pair(ab[r][j], args.inv_tau);
+                af[r][j] = log2_alpha_pair<MODE != kUnit>(af[r][j], args.inv_tau);
+                ab[r][j] = log2_alpha_pair<MODE != kUnit>(ab[r][j], args.inv_tau);
             }
             af[r][j] = movmatrix(af[r][j]);
             ab[r][j] = movmatrix(ab[r][j]);
@@ -218,14 +218,26 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                             unpack2(fmul2(pack2(b0, b1), pack2(kLog2e, kLog2e)), b0, b1);
                             unpack2(fmul2(pack2(x0, x1), pack2(kLog2e, kLog2e)), x0, x1);
                         }
-                        // the decaying factors on the special-function unit, the growing ones as their packed reciprocals
-                        const uint32_t ef = pack_bf16(ex2(b0), ex2(b1)), eb = pack_bf16(ex2(x0), ex2(x1));
-                        kfw[2 * jj + r] = mul_bf16x2(kr[r][j], rcp_bf16x2(ef));
-                        kbw[2 * jj + r] = mul_bf16x2(kr[r][j], eb);
-                        if (MODE != kSummary) {
+                        if constexpr (MODE == kUnit) {
+                            // the decaying factors on the special-function unit, the growing ones as their packed reciprocals
+                            const uint32_t ef = pack_bf16(ex2(b0), ex2(b1)), eb = pack_bf16(ex2(x0), ex2(x1));
                             const uint32_t hq = mul_bf16x2(qr[r][j], 0x3F003F00u);   // the 1/2 of the result: exact
+                            kfw[2 * jj + r] = mul_bf16x2(kr[r][j], rcp_bf16x2(ef));
+                            kbw[2 * jj + r] = mul_bf16x2(kr[r][j], eb);
                             qf[m][2 * jj + r] = mul_bf16x2(hq, ef);
                             qb[m][2 * jj + r] = mul_bf16x2(hq, rcp_bf16x2(eb));
+                        } else {
+                            // Factor and product in fp32, one rounding: what the packed reciprocals are low by on average would
+                            // pass into the states and on from chunk to chunk (with them 32 x 4096 tokens, gate logits around 4,
+                            // were 4.8e-3 off in 2-norm, the tcgen05 forms 4.5e-3; this way 3.3e-3 in the same time).
+                            const f32x2 k2 = widen(kr[r][j]);
+                            kfw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(-b0), ex2(-b1))));
+                            kbw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(x0), ex2(x1))));
+                            if (MODE != kSummary) {
+                                const f32x2 q2 = fmul2(widen(qr[r][j]), pack2(0.5f, 0.5f));   // the 1/2 of the result
+                                qf[m][2 * jj + r] = pack_f32x2(fmul2(q2, pack2(ex2(b0), ex2(b1))));
+                                qb[m][2 * jj + r] = pack_f32x2(fmul2(q2, pack2(ex2(-x0), ex2(-x1))));
+                            }
                         }
                     }
                 } else {

@@ -498,6 +498,24 @@ def test_fused_gates_match_unfused_chain_closely():
     assert np.abs(fa - fb).max() <= 1e-2 * np.abs(fa).max()
 
 
+def test_fused_gates_of_open_logits_carry_no_bias():
+    """With q, k and v constant the output is a sum of decays over some 500 tokens, which a bias of the log gates moves by as
+    much as it is: against the gates of vig_gate_prep_bf16 (relative error 2e-5 before the rounding to bf16, whose own errors
+    average out over 524 K gates), the mean output may move by the two evaluations' errors and the rounding of 16 K distinct
+    results (2^-9 / sqrt(3) / 128 = 9e-6), well inside 4e-4.  A polynomial 0.2 % off there moves it by 1.2e-3."""
+    L, dk, dv = 4096, 16, 32
+    rng = torch.Generator(device="cuda").manual_seed(23)
+    q = torch.full((1, 4, L, dk), 1 / 16, device="cuda", dtype=torch.bfloat16)
+    k, v = torch.ones_like(q), torch.ones(1, 4, L, dv, device="cuda", dtype=torch.bfloat16)
+    g = [(torch.randn(1, 4, L, dk, generator=rng, device="cuda") + 4).bfloat16() for _ in range(2)]
+    la, out = [torch.empty_like(x) for x in g], [torch.empty_like(v) for _ in range(2)]
+    vig.vig_gate_prep_bf16(g[0], g[1], la[0], la[1], 16.0)
+    vig.vig_bigla_fwd_bf16(q, k, v, la[0], la[1], out[0])
+    vig.vig_bigla_fwd_gates_bf16(q, k, v, g[0], g[1], out[1], 16.0)
+    a, b = (float(o.double().mean()) for o in out)
+    assert abs(b / a - 1) <= 4e-4
+
+
 @pytest.mark.parametrize("idx", [0, 3, 4])
 def test_host_entry_point_matches_device_path(oracle, idx):
     """Host buffers in and out (pinned and pageable), the batch cut into slices inside the call: the same bits as the
