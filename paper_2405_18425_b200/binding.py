@@ -80,6 +80,8 @@ def load() -> ctypes.CDLL:
         lib.vig_test_take_fallback_count.restype = ci
         lib.vig_test_expire_next_wait.argtypes = []
         lib.vig_test_expire_next_wait.restype = None
+        lib.vig_test_host_copy_usable.argtypes = [vp, ctypes.c_size_t]
+        lib.vig_test_host_copy_usable.restype = ci
         lib.vig_kernel_launch_count.argtypes = []
         lib.vig_kernel_launch_count.restype = ctypes.c_ulonglong
         try:
@@ -270,6 +272,11 @@ def vig_test_take_fallback_count(stream=None) -> int:
 def vig_test_expire_next_wait() -> None:
     """Test hook: the next single-block tensor-core launch lets one bounded device-side wait run out."""
     load().vig_test_expire_next_wait()
+
+
+def vig_test_host_copy_usable(address: int, nbytes: int) -> bool:
+    """Test hook: whether the host entry point would let a kernel touch these bytes of host memory (launches nothing)."""
+    return bool(load().vig_test_host_copy_usable(address, nbytes))
 
 
 def vig_kernel_launch_count() -> int:

@@ -503,8 +503,8 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
     // The way back by a kernel, beside the copies to the device; the way in by a kernel as well where the fixed cost of five
     // engine copies (20 us more) outweighs the engine's higher rate (7 %).  Pageable memory takes the engines.
     const bool out_kernel = whole && host_copy_usable(out, out_bytes);
-    const bool in_kernel = out_kernel && in_bytes <= (8u << 20) && host_copy_usable(q, 16) && host_copy_usable(k, 16) && host_copy_usable(v, 16) &&
-                           host_copy_usable(g_fwd, 16) && host_copy_usable(g_bwd, 16);
+    const bool in_kernel = out_kernel && in_bytes <= (8u << 20) && host_copy_usable(q, units * unit_k) && host_copy_usable(k, units * unit_k) &&
+                           host_copy_usable(v, units * unit_v) && host_copy_usable(g_fwd, units * unit_k) && host_copy_usable(g_bwd, units * unit_k);
     auto copy_in = [&](size_t ok_, size_t ov, size_t nbk, size_t nbv, cudaStream_t s) {
         const HostCopy c[5] = {{(const char*)g_fwd + ok_, dgf + ok_, nbk},
                                {(const char*)g_bwd + ok_, dgb + ok_, nbk},
@@ -604,6 +604,8 @@ int vig_test_take_fallback_count(void* stream) {
         return VIG_ERR_CUDA;
     return n;
 }
+
+int vig_test_host_copy_usable(const void* host, size_t bytes) { return host_copy_usable(host, bytes) ? 1 : 0; }
 
 void vig_test_expire_next_wait(void) { g_expire_next_wait.store(1, std::memory_order_relaxed); }
 

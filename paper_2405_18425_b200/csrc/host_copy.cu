@@ -4,6 +4,8 @@
 // can be paced: at full rate either way the link carries about 70 GB/s in both directions together, and the writes out,
 // which share their lane with the requests of the copies in, hold those back more than their share (57.8 MB in, 19.3 MB out
 // in three slices: 1.38 ms at full rate, 1.33 ms from one or two blocks).
+#include <cuda.h>
+
 #include <cstring>
 
 #include "ptx.cuh"
@@ -37,14 +39,35 @@ __global__ void __launch_bounds__(512) host_copy_kernel(const CopySet s) {
 
 }  // namespace
 
+// Every byte has to be mapped: a kernel that runs past the end of a registered range faults, where an engine copy returns an
+// error.  Ranges that follow one another without a gap (memory registered piece by piece) will do.
 bool host_copy_usable(const void* host, size_t bytes) {
-    if ((reinterpret_cast<uintptr_t>(host) & 15) != 0 || bytes % 16 != 0) return false;
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
-        cudaGetLastError();   // (nothing of the failed query is left behind)
-        return false;
+    if ((reinterpret_cast<uintptr_t>(host) & 15) != 0 || bytes == 0 || bytes % 16 != 0) return false;
+    using AttributeFn = CUresult (*)(void*, CUpointer_attribute, CUdeviceptr);
+    static const AttributeFn attribute = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &f, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) f = nullptr;
+        return reinterpret_cast<AttributeFn>(f);
+    }();
+    if (!attribute) return false;
+    uintptr_t p = reinterpret_cast<uintptr_t>(host);
+    const uintptr_t end = p + bytes;
+    for (int ranges = 0; p < end; ++ranges) {
+        cudaPointerAttributes at;
+        if (ranges == 64 || cudaPointerGetAttributes(&at, reinterpret_cast<void*>(p)) != cudaSuccess) {
+            cudaGetLastError();   // (nothing of the failed query is left behind)
+            return false;
+        }
+        if (at.type != cudaMemoryTypeHost || reinterpret_cast<uintptr_t>(at.devicePointer) != p) return false;   // pinned, and mapped at its own address
+        CUdeviceptr start = 0;
+        size_t size = 0;
+        if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)p) != CUDA_SUCCESS ||
+            attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)p) != CUDA_SUCCESS || start + size <= p)
+            return false;
+        p = start + size;
     }
-    return at.type == cudaMemoryTypeHost && at.devicePointer == host;   // pinned, and mapped at its own address
+    return true;
 }
 
 cudaError_t launch_host_copy(const HostCopy* copies, int n, int max_blocks, cudaStream_t stream) {

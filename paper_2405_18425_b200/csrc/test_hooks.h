@@ -14,6 +14,8 @@
 #ifndef VIG_TEST_HOOKS_H
 #define VIG_TEST_HOOKS_H
 
+#include <stddef.h>
+
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -31,6 +33,10 @@ int vig_test_take_fallback_count(void* stream);
  * microseconds, the blocks finish their unit without storing anything, and vig_last_device_status reports
  * VIG_ERR_DEVICE_TIMEOUT.  Nothing faults and nothing spins beyond that limit. */
 void vig_test_expire_next_wait(void);
+
+/* 1 if the host entry point would let a kernel read or write these bytes of host memory (all of them pinned and mapped,
+ * both ends 16-byte aligned), 0 if it would leave them to a copy engine.  Launches nothing. */
+int vig_test_host_copy_usable(const void* host, size_t bytes);
 
 #ifdef __cplusplus
 }

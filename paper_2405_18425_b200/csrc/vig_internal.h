@@ -124,7 +124,7 @@ struct HostCopy {
     void* dst;
     size_t bytes;   // a multiple of 16; both addresses 16-byte aligned
 };
-bool host_copy_usable(const void* host, size_t bytes);   // pinned and mapped, aligned
+bool host_copy_usable(const void* host, size_t bytes);   // all of it pinned and mapped, aligned
 cudaError_t launch_host_copy(const HostCopy* copies, int n, int max_blocks, cudaStream_t stream);
 
 // Launch with programmatic stream serialization: the kernel's prologue (everything before its pdl_wait) may overlap

@@ -1,6 +1,8 @@
 """GPU parity: the CUDA path, called through the C ABI, against the fp64 oracle on the same seeded
 inputs.  Bar: max|gpu - oracle| <= 1e-4 * max|oracle| for fp32 storage and <= 2e-2 * max|oracle|
 for bf16 storage, the maximum taken over the whole output tensor."""
+import ctypes
+import mmap
 import os
 
 import numpy as np
@@ -544,6 +546,31 @@ def test_host_entry_point_matches_device_path(oracle, idx):
     out_n = np.empty_like(x["v"])
     vig.vig_bigla_fwd_host(x["q"], x["k"], x["v"], x["g_fwd"], x["g_bwd"], out_n, cfg.tau, code)
     np.testing.assert_array_equal(out_n, ref_bytes)
+
+
+def test_host_memory_is_touched_by_kernels_only_where_all_of_it_is_mapped():
+    """The predicate alone, nothing is launched: part of a range registered, two registrations side by side, a gap between
+    them, pageable memory, addresses and sizes that are not whole 16-byte pieces."""
+    page, rt = mmap.PAGESIZE, torch.cuda.cudart()
+    torch.cuda.init()
+    area = mmap.mmap(-1, 16 * page)
+    base = ctypes.addressof(ctypes.c_char.from_buffer(area))
+    usable = lambda first, n: vig.vig_test_host_copy_usable(base + int(first * page), int(n * page))
+    assert not usable(0, 1)
+    for first, n in ((0, 4), (4, 2), (8, 3)):
+        assert int(rt.cudaHostRegister(base + first * page, n * page, 0)) == 0
+    try:
+        assert usable(0, 4) and usable(1, 3) and usable(2.5, 1) and usable(8, 3)
+        assert usable(0, 6)                                          # two registrations, no gap
+        assert not usable(4, 3) and not usable(4, 4) and not usable(0, 7) and not usable(5, 4)   # runs past the end; both ends mapped, a gap inside
+        assert not usable(9, 3) and not usable(6, 1)
+        assert not vig.vig_test_host_copy_usable(base + 8, 64) and not vig.vig_test_host_copy_usable(base, 72)
+    finally:
+        for first in (0, 4, 8):
+            rt.cudaHostUnregister(base + first * page)
+    assert not usable(0, 4)
+    pinned = torch.empty(1 << 20, dtype=torch.uint8, pin_memory=True)
+    assert vig.vig_test_host_copy_usable(pinned.data_ptr(), pinned.numel())
 
 
 def test_workspace_variant_and_determinism(oracle):
