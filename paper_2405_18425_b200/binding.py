@@ -128,7 +128,8 @@ def _dev(*tensors):
 
 
 def _device_call(name, v, tau, stream, *tensors, same_dtype=False):
-    """Calls a device entry point: sizes from the first tensor and, unless v is -1, the last dimension of tensor v."""
+    """Calls a device entry point: sizes from the first tensor and, unless v is -1, the last dimension of tensor v.  tau: a
+    float exactly where the entry point has one (the native module tells the signatures apart by it), else None."""
     if _lib is None:
         load()
     status = _call(_addr[name], None if stream is None else _stream(stream), v, same_dtype, tau, *tensors)
@@ -172,7 +173,7 @@ def vig_bigla_fwd_ws_bf16(q, k, v, log_alpha_fwd, log_alpha_bwd, out, ws, stream
 
 
 def _gate_prep(fn_name, g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd, tau, stream):
-    _device_call(fn_name, -1, tau, stream, g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd)
+    _device_call(fn_name, -1, float(tau), stream, g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd)
     return log_alpha_fwd, log_alpha_bwd
 
 
@@ -186,13 +187,13 @@ def vig_gate_prep_f32(g_fwd, g_bwd, log_alpha_fwd, log_alpha_bwd, tau=16.0, stre
 
 def vig_bigla_fwd_gates_bf16(q, k, v, g_fwd, g_bwd, out, tau=16.0, stream=None):
     """Forward pass from the gate logits: log alpha = logsigmoid(g) / tau is prepared inside the call."""
-    _device_call("vig_bigla_fwd_gates_bf16", 2, tau, stream, q, k, v, g_fwd, g_bwd, out)
+    _device_call("vig_bigla_fwd_gates_bf16", 2, float(tau), stream, q, k, v, g_fwd, g_bwd, out)
     return out
 
 
 def vig_bigla_fwd_blend_bf16(q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out, tau=16.0, stream=None):
     """Forward pass from the gate logits with the 2-D gate blend of Eq. 7 in the same call."""
-    _device_call("vig_bigla_fwd_blend_bf16", 2, tau, stream, q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out)
+    _device_call("vig_bigla_fwd_blend_bf16", 2, float(tau), stream, q, k, v, g_fwd, g_bwd, o_local, gate2d_logits, out)
     return out
 
 
@@ -213,7 +214,7 @@ def vig_bigla_bwd(q, k, v, log_alpha_fwd, log_alpha_bwd, d_out, dq, dk, dv, dlog
 
 def vig_gate_prep_bwd(g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd, tau=16.0, stream=None):
     """Gradient through the gate preparation: dg = dlog_alpha * sigmoid(-g) / tau, both directions."""
-    _device_call(_by_dtype(g_fwd, "vig_gate_prep_bwd"), -1, tau, stream, g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd)
+    _device_call(_by_dtype(g_fwd, "vig_gate_prep_bwd"), -1, float(tau), stream, g_fwd, g_bwd, dlog_alpha_fwd, dlog_alpha_bwd, dg_fwd, dg_bwd)
     return dg_fwd, dg_bwd
 
 

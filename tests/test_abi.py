@@ -134,6 +134,21 @@ def test_binding_refuses_cpu_tensors(lib):
         vig.vig_bigla_fwd_f32(t, t, t, t, t, t)
 
 
+@pytest.mark.parametrize("call", [
+    lambda t, tau: vig.vig_gate_prep_f32(t, t, t, t, tau),
+    lambda t, tau: vig.vig_bigla_fwd_gates_bf16(t, t, t, t, t, t, tau),
+    lambda t, tau: vig.vig_bigla_fwd_blend_bf16(t, t, t, t, t, t, t, t, tau),
+    lambda t, tau: vig.vig_gate_prep_bwd(t, t, t, t, t, t, tau)])
+def test_binding_refuses_a_temperature_that_is_no_number(lib, call):
+    """None included, which the native module takes for an entry point without a temperature: it would call one that has it
+    with whatever its register holds."""
+    import torch
+
+    for tau in (None, "warm", object()):
+        with pytest.raises((TypeError, ValueError), match="float"):
+            call(torch.zeros(1, 1, 4, 16), tau)
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     from paper_2405_18425_b200 import binding
 
