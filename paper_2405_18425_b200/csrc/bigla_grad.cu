@@ -572,7 +572,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const size_t at = (unit * L + row0 + 16 * wt + g) * DK + 2 * c;
         const bool in0 = row0 + 16 * wt + g < L, in1 = row0 + 16 * wt + 8 + g < L;
         auto word = [&](const __nv_bfloat16* p, int j, int r) {
-            return (r ? in1 : in0) ? __ldg(reinterpret_cast<const uint32_t*>(p + at + 8 * r * DK + 8 * j)) : 0u;
+            return (r ? in1 : in0) ? *reinterpret_cast<const uint32_t*>(p + at + 8 * r * DK + 8 * j) : 0u;
         };
         uint32_t lf[NP][2], lb[NP][2], qw[NP][2], kw[NP][2];
 #pragma unroll

@@ -199,3 +199,39 @@ def test_f32_walks_in_segments(oracle, units, L, dk, dv):
     torch.cuda.synchronize()
     f = lambda a: synth.stored_to_f64(a, "f32")
     assert rel_err(device_to_f64(out, "f32"), oracle.bigla_fwd(f(x["q"]), f(x["k"]), f(x["v"]), f(la[0]), f(la[1]), nthreads=4)) <= TOL["f32"]
+
+
+@pytest.mark.parametrize("units,L", [(3, 100), (200, 196), (4, 700)])
+def test_chain_of_dependent_launches_sees_what_the_last_one_wrote(units, L):
+    """Gate preparation, forward and gradient back to back on the same buffers, the contents changing from pass to pass: each
+    kernel starts while the one before it, which writes its inputs, may still be running."""
+    rng = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda d: torch.randn(1, units, L, d, generator=rng, device="cuda").bfloat16()
+    sets = [dict(q=mk(24) * 24 ** -0.5, k=mk(24), v=mk(48), gf=mk(24), gb=mk(24), g=mk(48)) for _ in range(3)]
+    now = {n: torch.empty_like(t) for n, t in sets[0].items()}
+    la = [torch.empty_like(now["gf"]) for _ in range(2)]
+
+    def step(keep):
+        out = [torch.empty_like(now[n]) for n in ("v", "q", "k", "v", "gf", "gb")] if keep is None else keep
+        vig.vig_gate_prep_bf16(now["gf"], now["gb"], la[0], la[1], 16.0)
+        vig.vig_bigla_fwd_bf16(now["q"], now["k"], now["v"], la[0], la[1], out[0])
+        vig.vig_bigla_bwd(now["q"], now["k"], now["v"], la[0], la[1], now["g"], *out[1:])
+        return out
+
+    alone = []
+    for s in sets:
+        for n in now:
+            now[n].copy_(s[n])
+        torch.cuda.synchronize()
+        alone.append(step(None))
+        torch.cuda.synchronize()
+    outs = [[[torch.empty_like(t) for t in alone[0]] for _ in sets] for _ in range(8)]
+    for rep in outs:
+        for s, keep in zip(sets, rep):
+            for n in now:
+                now[n].copy_(s[n])
+            step(keep)
+    torch.cuda.synchronize()
+    for rep in outs:
+        for got, want in zip(rep, alone):
+            assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
