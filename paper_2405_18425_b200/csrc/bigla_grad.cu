@@ -216,8 +216,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         mbar_init(bar, 1);
         mbar_init(bar + 8, 1);
         mbar_init(bar + 32, 1);
-        state_word[0] = 0;
-        state_word[1] = 0;
+        state_word[0] = 0;   // (the other word is written by the other block alone, and read once that has landed)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();
@@ -252,7 +251,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         }
     }
     __syncthreads();
-    if (MODE == kPair) cluster_arrive_relaxed();   // the other block may be written to once it runs
+    if (MODE == kPair) cluster_arrive_relaxed();   // the other block may be written to once it runs (nothing of its own goes where that lands)
     bool ok = mbar_wait_bounded(bar, 0);
 
     // ---- this warp's 16 rows; the gate tiles turned, as B operands of products over the tokens ----
@@ -507,7 +506,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const uint32_t st_left = tst, st_right = tst + (MODE == kMain ? 4 : 0) * kState;
     if (MODE == kPair) {
         const int here = __syncthreads_or(!(mbar_wait_bounded(bar + 8, 0) && ok)) ? 2 : 0;
-        const int word = state_word[0] | here | state_word[1];
+        const int word = here ? here : state_word[0] | state_word[1];
         if (word) {
             if (word & 2) {
                 if (chunk == 0) mbar_wait_bounded(bar + 32, 0);   // (the other block may not know and send its sums)
