@@ -32,6 +32,7 @@ from .binding import (  # noqa: F401
     vig_test_set_kernel_preference,
     vig_test_take_fallback_count,
     vig_test_expire_next_wait,
+    vig_test_expire_next_exchange,
     vig_test_host_copy_usable,
     VIG_TEST_KERNEL_AUTO,
     VIG_TEST_KERNEL_SIMT,

@@ -78,8 +78,9 @@ def load() -> ctypes.CDLL:
         lib.vig_test_set_kernel_preference.restype = ci
         lib.vig_test_take_fallback_count.argtypes = [vp]
         lib.vig_test_take_fallback_count.restype = ci
-        lib.vig_test_expire_next_wait.argtypes = []
-        lib.vig_test_expire_next_wait.restype = None
+        for name in ("vig_test_expire_next_wait", "vig_test_expire_next_exchange"):
+            getattr(lib, name).argtypes = []
+            getattr(lib, name).restype = None
         lib.vig_test_host_copy_usable.argtypes = [vp, ctypes.c_size_t]
         lib.vig_test_host_copy_usable.restype = ci
         lib.vig_kernel_launch_count.argtypes = []
@@ -271,8 +272,13 @@ def vig_test_take_fallback_count(stream=None) -> int:
 
 
 def vig_test_expire_next_wait() -> None:
-    """Test hook: the next single-block tensor-core launch lets one bounded device-side wait run out."""
+    """Test hook: the next forward or gradient call on the tensor cores lets one bounded device-side wait run out."""
     load().vig_test_expire_next_wait()
+
+
+def vig_test_expire_next_exchange() -> None:
+    """Test hook: the next gradient of two chunks lets the left one's wait for the right one's sums run out."""
+    load().vig_test_expire_next_exchange()
 
 
 def vig_test_host_copy_usable(address: int, nbytes: int) -> bool:

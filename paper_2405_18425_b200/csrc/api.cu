@@ -11,7 +11,7 @@ namespace vig {
 // [0]: the device status word (bit flags, kDevStatus*);  [1]: units the tensor-core kernels handed to their in-kernel
 // recurrence since the counter was last read (a test aid: kernels find it one word behind the status word).
 __device__ int g_device_status[2] = {0, 0};
-static std::atomic<int> g_expire_next_wait{0};   // test hook: the next single-block launch lets one bounded wait run out
+static std::atomic<int> g_expire_next_wait{0};   // test hook: the next launch that takes it lets one bounded wait run out
 int take_expire_next_wait() { return g_expire_next_wait.exchange(0, std::memory_order_relaxed); }
 
 static std::atomic<unsigned long long> g_launches{0};
@@ -608,6 +608,7 @@ int vig_test_take_fallback_count(void* stream) {
 int vig_test_host_copy_usable(const void* host, size_t bytes) { return host_copy_usable(host, bytes) ? 1 : 0; }
 
 void vig_test_expire_next_wait(void) { g_expire_next_wait.store(1, std::memory_order_relaxed); }
+void vig_test_expire_next_exchange(void) { g_expire_next_wait.store(2, std::memory_order_relaxed); }
 
 unsigned long long vig_kernel_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 

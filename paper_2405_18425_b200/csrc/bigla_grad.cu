@@ -52,10 +52,11 @@ struct GArgs {
     float* u;               // [unit][chunk][kind][DV][DK] fp32: the chunks' own states (kinds S>, Z<, S<, Z>)
     uint8_t* img;           // [unit][chunk][kind][hi, lo][DV][64 B]: the states entering a chunk, as shared-memory tiles
     float* decay;           // [unit][chunk][2][32]: products of alpha>, alpha< over the chunk
-    int* flags;             // [unit][chunk]: gates out of range
+    int* flags;             // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
     long long chunks;       // of the call
     int ahead;              // the chunk this many blocks on is pulled into L2
     int* dev_status;
+    int expire_wait;        // test hook, 1: every block lets one bounded wait, on an mbarrier nothing completes, run out; 2: a pair's left block its last
 };
 
 // Operand tiles [rows][32] bf16 (64-byte rows), in this order behind the v and g tiles.  As loaded: q in kQf, k in kKf,
@@ -202,7 +203,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const bool live = wt >= 0 && wt < nT;
     const GLayout<DV> lay(tiles, MODE);
     const uint32_t base = smem_u32(smem), tv = base, tg = base + lay.g, top = base + lay.op, tst = base + lay.st;
-    const uint32_t bar = base + lay.bar;   // inputs landed; + 8: states landed; + 32: a pair's sums of E landed
+    const uint32_t bar = base + lay.bar;   // inputs landed; + 8: states landed; + 24: never completed, for the test hook; + 32: a pair's sums of E landed
     auto op = [&](int o) { return top + (uint32_t)o * lay.op_bytes; };
     float* totals = reinterpret_cast<float*>(smem + lay.totals);
     float* ends = reinterpret_cast<float*>(smem + lay.ends);
@@ -215,6 +216,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 8, 1);
+        mbar_init(bar + 24, 1);
         mbar_init(bar + 32, 1);
         state_word[0] = 0;   // (the other word is written by the other block alone, and read once that has landed)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -252,7 +254,9 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     }
     __syncthreads();
     if (MODE == kPair) cluster_arrive_relaxed();   // the other block may be written to once it runs (nothing of its own goes where that lands)
-    bool ok = mbar_wait_bounded(bar, 0);
+    bool ok = true;
+    if (a.expire_wait == 1 && tid == 0) ok = mbar_wait_bounded(bar + 24, 0, 64);   // test hook: this wait cannot succeed
+    ok = mbar_wait_bounded(bar, 0) && ok;
 
     // ---- this warp's 16 rows; the gate tiles turned, as B operands of products over the tokens ----
     uint32_t qa[MP][4], ka[MP][4], fa[MP][4], ba[MP][4];
@@ -338,6 +342,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         cluster_wait();
     } else if (!ok) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(a.dev_status, kDevStatusTimeout);
+        if (MODE == kSummary && tid == 0) a.flags[unit * nch + chunk] = 2;   // (nor by the launches behind this one)
         if (MODE == kMain) mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
         return;
     }
@@ -413,9 +418,11 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     if (MODE == kMain) {
         int slow = 0;
         for (int x = tid; x < nch; x += blockDim.x) slow |= a.flags[unit * nch + x];
+        const bool missing = __syncthreads_or(slow & 2);
         if (__syncthreads_or(slow)) {
-            if (chunk == 0 && tid == 0) atomicAdd(a.dev_status + 1, 1);
             mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
+            if (missing) return;             // a summary of this unit did not get its inputs, and has said so
+            if (chunk == 0 && tid == 0) atomicAdd(a.dev_status + 1, 1);
             gradient_by_recurrence<DK, DV>(a, unit, chunk * nw + w, nch * nw, lane);
             return;
         }
@@ -509,7 +516,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         const int word = here ? here : state_word[0] | state_word[1];
         if (word) {
             if (word & 2) {
-                if (chunk == 0) mbar_wait_bounded(bar + 32, 0);   // (the other block may not know and send its sums)
+                if (chunk == 0 && ok && here) mbar_wait_bounded(bar + 32, 0);   // (the other block does not know and may send its sums)
                 if (tid == 0) atomicOr(a.dev_status, kDevStatusTimeout);
                 return;
             }
@@ -799,8 +806,9 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 st_async1(at, __float_as_uint(s0), peer_bar);
                 st_async1(at + 4, __float_as_uint(s1), peer_bar);
             }
-        } else if (!mbar_wait_bounded(bar + 32, 0)) {
-            atomicOr(a.dev_status, kDevStatusTimeout);
+        } else if (!__syncthreads_and(mbar_wait_bounded(bar + 32, 0) && a.expire_wait != 2)) {   // no gate gradients from sums that are not there
+            if (tid == 0) atomicOr(a.dev_status, kDevStatusTimeout);
+            return;
         }
     }
     if (scan) {
@@ -984,6 +992,7 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
             else
                 e = launch_pdl(grad_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 4, (kWork + 255) / 256), dim3(256), 0, stream, a);
         }
+        a.expire_wait = 0;   // (of a long call the first launch)
         if (e == cudaSuccess)
             e = launch_grad(bigla_grad_kernel<DK, DV, kMain>, grid, threads(kMain), GLayout<DV>(p.tiles, kMain).total, false, stream, tq, tk, tf, tb, tv, tg, a);
     }
@@ -1008,7 +1017,7 @@ cudaError_t launch_bigla_grad(const __nv_bfloat16* q, const __nv_bfloat16* k, co
     char* b = static_cast<char*>(scratch);
     GArgs a{q, k, v, la_f, la_b, d_out, dq, dk_out, dv_out, dla_f, dla_b, L, p.nch, p.tiles,
             reinterpret_cast<float*>(b + s.u), reinterpret_cast<uint8_t*>(b + s.img), reinterpret_cast<float*>(b + s.decay),
-            reinterpret_cast<int*>(b + s.flags), units * p.nch, 0, device_status_ptr()};
+            reinterpret_cast<int*>(b + s.flags), units * p.nch, 0, device_status_ptr(), take_expire_next_wait()};
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_) \
     if (dk == DK_ && dv == DV_) return launch_grad_t<DK_, DV_>(a, p, units, stream);

@@ -49,7 +49,7 @@ struct MArgs {
     float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
     uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
     float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
-    int* flags;        // [unit][chunk]: gates out of range
+    int* flags;        // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
     int* dev_status;
     float inv_tau;
     int ahead;         // the block this many further on has its inputs pulled into L2
@@ -254,6 +254,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     ok = mbar_wait_bounded(bar, 0) && ok;
     if (!__syncthreads_and(ok)) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
+        if (MODE == kSummary && tid == 0) args.flags[blockIdx.x] = 2;   // (nor by the launches behind this one)
         if (MODE == kMain) mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
         return;
     }
@@ -267,8 +268,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     if (MODE == kMain) {
         int any = 0;
         for (int x = tid; x < nch; x += blockDim.x) any |= args.flags[unit * nch + x];
+        const bool missing = __syncthreads_or(any & 2);
         redo = __syncthreads_or(any);
         if (redo) mbar_wait_bounded(bar + 8, 0);
+        if (missing) return;   // a summary of this unit did not get its inputs, and has said so
     }
     if (redo) {   // gates beyond the range of the factorised tiles: Eq. 6 step by step, over the dead tiles, by one block of the unit
         if (chunk != 0) return;
@@ -554,7 +557,7 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
 }
 
 template <int DK, int DV, bool GATES>
-cudaError_t launch_chunks(const MArgs& a, long long units, cudaStream_t stream) {
+cudaError_t launch_chunks(MArgs a, long long units, cudaStream_t stream) {
     CUtensorMap tv;
     if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
@@ -566,6 +569,7 @@ cudaError_t launch_chunks(const MArgs& a, long long units, cudaStream_t stream) 
         e = launch_pdl(mma_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 2, (kWork + 255) / 256), dim3(256), 0, stream, a);
     count_launch();
     if (e != cudaSuccess) return e;
+    a.expire_wait = 0;   // (of a long call the first launch)
     return launch_mma_t<DK, DV, GATES, 8, kMain>(a, tv, a.tiles, stream);
 }
 
@@ -607,7 +611,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
     a.L = L; a.blocks = units;
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
-    a.expire_wait = take_expire_next_wait();
+    a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_) \
@@ -655,6 +659,7 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
     a.decay = reinterpret_cast<float*>(b + p.decay);
     a.flags = reinterpret_cast<int*>(b + p.flags);
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
+    a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_)        \

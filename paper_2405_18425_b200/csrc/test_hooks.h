@@ -28,11 +28,14 @@ int vig_test_set_kernel_preference(int preference);
  * (negative: a vig_status error). */
 int vig_test_take_fallback_count(void* stream);
 
-/* The next launch of the single-block tensor-core kernel (sequences of at most 256 tokens) makes every block wait, with
- * a limit of a few dozen polls, on an mbarrier that nothing ever completes: the bounded wait runs out within
- * microseconds, the blocks finish their unit without storing anything, and vig_last_device_status reports
- * VIG_ERR_DEVICE_TIMEOUT.  Nothing faults and nothing spins beyond that limit. */
+/* In the next call of the forward pass (one launch for units of at most 256 tokens, the warp-tile launches beyond) or of the
+ * tensor-core gradient, the blocks of the first launch wait, with a limit of a few dozen polls, on an mbarrier that nothing
+ * ever completes: the bounded wait runs out within microseconds, nothing is stored, and vig_last_device_status reports
+ * VIG_ERR_DEVICE_TIMEOUT.  Nothing faults and nothing spins beyond that limit.
+ * vig_test_expire_next_exchange: the same for the last wait of a gradient of two chunks, the left one's for the right one's
+ * sums: the gate gradients of the left chunk are not stored. */
 void vig_test_expire_next_wait(void);
+void vig_test_expire_next_exchange(void);
 
 /* 1 if the host entry point would let a kernel read or write these bytes of host memory (all of them pinned and mapped,
  * both ends 16-byte aligned), 0 if it would leave them to a copy engine.  Launches nothing. */

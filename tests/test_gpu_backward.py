@@ -235,3 +235,45 @@ def test_chain_of_dependent_launches_sees_what_the_last_one_wrote(units, L):
     for rep in outs:
         for got, want in zip(rep, alone):
             assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
+
+
+def _gradient_call(L):
+    cfg, x = random_problem(4800 + L, 2, 2, L, 24, 48, "bf16", gate_mean=1.0)
+    d = {n: to_device(a, "bf16") for n, a in x.items()}
+    d["d_out"] = to_device(synth.make_grad_input(cfg), "bf16")
+    la = [torch.empty_like(d["g_fwd"]) for _ in range(2)]
+    vig.vig_gate_prep_bf16(d["g_fwd"], d["g_bwd"], *la, cfg.tau)
+
+    def call():
+        outs = [torch.full_like(d[n], 7.0) for n in ("q", "k", "v", "q", "q")]
+        vig.vig_bigla_bwd(d["q"], d["k"], d["v"], *la, d["d_out"], *outs)
+        torch.cuda.synchronize()
+        return outs
+    return call
+
+
+@pytest.mark.parametrize("L", [60, 196, 400])
+def test_gradient_whose_wait_expires_stores_nothing(L):
+    """One chunk, a pair, chunks through scratch (where the first of three launches lets its wait run out, and the last must
+    not go by what that did not write): the status word says so once, and the next call is as before."""
+    call = _gradient_call(L)
+    want = call()
+    assert vig.vig_last_device_status() == 0
+    vig.vig_test_expire_next_wait()
+    assert all(bool((o == 7.0).all()) for o in call())
+    assert vig.vig_last_device_status() == -7 and vig.vig_last_device_status() == 0
+    assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(call(), want))
+
+
+def test_pair_whose_exchange_expires_stores_no_gate_gradients():
+    """The left chunk of a pair (112 of 196 tokens) without the right one's sums: its gate gradients stay unwritten."""
+    call = _gradient_call(196)
+    want = call()
+    vig.vig_test_expire_next_exchange()
+    got = call()
+    assert vig.vig_last_device_status() == -7 and vig.vig_last_device_status() == 0
+    same = lambda a, b: torch.equal(a.view(torch.int16), b.view(torch.int16))
+    for a, b in zip(got[:3], want[:3]):
+        assert same(a, b)
+    for a, b in zip(got[3:], want[3:]):
+        assert bool((a[:, :, :112] == 7.0).all()) and same(a[:, :, 112:].contiguous(), b[:, :, 112:].contiguous())

@@ -288,6 +288,26 @@ def test_expired_device_wait_is_reported_and_leaves_the_library_usable(oracle):
     assert rel_err(device_to_f64(out, "bf16"), oracle_out(oracle, x["q"], x["k"], x["v"], la_f, la_b, "bf16")) <= TOL["bf16"]
 
 
+@pytest.mark.parametrize("L", [60, 300])
+def test_expired_wait_of_the_warp_tile_forms_stores_nothing(L):
+    """A unit in one block, and chunks in three launches, of which the last must not go by what the first did not write."""
+    cfg, x = random_problem(1950 + L, 2, 2, L, 16, 32, "bf16")
+    d = {n: to_device(a, "bf16") for n, a in x.items()}
+
+    def call():
+        out = torch.full_like(d["v"], 7.0)
+        vig.vig_bigla_fwd_gates_bf16(d["q"], d["k"], d["v"], d["g_fwd"], d["g_bwd"], out, cfg.tau)
+        torch.cuda.synchronize()
+        return out
+
+    want = call()
+    assert vig.vig_last_device_status() == 0
+    vig.vig_test_expire_next_wait()
+    assert bool((call() == 7.0).all())
+    assert vig.vig_last_device_status() == -7 and vig.vig_last_device_status() == 0
+    assert torch.equal(call().view(torch.int16), want.view(torch.int16))
+
+
 @pytest.mark.parametrize("name", [c.name for c in synth.SWEEP_CONFIGS])
 def test_second_workload_resolution_sweep_and_hierarchical_stages(oracle, name):
     """The resolution sweep (L = 196 .. 16384) and the stage shapes of the hierarchical variant (dk = 16, dv = 32,
