@@ -66,6 +66,13 @@ static bool use_mma_chunks(long long units, int L, int dk, int dv, bool gates) {
            mma_chunks_preferred(units, L, dk, dv, gates);
 }
 
+// Whether a bf16 call from gate logits takes the segmented launch, whose blocks wait for one another and are sized to fill the
+// chip: nothing else may hold an SM meanwhile.
+static bool takes_segments(long long units, int L, int dk, int dv) {
+    return kernel_preference() != VIG_TEST_KERNEL_SIMT && tc_supported(dk, dv) && !umma_supported(dk, dv, L) &&
+           !use_mma_chunks(units, L, dk, dv, true) && !use_mma_chunks(units, L, dk, dv, false) && use_segments(units, L, dk, dv);
+}
+
 // Scratch of the tcgen05 forms.
 static size_t umma_workspace_bytes(long long units, int L, int dk, int dv) {
     return use_segments(units, L, dk, dv) ? umma_seg_workspace_bytes(units, L) : umma_long_workspace_bytes(units, L, dk, dv);
@@ -500,9 +507,18 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
     // A unit's bytes are multiples of 16 whenever dk and dv are multiples of 8 (bf16) or 4 (fp32).
     const size_t in_bytes = units * (4 * unit_k + unit_v), out_bytes = units * unit_v;
     const bool whole = unit_k % 16 == 0 && unit_v % 16 == 0;
+    // Slices of whole units: while slice i + 1 travels to the device, the kernels of slice i run and slice i - 1 travels back.
+    // The way in bounds the call (55 GB/s), and what comes after the last copy in is pure addition, so each slice is about
+    // 0.35 of the one before: just enough for its way in to cover the way back of that one (a third of the bytes).  More
+    // slices only pay for larger results.  Small results, and unit sizes that would misalign a slice, go through the caller's
+    // stream in one piece.
+    int nsl = out_bytes >= (8u << 20) ? 3 : (out_bytes >= (1u << 20) ? 2 : 1);
+    if (!whole || units < 8) nsl = 1;
     // The way back by a kernel, beside the copies to the device; the way in by a kernel as well where the fixed cost of five
-    // engine copies (20 us more) outweighs the engine's higher rate (7 %).  Pageable memory takes the engines.
-    const bool out_kernel = whole && host_copy_usable(out, out_bytes);
+    // engine copies (20 us more) outweighs the engine's higher rate (7 %).  Pageable memory takes the engines, and so do slices
+    // beside the segmented launch: a copy kernel there keeps blocks that others spin on from starting until the link is done.
+    const bool engines = !whole || (nsl > 1 && dtype == VIG_DTYPE_BF16 && takes_segments(units, L, dk, dv));
+    const bool out_kernel = !engines && host_copy_usable(out, out_bytes);
     const bool in_kernel = out_kernel && in_bytes <= (8u << 20) && host_copy_usable(q, units * unit_k) && host_copy_usable(k, units * unit_k) &&
                            host_copy_usable(v, units * unit_v) && host_copy_usable(g_fwd, units * unit_k) && host_copy_usable(g_bwd, units * unit_k);
     auto copy_in = [&](size_t ok_, size_t ov, size_t nbk, size_t nbv, cudaStream_t s) {
@@ -516,13 +532,6 @@ int vig_bigla_fwd_host(const void* q, const void* k, const void* v, const void* 
         for (const HostCopy& x : c) good = good && cudaMemcpyAsync(x.dst, x.src, x.bytes, cudaMemcpyHostToDevice, s) == cudaSuccess;
         return good;
     };
-    // Slices of whole units: while slice i + 1 travels to the device, the kernels of slice i run and slice i - 1 travels back.
-    // The way in bounds the call (55 GB/s), and what comes after the last copy in is pure addition, so each slice is about
-    // 0.35 of the one before: just enough for its way in to cover the way back of that one (a third of the bytes).  More
-    // slices only pay for larger results.  Small results, and unit sizes that would misalign a slice, go through the caller's
-    // stream in one piece.
-    int nsl = out_bytes >= (8u << 20) ? 3 : (out_bytes >= (1u << 20) ? 2 : 1);
-    if (!whole || units < 8) nsl = 1;
     auto copy_out = [&](size_t ov, size_t nbv, cudaStream_t s) {
         const HostCopy c = {dout + ov, (char*)out + ov, nbv};
         return out_kernel ? launch_host_copy(&c, 1, nsl > 1 ? 2 : 32, s) == cudaSuccess : cudaMemcpyAsync(c.dst, c.src, nbv, cudaMemcpyDeviceToHost, s) == cudaSuccess;

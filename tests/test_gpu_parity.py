@@ -568,6 +568,22 @@ def test_host_entry_point_matches_device_path(oracle, idx):
     np.testing.assert_array_equal(out_n, ref_bytes)
 
 
+def test_host_slices_beside_the_segmented_launch_travel_by_the_copy_engines(segment_path):
+    """The segmented launch counts on every SM: a sliced host call of that form launches its own kernels alone (gate preparation
+    and the segments per slice), and its results are those of the device call, bit for bit."""
+    cfg, x = random_problem(2700, 96, 1, 400, 32, 64, "bf16")
+    host = {n: torch.from_numpy(a.view(np.int16)).pin_memory() for n, a in x.items()}
+    out_h = torch.zeros(x["v"].shape, dtype=torch.int16).pin_memory()
+    before = vig.vig_kernel_launch_count()
+    vig.vig_bigla_fwd_host(host["q"], host["k"], host["v"], host["g_fwd"], host["g_bwd"], out_h, cfg.tau, vig.VIG_DTYPE_BF16)
+    assert vig.vig_kernel_launch_count() - before == 4
+    assert vig.vig_last_device_status() == 0
+    d = {n: to_device(a, "bf16") for n, a in x.items()}
+    out_d = torch.empty_like(d["v"])
+    vig.vig_bigla_fwd_gates_bf16(d["q"], d["k"], d["v"], d["g_fwd"], d["g_bwd"], out_d, cfg.tau)
+    np.testing.assert_array_equal(out_h.numpy().view(np.uint16), to_stored(out_d, "bf16"))
+
+
 def test_host_memory_is_touched_by_kernels_only_where_all_of_it_is_mapped():
     """The predicate alone, nothing is launched: part of a range registered, two registrations side by side, a gap between
     them, pageable memory, addresses and sizes that are not whole 16-byte pieces."""
