@@ -38,4 +38,6 @@ from .binding import (  # noqa: F401
     VIG_TEST_KERNEL_SIMT,
     VIG_TEST_KERNEL_CHUNK_TASKS,
     VIG_TEST_KERNEL_SEGMENTS,
+    VIG_TEST_KERNEL_TCGEN05,
+    VIG_TEST_KERNEL_WARP_TILES,
 )

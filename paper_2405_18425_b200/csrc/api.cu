@@ -62,8 +62,9 @@ static bool use_segments(long long units, int L, int dk, int dv) {
 }
 
 static bool use_mma_chunks(long long units, int L, int dk, int dv, bool gates) {
-    return kernel_preference() == VIG_TEST_KERNEL_AUTO && !umma_supported(dk, dv, L) && mma_chunks_supported(units, L, dk, dv) &&
-           mma_chunks_preferred(units, L, dk, dv, gates);
+    if (umma_supported(dk, dv, L) || !mma_chunks_supported(units, L, dk, dv)) return false;
+    const int pref = kernel_preference();
+    return pref == VIG_TEST_KERNEL_AUTO ? mma_chunks_preferred(units, L, dk, dv, gates) : pref == VIG_TEST_KERNEL_WARP_TILES;
 }
 
 // Whether a bf16 call from gate logits takes the segmented launch, whose blocks wait for one another and are sized to fill the
@@ -200,7 +201,8 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     if (empty) return VIG_OK;
     const long long units = (long long)B * H;
     using bf = __nv_bfloat16;
-    if (tc_supported(dk, dv) && umma_supported(dk, dv, L) && kernel_preference() == VIG_TEST_KERNEL_AUTO) {
+    const int pref = kernel_preference();
+    if (tc_supported(dk, dv) && umma_supported(dk, dv, L) && (pref == VIG_TEST_KERNEL_AUTO || pref >= VIG_TEST_KERNEL_TCGEN05)) {
         cudaError_t e = launch_bigla_umma((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out,
                                           units, L, dk, dv, tau, stream);
         if (e == cudaSuccess && o_local)
@@ -598,7 +600,7 @@ int vig_last_device_status(void* stream) {
 
 int vig_test_set_kernel_preference(int preference) {
     if (preference != VIG_TEST_KERNEL_AUTO && preference != VIG_TEST_KERNEL_SIMT && preference != VIG_TEST_KERNEL_CHUNK_TASKS &&
-        preference != VIG_TEST_KERNEL_SEGMENTS)
+        preference != VIG_TEST_KERNEL_SEGMENTS && preference != VIG_TEST_KERNEL_TCGEN05 && preference != VIG_TEST_KERNEL_WARP_TILES)
         return VIG_ERR_UNSUPPORTED;
     g_kernel_pref.store(preference, std::memory_order_relaxed);
     return VIG_OK;

@@ -38,6 +38,7 @@
 #include "recurrence.cuh"
 #include "tma_host.h"
 #include "umma.cuh"
+#include "test_hooks.h"
 #include "vig_internal.h"
 
 namespace vig {
@@ -1036,7 +1037,9 @@ cudaError_t launch_bigla_umma_seg(const __nv_bfloat16* q, const __nv_bfloat16* k
 cudaError_t launch_bigla_umma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                               const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                               int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
-    if (mma_preferred(units, L, dk, dv, gate_tau > 0.f)) return launch_bigla_mma(q, k, v, la_f, la_b, out, units, L, dk, dv, gate_tau, stream);
+    const int pref = kernel_preference();
+    if (pref == VIG_TEST_KERNEL_WARP_TILES || (pref != VIG_TEST_KERNEL_TCGEN05 && mma_preferred(units, L, dk, dv, gate_tau > 0.f)))
+        return launch_bigla_mma(q, k, v, la_f, la_b, out, units, L, dk, dv, gate_tau, stream);
 #define VIG_CASE(DK_, DV_)                                                                                              \
     if (dk == DK_ && dv == DV_)                                                                                         \
         return gate_tau > 0.f ? launch_umma_t<DK_, DV_, true>(q, k, v, la_f, la_b, out, units, L, gate_tau, stream)     \

@@ -8,6 +8,9 @@
  *   VIG_TEST_KERNEL_CHUNK_TASKS  sequences of more than 256 tokens always take the three chunk-task launches
  *   VIG_TEST_KERNEL_SEGMENTS     sequences of 257 .. 8192 tokens always take the segmented single launch
  *                          (the default chooses between the two by segment count and unit count).
+ *   VIG_TEST_KERNEL_TCGEN05      always the tcgen05 kernels: the single-block one up to 256 tokens, chunk tasks or segments beyond
+ *   VIG_TEST_KERNEL_WARP_TILES   always the kernels of one warp per 16 tokens, one block per unit or per chunk
+ *                          (the default chooses between these by head size, length and unit count).
  *                          vig_bigla_workspace_bytes follows the setting: query it under the setting the call
  *                          will run with
  * Returns VIG_OK, or VIG_ERR_UNSUPPORTED for an unknown value (the setting is then unchanged). */
@@ -20,7 +23,8 @@
 extern "C" {
 #endif
 
-enum vig_test_kernel { VIG_TEST_KERNEL_AUTO = 0, VIG_TEST_KERNEL_SIMT = 2, VIG_TEST_KERNEL_CHUNK_TASKS = 3, VIG_TEST_KERNEL_SEGMENTS = 4 };
+enum vig_test_kernel { VIG_TEST_KERNEL_AUTO = 0, VIG_TEST_KERNEL_SIMT = 2, VIG_TEST_KERNEL_CHUNK_TASKS = 3, VIG_TEST_KERNEL_SEGMENTS = 4,
+                       VIG_TEST_KERNEL_TCGEN05 = 5, VIG_TEST_KERNEL_WARP_TILES = 6 };
 int vig_test_set_kernel_preference(int preference);
 
 /* Synchronises `stream`, then returns and clears the number of (batch, head) units that the tensor-core kernels of the

@@ -118,6 +118,15 @@ def test_fused_blend_on_a_unit_handed_to_the_recurrence(oracle):
     assert rel_err(got, ref) <= TOL["bf16"]
 
 
+@pytest.mark.parametrize("pref", [vig.VIG_TEST_KERNEL_TCGEN05, vig.VIG_TEST_KERNEL_WARP_TILES])
+def test_fused_blend_on_a_handed_over_unit_of_either_form(oracle, pref):
+    vig.vig_test_set_kernel_preference(pref)
+    try:
+        test_fused_blend_on_a_unit_handed_to_the_recurrence(oracle)
+    finally:
+        vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_AUTO)
+
+
 def test_dwconv3x3_many_channels_in_slabs(oracle):
     """More than 256 sixteen-byte channel groups: the groups are split over the grid's second dimension, raggedly."""
     rng = np.random.default_rng(77)

@@ -707,6 +707,47 @@ def test_every_kernel_family_meets_the_bar(oracle, pref, dk, dv, L):
     assert rel_err(got, ref) <= TOL["bf16"]
 
 
+@pytest.fixture(params=[vig.VIG_TEST_KERNEL_TCGEN05, vig.VIG_TEST_KERNEL_WARP_TILES], ids=["tcgen05", "warp_tiles"])
+def either_form(request):
+    """The tcgen05 kernels, then the kernels of one warp per 16 tokens, whatever the default dispatch takes."""
+    vig.vig_test_set_kernel_preference(request.param)
+    yield request.param
+    vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_AUTO)
+
+
+@pytest.mark.parametrize("dk,dv", [(16, 32), (16, 64), (24, 48), (32, 32), (32, 64)])
+@pytest.mark.parametrize("L", [1, 40, 128, 129, 196, 256, 300, 700])
+def test_either_form_meets_the_bar(oracle, either_form, dk, dv, L):
+    cfg, x = random_problem(650 + L, 3, 2, L, dk, dv, "bf16", gate_mean=1.0)
+    for run in (_run_unfused, _run_fused):
+        got, ref = run(oracle, cfg, x)
+        assert np.isfinite(got).all()
+        assert rel_err(got, ref) <= TOL["bf16"]
+
+
+def test_either_form_hands_units_over(oracle, either_form):
+    """Units whose gates leave the range of the factorised tiles, counted, beside ordinary ones; logits at both asymptotes."""
+    test_fallback_counter_counts_out_of_range_units(oracle)
+    test_mixed_units_fast_and_exact_paths(oracle)
+    test_fused_gates_temperature_and_extreme_logits(oracle, 16.0)
+
+
+@pytest.mark.parametrize("case", ["alpha_one", "closed", "wall", "mixed", "steep"])
+def test_either_form_with_degenerate_gates(oracle, either_form, case):
+    test_degenerate_gates(oracle, case, "bf16", 32, 64, 196)
+    test_degenerate_gates(oracle, case, "bf16", 24, 48, 700)
+
+
+@pytest.mark.parametrize("gate", [-0.45, "mix"])
+def test_either_form_with_steep_gates_inside_its_range(oracle, either_form, gate):
+    test_steep_gates_inside_the_factorised_range(oracle, 32, 64, 196, gate)
+    test_steep_gates_inside_the_factorised_range(oracle, 24, 48, 700, gate)
+
+
+def test_either_form_reports_an_expired_wait(oracle, either_form):
+    test_expired_device_wait_is_reported_and_leaves_the_library_usable(oracle)
+
+
 def test_kernel_preference_rejects_unknown_values():
     lib = vig.load()
     assert lib.vig_test_set_kernel_preference(7) == -3
