@@ -212,7 +212,6 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const Tile<64> t64(lane);
     const Tile<RV> tvv(lane);
 
-    pdl_launch_dependents();
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 8, 1);
@@ -222,6 +221,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();
+    pdl_launch_dependents();
     if (tid == 0) {
         mbar_expect_tx(bar, 4 * lay.op_bytes + 2 * lay.g);
         tma_load_3d(op(kQb), &tm_f, 0, row0, (int)unit, bar);
@@ -854,8 +854,8 @@ __global__ void __launch_bounds__(256) grad_fold_kernel(const GArgs a) {
     const float* own0 = a.u + ((first * 4 + kind) * DV + n) * DK + 4 * p;
     const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
     uint8_t* img = a.img + (first * 4 + kind) * 2 * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
     auto walk = [&](bool emit) {
         const float *own_p = own0, *dec_p = dec0;

@@ -100,7 +100,6 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     float* totals = reinterpret_cast<float*>(smem + lay.totals);
     volatile int* slow = reinterpret_cast<volatile int*>(smem + lay.bar + 32);
 
-    pdl_launch_dependents();
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_init(bar + 8, MODE == kMain ? 1 : 2 * MV);   // the states: one bulk copy, or one arrival per piece formed here
@@ -109,6 +108,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     pdl_wait();
+    pdl_launch_dependents();
     if (tid == 0) {
         mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
         tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
@@ -456,8 +456,8 @@ __global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a) {
     const float* own0 = a.u + ((first * 2 + dir) * DV + n) * DK + 4 * p;
     const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
     uint8_t* img = a.img + (first * 2 + dir) * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
     auto walk = [&](bool emit) {
         const float *own_p = own0, *dec_p = dec0;

@@ -212,7 +212,6 @@ bigla_umma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tma_load_3d(t_v, &tm_v, 0, r0, unit, bar_v);
     };
 
-    pdl_launch_dependents();   // the next kernel's set-up may overlap this grid
     if (warp == 2 && elect_one()) {
         // Warm L2 with this block's first unit while the kernel before this one in the stream still runs: a prefetch
         // consumes nothing, and L2 stays coherent with whatever that kernel is still writing.
@@ -255,6 +254,7 @@ bigla_umma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     zero_tail_rows();
     if (tid < 128) dec[tid] = 0.f;   // key dims a narrow head never writes
     pdl_wait();   // nothing above touches global memory: it may run while the previous kernel in the stream drains
+    pdl_launch_dependents();
     if (warp == 0 && elect_one()) {
         load_gates(group, 2 * lay.tile);
         load_qk(group, 0);

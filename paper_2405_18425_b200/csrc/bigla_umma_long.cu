@@ -157,7 +157,6 @@ bigla_long_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tma_load_3d(t_v, &tm_v, 0, task_chunk(t) * kChunk, task_unit(t), bar_v);
     };
 
-    pdl_launch_dependents();   // the next kernel's set-up may overlap this grid
     if (wq == 2 && blockIdx.x < args.tasks && elect_one()) {
         // Warm L2 with this block's first task while the kernel before this one in the stream still runs: a prefetch
         // consumes nothing, and L2 stays coherent with whatever that kernel is still writing.  The main launch only
@@ -190,6 +189,7 @@ bigla_long_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     build_zero_one_tile(bp + Y::zf, tid + kLThreads);
     if (tid < 64) totals[tid] = 0.f;   // key dims a narrow head never writes
     pdl_wait();   // nothing above touches global memory: it may run while the previous kernel in the stream drains
+    pdl_launch_dependents();
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -529,8 +529,8 @@ bigla_long_fold_kernel(const uint8_t* ws_slots, uint8_t* ws_img, const float* ws
     constexpr int kBatch = 32;
     const int unit = blockIdx.x, dir = blockIdx.y;
     const int i = blockIdx.z * kFoldRows + threadIdx.x / C4, c = threadIdx.x % C4;
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     int flagged = 0;
     for (int m = threadIdx.x; m < nch; m += blockDim.x) flagged |= ws_cflags[(size_t)unit * nch + m];
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);

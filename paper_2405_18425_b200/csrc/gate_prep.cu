@@ -39,8 +39,8 @@ __device__ __forceinline__ uint4 log_alpha_bf16x8(uint4 raw, float inv_tau) {
 template <typename T>
 __global__ void __launch_bounds__(256) gate_prep_kernel(const T* g_f, const T* g_b, T* la_f, T* la_b, long long n, float inv_tau) {
     // no __restrict__: the output may alias the input (in-place call)
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     const T* g = blockIdx.y == 0 ? g_f : g_b;
     T* la = blockIdx.y == 0 ? la_f : la_b;
     constexpr int V = 16 / sizeof(T);
@@ -89,8 +89,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) gate_prep_bwd_kernel(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n,
                                                             float inv_tau) {
     // no __restrict__: the output may be the incoming gradient's buffer
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     const T* g = blockIdx.y == 0 ? g_f : g_b;
     const T* d = blockIdx.y == 0 ? d_f : d_b;
     T* o = blockIdx.y == 0 ? o_f : o_b;

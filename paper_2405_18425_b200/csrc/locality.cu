@@ -77,7 +77,6 @@ __global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ 
     const uint32_t tile_bytes = (uint32_t)(th + 2) * (tw + 2) * gpb * 16;
     const uint32_t buf_pitch = (tile_bytes + 127) / 128 * 128;
     const uint32_t bar0 = smem_u32(dw_bar);
-    pdl_launch_dependents();
     if (threadIdx.x == 0) {
         mbar_init(bar0, 1);
         mbar_init(bar0 + 8, 1);
@@ -93,6 +92,7 @@ __global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ 
         tma_load_4d(smem_u32(dw_smem) + buf * buf_pitch, &tm_x, c_slab, j0 - 1, i0 - 1, n, bar0 + 8 * buf);
     };
     pdl_wait();   // x may be the output of the kernel before this one in the stream
+    pdl_launch_dependents();
     if (threadIdx.x == 0 && (int)blockIdx.x < tasks) issue(blockIdx.x, 0);
     f32x2 wr[9][V / 2], br[V / 2];   // filter taps and biases of the thread's channels as fp32 pairs
 #pragma unroll
@@ -185,8 +185,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) gate_blend_kernel(const T* o_local, const T* z, const T* o_global, T* out, long long n) {
     // no __restrict__: out may be o_global (in-place call)
     constexpr int V = Vec<T>::N;
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
     const long long nvec = n / V, stride = (long long)gridDim.x * blockDim.x;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < nvec; x += stride) {
         float a[V], b[V], c[V];

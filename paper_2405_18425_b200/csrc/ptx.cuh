@@ -83,6 +83,9 @@ __device__ __forceinline__ void named_bar(int id, int count) {
 // exited).  `pdl_wait`: blocks until every kernel this grid depends on has completed and its memory operations are
 // visible; a no-op for an ordinary launch.  The kernels here execute it before their first global-memory read into
 // shared memory or registers and before any write; prefetches into L2, which consume nothing, may precede it.
+// They let the next kernel start behind their own wait: before it, a run of small launches is let in several kernels deep, and the
+// blocks of one kernel, waiting, crowd those of another onto the same SMs (64 units of 196 tokens, 32 x 64, from logits: 11.7 us
+// a call, 7.6 this way; one sequence of 9762 tokens 23.3 and 14.7).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

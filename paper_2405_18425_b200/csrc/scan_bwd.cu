@@ -58,8 +58,8 @@ __global__ void __launch_bounds__(bwd_max_warps(CN) * 32, CN <= 16 ? 2 : 1) scan
     float* gs = vs + TG * kPitch;
     ulonglong2* st = reinterpret_cast<ulonglong2*>(sb_smem + nw * bwd_stage_floats(CN));   // [warp][kind][CN / 4][lane]
     float* dec = sb_smem + nw * bwd_stage_floats(CN) + (size_t)nw * 4 * kRows * DVP;       // [warp][kind][8]
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
 
     // the next TG tokens of a walk (t = base + step n) on their way; Z decays by the other direction's gate of the token before
     T rk, rq, rs, rz;

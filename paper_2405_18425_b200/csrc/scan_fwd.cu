@@ -50,8 +50,8 @@ __global__ void __launch_bounds__(scan_max_warps(RPL) * 32, RPL <= 8 ? 2 : 1) sc
     float* ks = xs + TG * DKP;
     float* as = ks + TG * DKP;
     float* vs = as + TG * DKP;                          // [TG][16]
-    pdl_launch_dependents();
     pdl_wait();
+    pdl_launch_dependents();
 
     // the next TG tokens of a walk (t = base + step n) on their way, four key dimensions (value columns) of a token per lane
     using P = Piece<T, VEC>;
