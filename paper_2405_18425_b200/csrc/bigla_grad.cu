@@ -27,7 +27,7 @@
 #include <atomic>
 
 #include "mma.cuh"
-#include "recurrence.cuh"
+#include "scan_bwd.cuh"
 #include "tma_host.h"
 #include "vig_internal.h"
 
@@ -99,84 +99,47 @@ __device__ __forceinline__ void st_async1(uint32_t addr, uint32_t v, uint32_t ba
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }   // orders no memory accesses
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
-// Sixteen bits of two words: an fp32 kept in two bf16 buffers.
-__device__ __forceinline__ void put_halves(__nv_bfloat16* hi, __nv_bfloat16* lo, float x) {
-    *reinterpret_cast<unsigned short*>(hi) = (unsigned short)(__float_as_uint(x) >> 16);
-    *reinterpret_cast<unsigned short*>(lo) = (unsigned short)(__float_as_uint(x) & 0xffffu);
-}
-__device__ __forceinline__ float get_halves(const __nv_bfloat16* hi, const __nv_bfloat16* lo) {
-    return __uint_as_float(((uint32_t)*reinterpret_cast<const unsigned short*>(hi) << 16) | *reinterpret_cast<const unsigned short*>(lo));
-}
-__device__ __forceinline__ float warp_sum(float x) {
-#pragma unroll
-    for (int m = 16; m >= 1; m >>= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
-    return x;
-}
-
-// A unit whose gates leave the range of the factorised tiles: the adjoint recurrences step by step in fp32.  A warp takes
-// one key dimension at a time (rows of S and Z over its lanes, sums over the value dimension by shuffles) for dq, dk and
-// the gate gradients, then one value column at a time for dv; the warps of all blocks of the unit share the work.  What
-// the ascending walk leaves for the descending one is kept, as fp32, in the four result buffers of that key dimension.
-template <int DK, int DV>
-__device__ __noinline__ void gradient_by_recurrence(const GArgs& a, size_t unit, int worker, int workers, int lane) {
-    const int L = a.L;
-    const size_t ok = unit * L * DK, ov = unit * L * DV;
-    constexpr int NC = (DV + 31) / 32;
-    for (int i = worker; i < DK; i += workers) {
-        for (int walk = 0; walk < 2; ++walk) {
-            float S[NC], Z[NC], run_f = 0.f, run_b = 0.f;
-#pragma unroll
-            for (int n = 0; n < NC; ++n) S[n] = Z[n] = 0.f;
-            const __nv_bfloat16 *ls = (walk == 0 ? a.la_f : a.la_b) + ok + i, *lz = (walk == 0 ? a.la_b : a.la_f) + ok + i;
-            for (int m = 0; m < L; ++m) {
-                const int t = walk == 0 ? m : L - 1 - m, tp = walk == 0 ? t - 1 : t + 1;
-                const size_t e = ok + (size_t)t * DK + i;
-                const float kk = __bfloat162float(a.k[e]), qq = __bfloat162float(a.q[e]);
-                const float ds = expf(__bfloat162float(ls[(size_t)t * DK])), dz = m > 0 ? expf(__bfloat162float(lz[(size_t)tp * DK])) : 0.f;
-                float aq = 0.f, ak = 0.f;
-#pragma unroll
-                for (int n = 0; n < NC; ++n) {
-                    const int j = lane + 32 * n;
-                    const float vj = j < DV ? __bfloat162float(a.v[ov + (size_t)t * DV + j]) : 0.f;
-                    const float gj = j < DV ? __bfloat162float(a.g[ov + (size_t)t * DV + j]) : 0.f;
-                    S[n] = fmaf(ds, S[n], kk * vj);
-                    Z[n] = fmaf(dz, Z[n], 0.5f * qq * gj);
-                    aq = fmaf(S[n], gj, aq);
-                    ak = fmaf(Z[n], vj, ak);
-                }
-                aq = 0.5f * warp_sum(aq);
-                ak = warp_sum(ak);
-                if (lane == 0) {
-                    if (walk == 0) {
-                        put_halves(a.dq + e, a.dk + e, aq);         // dq>
-                        put_halves(a.dla_f + e, a.dla_b + e, ak);   // dk<
-                    } else {
-                        const float qf = get_halves(a.dq + e, a.dk + e), kb = get_halves(a.dla_f + e, a.dla_b + e);
-                        run_f += qq * qf - kk * ak;
-                        a.dq[e] = __float2bfloat16_rn(qf + aq);
-                        a.dk[e] = __float2bfloat16_rn(ak + kb);
-                        a.dla_f[e] = __float2bfloat16_rn(run_f);
-                        a.dla_b[e] = __float2bfloat16_rn(-run_b);
-                        run_b += qq * aq - kk * kb;
-                    }
-                }
-            }
-        }
+// dq>, dk< of an element between the walks of gradient_by_walks, as fp32 in two bf16 result buffers each (written over at the end).
+struct ResultPairs {
+    __nv_bfloat16 *dq, *dk, *dla_f, *dla_b;
+    static __device__ __forceinline__ void put_halves(__nv_bfloat16* hi, __nv_bfloat16* lo, float x) {
+        *reinterpret_cast<unsigned short*>(hi) = (unsigned short)(__float_as_uint(x) >> 16);
+        *reinterpret_cast<unsigned short*>(lo) = (unsigned short)(__float_as_uint(x) & 0xffffu);
     }
-    for (int j = worker; j < DV; j += workers) {   // lanes are key dimensions
-        const bool live = lane < DK;
-        for (int walk = 0; walk < 2; ++walk) {
-            float Z = 0.f;
-            const __nv_bfloat16* lz = walk == 0 ? a.la_b : a.la_f;
-            for (int m = 0; m < L; ++m) {
-                const int t = walk == 0 ? m : L - 1 - m, tp = walk == 0 ? t - 1 : t + 1;
-                const size_t e = ok + (size_t)t * DK + lane, o = ov + (size_t)t * DV + j;
-                const float dz = live && m > 0 ? expf(__bfloat162float(lz[ok + (size_t)tp * DK + lane])) : 0.f;
-                Z = fmaf(dz, Z, live ? 0.5f * __bfloat162float(a.q[e]) * __bfloat162float(a.g[o]) : 0.f);
-                const float s = warp_sum(live ? __bfloat162float(a.k[e]) * Z : 0.f);
-                if (lane == 0) a.dv[o] = __float2bfloat16_rn(walk == 0 ? s : __bfloat162float(a.dv[o]) + s);
-            }
-        }
+    static __device__ __forceinline__ float get_halves(const __nv_bfloat16* hi, const __nv_bfloat16* lo) {
+        return __uint_as_float(((uint32_t)*reinterpret_cast<const unsigned short*>(hi) << 16) | *reinterpret_cast<const unsigned short*>(lo));
+    }
+    __device__ __forceinline__ void put(size_t e, float2 x) const {
+        put_halves(dq + e, dk + e, x.x);
+        put_halves(dla_f + e, dla_b + e, x.y);
+    }
+    __device__ __forceinline__ float2 get(size_t e) const { return make_float2(get_halves(dq + e, dk + e), get_halves(dla_f + e, dla_b + e)); }
+};
+struct WalkArgs {
+    scan::ScanBwdArgs<__nv_bfloat16> bwd;
+    scan::ScanArgs<__nv_bfloat16> fwd;
+    ResultPairs pairs;
+};
+
+// A unit whose gates leave the range of the factorised tiles: the fp32 walks of any decay (scan_bwd.cuh for dq, dk and the gate
+// gradients, scan_fwd.cuh on (k, q, d_out) for dv), a sequence cut into as many segments as the block has warps, or room for in
+// the shared memory of its dead tiles.  The unit's slabs of eight key dimensions and of sixteen value columns are dealt out
+// over its blocks.  Every thread of the block calls it.  768 such units of 196 tokens (32, 64): 10.9 ms with one key dimension
+// or value column a warp, serial over the tokens.
+template <int DK, int DV>
+__device__ __noinline__ void gradient_by_walks(WalkArgs x, size_t unit, int block, int blocks, float* smem, uint32_t smem_bytes) {
+    constexpr int kBwdSlabs = DK / scan::kRows, kSlabs = kBwdSlabs + DV / scan::kCols, RPL = DK <= 16 ? 4 : 8;
+    constexpr size_t kBwd = scan::bwd_stage_floats(DV / 4) + scan::bwd_fold_floats(DV / 4);
+    constexpr size_t kFwd = scan::scan_stage_floats(RPL) > scan::scan_fold_floats(RPL) ? scan::scan_stage_floats(RPL) : scan::scan_fold_floats(RPL);
+    constexpr int kPerWarp = (int)(4 * (kBwd > kFwd ? kBwd : kFwd));
+    const int L = x.bwd.L, w = threadIdx.x >> 5;
+    int nw = max(1, min(min((int)blockDim.x >> 5, scan::bwd_max_warps(DV / 4)), (int)smem_bytes / kPerWarp));
+    x.bwd.seg_len = x.fwd.seg_len = ((L + nw - 1) / nw + scan::TG - 1) / scan::TG * scan::TG;
+    nw = (L + x.bwd.seg_len - 1) / x.bwd.seg_len;
+    for (int slab = block; slab < kSlabs; slab += blocks) {
+        __syncthreads();   // the tiles, or the slab before
+        if (slab < kBwdSlabs) scan::scan_bwd_slab<__nv_bfloat16, DV / 4, true>(x.bwd, x.pairs, unit, slab, w, nw, smem);
+        else scan::scan_fwd_slab<__nv_bfloat16, RPL, true>(x.fwd, unit, slab - kBwdSlabs, w, nw, smem);
     }
 }
 
@@ -220,6 +183,11 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         state_word[0] = 0;   // (the other word is written by the other block alone, and read once that has landed)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    auto walk_args = [&] {   // the adjoint walk for dv: (k, q, d_out), the gates exchanged and moved by one token
+        return WalkArgs{{a.q, a.k, a.v, a.la_f, a.la_b, a.g, a.dq, a.dk, a.dla_f, a.dla_b, a.L, DK, DV, 0},
+                        {a.k, a.q, a.g, a.la_b, a.la_f, a.dv, a.L, DK, DV, 0, -1, 1},
+                        {a.dq, a.dk, a.dla_f, a.dla_b}};
+    };
     pdl_wait();
     pdl_launch_dependents();
     if (tid == 0) {
@@ -423,13 +391,13 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
             if (missing) return;             // a summary of this unit did not get its inputs, and has said so
             if (chunk == 0 && tid == 0) atomicAdd(a.dev_status + 1, 1);
-            gradient_by_recurrence<DK, DV>(a, unit, chunk * nw + w, nch * nw, lane);
+            gradient_by_walks<DK, DV>(walk_args(), unit, chunk, nch, reinterpret_cast<float*>(smem), lay.bar);
             return;
         }
     }
     if (MODE == kSingle && state_word[0]) {
         if (tid == 0) atomicAdd(a.dev_status + 1, 1);
-        gradient_by_recurrence<DK, DV>(a, unit, w, nw, lane);
+        gradient_by_walks<DK, DV>(walk_args(), unit, 0, 1, reinterpret_cast<float*>(smem), lay.bar);
         return;
     }
 
@@ -521,7 +489,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                 return;
             }
             if (chunk == 0 && tid == 0) atomicAdd(a.dev_status + 1, 1);
-            gradient_by_recurrence<DK, DV>(a, unit, chunk * nw + w, nch * nw, lane);
+            gradient_by_walks<DK, DV>(walk_args(), unit, chunk, nch, reinterpret_cast<float*>(smem), lay.bar);
             return;
         }
     }

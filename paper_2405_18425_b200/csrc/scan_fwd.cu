@@ -1,229 +1,20 @@
-// BiGLA forward (paper Eq. 6) step by step in fp32 on the CUDA cores: the fp32 entry point, and the bf16 head sizes the
-// tensor-core kernels do not cover.  No factorised gates, so any decay is in range.
-//
-// Column j of the state depends on column j of v alone, so a block takes sixteen value columns of one unit, and its warps
-// take the sequence in segments that are walked at the same time: every warp first finds, in one ascending pass, what its
-// tokens add to either state and by how much they shrink what enters it; each then folds the segments before it (forward)
-// and after it (backward) and walks its tokens up and down from those states.  What bounds it is the chain of tokens a
-// warp walks (about 50 instructions each), so few units are cut into many segments; enough units to fill the chip are
-// walked whole, without the first pass.  48 units of 196 tokens, 32 x 64, fp32: 31 us; one block of 128 threads per unit,
-// one direction after the other, took 256 us.
-//
-// Lane (rg, cp) keeps rows [rg RPL, rg RPL + RPL) of columns 2 cp, 2 cp + 1 as packed pairs of rows, so that the rows of q,
-// k and the gates come from shared memory as the operands they are.  Tokens are staged TG at a time by the warp that walks
-// them, the next TG on their way in registers meanwhile; no barrier but the two around the fold.
+// Launch of the fp32 forward walks (scan_fwd.cuh): a block per unit and sixteen value columns.
 #include <atomic>
 
-#include "ptx.cuh"
-#include "recurrence.cuh"
+#include "scan_fwd.cuh"
 #include "vig_internal.h"
 
 namespace vig {
 namespace {
 
-constexpr int kCols = 16;   // value columns of a block
-
-template <typename T>
-struct ScanArgs {
-    const T *q, *k, *v, *gf, *gb;   // log gates of the two directions; the gate of token t is element t + sf (t + sb), 0 outside
-    T* out;
-    int L, dk, dv, seg_len, sf, sb;
-};
-
-
-constexpr int TG = 4;   // tokens staged at once
-constexpr int scan_max_warps(int rpl) { return rpl <= 16 ? 8 : 1; }   // segments per block (32 rows a lane: no registers for the first pass)
-constexpr size_t scan_stage_floats(int rpl) { return (size_t)TG * (3 * 4 * rpl + kCols); }
-constexpr size_t scan_fold_floats(int rpl) { return (size_t)2 * 4 * rpl * (kCols + 1); }
+using namespace scan;
 
 template <typename T, int RPL, bool VEC>
 __global__ void __launch_bounds__(scan_max_warps(RPL) * 32, RPL <= 8 ? 2 : 1) scan_fwd_kernel(const ScanArgs<T> a) {
-    constexpr int DKP = 4 * RPL, R2 = RPL / 2, HC = (RPL + 7) / 8;
     extern __shared__ __align__(16) float sc_smem[];
-    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, nw = blockDim.x >> 5;
-    const int cp = lane & 7, rg = lane >> 3;
-    const int L = a.L, dk = a.dk, dv = a.dv;
-    const size_t unit = blockIdx.x, ok = unit * L * dk, ov = unit * L * dv;
-    const int col0 = blockIdx.y * kCols;
-    const int s0 = w * a.seg_len, s1 = min(L, s0 + a.seg_len);
-    float* xs = sc_smem + w * scan_stage_floats(RPL);   // [TG][DKP]: q (walks) or the gates of the backward direction (first pass)
-    float* ks = xs + TG * DKP;
-    float* as = ks + TG * DKP;
-    float* vs = as + TG * DKP;                          // [TG][16]
     pdl_wait();
     pdl_launch_dependents();
-
-    // the next TG tokens of a walk (t = base + step n) on their way, four key dimensions (value columns) of a token per lane
-    using P = Piece<T, VEC>;
-    P rx[HC], rk[HC], ra[HC], rv;
-    auto fetch = [&](int base, int step, const T* x, int sx, const T* ga, int sa) {
-#pragma unroll
-        for (int h = 0; h < HC; ++h) {
-            const int y = lane + 32 * h, t = base + step * (y / RPL), d = 4 * (y % RPL);   // (RPL = 4: the upper half of the warp has nothing to do)
-            const int n = t >= s0 && t < s1 && y < TG * RPL ? dk - d : 0;
-            rx[h].load(x + (ptrdiff_t)(t + sx) * dk + d, t + sx >= 0 && t + sx < L ? n : 0);
-            rk[h].load(a.k + ok + (ptrdiff_t)t * dk + d, n);
-            ra[h].load(ga + (ptrdiff_t)(t + sa) * dk + d, t + sa >= 0 && t + sa < L ? n : 0);
-        }
-        const int t = base + step * (lane >> 2), j = col0 + 4 * (lane & 3);
-        rv.load(a.v + ov + (ptrdiff_t)t * dv + j, lane < TG * kCols / 4 && t >= s0 && t < s1 ? dv - j : 0);
-    };
-    // ... and into shared memory (tokens outside the segment: k = q = 0, gate 1)
-    auto commit = [&](bool x_is_gate) {
-        __syncwarp();
-#pragma unroll
-        for (int h = 0; h < HC; ++h) {
-            const int y = lane + 32 * h;
-            if (RPL >= 8 || y < TG * RPL) {   // (the pieces of a token are consecutive: y is also the place)
-                float4 x = rx[h].get(), g = ra[h].get();
-                if (x_is_gate) x = make_float4(expf(x.x), expf(x.y), expf(x.z), expf(x.w));
-                reinterpret_cast<float4*>(xs)[y] = x;
-                reinterpret_cast<float4*>(ks)[y] = rk[h].get();
-                reinterpret_cast<float4*>(as)[y] = make_float4(expf(g.x), expf(g.y), expf(g.z), expf(g.w));
-            }
-        }
-        if (lane < TG * kCols / 4) reinterpret_cast<float4*>(vs)[lane] = rv.get();
-        __syncwarp();
-    };
-    auto rows = [&](const float* p, int n, f32x2 (&r)[R2]) {
-        const ulonglong2* s = reinterpret_cast<const ulonglong2*>(p + n * DKP + rg * RPL);
-#pragma unroll
-        for (int x = 0; x < R2 / 2; ++x) {
-            const ulonglong2 u = s[x];
-            r[2 * x] = u.x;
-            r[2 * x + 1] = u.y;
-        }
-    };
-    auto cols = [&](int n, f32x2& v0, f32x2& v1) {
-        const float2 v = *reinterpret_cast<const float2*>(vs + n * kCols + 2 * cp);
-        v0 = pack2(v.x, v.x);
-        v1 = pack2(v.y, v.y);
-    };
-
-    f32x2 S[R2][2], X[R2][2];   // the states that enter the segment from the left and from the right
-#pragma unroll
-    for (int r = 0; r < R2; ++r) S[r][0] = S[r][1] = X[r][0] = X[r][1] = 0ull;   // (+0, +0)
-    if (scan_max_warps(RPL) > 1 && nw > 1) {
-        // ---- first pass: forward state left behind (S) and its decay (D); backward state at the first token (X), the running
-        // product of the backward gates (P) turning the recurrence into a sum that also runs upwards ----
-        f32x2 D[R2], P[R2];
-        const f32x2 one = pack2(1.f, 1.f);
-#pragma unroll
-        for (int r = 0; r < R2; ++r) D[r] = P[r] = one;
-        fetch(s0, 1, a.gb + ok, a.sb, a.gf + ok, a.sf);
-        for (int t0 = s0; t0 < s1; t0 += TG) {
-            commit(true);
-            if (t0 + TG < s1) fetch(t0 + TG, 1, a.gb + ok, a.sb, a.gf + ok, a.sf);
-#pragma unroll
-            for (int n = 0; n < TG; ++n) {
-                f32x2 kk[R2], af[R2], ab[R2], v0, v1;
-                rows(ks, n, kk);
-                rows(as, n, af);
-                rows(xs, n, ab);
-                cols(n, v0, v1);
-#pragma unroll
-                for (int r = 0; r < R2; ++r) {
-                    S[r][0] = ffma2(af[r], S[r][0], fmul2(kk[r], v0));
-                    S[r][1] = ffma2(af[r], S[r][1], fmul2(kk[r], v1));
-                    const f32x2 pk = fmul2(P[r], kk[r]);
-                    X[r][0] = ffma2(pk, v0, X[r][0]);
-                    X[r][1] = ffma2(pk, v1, X[r][1]);
-                    D[r] = fmul2(D[r], af[r]);
-                    P[r] = fmul2(P[r], ab[r]);
-                }
-            }
-        }
-        __syncthreads();   // the fold area lies over the staging
-        ulonglong2* st = reinterpret_cast<ulonglong2*>(sc_smem);                    // [warp][dir][R2][lane]
-        f32x2* dec = reinterpret_cast<f32x2*>(sc_smem + (size_t)nw * 2 * DKP * kCols);   // [warp][dir][DKP / 2]
-#pragma unroll
-        for (int r = 0; r < R2; ++r) {
-            st[((w * 2) * R2 + r) * 32 + lane] = make_ulonglong2(S[r][0], S[r][1]);
-            st[((w * 2 + 1) * R2 + r) * 32 + lane] = make_ulonglong2(X[r][0], X[r][1]);
-            if (cp == 0) {
-                dec[(w * 2) * (DKP / 2) + rg * R2 + r] = D[r];
-                dec[(w * 2 + 1) * (DKP / 2) + rg * R2 + r] = P[r];
-            }
-            S[r][0] = S[r][1] = X[r][0] = X[r][1] = 0ull;
-        }
-        __syncthreads();
-        auto fold = [&](int s, int dir, f32x2 (&to)[R2][2]) {
-#pragma unroll
-            for (int r = 0; r < R2; ++r) {
-                const ulonglong2 e = st[((s * 2 + dir) * R2 + r) * 32 + lane];
-                const f32x2 d = dec[(s * 2 + dir) * (DKP / 2) + rg * R2 + r];
-                to[r][0] = ffma2(d, to[r][0], e.x);
-                to[r][1] = ffma2(d, to[r][1], e.y);
-            }
-        };
-        for (int s = 0; s < w; ++s) fold(s, 0, S);
-        for (int s = nw - 1; s > w; --s) fold(s, 1, X);
-        __syncthreads();
-    }
-
-    // ---- the walks: up (o> into `out`), then down ((o> + o<) / 2); the same lane writes and reads back an element ----
-#pragma unroll 1
-    for (int walk = 0; walk < 2; ++walk) {
-        const int step = walk == 0 ? 1 : -1;
-        const T* ga = (walk == 0 ? a.gf : a.gb) + ok;
-        const int sa = walk == 0 ? a.sf : a.sb, first = walk == 0 ? s0 : s1 - 1;
-        if (walk == 1) {
-#pragma unroll
-            for (int r = 0; r < R2; ++r) {
-                S[r][0] = X[r][0];
-                S[r][1] = X[r][1];
-            }
-        }
-        fetch(first, step, a.q + ok, 0, ga, sa);
-        for (int m = 0; m < s1 - s0; m += TG) {
-            const int base = first + step * m;
-            commit(false);
-            if (m + TG < s1 - s0) fetch(base + step * TG, step, a.q + ok, 0, ga, sa);
-            T up[2];
-            if (walk == 1) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int t = base - rg, j = col0 + 2 * cp + h;
-                    up[h] = t >= s0 && j < dv ? a.out[ov + (size_t)t * dv + j] : T(0.f);
-                }
-            }
-            float o[4][2];
-#pragma unroll
-            for (int n = 0; n < 4; ++n) {
-                f32x2 qq[R2], kk[R2], af[R2], v0, v1, a0 = 0ull, a1 = 0ull;
-                rows(xs, n, qq);
-                rows(ks, n, kk);
-                rows(as, n, af);
-                cols(n, v0, v1);
-#pragma unroll
-                for (int r = 0; r < R2; ++r) {
-                    S[r][0] = ffma2(af[r], S[r][0], fmul2(kk[r], v0));   // S_t = G_t . S_prev + k_t^T v_t
-                    S[r][1] = ffma2(af[r], S[r][1], fmul2(kk[r], v1));
-                    a0 = ffma2(qq[r], S[r][0], a0);                      // o_t = q_t S_t
-                    a1 = ffma2(qq[r], S[r][1], a1);
-                }
-                o[n][0] = sum2(a0);
-                o[n][1] = sum2(a1);
-            }
-            // sums over the four row groups, token n to the lanes of row group n
-            float h2[2][2], o1[2];
-            const bool hi = rg & 2, odd = rg & 1;
-#pragma unroll
-            for (int n = 0; n < 2; ++n)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) h2[n][h] = (hi ? o[n + 2][h] : o[n][h]) + __shfl_xor_sync(0xffffffffu, hi ? o[n][h] : o[n + 2][h], 16);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) o1[h] = (odd ? h2[1][h] : h2[0][h]) + __shfl_xor_sync(0xffffffffu, odd ? h2[0][h] : h2[1][h], 8);
-            const int t = base + step * rg;
-            if (t >= s0 && t < s1) {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int j = col0 + 2 * cp + h;
-                    if (j < dv) rec_store(a.out + ov + (size_t)t * dv + j, walk == 0 ? o1[h] : 0.5f * (rec_to_float(up[h]) + o1[h]));
-                }
-            }
-        }
-    }
+    scan_fwd_slab<T, RPL, VEC>(a, blockIdx.x, blockIdx.y, threadIdx.x >> 5, blockDim.x >> 5, sc_smem);
 }
 
 template <typename T, int RPL, bool VEC>
