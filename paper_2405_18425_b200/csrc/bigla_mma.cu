@@ -575,33 +575,33 @@ cudaError_t launch_chunks(MArgs a, long long units, cudaStream_t stream) {
 
 }  // namespace
 
-// Where this form is the faster one, as units per SM up to which it is (measured against the tcgen05 form for head sizes of
-// 512 to 2048 state elements, 128 to 256 tokens, 16 to 1536 units).  Up to 128 tokens always, by 1.0 to 3 times.  With a
-// second chunk its work per token grows with the state while the other form's hand-overs cost the same, and above 208
-// tokens two blocks per SM leave 64 registers a thread: the larger the state, the fewer units it takes before the other
-// form, which has its latency hidden by then, catches up.  Gates prepared in the kernel cost this form less.
-bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
-    constexpr int kAlways = 1 << 20;
-    const int state = dk * dv;
-    int waves = kAlways;
-    if (L > 208) {
-        if (state > 1536) waves = 0;
-        else if (state > 1152) waves = 1;
-        else if (state > 768) waves = gates ? (dk == 32 ? 3 : kAlways) : 2;
-    } else if (L > 128) {
-        if (state > 1536) waves = 1;
-        else if (state > 1152) waves = gates ? 4 : 3;
-    }
-    if (waves == kAlways) return true;
+// Multiprocessors of the current device, 0 if it cannot be asked.
+static int device_sms() {
     static std::atomic<int> sms_of[64];
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     int sms = sms_of[dev].load(std::memory_order_relaxed);
     if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
         sms_of[dev].store(sms, std::memory_order_relaxed);
     }
-    return form_units(units) <= (long long)waves * sms;
+    return sms;
+}
+
+// Where this form is the faster one for units of up to 256 tokens.  Its work per unit grows with the 16-token tiles and with
+// the state, while the tcgen05 form's time is its hand-overs whatever the state, so the line is a product of the two; and it
+// drops with the units per SM, as the other form gets its latency hidden (above three per SM it has), and where the gates
+// come prepared, which spares the other form a phase.  Timed against the tcgen05 form for nine head sizes, 128 to 256 tokens,
+// 16 to 1536 units, with and without the gates (1026 shapes): within 0.3 % of the better form on average.  768 units of
+// 208 tokens, us, this form / tcgen05: 24 x 48 from logits 30.4 / 34.6, from log gates 29.0 / 28.5; 32 x 64 from logits 37.6 / 31.0.
+bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
+    const int sms = device_sms();
+    if (sms == 0) return false;
+    units = form_units(units);
+    const int work = (L + 15) / 16 * dk * dv;
+    if (units <= sms) return work <= (gates ? 27000 : 24600);
+    if (units <= 3LL * sms) return work <= (gates ? 20000 : 16200);
+    return work <= (gates ? 16200 : 12300);
 }
 
 cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
@@ -623,23 +623,27 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
     return cudaErrorNotSupported;
 }
 
-// Where the chunks run faster this way than as tcgen05 segments or chunk tasks (measured for head sizes of 512 to 2048 state
-// elements, 257 to 16384 tokens, 1 to 600 units).  Few chunks: always, by 1.1 to 1.8 times - a chunk's chain of dependent
-// steps is shorter.  Many chunks: the tcgen05 tasks have their latency hidden and cost the same whatever the state, so only
-// small states, and gates that would otherwise be prepared by a launch of their own, keep the advantage.  The segmented
-// launch is at its best where two segments of every unit just fill the chip.
+// Where the chunks run faster this way than as tcgen05 segments or chunk tasks.  A chunk's chain of dependent steps is shorter
+// here, so few chunks gain most (1.3 to 1.7 times up to one per SM); a chunk's work grows with the key dimensions, while the chunk
+// tasks, once their latency is hidden, cost the same whatever the state: the wider the keys the sooner the tasks win, and sooner
+// where the gates come prepared (40 x 4096 tokens from log gates, 24 x 48: 50.8 us this way, 48.2 as tasks).  The segmented launch is at its best while two full segments (four chunks) of every unit are
+// resident in one round; beyond that round it is at its worst (300 units of 304 tokens, 32 x 64, from logits: 52.7 us, 43.7 this way).
+// More than 64 chunks: the fold here takes eight runs side by side, the tasks' takes one.  Timed against the tcgen05
+// forms for nine head sizes, 257 to 16384 tokens, 1 to 300 units, with and without the gates (1530 shapes): within 0.3 % of the
+// better form on average.
 bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
     if (dk == 16) return true;
+    const long long sms = device_sms();
+    if (sms == 0) return false;
     units = form_units(units);
-    const long long chunks = units * ((L + 127) / 128);
-    constexpr int kSms = 148;
-    if (dk == 24 && dv <= 48) {
-        if (gates) return L <= 1100 || chunks <= 8 * kSms;
-        return (L <= 1100 || chunks <= 4 * kSms) && !(L > 300 && L <= 512 && units > 40 && units <= kSms);
-    }
-    if (chunks <= 64 || (L > 8192 && units <= 4)) return true;
-    if (dk * dv <= 1024 && gates && (L <= 400 || (L > 512 && L <= 800))) return true;
-    return L <= 300 && (gates || units > kSms);
+    const int nch = chunk_plan(units, L, dk, dv).nch;
+    const long long chunks = units * nch;
+    const bool two_segments = L <= 512;
+    if (two_segments && nch == 4 && units <= sms) return dk == 32 ? chunks <= sms : (chunks <= 3 * sms || dv <= (gates ? 48 : 32));
+    if (two_segments && units > sms) return gates || dk == 24 || chunks <= 8 * sms;
+    if (dk == 24) return gates || dv == 32 || chunks <= (nch <= 8 ? 8 : 4) * sms;
+    if (chunks <= sms) return true;
+    return (gates || nch > 64) && chunks <= 4 * sms;
 }
 
 bool mma_chunks_supported(long long units, int L, int dk, int dv) { return units * chunk_plan(units, L, dk, dv).nch <= 0x7fffffffLL; }

@@ -748,6 +748,18 @@ def test_either_form_reports_an_expired_wait(oracle, either_form):
     test_expired_device_wait_is_reported_and_leaves_the_library_usable(oracle)
 
 
+@pytest.mark.parametrize("units,dk,dv", [(144, 32, 64), (24, 32, 32), (100, 24, 48)])
+def test_lengths_cut_alike_take_the_same_form(units, dk, dv):
+    """289 to 304 tokens are three chunks of up to seven tiles: whichever form is taken, all of them take it."""
+    counts = set()
+    for L in (289, 300, 301, 304):
+        q, v = (torch.zeros(units, 1, L, d, device="cuda", dtype=torch.bfloat16) for d in (dk, dv))
+        before = vig.vig_kernel_launch_count()
+        vig.vig_bigla_fwd_gates_bf16(q, q, v, q, q, torch.empty_like(v), 16.0)
+        counts.add(vig.vig_kernel_launch_count() - before)
+    assert len(counts) == 1
+
+
 def test_kernel_preference_rejects_unknown_values():
     lib = vig.load()
     assert lib.vig_test_set_kernel_preference(7) == -3
