@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a) {
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
 cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t stream) {
     const int threads = (tiles < 2 ? 2 : tiles) * 32;
-    const size_t smem = MLayout<DV>(tiles, MODE == kMain || (MODE == kUnit && tiles > 8)).total, rec = (size_t)rec_plan(threads, DK, DV).smem_floats * 4;
+    const size_t smem = MLayout<DV>(tiles, MODE == kMain || (MODE == kUnit && tiles > 8)).total, rec = (size_t)rec_plan(threads < kRecThreads ? threads : kRecThreads, DK, DV).smem_floats * 4;
     static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -1,7 +1,6 @@
 // Step-by-step evaluation of the BiGLA recurrences (paper Eq. 6) by one thread block for one
-// (batch, head) unit, in fp32 on the CUDA cores.  Used as the fp32 entry point's kernel, as the
-// bf16 entry point's kernel for head sizes the tensor-core kernel does not cover, and inside the
-// tensor-core kernel for units whose gates leave the range its factorised tiles can represent.
+// (batch, head) unit, in fp32 on the CUDA cores: inside the tensor-core kernels of the forward pass, for units whose
+// gates leave the range their factorised tiles can represent.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -10,6 +9,8 @@ namespace vig {
 
 constexpr int kRecTT = 16;   // time steps staged in shared memory at once
 constexpr int kRecR = 32;    // max state rows (key dims) held per thread
+constexpr int kRecThreads = 256;   // threads of a larger block that take part: more of them only add partial sums to put together
+                                   // (512 such units of 196 tokens, 24 x 48: 785 us with all 416 threads of a block, 571 with 256)
 
 struct RecPlan {
     int P;    // thread groups along the key dimension
@@ -69,7 +70,8 @@ struct Piece<__nv_bfloat16, true> {
 template <typename T>
 __device__ void recurrence_unit(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, T* out,
                                 int L, int dk, int dv, float* ws, float gate_inv_tau = 0.f) {
-    const int nt = blockDim.x, tid = threadIdx.x;
+    const int nt = min((int)blockDim.x, kRecThreads), tid = threadIdx.x;
+    const int first = tid < nt ? tid : 1 << 30;   // of this thread's share of every loop below (none for the threads that are left over)
     const RecPlan pl = rec_plan(nt, dk, dv);
     float* qs = ws;
     float* ks = qs + kRecTT * dk;
@@ -78,7 +80,7 @@ __device__ void recurrence_unit(const T* q, const T* k, const T* v, const T* la_
     float* part = vs + kRecTT * dv;
 
     const int p = tid / dv, j = tid - p * dv;
-    const bool active = p < pl.P;
+    const bool active = tid < nt && p < pl.P;
     const int i0 = p * pl.Rn;
     const int rn = active ? min(pl.Rn, dk - i0) : 0;
     const int nchunk = (L + kRecTT - 1) / kRecTT;
@@ -92,7 +94,7 @@ __device__ void recurrence_unit(const T* q, const T* k, const T* v, const T* la_
             const int c = dir == 0 ? cc : nchunk - 1 - cc;
             const int t0 = c * kRecTT;
             const int nv = min(kRecTT, L - t0);
-            for (int x = tid; x < nv * dk; x += nt) {
+            for (int x = first; x < nv * dk; x += nt) {
                 const size_t g = (size_t)t0 * dk + x;
                 qs[x] = rec_to_float(q[g]);
                 ks[x] = rec_to_float(k[g]);
@@ -100,7 +102,7 @@ __device__ void recurrence_unit(const T* q, const T* k, const T* v, const T* la_
                 if (gate_inv_tau > 0.f) a = (fminf(a, 0.f) - log1pf(expf(-fabsf(a)))) * gate_inv_tau;
                 es[x] = expf(a);   // alpha_t[i]
             }
-            for (int x = tid; x < nv * dv; x += nt) vs[x] = rec_to_float(v[(size_t)t0 * dv + x]);
+            for (int x = first; x < nv * dv; x += nt) vs[x] = rec_to_float(v[(size_t)t0 * dv + x]);
             __syncthreads();
             if (active) {
                 for (int n = 0; n < nv; ++n) {
@@ -121,7 +123,7 @@ __device__ void recurrence_unit(const T* q, const T* k, const T* v, const T* la_
                 }
             }
             __syncthreads();
-            for (int x = tid; x < nv * dv; x += nt) {
+            for (int x = first; x < nv * dv; x += nt) {
                 float o = 0.f;
                 for (int pp = 0; pp < pl.P; ++pp) o += part[pp * kRecTT * dv + x];
                 T* dst = out + (size_t)t0 * dv + x;
