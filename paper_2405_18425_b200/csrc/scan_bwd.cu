@@ -32,10 +32,11 @@ cudaError_t launch_scan_bwd_t(ScanBwdArgs<T> a, float2* pairs, long long units, 
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
-    // Segments: about sixteen warps per SM over the whole call, in whole groups of TG tokens; a call that has them without
-    // splitting walks whole sequences and skips the first pass.
+    // Segments: about sixteen warps per SM over the whole call, in whole groups of TG tokens; a call that nearly has them
+    // without splitting walks whole sequences and skips the first pass, which costs half as much again.
     const int slabs = (a.dk + kRows - 1) / kRows;
-    long long want = (16LL * sms + units * slabs - 1) / (units * slabs);
+    long long want = (16LL * sms + units * slabs / 2) / (units * slabs);
+    if (want < 1) want = 1;
     if (want > kMaxWarps) want = kMaxWarps;
     a.seg_len = (int)(((a.L + want - 1) / want + TG - 1) / TG * TG);
     const int nw = (a.L + a.seg_len - 1) / a.seg_len;
