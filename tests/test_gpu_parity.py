@@ -568,6 +568,29 @@ def test_host_entry_point_matches_device_path(oracle, idx):
     np.testing.assert_array_equal(out_n, ref_bytes)
 
 
+@pytest.mark.parametrize("dtype,units,L,dk,dv", [("bf16", 768, 196, 32, 64), ("bf16", 110, 700, 32, 64), ("f32", 400, 196, 32, 64)])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_slices_have_the_bits_of_the_whole_batch(dtype, units, L, dk, dv, pinned):
+    """Three slices, of which the last alone would take another form (fewer units per SM, fewer chunks, longer segments): pinned
+    buffers (results by a kernel) and pageable ones (the engines) against the device call on the whole batch."""
+    t = torch.bfloat16 if dtype == "bf16" else torch.float32
+    rng = torch.Generator(device="cuda").manual_seed(units)
+    q, k, v, gf, gb = ((torch.randn(units, 1, L, d, generator=rng, device="cuda") * s).to(t)
+                       for d, s in ((dk, dk ** -0.5), (dk, 1), (dv, 1), (dk, 1), (dk, 1)))
+    want, la = torch.empty_like(v), [torch.empty_like(gf) for _ in range(2)]
+    if dtype == "f32":
+        vig.vig_gate_prep_f32(gf, gb, *la, 16.0)
+        vig.vig_bigla_fwd_f32(q, k, v, *la, want)
+    else:
+        vig.vig_bigla_fwd_gates_bf16(q, k, v, gf, gb, want, 16.0)
+    host = [torch.empty(x.shape, dtype=t, pin_memory=pinned).copy_(x) for x in (q, k, v, gf, gb)]
+    out = torch.empty(v.shape, dtype=t, pin_memory=pinned)
+    vig.vig_bigla_fwd_host(*host, out, 16.0, vig.VIG_DTYPE_F32 if dtype == "f32" else vig.VIG_DTYPE_BF16)
+    assert vig.vig_last_device_status() == 0
+    bits = torch.int32 if dtype == "f32" else torch.int16
+    assert torch.equal(out.view(bits), want.cpu().view(bits))
+
+
 def test_host_slices_beside_the_segmented_launch_travel_by_the_copy_engines(segment_path):
     """The segmented launch counts on every SM: a sliced host call of that form launches its own kernels alone (gate preparation
     and the segments per slice), and its results are those of the device call, bit for bit."""
