@@ -196,7 +196,7 @@ int vig_bigla_fwd_blend_bf16(const void* q, const void* k, const void* v,
  * chunk: one launch up to 224 tokens, three (the chunks' own states, a fold over the chunks, the chunks) beyond.  Operands
  * of dq, dk and the gate gradients are taken as two bf16 each, so they carry about sixteen significant bits before the
  * rounding to bf16; dv takes one bf16 per operand like the forward pass.  A unit whose gates decay by more than e^-60
- * inside one chunk is computed by an in-kernel fp32 recurrence.  Everything else takes fp32 walks over the sequence on the
+ * inside one chunk takes the fp32 walks inside the kernel.  Everything else takes fp32 walks over the sequence on the
  * CUDA cores: dv as the forward walk on (k, q, d_out) with the gates moved by one token, dq and dk from the four states,
  * the gate gradients as running sums of q * dq - k * dk per direction; sequences are walked in segments side by side.
  * Scratch (the chunks' or segments' states, partial results) comes from the library's pool, stream-ordered.

@@ -10,7 +10,7 @@ namespace vig {
 constexpr int kRecTT = 16;   // time steps staged in shared memory at once
 constexpr int kRecR = 32;    // max state rows (key dims) held per thread
 constexpr int kRecThreads = 256;   // threads of a larger block that take part: more of them only add partial sums to put together
-                                   // (512 such units of 196 tokens, 24 x 48: 785 us with all 416 threads of a block, 571 with 256)
+                                   // (512 such units of 196 tokens, 24 x 48: 787 us with all 416 threads of a block, 579 with 256)
 
 struct RecPlan {
     int P;    // thread groups along the key dimension
