@@ -47,7 +47,7 @@ def _check(got, ref, dtype, label=""):
 @pytest.mark.parametrize("L", [1, 2, 15, 16, 17, 100, 196, 300])
 def test_bf16_gradient_small_and_ragged(oracle, dk, dv, L):
     """Lengths below, at and across the sixteen-token staging, one and two tokens, head sizes on and off the
-    tensor-core path of the forward pass that supplies dv."""
+    tensor-core gradient's."""
     cfg, x = random_problem(4000 + L, 2, 2, L, dk, dv, "bf16", gate_mean=1.0)
     got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
     _check(got, ref, "bf16")
@@ -69,11 +69,11 @@ def test_gradient_strong_gates(oracle):
 
 
 def test_bf16_gradient_with_a_unit_beyond_the_tensor_core_range(oracle):
-    """One unit whose gates sum to about -80 over a chunk: the forward kernel that supplies dv hands that unit to its
-    in-kernel recurrence (the counter says so); all five gradients must still meet the bar."""
+    """One unit whose gates sum to about -80 over a chunk: the tensor-core gradient hands that unit to the walks in the
+    kernel (the counter says so); all five gradients must still meet the bar."""
     cfg, x = random_problem(4300, 2, 3, 196, 32, 64, "bf16", gate_mean=1.0)
     g = synth.stored_to_f64(x["g_bwd"], "bf16").copy()
-    g[1, 1, 10:140] = -10.0            # log alpha< = -10 / 16 per token; moved by one token it gates dv's forward pass
+    g[1, 1, 10:140] = -10.0            # log alpha< = -10 / 16 per token
     x["g_bwd"] = synth.store(g, "bf16")
     vig.vig_test_take_fallback_count()
     got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
@@ -138,7 +138,7 @@ def test_gate_prep_gradient_matches_oracle(oracle, dtype, shape):
 
 @pytest.mark.parametrize("B,H,L,dk,dv", [(16, 4, 196, 32, 64), (2, 2, 1100, 24, 48), (3, 2, 300, 40, 72)])
 def test_gradient_is_bitwise_reproducible(B, H, L, dk, dv):
-    """Whole units, segmented walks and the element-wise staging: four calls on the same inputs give the same bytes (the
+    """A pair of chunks, chunks through scratch and the walks: four calls on the same inputs give the same bytes (the
     asynchronous staging and the in-place results leave no room for a race that this would not show sooner or later)."""
     cfg, x = random_problem(4400 + L, B, H, L, dk, dv, "bf16", gate_mean=1.0)
     d = {n: to_device(a, "bf16") for n, a in x.items()}
