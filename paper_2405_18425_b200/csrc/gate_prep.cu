@@ -83,9 +83,8 @@ __device__ __forceinline__ float gate_grad_of(float g, float d, float inv_tau) {
 }
 
 // 16-byte vector body with a scalar tail; blockIdx.y picks the direction.  Bound by memory traffic and, with the exact fp32
-// division, by issue slots as much (0.7 an SM quarter and cycle); bf16: eight loads in flight a thread and half the threads, with
-// what it follows in a training step of 150528 x 32 gates 2.5 us less than one pair of loads a thread.  fp32, with the exact
-// division, is better off with one pair and all the threads (the same gates: 19.8 us, 21.0 with eight loads).
+// division, by issue slots as much (0.7 an SM quarter and cycle); eight loads in flight a thread and half the threads: with
+// what it follows in a training step of 150528 x 32 gates 2.5 us less than one pair of loads a thread.
 template <typename T>
 __global__ void __launch_bounds__(256) gate_prep_bwd_kernel(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n,
                                                             float inv_tau) {
@@ -95,7 +94,7 @@ __global__ void __launch_bounds__(256) gate_prep_bwd_kernel(const T* g_f, const 
     const T* g = blockIdx.y == 0 ? g_f : g_b;
     const T* d = blockIdx.y == 0 ? d_f : d_b;
     T* o = blockIdx.y == 0 ? o_f : o_b;
-    constexpr int V = 16 / sizeof(T), kBatch = sizeof(T) == 4 ? 1 : 4;   // 16-byte pieces of either input that a thread has in flight
+    constexpr int V = 16 / sizeof(T), kBatch = 4;   // 16-byte pieces of either input that a thread has in flight
     const long long nvec = n / V, stride = (long long)gridDim.x * blockDim.x;
     auto piece = [&](uint4 rg, uint4 rd, long long x) {
         if constexpr (sizeof(T) == 4) {
@@ -152,6 +151,8 @@ template <typename T>
 cudaError_t launch_gate_prep_bwd(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n, float tau,
                                  cudaStream_t stream) {
     long long blocks = 1;
+    // fp32, with the exact division, wants the threads more than the loads in flight: 19.7 us with four blocks per SM, 20.6 with two
+    // (768 units of 196 tokens, 32 key dimensions); bf16 12.9 and 10.5
     const cudaError_t e = gate_blocks(n, 16 / (int)sizeof(T), sizeof(T) == 4 ? 4 : 2, &blocks);
     if (e != cudaSuccess) return e;
     const cudaError_t le = launch_pdl(gate_prep_bwd_kernel<T>, dim3((unsigned)blocks, 2), dim3(256), 0, stream, g_f, g_b, d_f, d_b, o_f, o_b, n,
