@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(256) gate_prep_bwd_kernel(const T* g_f, const 
     }
 }
 
-static cudaError_t gate_blocks(long long n, int vec, int per_sm, long long* blocks) {
+static cudaError_t gate_blocks(long long n, int vec, long long* blocks) {
     static std::atomic<int> sms_of[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
@@ -142,7 +142,7 @@ static cudaError_t gate_blocks(long long n, int vec, int per_sm, long long* bloc
     }
     long long b = (n / vec + 255) / 256;
     if (b < 1) b = 1;
-    if (b > (long long)per_sm * sms) b = (long long)per_sm * sms;
+    if (b > 2LL * sms) b = 2LL * sms;
     *blocks = b;
     return cudaSuccess;
 }
@@ -151,9 +151,7 @@ template <typename T>
 cudaError_t launch_gate_prep_bwd(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n, float tau,
                                  cudaStream_t stream) {
     long long blocks = 1;
-    // fp32, with the exact division, wants the threads more than the loads in flight: 19.7 us with four blocks per SM, 20.6 with two
-    // (768 units of 196 tokens, 32 key dimensions); bf16 12.9 and 10.5
-    const cudaError_t e = gate_blocks(n, 16 / (int)sizeof(T), sizeof(T) == 4 ? 4 : 2, &blocks);
+    const cudaError_t e = gate_blocks(n, 16 / (int)sizeof(T), &blocks);
     if (e != cudaSuccess) return e;
     const cudaError_t le = launch_pdl(gate_prep_bwd_kernel<T>, dim3((unsigned)blocks, 2), dim3(256), 0, stream, g_f, g_b, d_f, d_b, o_f, o_b, n,
                                       1.0f / tau);
