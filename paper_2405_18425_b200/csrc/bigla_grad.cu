@@ -188,8 +188,12 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         {a.k, a.q, a.g, a.la_b, a.la_f, a.dv, a.L, DK, DV, 0, -1, 1},
                         {a.dq, a.dk, a.dla_f, a.dla_b}};
     };
-    pdl_wait();
-    pdl_launch_dependents();
+    // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
+    // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
+    if (MODE != kMain) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     if (tid == 0) {
         mbar_expect_tx(bar, 4 * lay.op_bytes + 2 * lay.g);
         tma_load_3d(op(kQb), &tm_f, 0, row0, (int)unit, bar);
@@ -198,10 +202,6 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         tma_load_3d(op(kKf), &tm_k, 0, row0, (int)unit, bar);
         tma_load_3d(tv, &tm_v, 0, row0, (int)unit, bar);
         tma_load_3d(tg, &tm_g, 0, row0, (int)unit, bar);
-        if (MODE == kMain) {
-            mbar_expect_tx(bar + 8, 8 * kState);
-            bulk_load(tst, a.img + (unit * nch + chunk) * 8 * kState, 8 * kState, bar + 8);
-        }
         if (MODE == kPair) {   // two states and a word from the other block; from the right one also its sums of E
             mbar_expect_tx(bar + 8, 4 * DV * NP * 16 + 4);
             mbar_expect_tx(bar + 32, 2 * DK * 4);
@@ -311,7 +311,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     } else if (!ok) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(a.dev_status, kDevStatusTimeout);
         if (MODE == kSummary && tid == 0) a.flags[unit * nch + chunk] = 2;   // (nor by the launches behind this one)
-        if (MODE == kMain) mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
+        if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
         return;
     }
 
@@ -388,11 +388,17 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         for (int x = tid; x < nch; x += blockDim.x) slow |= a.flags[unit * nch + x];
         const bool missing = __syncthreads_or(slow & 2);
         if (__syncthreads_or(slow)) {
-            mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
+            pdl_wait();
             if (missing) return;             // a summary of this unit did not get its inputs, and has said so
             if (chunk == 0 && tid == 0) atomicAdd(a.dev_status + 1, 1);
             gradient_by_walks<DK, DV>(walk_args(), unit, chunk, nch, reinterpret_cast<float*>(smem), lay.bar);
             return;
+        }
+        if (w == 0) pdl_wait();   // the fold
+        if (tid == 0) {
+            pdl_launch_dependents();
+            mbar_expect_tx(bar + 8, 8 * kState);
+            bulk_load(tst, a.img + (unit * nch + chunk) * 8 * kState, 8 * kState, bar + 8);
         }
     }
     if (MODE == kSingle && state_word[0]) {

@@ -107,15 +107,15 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         *slow = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    pdl_wait();
-    pdl_launch_dependents();
+    // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
+    // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
+    if (MODE != kMain) {
+        pdl_wait();
+        pdl_launch_dependents();
+    }
     if (tid == 0) {
         mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
         tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
-        if (MODE == kMain) {
-            mbar_expect_tx(bar + 8, 2 * kState);
-            bulk_load(tst, args.img + (size_t)blockIdx.x * 2 * kState, 2 * kState, bar + 8);
-        }
     }
 
     // ---- this warp's 16 rows (g and g + 8) in fragment order: pair j of lane c ----
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     if (!__syncthreads_and(ok)) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
         if (MODE == kSummary && tid == 0) args.flags[blockIdx.x] = 2;   // (nor by the launches behind this one)
-        if (MODE == kMain) mbar_wait_bounded(bar + 8, 0);   // (the block must not end under a copy in flight)
+        if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
         return;
     }
     if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
@@ -270,8 +270,13 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         for (int x = tid; x < nch; x += blockDim.x) any |= args.flags[unit * nch + x];
         const bool missing = __syncthreads_or(any & 2);
         redo = __syncthreads_or(any);
-        if (redo) mbar_wait_bounded(bar + 8, 0);
+        if (w == 0 || redo) pdl_wait();   // the fold
         if (missing) return;   // a summary of this unit did not get its inputs, and has said so
+        if (tid == 0 && !redo) {
+            pdl_launch_dependents();
+            mbar_expect_tx(bar + 8, 2 * kState);
+            bulk_load(tst, args.img + (size_t)blockIdx.x * 2 * kState, 2 * kState, bar + 8);
+        }
     }
     if (redo) {   // gates beyond the range of the factorised tiles: Eq. 6 step by step, over the dead tiles, by one block of the unit
         if (chunk != 0) return;
