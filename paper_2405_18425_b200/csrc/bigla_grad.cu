@@ -166,7 +166,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     const bool live = wt >= 0 && wt < nT;
     const GLayout<DV> lay(tiles, MODE);
     const uint32_t base = smem_u32(smem), tv = base, tg = base + lay.g, top = base + lay.op, tst = base + lay.st;
-    const uint32_t bar = base + lay.bar;   // inputs landed; + 8: states landed; + 24: never completed, for the test hook; + 32: a pair's sums of E landed
+    const uint32_t bar = base + lay.bar;   // q, k, gates landed; + 40: v, g landed; + 8: states landed; + 24: never completed, for the test hook; + 32: a pair's sums of E landed
     auto op = [&](int o) { return top + (uint32_t)o * lay.op_bytes; };
     float* totals = reinterpret_cast<float*>(smem + lay.totals);
     float* ends = reinterpret_cast<float*>(smem + lay.ends);
@@ -180,6 +180,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         mbar_init(bar + 8, 1);
         mbar_init(bar + 24, 1);
         mbar_init(bar + 32, 1);
+        mbar_init(bar + 40, 1);
         state_word[0] = 0;   // (the other word is written by the other block alone, and read once that has landed)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -195,13 +196,14 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
         pdl_launch_dependents();
     }
     if (tid == 0) {
-        mbar_expect_tx(bar, 4 * lay.op_bytes + 2 * lay.g);
+        mbar_expect_tx(bar, 4 * lay.op_bytes);   // (v and g, which nothing needs before the operands are scaled, behind a barrier of their own)
         tma_load_3d(op(kQb), &tm_f, 0, row0, (int)unit, bar);
         tma_load_3d(op(kKb), &tm_b, 0, row0, (int)unit, bar);
         tma_load_3d(op(kQf), &tm_q, 0, row0, (int)unit, bar);
         tma_load_3d(op(kKf), &tm_k, 0, row0, (int)unit, bar);
-        tma_load_3d(tv, &tm_v, 0, row0, (int)unit, bar);
-        tma_load_3d(tg, &tm_g, 0, row0, (int)unit, bar);
+        mbar_expect_tx(bar + 40, 2 * lay.g);
+        tma_load_3d(tv, &tm_v, 0, row0, (int)unit, bar + 40);
+        tma_load_3d(tg, &tm_g, 0, row0, (int)unit, bar + 40);
         if (MODE == kPair) {   // two states and a word from the other block; from the right one also its sums of E
             mbar_expect_tx(bar + 8, 4 * DV * NP * 16 + 4);
             mbar_expect_tx(bar + 32, 2 * DK * 4);
@@ -305,6 +307,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             t64.store(op(kQb + 1), 16 * wt, m, qbl[0], qbl[1], qbl[2], qbl[3]);
         }
     }
+    ok = mbar_wait_bounded(bar + 40, 0) && ok;
     ok = __syncthreads_and(ok);
     if (MODE == kPair) {
         cluster_wait();
