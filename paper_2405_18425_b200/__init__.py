@@ -40,4 +40,5 @@ from .binding import (  # noqa: F401
     VIG_TEST_KERNEL_SEGMENTS,
     VIG_TEST_KERNEL_TCGEN05,
     VIG_TEST_KERNEL_WARP_TILES,
+    VIG_TEST_KERNEL_CLUSTERS,
 )

@@ -259,7 +259,7 @@ def vig_last_device_status(stream=None) -> int:
 
 
 VIG_TEST_KERNEL_AUTO, VIG_TEST_KERNEL_SIMT, VIG_TEST_KERNEL_CHUNK_TASKS, VIG_TEST_KERNEL_SEGMENTS = 0, 2, 3, 4
-VIG_TEST_KERNEL_TCGEN05, VIG_TEST_KERNEL_WARP_TILES = 5, 6
+VIG_TEST_KERNEL_TCGEN05, VIG_TEST_KERNEL_WARP_TILES, VIG_TEST_KERNEL_CLUSTERS = 5, 6, 8
 
 
 def vig_test_set_kernel_preference(preference: int) -> None:

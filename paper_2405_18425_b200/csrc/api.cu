@@ -67,11 +67,18 @@ static bool use_mma_chunks(long long units, int L, int dk, int dv, bool gates) {
     return pref == VIG_TEST_KERNEL_AUTO ? mma_chunks_preferred(units, L, dk, dv, gates) : pref == VIG_TEST_KERNEL_WARP_TILES;
 }
 
+// Units of a few chunks in one launch, a cluster of blocks per unit.
+static bool use_mma_cluster(long long units, int L, int dk, int dv, bool gates) {
+    if (!mma_cluster_supported(units, L, dk, dv)) return false;
+    const int pref = kernel_preference();
+    return pref == VIG_TEST_KERNEL_AUTO ? mma_cluster_preferred(units, L, dk, dv, gates) : pref == VIG_TEST_KERNEL_CLUSTERS;
+}
+
 // Whether a bf16 call from gate logits takes the segmented launch, whose blocks wait for one another and are sized to fill the
 // chip: nothing else may hold an SM meanwhile.
 static bool takes_segments(long long units, int L, int dk, int dv) {
     return kernel_preference() != VIG_TEST_KERNEL_SIMT && tc_supported(dk, dv) && !umma_supported(dk, dv, L) &&
-           !use_mma_chunks(units, L, dk, dv, true) && !use_mma_chunks(units, L, dk, dv, false) && use_segments(units, L, dk, dv);
+           !use_mma_cluster(units, L, dk, dv, true) && !use_mma_cluster(units, L, dk, dv, false) && !use_mma_chunks(units, L, dk, dv, true) && !use_mma_chunks(units, L, dk, dv, false) && use_segments(units, L, dk, dv);
 }
 
 // Scratch of the tcgen05 forms.
@@ -95,6 +102,7 @@ size_t tc_least_workspace_bytes(long long units, int L, int dk, int dv) {
 cudaError_t launch_bigla_tc(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                             const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                             int L, int dk, int dv, void* ws, size_t ws_bytes, cudaStream_t stream) {
+    if (use_mma_cluster(units, L, dk, dv, false)) return launch_bigla_mma_cluster(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, stream);
     if (umma_supported(dk, dv, L)) return launch_bigla_umma(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, stream);
     if (use_mma_chunks(units, L, dk, dv, false) && ws_bytes >= mma_chunks_workspace_bytes(units, L, dk, dv))
         return launch_bigla_mma_chunks(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, ws, stream);
@@ -166,11 +174,12 @@ static int fwd_bf16_impl(const void* q, const void* k, const void* v, const void
         }
         if (empty) return VIG_OK;
         void* scratch = ws;
-        if (own_ws && need > 0) {
+        const bool alloc = own_ws && need > 0 && !use_mma_cluster(units, L, dk, dv, false);   // (clusters use none)
+        if (alloc) {
             if (pool_alloc(&scratch, need, stream) != cudaSuccess) return VIG_ERR_CUDA;
         }
         cudaError_t e = launch_bigla_tc(q_, k_, v_, f_, b_, (bf*)out, units, L, dk, dv, scratch, own_ws ? need : ws_bytes, stream);
-        if (own_ws && need > 0) {
+        if (alloc) {
             if (cudaFreeAsync(scratch, stream) != cudaSuccess) return VIG_ERR_CUDA;
         }
         return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
@@ -202,6 +211,13 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     const long long units = (long long)B * H;
     using bf = __nv_bfloat16;
     const int pref = kernel_preference();
+    if (tc_supported(dk, dv) && use_mma_cluster(units, L, dk, dv, true)) {
+        cudaError_t e = launch_bigla_mma_cluster((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out, units, L, dk, dv,
+                                                 tau, stream);
+        if (e == cudaSuccess && o_local)
+            e = launch_gate_blend<bf>((const bf*)o_local, (const bf*)z2d, (const bf*)out, (bf*)out, (long long)units * L * dv, stream);
+        return e == cudaSuccess ? VIG_OK : VIG_ERR_CUDA;
+    }
     if (tc_supported(dk, dv) && umma_supported(dk, dv, L) && (pref == VIG_TEST_KERNEL_AUTO || pref >= VIG_TEST_KERNEL_TCGEN05)) {
         cudaError_t e = launch_bigla_umma((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out,
                                           units, L, dk, dv, tau, stream);
@@ -600,7 +616,8 @@ int vig_last_device_status(void* stream) {
 
 int vig_test_set_kernel_preference(int preference) {
     if (preference != VIG_TEST_KERNEL_AUTO && preference != VIG_TEST_KERNEL_SIMT && preference != VIG_TEST_KERNEL_CHUNK_TASKS &&
-        preference != VIG_TEST_KERNEL_SEGMENTS && preference != VIG_TEST_KERNEL_TCGEN05 && preference != VIG_TEST_KERNEL_WARP_TILES)
+        preference != VIG_TEST_KERNEL_SEGMENTS && preference != VIG_TEST_KERNEL_TCGEN05 && preference != VIG_TEST_KERNEL_WARP_TILES &&
+        preference != VIG_TEST_KERNEL_CLUSTERS)
         return VIG_ERR_UNSUPPORTED;
     g_kernel_pref.store(preference, std::memory_order_relaxed);
     return VIG_OK;

@@ -80,25 +80,6 @@ struct GLayout {
     }
 };
 
-__device__ __forceinline__ uint32_t cluster_peer(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-// Asynchronous stores to the other block's shared memory, counted by an mbarrier of that block.  Nothing waits for them
-// here: a releasing arrive or a cluster barrier after ordinary remote stores stalls its warp for about 6000 cycles beside
-// two blocks' ldmatrix traffic.
-__device__ __forceinline__ void st_async4(uint32_t addr, const uint32_t (&v)[4], uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1,%2,%3,%4}, [%5];" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-                 "r"(v[3]), "r"(bar)
-                 : "memory");
-}
-__device__ __forceinline__ void st_async1(uint32_t addr, uint32_t v, uint32_t bar) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(addr), "r"(v), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }   // orders no memory accesses
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
 // dq>, dk< of an element between the walks of gradient_by_walks, as fp32 in two bf16 result buffers each (written over at the end).
 struct ResultPairs {
     __nv_bfloat16 *dq, *dk, *dla_f, *dla_b;
@@ -372,8 +353,8 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                     if (c < NP) {
                         const uint32_t at = cluster_peer(tst + (uint32_t)(kind & 1) * 2 * kState + n * 64 + ((c ^ ((n >> 1) & 3)) << 4), 1 - chunk);
                         const uint32_t peer_bar = cluster_peer(bar + 8, 1 - chunk);
-                        st_async4(at, hi, peer_bar);
-                        st_async4(at + kState, lo, peer_bar);
+                        st_async4(at, hi[0], hi[1], hi[2], hi[3], peer_bar);
+                        st_async4(at + kState, lo[0], lo[1], lo[2], lo[3], peer_bar);
                     }
                 }
             }
@@ -907,21 +888,8 @@ GScratch grad_scratch(const GPlan& p, long long units, int dk, int dv) {
 
 template <typename... KArgs, typename... Args>
 cudaError_t launch_grad(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem, bool pair, cudaStream_t stream, Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pair ? 2 : 1;
     count_launch();
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return launch_pdl_cluster(kernel, dim3(grid), dim3(threads), smem, pair ? 2 : 1, stream, static_cast<KArgs>(args)...);
 }
 
 template <int DK, int DV>

@@ -36,7 +36,7 @@ using namespace wmma16;
 
 #pragma nv_diag_suppress 128   // the summary instances return half way: the loops behind that are not reachable in them
 
-enum { kUnit = 0, kSummary = 1, kMain = 2 };
+enum { kUnit = 0, kSummary = 1, kMain = 2, kCluster = 3 };
 constexpr int kChunkTiles = 8;        // 16-token tiles of a chunk at most
 constexpr float kGateRange = 60.f;    // largest decay of a chunk, as -log, that the factorised tiles take
 
@@ -56,21 +56,26 @@ struct MArgs {
     int expire_wait;   // test hook: every block lets one bounded wait, on an mbarrier nothing completes, run out
 };
 
-// Shared memory: v [rows][RV], k~> and k~< [rows][64 B], the two states [DV][64 B], gate totals [tile][2][32] fp32.
+// Shared memory: v [rows][RV], k~> and k~< [rows][64 B], the two states [DV][64 B], gate totals [tile][2][32] fp32; chunks of a
+// cluster: a slot for each of the other chunks (the state it adds, [DV][DK] fp32, its decay [DK] and a status word), then the
+// decay of its own that it needs.
 template <int DV>
 struct MLayout {
     static constexpr uint32_t kVRow = DV == 32 ? 64 : 128, kState = DV * 64;
-    uint32_t kf, kb, st, totals, bar, total;
-    __host__ __device__ MLayout(int tiles, bool states) {
+    uint32_t kf, kb, st, totals, slots, bar, total;
+    __host__ __device__ MLayout(int tiles, bool states, uint32_t slot_bytes = 0) {
         const uint32_t rows = tiles * 16u;
         kf = rows * kVRow;
         kb = kf + rows * 64;
         st = kb + rows * 64;
         totals = st + (states ? 2 * kState : 0);
-        bar = totals + tiles * 256u;
+        slots = totals + tiles * 256u;
+        bar = slots + slot_bytes;
         total = bar + 64;
     }
 };
+constexpr uint32_t slot_bytes(int dk, int dv) { return dv * dk * 4u + 144u; }   // (the decay behind the state, the word 128 bytes on)
+constexpr uint32_t all_slots(int dk, int dv, int nch) { return (nch - 1) * slot_bytes(dk, dv) + 128u; }
 
 // Blocks per SM the registers are held to (four blocks of the other forms would leave 64 registers a thread: 19 us against 15
 // at 768 units of 100 tokens, 32 x 64).
@@ -95,14 +100,14 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     const int tok0 = chunk * tiles * 16, T = min(tiles, Tall - chunk * tiles);   // this block's first token and its tiles
     const bool live = w < T;                          // (blocks have two warps at least: the in-kernel recurrence needs them)
     const int ch = kTwo ? w >> 3 : 0, c0 = 8 * ch;    // this warp's chunk and its first tile
-    const MLayout<DV> lay(tiles, kTwo ? Tall > 8 : MODE == kMain);
+    const MLayout<DV> lay(tiles, kTwo ? Tall > 8 : MODE == kMain || MODE == kCluster, MODE == kCluster ? all_slots(DK, DV, nch) : 0u);
     const uint32_t base = smem_u32(smem), tv = base, tkf = base + lay.kf, tkb = base + lay.kb, tst = base + lay.st, bar = base + lay.bar;
     float* totals = reinterpret_cast<float*>(smem + lay.totals);
     volatile int* slow = reinterpret_cast<volatile int*>(smem + lay.bar + 32);
 
     if (tid == 0) {
         mbar_init(bar, 1);
-        mbar_init(bar + 8, MODE == kMain ? 1 : 2 * MV);   // the states: one bulk copy, or one arrival per piece formed here
+        mbar_init(bar + 8, MODE == kMain || MODE == kCluster ? 1 : 2 * MV);   // the states: one bulk copy, the other chunks' slots, or one arrival per piece formed here
         mbar_init(bar + 16, 1);       // never completed: only the test hook waits on it
         *slow = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -116,6 +121,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     if (tid == 0) {
         mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
         tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
+        if (MODE == kCluster) mbar_expect_tx(bar + 8, (nch - 1) * (DV * DK * 4 + DK * 4 + 4));
     }
 
     // ---- this warp's 16 rows (g and g + 8) in fragment order: pair j of lane c ----
@@ -171,6 +177,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         }
     }
     __syncthreads();
+    if (MODE == kCluster) cluster_arrive_relaxed();   // the other chunks may write here once this one's barriers stand
     // sums over tiles [from, to) of one direction
     auto sum_totals = [&](int dir, int from, int to, f32x2 (&s)[NP]) {
 #pragma unroll
@@ -252,7 +259,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     bool ok = true;
     if (args.expire_wait && tid == 0) ok = mbar_wait_bounded(bar + 16, 0, 64);   // test hook: this wait cannot succeed
     ok = mbar_wait_bounded(bar, 0) && ok;
-    if (!__syncthreads_and(ok)) {   // a load that never lands: report it and leave, all threads together, nothing stored
+    ok = __syncthreads_and(ok);
+    if (MODE == kCluster) {
+        cluster_wait();
+    } else if (!ok) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
         if (MODE == kSummary && tid == 0) args.flags[blockIdx.x] = 2;   // (nor by the launches behind this one)
         if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
@@ -287,16 +297,25 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                                        reinterpret_cast<float*>(smem), args.inv_tau);
         return;
     }
-    if (!live) return;
+    if (MODE != kCluster && !live) return;
     const Tile<64> t64(lane);
     const Tile<RV> tvv(lane);
+    float* slots = reinterpret_cast<float*>(smem + lay.slots);
+    constexpr int kSlotFloats = slot_bytes(DK, DV) / 4, kStateFloats = DV * DK;
+    // Place of a key dimension (a column of the operand tiles) in a row of a slot: pairs of a lane's pairs side by side.
+    auto slot_place = [](int col) {
+        const int j = col >> 3, m = j >> 1, cc = (col & 7) >> 1;
+        return 16 * m + (2 * m + 1 < NP ? 4 * cc + 2 * (j & 1) : 2 * cc) + (col & 1);
+    };
 
     // ---- the states the chunks hand each other, transposed: rows of v times k~ over the tokens, 16 value columns a job; the
     // last warps first: theirs is the shorter chunk ----
-    if (MODE == kSummary || (kTwo && T > 8)) {
-        for (int job = T - 1 - w; job < 2 * MV; job += T) {
-            const int dir = job & 1, mt = job >> 1;   // two chunks: dir 0: chunk 0 -> 1 (forward), dir 1: chunk 1 -> 0
-            const int t0 = MODE == kSummary || dir == 0 ? 0 : 8, t1 = kTwo && dir == 0 ? 8 : T;
+    if (MODE == kSummary || MODE == kCluster || (kTwo && T > 8)) {
+        // (in a cluster the first chunk owes nobody S<, the last nobody S>)
+        const int dirs = MODE == kCluster ? (chunk > 0) + (chunk + 1 < nch) : 2;
+        for (int job = live ? T - 1 - w : 2 * MV; job < dirs * MV; job += T) {
+            const int dir = dirs == 2 ? job & 1 : (chunk == 0 ? 0 : 1), mt = dirs == 2 ? job >> 1 : job;   // two chunks: dir 0: chunk 0 -> 1 (forward), dir 1: chunk 1 -> 0
+            const int t0 = !kTwo || dir == 0 ? 0 : 8, t1 = kTwo && dir == 0 ? 8 : T;
             float u[2 * MP][4];
 #pragma unroll
             for (int j = 0; j < 2 * MP; ++j)
@@ -324,8 +343,12 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                 // sequences: the forward state alone decays to the chunk's end
                 float d0, d1;
                 unpack2(GATES ? dec[j] : fmul2(dec[j], pack2(kLog2e, kLog2e)), d0, d1);
-                d0 = MODE == kSummary && dir == 1 ? 1.f : ex2(d0);
-                d1 = MODE == kSummary && dir == 1 ? 1.f : ex2(d1);
+                d0 = !kTwo && dir == 1 ? 1.f : ex2(d0);
+                d1 = !kTwo && dir == 1 ? 1.f : ex2(d1);
+                if (MODE == kCluster) {
+                    u[j][0] *= d0; u[j][1] *= d1; u[j][2] *= d0; u[j][3] *= d1;
+                    continue;
+                }
 #pragma unroll
                 for (int r = 0; r < 2; ++r) {
                     const int n = 16 * mt + 8 * r + g;
@@ -336,10 +359,49 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                         *reinterpret_cast<uint32_t*>(smem + lay.st + dir * kState + n * 64 + ((j ^ ((n >> 1) & 3)) << 4) + 4 * c) = pack_bf16(u0, u1);
                 }
             }
+            if (MODE == kCluster) {   // to every chunk behind (S>) or before (S<) this one
+                const int p0 = dir == 0 ? chunk + 1 : 0, p1 = dir == 0 ? nch : chunk;
+                const uint32_t at = base + lay.slots + (dir == 0 ? chunk : chunk - 1) * slot_bytes(DK, DV) + (16 * mt + g) * (DK * 4);
+#pragma unroll 1
+                for (int p = p0; p < p1; ++p) {
+                    const uint32_t to = cluster_peer(at, p), peer_bar = cluster_peer(bar + 8, p);
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int m = 0; m < MP; ++m) {
+                            if (2 * m + 1 < NP)
+                                st_async4(to + 8 * r * DK * 4 + 64 * m + 16 * c, __float_as_uint(u[2 * m][2 * r]), __float_as_uint(u[2 * m][2 * r + 1]),
+                                          __float_as_uint(u[2 * m + 1][2 * r]), __float_as_uint(u[2 * m + 1][2 * r + 1]), peer_bar);
+                            else
+                                st_async2(to + 8 * r * DK * 4 + 64 * m + 8 * c, __float_as_uint(u[2 * m][2 * r]), __float_as_uint(u[2 * m][2 * r + 1]), peer_bar);
+                        }
+                }
+            }
             __syncwarp();
             if (kTwo && lane == 0) mbar_arrive(bar + 8);
         }
         if (MODE == kSummary) return;
+    }
+    if (MODE == kCluster && w == 0) {   // the decay across this chunk, and whether anything is wrong here
+        const int word = (*slow ? 1 : 0) | (ok ? 0 : 2);
+        if (lane < DK) {
+            float s0 = 0.f, s1 = 0.f;
+            for (int x = 0; x < T; ++x) {
+                s0 += totals[(x * 2) * 32 + lane];
+                s1 += totals[(x * 2 + 1) * 32 + lane];
+            }
+            s0 = ex2(GATES ? s0 : s0 * kLog2e);
+            s1 = ex2(GATES ? s1 : s1 * kLog2e);
+            slots[(nch - 1) * kSlotFloats + slot_place(lane)] = s1;   // its own, of S< across this chunk
+#pragma unroll 1
+            for (int p = 0; p < nch; ++p) {
+                if (p == chunk) continue;
+                const uint32_t at = base + lay.slots + (p > chunk ? chunk : chunk - 1) * slot_bytes(DK, DV) + kStateFloats * 4;
+                const uint32_t peer_bar = cluster_peer(bar + 8, p);
+                st_async1(cluster_peer(at + slot_place(lane) * 4, p), __float_as_uint(p > chunk ? s0 : s1), peer_bar);
+                if (lane == 0) st_async1(cluster_peer(at + 128, p), (uint32_t)word, peer_bar);
+            }
+        }
     }
 
     // ---- this warp's rows against the tiles of its chunk: forward products up to the diagonal tile, backward ones from it on
@@ -379,7 +441,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
             mma_k16(o[2 * n2 + 1], p, r[2], r[3]);
         }
     };
-    {
+    if (live) {
         uint32_t kt = tkf + (uint32_t)c0 * 1024, vt = tv + (uint32_t)c0 * 16 * RV;
 #pragma unroll 1
         for (int j = 0; j < mine; ++j, kt += 1024, vt += 16 * RV) tile(qf, kt, vt, 0);
@@ -393,8 +455,56 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
             tile(qb, kt, vt, 0);
         }
     }
-    if (MODE == kMain || (kTwo && T > 8)) {
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded(bar + 8, 0))) {   // (never expected where the warps of this block form the states)
+    if (MODE == kCluster) {
+        // ---- the states that enter this chunk, from what the chunks before and behind it add: in(c + 1) = d>(c) in(c) + own(c),
+        // in(c - 1) = d<(c) in(c) + own(c), the latter stored times this chunk's d<, as the fold of the long form does ----
+        const bool got = __syncthreads_and(mbar_wait_bounded(bar + 8, 0) && ok);
+        int word = got ? *slow : 2;
+        for (int x = 0; got && x + 1 < nch; ++x) word |= *reinterpret_cast<const int*>(slots + x * kSlotFloats + kStateFloats + 32);
+        if (word) {   // (every block has all that is sent to it by now, so none is written to after its end)
+            if (word & 2) {
+                if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
+                return;
+            }
+            if (chunk != 0) return;
+            if (tid == 0) atomicAdd(args.dev_status + 1, 1);
+            __syncthreads();
+            const size_t okk = unit * L * DK, ov = unit * L * DV;
+            recurrence_unit<__nv_bfloat16>(args.q + okk, args.k + okk, args.v + ov, args.la_f + okk, args.la_b + okk, args.out + ov, L, DK, DV,
+                                           reinterpret_cast<float*>(smem), args.inv_tau);
+            return;
+        }
+        constexpr int P = DK / 4;
+        const float4* own = reinterpret_cast<const float4*>(slots + (nch - 1) * kSlotFloats);
+        for (int x = tid; x < 2 * DV * P; x += blockDim.x) {
+            const int dir = x >= DV * P, y = dir ? x - DV * P : x, n = y / P, p = y % P;
+            float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int first = dir == 0 ? 0 : nch - 2, last = dir == 0 ? chunk : chunk - 1, step = dir == 0 ? 1 : -1;
+#pragma unroll 1
+            for (int s = first; s != last; s += step) {
+                const float4 u = *reinterpret_cast<const float4*>(slots + s * kSlotFloats + n * DK + 4 * p);
+                const float4 d = *reinterpret_cast<const float4*>(slots + s * kSlotFloats + kStateFloats + 4 * p);
+                carry = make_float4(fmaf(d.x, carry.x, u.x), fmaf(d.y, carry.y, u.y), fmaf(d.z, carry.z, u.z), fmaf(d.w, carry.w, u.w));
+            }
+            if (dir == 1) {
+                const float4 d = own[p];
+                carry = make_float4(carry.x * d.x, carry.y * d.y, carry.z * d.z, carry.w * d.w);
+            }
+            const int m = p >> 2, cc = p & 3;
+            uint8_t* row = smem + lay.st + dir * kState + n * 64;
+            auto at = [&](int j) { return row + ((j ^ ((n >> 1) & 3)) << 4); };
+            if (2 * m + 1 < NP) {
+                *reinterpret_cast<uint32_t*>(at(2 * m) + 4 * cc) = pack_bf16(carry.x, carry.y);
+                *reinterpret_cast<uint32_t*>(at(2 * m + 1) + 4 * cc) = pack_bf16(carry.z, carry.w);
+            } else {
+                *reinterpret_cast<uint2*>(at(2 * m) + 8 * cc) = make_uint2(pack_bf16(carry.x, carry.y), pack_bf16(carry.z, carry.w));
+            }
+        }
+        __syncthreads();
+        if (!live) return;
+    }
+    if (MODE == kMain || MODE == kCluster || (kTwo && T > 8)) {
+        if (MODE != kCluster && !__all_sync(0xffffffffu, mbar_wait_bounded(bar + 8, 0))) {   // (never expected where the warps of this block form the states)
             if (lane == 0) atomicOr(args.dev_status, kDevStatusTimeout);
             return;
         }
@@ -415,7 +525,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                 }
             }
         };
-        if (MODE == kMain) {   // (the first chunk's S> and the last one's S< are zero)
+        if (MODE == kMain || MODE == kCluster) {   // (the first chunk's S> and the last one's S< are zero)
             if (chunk > 0) state(qf, tst);
             if (chunk + 1 < nch) state(qb, tst + kState);
         } else if (ch == 0) {
@@ -510,7 +620,7 @@ __global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a) {
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
 cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t stream) {
     const int threads = (tiles < 2 ? 2 : tiles) * 32;
-    const size_t smem = MLayout<DV>(tiles, MODE == kMain || (MODE == kUnit && tiles > 8)).total, rec = (size_t)rec_plan(threads < kRecThreads ? threads : kRecThreads, DK, DV).smem_floats * 4;
+    const size_t smem = MLayout<DV>(tiles, MODE == kMain || MODE == kCluster || (MODE == kUnit && tiles > 8), MODE == kCluster ? all_slots(DK, DV, a.nch) : 0u).total, rec = (size_t)rec_plan(threads < kRecThreads ? threads : kRecThreads, DK, DV).smem_floats * 4;
     static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -519,13 +629,14 @@ cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t
     int sms = sms_of[dev].load(std::memory_order_acquire);
     if (sms == 0) {
         auto kernel = bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>;
-        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MODE == kCluster ? 112 * 1024 : 100 * 1024)) != cudaSuccess) return e;
         if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
     a.ahead = mma_blocks_per_sm(DK, DV, MAXT, MODE) * sms;
-    const cudaError_t le = launch_pdl(bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>, dim3((unsigned)a.blocks), dim3(threads), smem > rec ? smem : rec, stream, tv, a);
+    const cudaError_t le = launch_pdl_cluster(bigla_mma_kernel<DK, DV, GATES, MAXT, MODE>, dim3((unsigned)a.blocks), dim3(threads), smem > rec ? smem : rec,
+                                              MODE == kCluster ? a.nch : 1, stream, tv, a);
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
 }
@@ -559,6 +670,14 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
     p.flags = p.decay + n * 64 * 4;
     p.total = (p.flags + n * 4 + 255) / 256 * 256;
     return p;
+}
+
+// One launch: the chunks of a unit are the blocks of a cluster.
+template <int DK, int DV, bool GATES>
+cudaError_t launch_cluster(MArgs a, long long units, cudaStream_t stream) {
+    CUtensorMap tv;
+    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
+    return launch_mma_t<DK, DV, GATES, 8, kCluster>(a, tv, a.tiles, stream);
 }
 
 template <int DK, int DV, bool GATES>
@@ -653,6 +772,30 @@ bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
 
 bool mma_chunks_supported(long long units, int L, int dk, int dv) { return units * chunk_plan(units, L, dk, dv).nch <= 0x7fffffffLL; }
 
+bool mma_cluster_supported(long long units, int L, int dk, int dv) {
+    const int nch = chunk_plan(units, L, dk, dv).nch;
+    return nch >= 2 && nch <= 8 && units * nch <= 0x7fffffffLL;
+}
+
+// Where one launch of clusters is the fastest form.  Against the three launches over chunks, the tcgen05 segments and chunk tasks
+// (564 shapes, six head sizes, 257 to 1024 tokens, 8 to 600 units): three chunks always (144 units of 300 tokens, 32 x 64, from
+// logits 19.7 us, 23.2 in three launches); four unless a large state meets what suits the segments, two of them for every unit
+// in one round, or comes with its gates prepared; more while the clusters of the call run side by side, since every chunk gives its states
+// to all the others and clusters of seven or eight blocks leave SMs without one (148 units of 1024 tokens, 32 x 64: 86 us, 59 in three
+// launches).  Within 1.0 % of the best form on average.  Units of one block otherwise (336 shapes): two chunks on SMs of their own
+// halve the chain of a large unit while SMs are free (one unit of 256 tokens, 32 x 64: 8.0 us, 10.3 and 11.2 in one block).
+bool mma_cluster_preferred(long long units, int L, int dk, int dv, bool gates) {
+    const long long sms = device_sms();
+    if (sms == 0) return false;
+    units = form_units(units);
+    const int nch = chunk_plan(units, L, dk, dv).nch, state = dk * dv;
+    const long long chunks = units * nch;
+    if (nch == 2) return 2 * units <= sms && (L + 15) / 16 * state >= 19900;
+    if (nch == 3 || state <= 512) return true;
+    if (nch == 4) return state <= 1152 || (units <= sms ? 10 * chunks <= 28 * sms : gates || state <= 1536);
+    return 10 * chunks <= (nch <= 6 ? 28 : (state <= 1152 ? 20 : 10)) * sms;
+}
+
 size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv) { return chunk_plan(units, L, dk, dv).total; }
 
 cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
@@ -674,6 +817,27 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
 #define VIG_CASE(DK_, DV_)        \
     if (dk == DK_ && dv == DV_) \
         return gate_tau > 0.f ? launch_chunks<DK_, DV_, true>(a, units, stream) : launch_chunks<DK_, DV_, false>(a, units, stream);
+    VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
+    VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
+    VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)
+#undef VIG_CASE
+    return cudaErrorNotSupported;
+}
+
+cudaError_t launch_bigla_mma_cluster(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                                     const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
+                                     int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
+    const ChunkPlan p = chunk_plan(units, L, dk, dv);
+    MArgs a{};
+    a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
+    a.L = L; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
+    a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
+    a.expire_wait = take_expire_next_wait() == 1;
+    a.dev_status = device_status_ptr();
+    if (!a.dev_status) return cudaErrorUnknown;
+#define VIG_CASE(DK_, DV_)        \
+    if (dk == DK_ && dv == DV_) \
+        return gate_tau > 0.f ? launch_cluster<DK_, DV_, true>(a, units, stream) : launch_cluster<DK_, DV_, false>(a, units, stream);
     VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
     VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
     VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)

@@ -10,6 +10,7 @@
  *                          (the default chooses between the two by segment count and unit count).
  *   VIG_TEST_KERNEL_TCGEN05      always the tcgen05 kernels: the single-block one up to 256 tokens, chunk tasks or segments beyond
  *   VIG_TEST_KERNEL_WARP_TILES   always the kernels of one warp per 16 tokens, one block per unit or per chunk
+ *   VIG_TEST_KERNEL_CLUSTERS     129 .. 1024 tokens: the blocks of up to 128 tokens of a unit always as one cluster
  *                          (the default chooses between these by head size, length and unit count).
  *                          vig_bigla_workspace_bytes follows the setting: query it under the setting the call
  *                          will run with
@@ -24,7 +25,7 @@ extern "C" {
 #endif
 
 enum vig_test_kernel { VIG_TEST_KERNEL_AUTO = 0, VIG_TEST_KERNEL_SIMT = 2, VIG_TEST_KERNEL_CHUNK_TASKS = 3, VIG_TEST_KERNEL_SEGMENTS = 4,
-                       VIG_TEST_KERNEL_TCGEN05 = 5, VIG_TEST_KERNEL_WARP_TILES = 6 };
+                       VIG_TEST_KERNEL_TCGEN05 = 5, VIG_TEST_KERNEL_WARP_TILES = 6, VIG_TEST_KERNEL_CLUSTERS = 8 };
 int vig_test_set_kernel_preference(int preference);
 
 /* Synchronises `stream`, then returns and clears the number of (batch, head) units that the tensor-core kernels of the

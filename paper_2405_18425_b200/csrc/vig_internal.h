@@ -76,6 +76,13 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
                                     const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                                     int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream);
 
+// Up to eight such chunks as the blocks of a cluster, states through distributed shared memory: one launch, no scratch.
+bool mma_cluster_supported(long long units, int L, int dk, int dv);
+bool mma_cluster_preferred(long long units, int L, int dk, int dv, bool gates);
+cudaError_t launch_bigla_mma_cluster(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
+                                     const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
+                                     int L, int dk, int dv, float gate_tau, cudaStream_t stream);
+
 // ---- Eq. 7 around the mixer: depth-wise 3 x 3 convolution (channels last) and the 2-D gate blend ----
 bool dwconv_supported(int C, size_t elem);
 template <typename T>
@@ -128,21 +135,29 @@ bool host_copy_usable(const void* host, size_t bytes);   // all of it pinned and
 cudaError_t launch_host_copy(const HostCopy* copies, int n, int max_blocks, cudaStream_t stream);
 
 // Launch with programmatic stream serialization: the kernel's prologue (everything before its pdl_wait) may overlap
-// the tail of the kernel before it in the stream.
+// the tail of the kernel before it in the stream.  cluster: blocks of a cluster (along x; the grid is a multiple of it).
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                              Args&&... args) {
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, int cluster, cudaStream_t stream,
+                                      Args&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                              Args&&... args) {
+    return launch_pdl_cluster(kernel, grid, block, smem, 1, stream, static_cast<KArgs>(args)...);
 }
 
 // Kernel family the bf16 entry points use (a vig_test_kernel value; test_hooks.h): the default unless a test changed it.

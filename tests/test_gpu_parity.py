@@ -787,3 +787,39 @@ def test_kernel_preference_rejects_unknown_values():
     lib = vig.load()
     assert lib.vig_test_set_kernel_preference(7) == -3
     assert lib.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_AUTO) == 0
+
+
+@pytest.fixture
+def cluster_form():
+    vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_CLUSTERS)
+    yield
+    vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_AUTO)
+
+
+@pytest.mark.parametrize("dk,dv", [(16, 32), (16, 64), (24, 48), (32, 32), (32, 64)])
+@pytest.mark.parametrize("L", [129, 200, 256, 257, 289, 400, 513, 1009, 1024])
+def test_chunks_of_a_cluster(oracle, cluster_form, dk, dv, L):
+    """Two to eight chunks, a last one of one token, of whole tiles and full; beyond 256 tokens with the bits of the three launches over
+    the same chunks, from log gates (gate logits: there the gates are prepared once and read twice, the same values)."""
+    cfg, x = random_problem(3100 + L, 3, 2, L, dk, dv, "bf16", gate_mean=1.0)
+    for run in (_run_unfused, _run_fused):
+        before = vig.vig_kernel_launch_count()
+        got, ref = run(oracle, cfg, x)
+        assert vig.vig_kernel_launch_count() - before == 1
+        assert np.isfinite(got).all() and rel_err(got, ref) <= TOL["bf16"]
+        if L > 256:
+            vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_WARP_TILES)
+            np.testing.assert_array_equal(run(oracle, cfg, x)[0], got)
+            vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_CLUSTERS)
+
+
+@pytest.mark.parametrize("case", ["closed", "wall", "mixed", "steep"])
+def test_chunks_of_a_cluster_with_degenerate_gates(oracle, cluster_form, case):
+    test_degenerate_gates(oracle, case, "bf16", 32, 64, 300)
+    test_degenerate_gates(oracle, case, "bf16", 24, 48, 1000)
+
+
+def test_expired_wait_in_a_cluster_and_in_the_chunk_launches(cluster_form):
+    test_expired_wait_of_the_warp_tile_forms_stores_nothing(700)
+    vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_WARP_TILES)
+    test_expired_wait_of_the_warp_tile_forms_stores_nothing(300)
