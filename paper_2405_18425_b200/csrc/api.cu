@@ -88,7 +88,7 @@ static size_t umma_workspace_bytes(long long units, int L, int dk, int dv) {
 
 size_t tc_workspace_bytes(long long units, int L, int dk, int dv) {
     if (umma_supported(dk, dv, L)) return 0;   // one thread block covers a unit
-    return use_mma_chunks(units, L, dk, dv, false) ? mma_chunks_workspace_bytes(units, L, dk, dv) : umma_workspace_bytes(units, L, dk, dv);
+    return use_mma_chunks(units, L, dk, dv, false) ? mma_chunks_workspace_bytes(units, L, dk, dv, false) : umma_workspace_bytes(units, L, dk, dv);
 }
 
 // The least a caller's scratch has to hold.
@@ -104,7 +104,7 @@ cudaError_t launch_bigla_tc(const __nv_bfloat16* q, const __nv_bfloat16* k, cons
                             int L, int dk, int dv, void* ws, size_t ws_bytes, cudaStream_t stream) {
     if (use_mma_cluster(units, L, dk, dv, false)) return launch_bigla_mma_cluster(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, stream);
     if (umma_supported(dk, dv, L)) return launch_bigla_umma(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, stream);
-    if (use_mma_chunks(units, L, dk, dv, false) && ws_bytes >= mma_chunks_workspace_bytes(units, L, dk, dv))
+    if (use_mma_chunks(units, L, dk, dv, false) && ws_bytes >= mma_chunks_workspace_bytes(units, L, dk, dv, false))
         return launch_bigla_mma_chunks(q, k, v, la_f, la_b, out, units, L, dk, dv, 0.f, ws, stream);
     if (use_segments(units, L, dk, dv)) return launch_bigla_umma_seg(q, k, v, la_f, la_b, out, units, L, dk, dv, ws, stream);
     return launch_bigla_umma_long(q, k, v, la_f, la_b, out, units, L, dk, dv, ws, stream);
@@ -227,7 +227,7 @@ static int fwd_gates_bf16_impl(const void* q, const void* k, const void* v, cons
     }
     if (tc_supported(dk, dv) && use_mma_chunks(units, L, dk, dv, true)) {
         void* ws = nullptr;
-        if (pool_alloc(&ws, mma_chunks_workspace_bytes(units, L, dk, dv), stream) != cudaSuccess) return VIG_ERR_CUDA;
+        if (pool_alloc(&ws, mma_chunks_workspace_bytes(units, L, dk, dv, true), stream) != cudaSuccess) return VIG_ERR_CUDA;
         cudaError_t e = launch_bigla_mma_chunks((const bf*)q, (const bf*)k, (const bf*)v, (const bf*)g_f, (const bf*)g_b, (bf*)out, units, L, dk, dv, tau,
                                                 ws, stream);
         if (cudaFreeAsync(ws, stream) != cudaSuccess) return VIG_ERR_CUDA;

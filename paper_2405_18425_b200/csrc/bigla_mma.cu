@@ -50,6 +50,8 @@ struct MArgs {
     uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
     float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
     int* flags;        // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
+    uint8_t* keys;     // GATES: [unit][chunk][k~>, k~<][rows][64 B]: the scaled keys of a chunk, as shared-memory tiles
+    __nv_bfloat16 *la2_f, *la2_b;   // GATES: log2 alpha as prepared by the summary launch
     int* dev_status;
     float inv_tau;
     int ahead;         // the block this many further on has its inputs pulled into L2
@@ -90,6 +92,9 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     constexpr int RV = MLayout<DV>::kVRow;
     constexpr uint32_t kState = MLayout<DV>::kState;
     constexpr bool kTwo = MODE == kUnit && MAXT > 8;   // units of two chunks
+    // From logits, the summary launch leaves the prepared gates and the scaled keys behind for the chunks' launch (the keys by one
+    // bulk copy of its tiles), which would spend a third of its instructions on doing both again.
+    constexpr bool kGiveKeys = GATES && MODE == kSummary, kTakeKeys = GATES && MODE == kMain;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int g = lane >> 2, c = lane & 3;
@@ -119,7 +124,8 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         pdl_launch_dependents();
     }
     if (tid == 0) {
-        mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
+        mbar_expect_tx(bar, (uint32_t)tiles * (16 * RV + (kTakeKeys ? 2048 : 0)));
+        if (kTakeKeys) bulk_load(tkf, args.keys + (size_t)blockIdx.x * tiles * 2048, tiles * 2048, bar);
         tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
         if (MODE == kCluster) mbar_expect_tx(bar + 8, (nch - 1) * (DV * DK * 4 + DK * 4 + 4));
     }
@@ -131,15 +137,15 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         const int row = tok0 + w * 16 + 8 * r + g;
         if (live && row < L) {
             const size_t at = (unit * L + row) * DK;
-            load_pairs<DK>(args.la_f + at, c, af[r]);
-            load_pairs<DK>(args.la_b + at, c, ab[r]);
-            load_pairs<DK>(args.k + at, c, kr[r]);
+            load_pairs<DK>((kTakeKeys ? args.la2_f : args.la_f) + at, c, af[r]);
+            load_pairs<DK>((kTakeKeys ? args.la2_b : args.la_b) + at, c, ab[r]);
+            if (!kTakeKeys) load_pairs<DK>(args.k + at, c, kr[r]);
             if (MODE != kSummary) load_pairs<DK>(args.q + at, c, qr[r]);
         } else {
 #pragma unroll
             for (int j = 0; j < NP; ++j) {   // rows past the end: q = k = 0 and no decay (GATES: a logit of 100, log alpha = 0)
                 qr[r][j] = kr[r][j] = 0u;
-                af[r][j] = ab[r][j] = GATES ? 0x42C842C8u : 0u;
+                af[r][j] = ab[r][j] = GATES && !kTakeKeys ? 0x42C842C8u : 0u;
             }
         }
     }
@@ -161,10 +167,27 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     for (int j = 0; j < NP; ++j) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            if (GATES) {
+            if (GATES && !kTakeKeys) {
                 af[r][j] = log2_alpha_pair<MODE != kUnit>(af[r][j], args.inv_tau);
                 ab[r][j] = log2_alpha_pair<MODE != kUnit>(ab[r][j], args.inv_tau);
             }
+        }
+    }
+    if (kGiveKeys) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int row = tok0 + w * 16 + 8 * r + g;
+            if (live && row < L) {
+                const size_t at = (unit * L + row) * DK;
+                store_pairs<DK>(args.la2_f + at, c, af[r]);
+                store_pairs<DK>(args.la2_b + at, c, ab[r]);
+            }
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
             af[r][j] = movmatrix(af[r][j]);
             ab[r][j] = movmatrix(ab[r][j]);
         }
@@ -237,9 +260,11 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                             // Factor and product in fp32, one rounding: what the packed reciprocals are low by on average would
                             // pass into the states and on from chunk to chunk (with them 32 x 4096 tokens, gate logits around 4,
                             // were 4.8e-3 off in 2-norm, the tcgen05 forms 4.5e-3; this way 3.3e-3 in the same time).
-                            const f32x2 k2 = widen(kr[r][j]);
-                            kfw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(-b0), ex2(-b1))));
-                            kbw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(x0), ex2(x1))));
+                            if (!kTakeKeys) {
+                                const f32x2 k2 = widen(kr[r][j]);
+                                kfw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(-b0), ex2(-b1))));
+                                kbw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(x0), ex2(x1))));
+                            }
                             if (MODE != kSummary) {
                                 const f32x2 q2 = fmul2(widen(qr[r][j]), pack2(0.5f, 0.5f));   // the 1/2 of the result
                                 qf[m][2 * jj + r] = pack_f32x2(fmul2(q2, pack2(ex2(b0), ex2(b1))));
@@ -252,10 +277,13 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                     for (int r = 0; r < 2; ++r) kfw[2 + r] = kbw[2 + r] = qf[m][2 + r] = qb[m][2 + r] = 0u;
                 }
             }
-            t64.store(tkf, 16 * w, m, kfw[0], kfw[1], kfw[2], kfw[3]);
-            t64.store(tkb, 16 * w, m, kbw[0], kbw[1], kbw[2], kbw[3]);
+            if (!kTakeKeys) {
+                t64.store(tkf, 16 * w, m, kfw[0], kfw[1], kfw[2], kfw[3]);
+                t64.store(tkb, 16 * w, m, kbw[0], kbw[1], kbw[2], kbw[3]);
+            }
         }
     }
+    if (kGiveKeys) fence_async_smem();   // (the tiles, for the bulk copy)
     bool ok = true;
     if (args.expire_wait && tid == 0) ok = mbar_wait_bounded(bar + 16, 0, 64);   // test hook: this wait cannot succeed
     ok = mbar_wait_bounded(bar, 0) && ok;
@@ -268,6 +296,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
         return;
     }
+    if (kGiveKeys && tid == 0) bulk_store(args.keys + (size_t)blockIdx.x * tiles * 2048, tkf, tiles * 2048);
     if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
         float s = 0.f;
         for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
@@ -380,7 +409,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
             __syncwarp();
             if (kTwo && lane == 0) mbar_arrive(bar + 8);
         }
-        if (MODE == kSummary) return;
+        if (MODE == kSummary) {
+            if (kGiveKeys && tid == 0) bulk_store_wait();   // (the tiles must outlast the copy)
+            return;
+        }
     }
     if (MODE == kCluster && w == 0) {   // the decay across this chunk, and whether anything is wrong here
         const int word = (*slow ? 1 : 0) | (ok ? 0 : 2);
@@ -655,9 +687,9 @@ cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
 // Sequences of any length: chunks of equal numbers of tiles.
 struct ChunkPlan {
     int nch, tiles;
-    size_t u, img, decay, flags, total;   // byte offsets in the scratch
+    size_t u, img, decay, flags, keys, la2, la2_bytes, total;   // byte offsets in the scratch
 };
-ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
+ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false) {
     ChunkPlan p;
     const int T = (L + 15) / 16;
     p.nch = (T + kChunkTiles - 1) / kChunkTiles;
@@ -668,7 +700,12 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv) {
     p.img = n * 2 * dk * dv * 4;
     p.decay = p.img + n * 2 * dv * 64;
     p.flags = p.decay + n * 64 * 4;
-    p.total = (p.flags + n * 4 + 255) / 256 * 256;
+    p.keys = p.la2 = p.total = (p.flags + n * 4 + 255) / 256 * 256;
+    p.la2_bytes = ((size_t)units * L * dk * 2 + 255) / 256 * 256;
+    if (gates) {
+        p.la2 = p.keys + n * p.tiles * 2048;
+        p.total = p.la2 + 2 * p.la2_bytes;
+    }
     return p;
 }
 
@@ -796,12 +833,12 @@ bool mma_cluster_preferred(long long units, int L, int dk, int dv, bool gates) {
     return 10 * chunks <= (nch <= 6 ? 28 : (state <= 1152 ? 20 : 10)) * sms;
 }
 
-size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv) { return chunk_plan(units, L, dk, dv).total; }
+size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv, bool gates) { return chunk_plan(units, L, dk, dv, gates).total; }
 
 cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                                     const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                                     int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream) {
-    const ChunkPlan p = chunk_plan(units, L, dk, dv);
+    const ChunkPlan p = chunk_plan(units, L, dk, dv, gate_tau > 0.f);
     char* b = static_cast<char*>(ws);
     MArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
@@ -810,6 +847,9 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
     a.img = reinterpret_cast<uint8_t*>(b + p.img);
     a.decay = reinterpret_cast<float*>(b + p.decay);
     a.flags = reinterpret_cast<int*>(b + p.flags);
+    a.keys = reinterpret_cast<uint8_t*>(b + p.keys);
+    a.la2_f = reinterpret_cast<__nv_bfloat16*>(b + p.la2);
+    a.la2_b = reinterpret_cast<__nv_bfloat16*>(b + p.la2 + p.la2_bytes);
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();

@@ -71,7 +71,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
 // prepared on the way as well.  mma_chunks_preferred: the shapes it is the faster form for.
 bool mma_chunks_supported(long long units, int L, int dk, int dv);
 bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates);
-size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv);
+size_t mma_chunks_workspace_bytes(long long units, int L, int dk, int dv, bool gates);
 cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,
                                     const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                                     int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream);
