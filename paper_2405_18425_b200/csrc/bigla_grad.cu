@@ -170,6 +170,21 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
                         {a.k, a.q, a.g, a.la_b, a.la_f, a.dv, a.L, DK, DV, 0, -1, 1},
                         {a.dq, a.dk, a.dla_f, a.dla_b}};
     };
+    auto pull = [&](long long block) {   // the tokens of a block into L2
+        const long long nu = block / nch;
+        const int nr = (int)(block % nch) * tiles * 16;
+        const size_t at = (size_t)nu * L + nr;
+        const uint32_t n = min(tiles * 16, L - nr);
+        prefetch_l2(a.la_f + at * DK, n * DK * 2);
+        prefetch_l2(a.la_b + at * DK, n * DK * 2);
+        prefetch_l2(a.q + at * DK, n * DK * 2);
+        prefetch_l2(a.k + at * DK, n * DK * 2);
+        prefetch_l2(a.v + at * DV, n * DV * 2);
+        prefetch_l2(a.g + at * DV, n * DV * 2);
+    };
+    // ... and those of the first round while the launch before still runs: a prefetch consumes nothing, and L2 stays coherent with
+    // what that launch still writes.
+    if (MODE != kMain && tid == 0 && (long long)blockIdx.x < a.ahead) pull(blockIdx.x);
     // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
     // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
     if (MODE != kMain) {
@@ -190,18 +205,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
             mbar_expect_tx(bar + 32, 2 * DK * 4);
         }
         const long long next = (long long)blockIdx.x + a.ahead;
-        if (next < a.chunks) {   // a block that starts when one of these is done finds its tokens in L2
-            const long long nu = next / nch;
-            const int nr = (int)(next % nch) * tiles * 16;
-            const size_t at = (size_t)nu * L + nr;
-            const uint32_t n = min(tiles * 16, L - nr);
-            prefetch_l2(a.la_f + at * DK, n * DK * 2);
-            prefetch_l2(a.la_b + at * DK, n * DK * 2);
-            prefetch_l2(a.q + at * DK, n * DK * 2);
-            prefetch_l2(a.k + at * DK, n * DK * 2);
-            prefetch_l2(a.v + at * DV, n * DV * 2);
-            prefetch_l2(a.g + at * DV, n * DV * 2);
-        }
+        if (next < a.chunks) pull(next);   // a block that starts when one of these is done finds its tokens in L2
     }
     __syncthreads();
     if (MODE == kPair) cluster_arrive_relaxed();   // the other block may be written to once it runs (nothing of its own goes where that lands)

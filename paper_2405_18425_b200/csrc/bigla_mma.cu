@@ -117,6 +117,18 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         *slow = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    auto pull = [&](size_t at, uint32_t n, bool rest, bool q) {   // n tokens from `at` into L2
+        if (rest) {
+            prefetch_l2(args.la_f + at * DK, n * DK * 2);
+            prefetch_l2(args.la_b + at * DK, n * DK * 2);
+            prefetch_l2(args.k + at * DK, n * DK * 2);
+            prefetch_l2(args.v + at * DV, n * DV * 2);
+        }
+        if (q) prefetch_l2(args.q + at * DK, n * DK * 2);
+    };
+    // A block that is let in while the launch before still runs has its tokens brought to L2 meanwhile (a prefetch consumes nothing,
+    // and L2 stays coherent with what that launch still writes); the blocks after the first round are pulled in by those of it.
+    if (MODE != kMain && tid == 32 && (int)blockIdx.x < args.ahead) pull(unit * L + tok0, min(tiles * 16, L - tok0), true, true);
     // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
     // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
     if (MODE != kMain) {
@@ -149,18 +161,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
             }
         }
     }
-    if (tid == 0 && blockIdx.x + (long long)args.ahead < args.blocks) {   // a block that starts when one of these is done finds its inputs in L2
+    if (MODE != kMain && tid == 0 && blockIdx.x + (long long)args.ahead < args.blocks) {   // a block that starts when one of these is done finds its inputs in L2
         const size_t next = blockIdx.x + (size_t)args.ahead;
         const int nr = MODE == kUnit ? 0 : (int)(next % (unsigned)nch) * tiles * 16;
-        const size_t at = (MODE == kUnit ? next : next / (unsigned)nch) * L + nr;
-        const uint32_t n = min(tiles * 16, L - nr);
-        if (MODE != kMain) {   // (the summary launch has just read everything but q)
-            prefetch_l2(args.la_f + at * DK, n * DK * 2);
-            prefetch_l2(args.la_b + at * DK, n * DK * 2);
-            prefetch_l2(args.k + at * DK, n * DK * 2);
-            prefetch_l2(args.v + at * DV, n * DV * 2);
-        }
-        if (MODE != kSummary) prefetch_l2(args.q + at * DK, n * DK * 2);
+        pull((MODE == kUnit ? next : next / (unsigned)nch) * L + nr, min(tiles * 16, L - nr), true, true);   // (q: of the chunks' launch as well)
     }
     // ---- gate totals of the tile; the gates turned, as B operands of products over the tokens ----
 #pragma unroll
@@ -751,18 +755,16 @@ static int device_sms() {
 
 // Where this form is the faster one for units of up to 256 tokens.  Its work per unit grows with the 16-token tiles and with
 // the state, while the tcgen05 form's time is its hand-overs whatever the state, so the line is a product of the two; and it
-// drops with the units per SM, as the other form gets its latency hidden (above three per SM it has), and where the gates
-// come prepared, which spares the other form a phase.  Timed against the tcgen05 form for nine head sizes, 128 to 256 tokens,
-// 16 to 1536 units, with and without the gates (1026 shapes): within 0.3 % of the better form on average.  768 units of
-// 208 tokens, us, this form / tcgen05: 24 x 48 from logits 30.4 / 34.6, from log gates 29.0 / 28.5; 32 x 64 from logits 37.6 / 31.0.
+// drops with the units per SM, as the other form gets its latency hidden, sooner where the gates come prepared, which spares
+// the other form a phase.  Timed against the tcgen05 form for six head sizes, 130 to 256 tokens, 1 to 1024 units, with and without
+// the gates (756 shapes): within 0.2 % of the better form on average.  512 units of 208 tokens, 24 x 48, us, this form / tcgen05:
+// from logits 20.4 / 23.7, from log gates 20.2 / 19.9; 768 of 208, 32 x 64, from logits 37.2 / 30.7.
 bool mma_preferred(long long units, int L, int dk, int dv, bool gates) {
     const int sms = device_sms();
     if (sms == 0) return false;
     units = form_units(units);
     const int work = (L + 15) / 16 * dk * dv;
-    if (units <= sms) return work <= (gates ? 27000 : 24600);
-    if (units <= 3LL * sms) return work <= (gates ? 20000 : 16200);
-    return work <= (gates ? 16200 : 12300);
+    return work <= (units <= sms ? 27000 : (gates || units <= 3LL * sms ? 20000 : 15200));
 }
 
 cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, const __nv_bfloat16* v,

@@ -35,15 +35,26 @@ __device__ __forceinline__ uint4 log_alpha_bf16x8(uint4 raw, float inv_tau) {
     return raw;
 }
 
+// The block's first four runs of 16-byte pieces of g into L2, while the launch before still runs.
+template <typename T>
+__device__ __forceinline__ void pull_batch(const T* g, long long nvec) {
+    if (threadIdx.x < 4) {
+        const long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x * ((long long)gridDim.x * blockDim.x);
+        const long long m = nvec - x < blockDim.x ? nvec - x : blockDim.x;
+        if (m > 0) prefetch_l2(reinterpret_cast<const uint4*>(g) + x, (uint32_t)m * 16);
+    }
+}
+
 // 16-byte vector body (4 floats or 8 bf16 per thread) with a scalar tail; blockIdx.y picks the direction.
 template <typename T>
 __global__ void __launch_bounds__(256) gate_prep_kernel(const T* g_f, const T* g_b, T* la_f, T* la_b, long long n, float inv_tau) {
     // no __restrict__: the output may alias the input (in-place call)
-    pdl_wait();
-    pdl_launch_dependents();
     const T* g = blockIdx.y == 0 ? g_f : g_b;
     T* la = blockIdx.y == 0 ? la_f : la_b;
     constexpr int V = 16 / sizeof(T);
+    pull_batch(g, n / V);
+    pdl_wait();
+    pdl_launch_dependents();
     const long long nvec = n / V;
     const long long stride = (long long)gridDim.x * blockDim.x;
     long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -89,11 +100,12 @@ template <typename T>
 __global__ void __launch_bounds__(256) gate_prep_bwd_kernel(const T* g_f, const T* g_b, const T* d_f, const T* d_b, T* o_f, T* o_b, long long n,
                                                             float inv_tau) {
     // no __restrict__: the output may be the incoming gradient's buffer
-    pdl_wait();
-    pdl_launch_dependents();
     const T* g = blockIdx.y == 0 ? g_f : g_b;
     const T* d = blockIdx.y == 0 ? d_f : d_b;
     T* o = blockIdx.y == 0 ? o_f : o_b;
+    pull_batch(g, n / (16 / (int)sizeof(T)));
+    pdl_wait();
+    pdl_launch_dependents();
     constexpr int V = 16 / sizeof(T), kBatch = 4;   // 16-byte pieces of either input that a thread has in flight
     const long long nvec = n / V, stride = (long long)gridDim.x * blockDim.x;
     auto piece = [&](uint4 rg, uint4 rd, long long x) {
