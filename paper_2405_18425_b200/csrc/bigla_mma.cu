@@ -79,10 +79,10 @@ struct MLayout {
 constexpr uint32_t slot_bytes(int dk, int dv) { return dv * dk * 4u + 144u; }   // (the decay behind the state, the word 128 bytes on)
 constexpr uint32_t all_slots(int dk, int dv, int nch) { return (nch - 1) * slot_bytes(dk, dv) + 128u; }
 
-// Blocks per SM the registers are held to (four blocks of the other forms would leave 64 registers a thread: 19 us against 15
-// at 768 units of 100 tokens, 32 x 64).
+// Blocks per SM the registers are held to (64 registers a thread for four: 19 us against 15 where the state is large, units of one block,
+// 768 of 100 tokens, 32 x 64; chunks of small states gain, 2 x 4 units of 16384 tokens, 24 x 48: 39.8 to 38.5).
 constexpr int mma_blocks_per_sm(int dk, int dv, int max_tiles, int mode) {
-    return max_tiles > 8 ? 2 : (mode == kSummary && dk * dv <= 1152 ? 4 : 3);
+    return max_tiles > 8 ? 2 : (mode != kUnit && dk * dv <= 1152 ? 4 : 3);
 }
 
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
