@@ -290,8 +290,11 @@ static int bwd_impl(const void* q, const void* k, const void* v, const void* la_
             if (e == cudaSuccess) st = fwd_bf16_impl(k, q, d_out, sf, sb, dv_out, B, H, L, dk, dv, nullptr, 0, true, stream);
         }
     }
-    if (!tc) e = launch_scan_fwd<T>(k_, q_, g_, f_, b_, (T*)dv_out, units, L, dk, dv, true, stream);
-    if (e == cudaSuccess && st == VIG_OK)
+    const bool together = !tc && bwd_in_one_launch(units, L, dk, dv);
+    if (together)
+        e = launch_scan_grad<T>(q_, k_, v_, f_, b_, g_, (T*)dq, (T*)dk_out, (T*)dv_out, (T*)dla_f, (T*)dla_b, scratch, units, L, dk, dv, stream);
+    else if (!tc) e = launch_scan_fwd<T>(k_, q_, g_, f_, b_, (T*)dv_out, units, L, dk, dv, true, stream);
+    if (!together && e == cudaSuccess && st == VIG_OK)
         e = launch_bigla_bwd<T>(q_, k_, v_, f_, b_, g_, (T*)dq, (T*)dk_out, (T*)dla_f, (T*)dla_b, (float*)(scratch + 2 * gate_bytes), units, L, dk, dv,
                                 stream);
     if (e != cudaSuccess) st = VIG_ERR_CUDA;

@@ -541,6 +541,14 @@ size_t bwd_scratch_bytes(long long units, int L, int dk, int dv) {
     return (p + st + de + to) * sizeof(float);
 }
 
+bool scan_grad_supported(int dk, int dv);
+bool bwd_in_one_launch(long long units, int L, int dk, int dv) {
+    int sms = 0, nseg, seg_len;
+    if (!scan_grad_supported(dk, dv) || sm_count_of_device(&sms) != cudaSuccess) return false;
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
+    return nseg == 1;
+}
+
 template <typename T>
 cudaError_t launch_shift_gates(const T* la_f, const T* la_b, T* out_f, T* out_b, long long units, int L, int dk, cudaStream_t stream) {
     const bool wide = (dk * sizeof(T)) % 16 == 0;   // (all four pointers are 16-byte aligned)
