@@ -75,7 +75,7 @@ struct GLayout {
         totals = st + (mode == kPair ? 2u : (mode == kMain ? 4u : 0u)) * 2 * kState;   // [tile][2][32] fp32
         ends = totals + tiles * 256u;                                                // [2][32] fp32
         part = ends + 256;                                                           // [warp][2][32] fp32
-        bar = part + warps * 256u;
+        bar = part + (mode == kSummary ? 0u : warps * 256u);
         total = bar + 64;
     }
 };
@@ -923,7 +923,10 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
         if (e != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
-    a.ahead = 2 * sms;   // two blocks per SM
+    // Two blocks per SM.  The summary launch of a long call fits three where they have one warp per tile: worth the uneven share of its
+    // jobs in the larger calls (training step of 8 x 4 units of 4096 tokens, 24 x 48: 159.5 to 154.3 us; 24 x 6 of 300, 32 x 64: 80.8 to 82.5).
+    const bool three = p.mode == kMain && units * p.nch > 4LL * sms && DK * DV > 512;
+    a.ahead = (three ? 3 : 2) * sms;
     const unsigned grid = (unsigned)(units * p.nch);
     auto threads = [&](int mode) { return 32 * grad_warps(mode, p.tiles); };
     if (p.mode == kSingle)
@@ -931,7 +934,7 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
     else if (p.mode == kPair)
         e = launch_grad(bigla_grad_kernel<DK, DV, kPair>, grid, threads(kPair), GLayout<DV>(p.tiles, kPair).total, true, stream, tq, tk, tf, tb, tv, tg, a);
     else {
-        e = launch_grad(bigla_grad_kernel<DK, DV, kSummary>, grid, threads(kSummary), GLayout<DV>(p.tiles, kSummary).total, false, stream, tq, tk, tf, tb, tv, tg, a);
+        e = launch_grad(bigla_grad_kernel<DK, DV, kSummary>, grid, three ? 32 * p.tiles : threads(kSummary), GLayout<DV>(p.tiles, kSummary).total, false, stream, tq, tk, tf, tb, tv, tg, a);
         if (e == cudaSuccess) {
             count_launch();
             constexpr int kGroups = 8, kWork = DK / 4 * DV;
@@ -942,6 +945,7 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
                 e = launch_pdl(grad_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 4, (kWork + 255) / 256), dim3(256), 0, stream, a);
         }
         a.expire_wait = 0;   // (of a long call the first launch)
+        a.ahead = 2 * sms;
         if (e == cudaSuccess)
             e = launch_grad(bigla_grad_kernel<DK, DV, kMain>, grid, threads(kMain), GLayout<DV>(p.tiles, kMain).total, false, stream, tq, tk, tf, tb, tv, tg, a);
     }
