@@ -26,6 +26,7 @@
 
 #include <atomic>
 
+#include "fold.cuh"
 #include "mma.cuh"
 #include "scan_bwd.cuh"
 #include "tma_host.h"
@@ -795,15 +796,11 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     }
 }
 
-// Second launch of a long call: the states entering every chunk, from the chunks' own: S> and Z< ascending, in(c + 1) =
-// d(c) in(c) + own(c); S< and Z> descending, in(c - 1) = d(c) in(c) + own(c).  A thread takes four key dimensions of one value
-// column over a run of chunks, eight loads in flight; GROUPS runs of a long sequence are taken side by side, first for what
-// each adds and by how much it decays, then from the carry of the runs before it.
-template <int DK, int DV, int GROUPS>
-__global__ void __launch_bounds__(256) grad_fold_kernel(const GArgs a) {
-    constexpr int P = DK / 4, kBatch = 8, kItems = 256 / GROUPS;
+// Second launch of a long call: the states entering every chunk, from the chunks' own: S> and Z< ascending, S< and Z> descending.
+template <int DK, int DV, int GROUPS, int RUN>
+__global__ void __launch_bounds__(kFoldThreads, fold_blocks_per_sm(RUN)) grad_fold_kernel(const GArgs a) {
+    constexpr int P = DK / 4, kItems = kFoldThreads / GROUPS;
     constexpr int kState = (int)GLayout<DV>::kState;
-    __shared__ float4 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
     const size_t unit = blockIdx.x;
     const int kind = blockIdx.y, dir = (kind == 0 || kind == 3) ? 0 : 1;   // S>, Z> decay by log alpha>
     const bool up = kind < 2;
@@ -811,58 +808,20 @@ __global__ void __launch_bounds__(256) grad_fold_kernel(const GArgs a) {
     const int run = (nch + GROUPS - 1) / GROUPS, i0 = min(nch, grp * run), i1 = min(nch, i0 + run);   // in walking order
     const bool in = x < P * DV;
     const int p = in ? x % P : 0, n = in ? x / P : 0;
-    const ptrdiff_t step = up ? 1 : -1;
+    const int step = up ? 1 : -1;
     const size_t first = unit * nch + (up ? i0 : nch - 1 - i0);
-    const float* own0 = a.u + ((first * 4 + kind) * DV + n) * DK + 4 * p;
-    const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
     uint8_t* img = a.img + (first * 4 + kind) * 2 * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
     pdl_wait();
     pdl_launch_dependents();
-    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
-    auto walk = [&](bool emit) {
-        const float *own_p = own0, *dec_p = dec0;
-        for (int b0 = i0; b0 < i1; b0 += kBatch) {
-            float4 own[kBatch], d[kBatch];
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                if (b0 + b < i1) {
-                    own[b] = *reinterpret_cast<const float4*>(own_p);
-                    d[b] = *reinterpret_cast<const float4*>(dec_p);
-                    own_p += step * (4 * DV * DK);
-                    dec_p += step * 64;
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                if (b0 + b < i1) {
-                    if (emit) {
-                        uint2 hi, lo;
-                        split_bf16(pack2(carry.x, carry.y), hi.x, lo.x);
-                        split_bf16(pack2(carry.z, carry.w), hi.y, lo.y);
-                        *reinterpret_cast<uint2*>(img) = hi;
-                        *reinterpret_cast<uint2*>(img + kState) = lo;
-                        img += step * (8 * kState);
-                    } else {
-                        all = make_float4(all.x * d[b].x, all.y * d[b].y, all.z * d[b].z, all.w * d[b].w);
-                    }
-                    carry = make_float4(fmaf(d[b].x, carry.x, own[b].x), fmaf(d[b].y, carry.y, own[b].y), fmaf(d[b].z, carry.z, own[b].z),
-                                        fmaf(d[b].w, carry.w, own[b].w));
-                }
-            }
-        }
-    };
-    if (GROUPS > 1) {
-        if (in) walk(false);
-        s_state[grp][item] = carry;
-        s_decay[grp][item] = all;
-        __syncthreads();
-        carry = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int y = 0; y < grp; ++y) {
-            const float4 s = s_state[y][item], d = s_decay[y][item];
-            carry = make_float4(fmaf(d.x, carry.x, s.x), fmaf(d.y, carry.y, s.y), fmaf(d.z, carry.z, s.z), fmaf(d.w, carry.w, s.w));
-        }
-    }
-    if (in) walk(true);
+    fold_runs<GROUPS, RUN>(a.u + ((first * 4 + kind) * DV + n) * DK + 4 * p, step * (4 * DV * DK), a.decay + first * 64 + dir * 32 + 4 * p, step * 64, run, i1 - i0, in,
+                      item, grp, [&](int i, float4 carry, float4) {
+                          uint2 hi, lo;
+                          split_bf16(pack2(carry.x, carry.y), hi.x, lo.x);
+                          split_bf16(pack2(carry.z, carry.w), hi.y, lo.y);
+                          uint8_t* to = img + (ptrdiff_t)(i * step) * (8 * kState);
+                          *reinterpret_cast<uint2*>(to) = hi;
+                          *reinterpret_cast<uint2*>(to + kState) = lo;
+                      });
 }
 
 // How a sequence is cut: one chunk of up to eight tiles, two of up to seven, else chunks of six.
@@ -937,12 +896,10 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
         e = launch_grad(bigla_grad_kernel<DK, DV, kSummary>, grid, three ? 32 * p.tiles : threads(kSummary), GLayout<DV>(p.tiles, kSummary).total, false, stream, tq, tk, tf, tb, tv, tg, a);
         if (e == cudaSuccess) {
             count_launch();
-            constexpr int kGroups = 8, kWork = DK / 4 * DV;
-            if (p.nch > 24)
-                e = launch_pdl(grad_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 4, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0,
-                               stream, a);
-            else
-                e = launch_pdl(grad_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 4, (kWork + 255) / 256), dim3(256), 0, stream, a);
+            e = with_fold_plan(p.nch, [&](auto groups, auto run) {
+                constexpr int kGroups = decltype(groups)::value, kItems = kFoldThreads / kGroups;
+                return launch_pdl(grad_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)units, 4, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
+            });
         }
         a.expire_wait = 0;   // (of a long call the first launch)
         a.ahead = 2 * sms;

@@ -24,6 +24,7 @@
 
 #include <atomic>
 
+#include "fold.cuh"
 #include "mma.cuh"
 #include "recurrence.cuh"
 #include "tma_host.h"
@@ -586,71 +587,28 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     }
 }
 
-// Second launch of a long call: the states that enter every chunk from what the chunks add, S> ascending, in(c + 1) =
-// d>(c) in(c) + own(c), S< descending, in(c - 1) = d<(c) in(c) + own(c), stored times d<(c), the decay from the chunk's end to
-// its start.  A thread takes four key dimensions of one value column over a run of chunks, eight loads in flight.  GROUPS
-// runs of a long sequence are taken side by side, first for what each adds and by how much it decays, then from the carry of
-// the runs before it (128 chunks as one run: 17.7 us, bound by the round trips of sixteen batches).
-template <int DK, int DV, int GROUPS>
-__global__ void __launch_bounds__(256) mma_fold_kernel(const MArgs a) {
-    constexpr int P = DK / 4, kBatch = 8, kItems = 256 / GROUPS;
+// Second launch of a long call: the states that enter every chunk from what the chunks add, S> ascending, S< descending, the latter
+// stored times d<(c), the decay from the chunk's end to its start.
+template <int DK, int DV, int GROUPS, int RUN>
+__global__ void __launch_bounds__(kFoldThreads, fold_blocks_per_sm(RUN)) mma_fold_kernel(const MArgs a) {
+    constexpr int P = DK / 4, kItems = kFoldThreads / GROUPS;
     constexpr int kState = (int)MLayout<DV>::kState;
-    __shared__ float4 s_state[GROUPS][kItems], s_decay[GROUPS][kItems];
     const size_t unit = blockIdx.x;
     const int dir = blockIdx.y, item = threadIdx.x % kItems, grp = threadIdx.x / kItems;
     const int x = blockIdx.z * kItems + item, nch = a.nch;
     const int run = (nch + GROUPS - 1) / GROUPS, i0 = min(nch, grp * run), i1 = min(nch, i0 + run);   // in walking order
     const bool in = x < P * DV;
     const int p = in ? x % P : 0, n = in ? x / P : 0;
-    const ptrdiff_t step = dir == 0 ? 1 : -1;
+    const int step = dir == 0 ? 1 : -1;
     const size_t first = unit * nch + (dir == 0 ? i0 : nch - 1 - i0);
-    const float* own0 = a.u + ((first * 2 + dir) * DV + n) * DK + 4 * p;
-    const float* dec0 = a.decay + first * 64 + dir * 32 + 4 * p;
     uint8_t* img = a.img + (first * 2 + dir) * kState + n * 64 + (((p >> 1) ^ ((n >> 1) & 3)) << 4) + 8 * (p & 1);
     pdl_wait();
     pdl_launch_dependents();
-    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), all = make_float4(1.f, 1.f, 1.f, 1.f);
-    auto walk = [&](bool emit) {
-        const float *own_p = own0, *dec_p = dec0;
-        for (int b0 = i0; b0 < i1; b0 += kBatch) {
-            float4 own[kBatch], d[kBatch];
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                if (b0 + b < i1) {
-                    own[b] = *reinterpret_cast<const float4*>(own_p);
-                    d[b] = *reinterpret_cast<const float4*>(dec_p);
-                    own_p += step * (2 * DV * DK);
-                    dec_p += step * 64;
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                if (b0 + b < i1) {
-                    if (emit) {
-                        *reinterpret_cast<uint2*>(img) = dir == 0 ? make_uint2(pack_bf16(carry.x, carry.y), pack_bf16(carry.z, carry.w))
-                                                                  : make_uint2(pack_bf16(carry.x * d[b].x, carry.y * d[b].y), pack_bf16(carry.z * d[b].z, carry.w * d[b].w));
-                        img += step * (2 * kState);
-                    } else {
-                        all = make_float4(all.x * d[b].x, all.y * d[b].y, all.z * d[b].z, all.w * d[b].w);
-                    }
-                    carry = make_float4(fmaf(d[b].x, carry.x, own[b].x), fmaf(d[b].y, carry.y, own[b].y), fmaf(d[b].z, carry.z, own[b].z),
-                                        fmaf(d[b].w, carry.w, own[b].w));
-                }
-            }
-        }
-    };
-    if (GROUPS > 1) {
-        if (in) walk(false);
-        s_state[grp][item] = carry;
-        s_decay[grp][item] = all;
-        __syncthreads();
-        carry = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int y = 0; y < grp; ++y) {
-            const float4 s = s_state[y][item], d = s_decay[y][item];
-            carry = make_float4(fmaf(d.x, carry.x, s.x), fmaf(d.y, carry.y, s.y), fmaf(d.z, carry.z, s.z), fmaf(d.w, carry.w, s.w));
-        }
-    }
-    if (in) walk(true);
+    fold_runs<GROUPS, RUN>(a.u + ((first * 2 + dir) * DV + n) * DK + 4 * p, step * (2 * DV * DK), a.decay + first * 64 + dir * 32 + 4 * p, step * 64, run, i1 - i0, in,
+                      item, grp, [&](int i, float4 carry, float4 d) {
+                          if (dir == 1) carry = make_float4(carry.x * d.x, carry.y * d.y, carry.z * d.z, carry.w * d.w);
+                          *reinterpret_cast<uint2*>(img + (ptrdiff_t)(i * step) * (2 * kState)) = make_uint2(pack_bf16(carry.x, carry.y), pack_bf16(carry.z, carry.w));
+                      });
 }
 
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
@@ -727,11 +685,10 @@ cudaError_t launch_chunks(MArgs a, long long units, cudaStream_t stream) {
     if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
     if (e != cudaSuccess) return e;
-    constexpr int kGroups = 8, kWork = DK / 4 * DV;
-    if (a.nch > 24)
-        e = launch_pdl(mma_fold_kernel<DK, DV, kGroups>, dim3((unsigned)units, 2, (kWork + 256 / kGroups - 1) / (256 / kGroups)), dim3(256), 0, stream, a);
-    else
-        e = launch_pdl(mma_fold_kernel<DK, DV, 1>, dim3((unsigned)units, 2, (kWork + 255) / 256), dim3(256), 0, stream, a);
+    e = with_fold_plan(a.nch, [&](auto groups, auto run) {
+        constexpr int kGroups = decltype(groups)::value, kItems = kFoldThreads / kGroups;
+        return launch_pdl(mma_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)units, 2, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
+    });
     count_launch();
     if (e != cudaSuccess) return e;
     a.expire_wait = 0;   // (of a long call the first launch)
