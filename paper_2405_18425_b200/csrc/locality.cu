@@ -91,6 +91,12 @@ __global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ 
         mbar_expect_tx(bar0 + 8 * buf, tile_bytes);
         tma_load_4d(smem_u32(dw_smem) + buf * buf_pitch, &tm_x, c_slab, j0 - 1, i0 - 1, n, bar0 + 8 * buf);
     };
+    if (threadIdx.x == 0) {   // the first tile and the filters to L2 while the launch before still runs (a prefetch consumes nothing)
+        const int task = blockIdx.x, j0 = (task % coltiles) * tw, i0 = ((task / coltiles) % rowsegs) * th, n = task / (coltiles * rowsegs);
+        if (task < tasks) tma_prefetch_4d(&tm_x, c_slab, j0 - 1, i0 - 1, n);
+        const int live = min(gpb * V, C - c_slab) * 9 * (int)sizeof(T);
+        prefetch_l2(w + (size_t)c_slab * 9, live & ~15);
+    }
     pdl_wait();   // x may be the output of the kernel before this one in the stream
     pdl_launch_dependents();
     if (threadIdx.x == 0 && (int)blockIdx.x < tasks) issue(blockIdx.x, 0);
