@@ -646,7 +646,24 @@ cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
     return launch_mma_t<DK, DV, GATES, 16, kUnit>(a, tv, T, stream);
 }
 
-// Sequences of any length: chunks of equal numbers of tiles.
+// Multiprocessors of the current device, 0 if it cannot be asked.
+static int device_sms() {
+    static std::atomic<int> sms_of[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int sms = sms_of[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+        sms_of[dev].store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
+
+// Sequences of any length: chunks of equal numbers of tiles, up to eight.  From logits, beyond eight chunks, the tiles are what makes
+// the rounds of blocks cheapest, a block's time being about that of its loads and hand-overs (eight tiles' worth) and of its tiles, short
+// of the 128 chunks up to which the fold keeps its runs short.  6 x 4 units of 1300 tokens, 24 x 64: 17.8 us a call, 20.6 with
+// eight tiles; 3 x 3 of 5000, 24 x 32: 16.4 and 18.3; 8 x 4 of 4096, 24 x 48: 37.4 and 37.8.  (From log gates the scratch may be the caller's,
+// whose size this keeps.)
 struct ChunkPlan {
     int nch, tiles;
     size_t u, img, decay, flags, keys, la2, la2_bytes, total;   // byte offsets in the scratch
@@ -654,9 +671,23 @@ struct ChunkPlan {
 ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false) {
     ChunkPlan p;
     const int T = (L + 15) / 16;
-    p.nch = (T + kChunkTiles - 1) / kChunkTiles;
-    p.tiles = (T + p.nch - 1) / p.nch;
-    p.nch = (T + p.tiles - 1) / p.tiles;
+    auto cut = [&](int tiles) {
+        p.nch = (T + tiles - 1) / tiles;
+        p.tiles = (T + p.nch - 1) / p.nch;
+        p.nch = (T + p.tiles - 1) / p.tiles;
+    };
+    cut(kChunkTiles);
+    const long long slots = (long long)mma_blocks_per_sm(dk, dv, kChunkTiles, kMain) * device_sms();
+    if (gates && p.nch > kChunkTiles && slots > 0) {
+        int best = p.tiles;
+        long long best_cost = -1;
+        for (int tiles = kChunkTiles; tiles >= 5; --tiles) {
+            const int nch = (T + tiles - 1) / tiles;
+            const long long cost = (form_units(units) * nch + slots - 1) / slots * (8 + tiles);
+            if (best_cost < 0 || (cost < best_cost && nch <= 128)) best = tiles, best_cost = cost;
+        }
+        cut(best);
+    }
     const size_t n = (size_t)units * p.nch;
     p.u = 0;
     p.img = n * 2 * dk * dv * 4;
@@ -696,19 +727,6 @@ cudaError_t launch_chunks(MArgs a, long long units, cudaStream_t stream) {
 }
 
 }  // namespace
-
-// Multiprocessors of the current device, 0 if it cannot be asked.
-static int device_sms() {
-    static std::atomic<int> sms_of[64];
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-    int sms = sms_of[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-        sms_of[dev].store(sms, std::memory_order_relaxed);
-    }
-    return sms;
-}
 
 // Where this form is the faster one for units of up to 256 tokens.  Its work per unit grows with the 16-token tiles and with
 // the state, while the tcgen05 form's time is its hand-overs whatever the state, so the line is a product of the two; and it

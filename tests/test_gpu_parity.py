@@ -823,3 +823,15 @@ def test_expired_wait_in_a_cluster_and_in_the_chunk_launches(cluster_form):
     test_expired_wait_of_the_warp_tile_forms_stores_nothing(700)
     vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_WARP_TILES)
     test_expired_wait_of_the_warp_tile_forms_stores_nothing(300)
+
+
+@pytest.mark.parametrize("units,L,dk,dv", [(24, 1300, 24, 64), (9, 5000, 24, 32), (1, 1040, 16, 32), (3, 16400, 32, 32)])
+def test_chunks_cut_for_whole_rounds(oracle, units, L, dk, dv):
+    """From logits the tiles of a chunk follow the call: five to eight of them, up to more than 128 chunks."""
+    cfg, x = random_problem(3300 + L, units, 1, L, dk, dv, "bf16", gate_mean=2.0)
+    vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_WARP_TILES)
+    try:
+        got, ref = _run_fused(oracle, cfg, x)
+    finally:
+        vig.vig_test_set_kernel_preference(vig.VIG_TEST_KERNEL_AUTO)
+    assert np.isfinite(got).all() and rel_err(got, ref) <= TOL["bf16"]
