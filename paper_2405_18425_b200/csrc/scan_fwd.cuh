@@ -20,7 +20,7 @@ namespace vig {
 namespace scan {
 
 constexpr int TG = 4;       // tokens staged at once
-constexpr int kCols = 16;   // value columns of a block
+constexpr int kCols = 16;   // value columns of a block of two columns a lane
 
 template <typename T>
 struct ScanArgs {
@@ -30,25 +30,25 @@ struct ScanArgs {
 };
 
 constexpr int scan_max_warps(int rpl) { return rpl <= 16 ? 8 : 1; }   // segments per block (32 rows a lane: no registers for the first pass)
-constexpr size_t scan_stage_floats(int rpl) { return (size_t)TG * (3 * 4 * rpl + kCols); }
-constexpr size_t scan_fold_floats(int rpl) { return (size_t)2 * 4 * rpl * (kCols + 1); }
+constexpr size_t scan_stage_floats(int rpl, int cpl = 2) { return (size_t)TG * (3 * 4 * rpl + 8 * cpl); }
+constexpr size_t scan_fold_floats(int rpl, int cpl = 2) { return (size_t)2 * 4 * rpl * (8 * cpl + 1); }
 
-// One slab of sixteen value columns of one unit by the first nw warps of a block (this one is number w), a segment of
+// One slab of 8 CPL value columns of one unit by the first nw warps of a block (this one is number w), a segment of
 // a.seg_len tokens each: nw of them cover the sequence.  Every thread of the block calls it: block barriers inside.
-template <typename T, int RPL, bool VEC>
+template <typename T, int RPL, bool VEC, int CPL = 2>
 __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit, int slab, int w, int nw, float* sc_smem) {
-    constexpr int DKP = 4 * RPL, R2 = RPL / 2, HC = (RPL + 7) / 8;
+    constexpr int DKP = 4 * RPL, R2 = RPL / 2, HC = (RPL + 7) / 8, kWide = 8 * CPL, kPieces = TG * kWide / 4;   // 4-column pieces of v in a group
     const int lane = threadIdx.x & 31;
     const int cp = lane & 7, rg = lane >> 3;
     const bool on = w < nw;
     const int L = a.L, dk = a.dk, dv = a.dv;
     const size_t ok = unit * L * dk, ov = unit * L * dv;
-    const int col0 = slab * kCols;
+    const int col0 = slab * kWide;
     const int s0 = w * a.seg_len, s1 = min(L, s0 + a.seg_len);
-    float* xs = sc_smem + w * scan_stage_floats(RPL);   // [TG][DKP]: q (walks) or the gates of the backward direction (first pass)
+    float* xs = sc_smem + w * scan_stage_floats(RPL, CPL);   // [TG][DKP]: q (walks) or the gates of the backward direction (first pass)
     float* ks = xs + TG * DKP;
     float* as = ks + TG * DKP;
-    float* vs = as + TG * DKP;                          // [TG][16]
+    float* vs = as + TG * DKP;                          // [TG][8 CPL]
 
     // the next TG tokens of a walk (t = base + step n) on their way, four key dimensions (value columns) of a token per lane
     using P = Piece<T, VEC>;
@@ -62,8 +62,8 @@ __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit,
             rk[h].load(a.k + ok + (ptrdiff_t)t * dk + d, n);
             ra[h].load(ga + (ptrdiff_t)(t + sa) * dk + d, t + sa >= 0 && t + sa < L ? n : 0);
         }
-        const int t = base + step * (lane >> 2), j = col0 + 4 * (lane & 3);
-        rv.load(a.v + ov + (ptrdiff_t)t * dv + j, lane < TG * kCols / 4 && t >= s0 && t < s1 ? dv - j : 0);
+        const int t = base + step * (lane / (kWide / 4)), j = col0 + 4 * (lane % (kWide / 4));
+        rv.load(a.v + ov + (ptrdiff_t)t * dv + j, lane < kPieces && t >= s0 && t < s1 ? dv - j : 0);
     };
     // ... and into shared memory (tokens outside the segment: k = q = 0, gate 1)
     auto commit = [&](bool x_is_gate) {
@@ -79,7 +79,7 @@ __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit,
                 reinterpret_cast<float4*>(as)[y] = make_float4(expf(g.x), expf(g.y), expf(g.z), expf(g.w));
             }
         }
-        if (lane < TG * kCols / 4) reinterpret_cast<float4*>(vs)[lane] = rv.get();
+        if (lane < kPieces) reinterpret_cast<float4*>(vs)[lane] = rv.get();
         __syncwarp();
     };
     auto rows = [&](const float* p, int n, f32x2 (&r)[R2]) {
@@ -91,15 +91,27 @@ __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit,
             r[2 * x + 1] = u.y;
         }
     };
-    auto cols = [&](int n, f32x2& v0, f32x2& v1) {
-        const float2 v = *reinterpret_cast<const float2*>(vs + n * kCols + 2 * cp);
-        v0 = pack2(v.x, v.x);
-        v1 = pack2(v.y, v.y);
+    // column h of this lane: two of them side by side, more of them eight apart (the eight lanes of a row group read whole lines)
+    auto column = [&](int h) { return CPL == 2 ? 2 * cp + h : 8 * h + cp; };
+    auto cols = [&](int n, f32x2 (&v2)[CPL]) {
+        if constexpr (CPL == 2) {
+            const float2 v = *reinterpret_cast<const float2*>(vs + n * kWide + 2 * cp);
+            v2[0] = pack2(v.x, v.x);
+            v2[1] = pack2(v.y, v.y);
+        } else {
+#pragma unroll
+            for (int h = 0; h < CPL; ++h) {
+                const float v = vs[n * kWide + column(h)];
+                v2[h] = pack2(v, v);
+            }
+        }
     };
 
-    f32x2 S[R2][2], X[R2][2];   // the states that enter the segment from the left and from the right
+    f32x2 S[R2][CPL], X[R2][CPL];   // the states that enter the segment from the left and from the right
 #pragma unroll
-    for (int r = 0; r < R2; ++r) S[r][0] = S[r][1] = X[r][0] = X[r][1] = 0ull;   // (+0, +0)
+    for (int r = 0; r < R2; ++r)
+#pragma unroll
+        for (int h = 0; h < CPL; ++h) S[r][h] = X[r][h] = 0ull;   // (+0, +0)
     if (scan_max_warps(RPL) > 1 && nw > 1) {
         // ---- first pass: forward state left behind (S) and its decay (D); backward state at the first token (X), the running
         // product of the backward gates (P) turning the recurrence into a sum that also runs upwards ----
@@ -113,46 +125,49 @@ __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit,
             if (t0 + TG < s1) fetch(t0 + TG, 1, a.gb + ok, a.sb, a.gf + ok, a.sf);
 #pragma unroll
             for (int n = 0; n < TG; ++n) {
-                f32x2 kk[R2], af[R2], ab[R2], v0, v1;
+                f32x2 kk[R2], af[R2], ab[R2], v2[CPL];
                 rows(ks, n, kk);
                 rows(as, n, af);
                 rows(xs, n, ab);
-                cols(n, v0, v1);
+                cols(n, v2);
 #pragma unroll
                 for (int r = 0; r < R2; ++r) {
-                    S[r][0] = ffma2(af[r], S[r][0], fmul2(kk[r], v0));
-                    S[r][1] = ffma2(af[r], S[r][1], fmul2(kk[r], v1));
                     const f32x2 pk = fmul2(P[r], kk[r]);
-                    X[r][0] = ffma2(pk, v0, X[r][0]);
-                    X[r][1] = ffma2(pk, v1, X[r][1]);
+#pragma unroll
+                    for (int h = 0; h < CPL; ++h) {
+                        S[r][h] = ffma2(af[r], S[r][h], fmul2(kk[r], v2[h]));
+                        X[r][h] = ffma2(pk, v2[h], X[r][h]);
+                    }
                     D[r] = fmul2(D[r], af[r]);
                     P[r] = fmul2(P[r], ab[r]);
                 }
             }
         }
         __syncthreads();   // the fold area lies over the staging
-        ulonglong2* st = reinterpret_cast<ulonglong2*>(sc_smem);                    // [warp][dir][R2][lane]
-        f32x2* dec = reinterpret_cast<f32x2*>(sc_smem + (size_t)nw * 2 * DKP * kCols);   // [warp][dir][DKP / 2]
+        f32x2* st = reinterpret_cast<f32x2*>(sc_smem);                                   // [warp][dir][R2][CPL][lane]
+        f32x2* dec = reinterpret_cast<f32x2*>(sc_smem + (size_t)nw * 2 * DKP * kWide);   // [warp][dir][DKP / 2]
 #pragma unroll
         for (int r = 0; r < R2; ++r) {
-            if (on) {
-                st[((w * 2) * R2 + r) * 32 + lane] = make_ulonglong2(S[r][0], S[r][1]);
-                st[((w * 2 + 1) * R2 + r) * 32 + lane] = make_ulonglong2(X[r][0], X[r][1]);
+#pragma unroll
+            for (int h = 0; h < CPL; ++h) {
+                if (on) {
+                    st[(((w * 2) * R2 + r) * CPL + h) * 32 + lane] = S[r][h];
+                    st[(((w * 2 + 1) * R2 + r) * CPL + h) * 32 + lane] = X[r][h];
+                }
+                S[r][h] = X[r][h] = 0ull;
             }
             if (on && cp == 0) {
                 dec[(w * 2) * (DKP / 2) + rg * R2 + r] = D[r];
                 dec[(w * 2 + 1) * (DKP / 2) + rg * R2 + r] = P[r];
             }
-            S[r][0] = S[r][1] = X[r][0] = X[r][1] = 0ull;
         }
         __syncthreads();
-        auto fold = [&](int s, int dir, f32x2 (&to)[R2][2]) {
+        auto fold = [&](int s, int dir, f32x2 (&to)[R2][CPL]) {
 #pragma unroll
             for (int r = 0; r < R2; ++r) {
-                const ulonglong2 e = st[((s * 2 + dir) * R2 + r) * 32 + lane];
                 const f32x2 d = dec[(s * 2 + dir) * (DKP / 2) + rg * R2 + r];
-                to[r][0] = ffma2(d, to[r][0], e.x);
-                to[r][1] = ffma2(d, to[r][1], e.y);
+#pragma unroll
+                for (int h = 0; h < CPL; ++h) to[r][h] = ffma2(d, to[r][h], st[(((s * 2 + dir) * R2 + r) * CPL + h) * 32 + lane]);
             }
         };
         for (int s = 0; s < w && on; ++s) fold(s, 0, S);
@@ -169,56 +184,58 @@ __device__ __forceinline__ void scan_fwd_slab(const ScanArgs<T>& a, size_t unit,
         const int sa = walk == 0 ? a.sf : a.sb, first = walk == 0 ? s0 : s1 - 1;
         if (walk == 1) {
 #pragma unroll
-            for (int r = 0; r < R2; ++r) {
-                S[r][0] = X[r][0];
-                S[r][1] = X[r][1];
-            }
+            for (int r = 0; r < R2; ++r)
+#pragma unroll
+                for (int h = 0; h < CPL; ++h) S[r][h] = X[r][h];
         }
         fetch(first, step, a.q + ok, 0, ga, sa);
         for (int m = 0; m < s1 - s0; m += TG) {
             const int base = first + step * m;
             commit(false);
             if (m + TG < s1 - s0) fetch(base + step * TG, step, a.q + ok, 0, ga, sa);
-            T up[2];
+            T up[CPL];
             if (walk == 1) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int t = base - rg, j = col0 + 2 * cp + h;
+                for (int h = 0; h < CPL; ++h) {
+                    const int t = base - rg, j = col0 + column(h);
                     up[h] = t >= s0 && j < dv ? a.out[ov + (size_t)t * dv + j] : T(0.f);
                 }
             }
-            float o[4][2];
+            float o[4][CPL];
 #pragma unroll
             for (int n = 0; n < 4; ++n) {
-                f32x2 qq[R2], kk[R2], af[R2], v0, v1, a0 = 0ull, a1 = 0ull;
+                f32x2 qq[R2], kk[R2], af[R2], v2[CPL], acc[CPL];
                 rows(xs, n, qq);
                 rows(ks, n, kk);
                 rows(as, n, af);
-                cols(n, v0, v1);
+                cols(n, v2);
+#pragma unroll
+                for (int h = 0; h < CPL; ++h) acc[h] = 0ull;
 #pragma unroll
                 for (int r = 0; r < R2; ++r) {
-                    S[r][0] = ffma2(af[r], S[r][0], fmul2(kk[r], v0));   // S_t = G_t . S_prev + k_t^T v_t
-                    S[r][1] = ffma2(af[r], S[r][1], fmul2(kk[r], v1));
-                    a0 = ffma2(qq[r], S[r][0], a0);                      // o_t = q_t S_t
-                    a1 = ffma2(qq[r], S[r][1], a1);
+#pragma unroll
+                    for (int h = 0; h < CPL; ++h) {
+                        S[r][h] = ffma2(af[r], S[r][h], fmul2(kk[r], v2[h]));   // S_t = G_t . S_prev + k_t^T v_t
+                        acc[h] = ffma2(qq[r], S[r][h], acc[h]);                 // o_t = q_t S_t
+                    }
                 }
-                o[n][0] = sum2(a0);
-                o[n][1] = sum2(a1);
+#pragma unroll
+                for (int h = 0; h < CPL; ++h) o[n][h] = sum2(acc[h]);
             }
             // sums over the four row groups, token n to the lanes of row group n
-            float h2[2][2], o1[2];
+            float h2[2][CPL], o1[CPL];
             const bool hi = rg & 2, odd = rg & 1;
 #pragma unroll
             for (int n = 0; n < 2; ++n)
 #pragma unroll
-                for (int h = 0; h < 2; ++h) h2[n][h] = (hi ? o[n + 2][h] : o[n][h]) + __shfl_xor_sync(0xffffffffu, hi ? o[n][h] : o[n + 2][h], 16);
+                for (int h = 0; h < CPL; ++h) h2[n][h] = (hi ? o[n + 2][h] : o[n][h]) + __shfl_xor_sync(0xffffffffu, hi ? o[n][h] : o[n + 2][h], 16);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) o1[h] = (odd ? h2[1][h] : h2[0][h]) + __shfl_xor_sync(0xffffffffu, odd ? h2[0][h] : h2[1][h], 8);
+            for (int h = 0; h < CPL; ++h) o1[h] = (odd ? h2[1][h] : h2[0][h]) + __shfl_xor_sync(0xffffffffu, odd ? h2[0][h] : h2[1][h], 8);
             const int t = base + step * rg;
             if (t >= s0 && t < s1) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int j = col0 + 2 * cp + h;
+                for (int h = 0; h < CPL; ++h) {
+                    const int j = col0 + column(h);
                     if (j < dv) rec_store(a.out + ov + (size_t)t * dv + j, walk == 0 ? o1[h] : 0.5f * (rec_to_float(up[h]) + o1[h]));
                 }
             }
