@@ -66,7 +66,8 @@ typedef enum vig_dtype { VIG_DTYPE_F32 = 0, VIG_DTYPE_BF16 = 1 } vig_dtype;
  *       recurrence (Eq. 6 step by step) instead of the factorised tiles.
  * f32:  dk <= 128, dv <= 256; fp32 walks on the CUDA cores, a sequence cut into segments that run side by side.
  * Sequences of at most 256 tokens run in one launch with a unit per thread block and use no scratch.
- * Longer ones are cut into 256-token segments (one launch; the blocks of a unit exchange segment
+ * Longer ones are cut into chunks of up to 128 tokens that are the blocks of one cluster (one launch, up to 1024 tokens, no scratch),
+ * into 256-token segments (one launch; the blocks of a unit exchange segment
  * summaries through scratch) or into 128-token chunk tasks (three launches; chunk summaries and
  * boundary states go through scratch), whichever suits the shape.  The library allocates and frees
  * that scratch on `stream` from a stream-ordered memory pool of its own (one per device, which keeps

@@ -1,7 +1,8 @@
 // bf16 BiGLA forward on the warp-level tensor-core instructions (mma.sync): one warp per 16 tokens, every product a chain of
 // 16 x 16 tiles whose scores stay in registers.  Units of at most 256 tokens are one block each; longer sequences are cut
-// into chunks of up to 128 tokens, one block each, in three launches: the state every chunk adds in either direction, a
-// fold over the chunks, the chunks themselves from the states that enter them.
+// into chunks of up to 128 tokens, one block each.  Up to eight chunks (1024 tokens): one launch, a cluster of blocks per unit, each of
+// which gives the others the state it adds through distributed shared memory.  Any length: three launches, the state every chunk adds in
+// either direction, a fold over the chunks, the chunks themselves from the states that enter them.
 //
 // With b_t the inclusive prefix sum of log alpha> and x_t the exclusive prefix sum of log alpha< (the backward decay from t
 // to s > t is exp(x_s - x_t): the gates t .. s-1), both from the start of a chunk of 128 tokens, Eq. 6 is, per chunk,

@@ -86,7 +86,8 @@ __device__ __forceinline__ void named_bar(int id, int count) {
 // programmatic stream serialization, may start its prologue once every block of this grid has executed this (or
 // exited).  `pdl_wait`: blocks until every kernel this grid depends on has completed and its memory operations are
 // visible; a no-op for an ordinary launch.  The kernels here execute it before their first global-memory read into
-// shared memory or registers and before any write; prefetches into L2, which consume nothing, may precede it.
+// shared memory or registers and before any write; prefetches into L2, which consume nothing, may precede it.  One exception: the last
+// launch of a chunked call reads inputs and flags at once and waits only for what the fold before it writes (see there).
 // They let the next kernel start behind their own wait: before it, a run of small launches is let in several kernels deep, and the
 // blocks of one kernel, waiting, crowd those of another onto the same SMs (64 units of 196 tokens, 32 x 64, from logits: 11.7 us
 // a call, 7.6 this way; one sequence of 9762 tokens 23.3 and 14.7).

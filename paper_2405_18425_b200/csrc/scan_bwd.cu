@@ -20,8 +20,8 @@ __global__ void __launch_bounds__(bwd_max_warps(CN) * 32, CN <= 16 ? 2 : 1) scan
 
 // Both in one launch, the longer walks first.  Either alone leaves SMs idle that hold one block beside SMs that hold two: 48 units
 // of 196 tokens, 32 x 64, fp32, 192 blocks each: 31 us and 51 us one after the other, 59 us together.
-template <typename T, int CN, int RPL>
-__global__ void __launch_bounds__(256, 2) scan_grad_kernel(const ScanBwdArgs<T> a, const FloatPairs pairs, const ScanArgs<T> f, int bwd_slabs, int bwd_warps,
+template <typename T, int CN, int RPL, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, WARPS > 8 ? 1 : 2) scan_grad_kernel(const ScanBwdArgs<T> a, const FloatPairs pairs, const ScanArgs<T> f, int bwd_slabs, int bwd_warps,
                                                            int fwd_warps) {
     extern __shared__ __align__(16) float sg_smem[];
     pdl_wait();
@@ -40,10 +40,10 @@ int segment_length(int L, long long blocks, int sms, int most) {
     return (int)(((L + want - 1) / want + TG - 1) / TG * TG);
 }
 
-template <typename T, int CN, int RPL>
+template <typename T, int CN, int RPL, int WARPS>
 cudaError_t launch_scan_grad_t(ScanBwdArgs<T> a, float2* pairs, ScanArgs<T> f, long long units, cudaStream_t stream) {
-    constexpr int kMaxWarps = 8;
-    static_assert(bwd_max_warps(CN) == kMaxWarps && scan_max_warps(RPL) == kMaxWarps, "");
+    constexpr int kMaxWarps = WARPS;
+    static_assert(bwd_max_warps(CN) == 8 && scan_max_warps(RPL) == 8, "");
     constexpr size_t kBwd = (bwd_stage_floats(CN) + bwd_fold_floats(CN)) * sizeof(float);
     constexpr size_t kFwd = (scan_stage_floats(RPL) > scan_fold_floats(RPL) ? scan_stage_floats(RPL) : scan_fold_floats(RPL)) * sizeof(float);
     constexpr size_t kPerWarp = kBwd > kFwd ? kBwd : kFwd;
@@ -54,15 +54,16 @@ cudaError_t launch_scan_grad_t(ScanBwdArgs<T> a, float2* pairs, ScanArgs<T> f, l
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     int sms = sms_of[dev].load(std::memory_order_acquire);
     if (sms == 0) {
-        if ((e = cudaFuncSetAttribute(scan_grad_kernel<T, CN, RPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxWarps * kPerWarp))) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(scan_grad_kernel<T, CN, RPL, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxWarps * kPerWarp))) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
     const int bs = (a.dk + kRows - 1) / kRows, fs = (f.dv + kCols - 1) / kCols;
-    a.seg_len = segment_length(a.L, units * bs, sms, kMaxWarps);
-    f.seg_len = segment_length(f.L, units * fs, sms, kMaxWarps);
+    const int most = WARPS > 8 ? many_segments(a.L) : kMaxWarps;
+    a.seg_len = segment_length(a.L, units * bs, sms, most);
+    f.seg_len = segment_length(f.L, units * fs, sms, most);
     const int nb = (a.L + a.seg_len - 1) / a.seg_len, nf = (f.L + f.seg_len - 1) / f.seg_len, nw = nb > nf ? nb : nf;
-    const cudaError_t le = launch_pdl(scan_grad_kernel<T, CN, RPL>, dim3((unsigned)units, (unsigned)(bs + fs)), dim3(nw * 32), nw * kPerWarp, stream, a,
+    const cudaError_t le = launch_pdl(scan_grad_kernel<T, CN, RPL, WARPS>, dim3((unsigned)units, (unsigned)(bs + fs)), dim3(nw * 32), nw * kPerWarp, stream, a,
                                       FloatPairs{pairs}, f, bs, nb, nf);
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
@@ -107,6 +108,9 @@ cudaError_t launch_scan_bwd(const T* q, const T* k, const T* v, const T* la_f, c
 }
 
 bool scan_grad_supported(int dk, int dv) { return dk <= 32 && dv <= 64 && dk % 4 == 0 && dv % 4 == 0; }
+bool scan_grad_many(long long units, int dk, int dv, int sms) {
+    return scan_grad_supported(dk, dv) && units * ((dk + kRows - 1) / kRows + (dv + kCols - 1) / kCols) <= sms;
+}
 
 template <typename T>
 cudaError_t launch_scan_grad(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, const T* d_out, T* dq, T* dk_out, T* dv_out, T* dla_f, T* dla_b,
@@ -114,10 +118,20 @@ cudaError_t launch_scan_grad(const T* q, const T* k, const T* v, const T* la_f, 
     const ScanBwdArgs<T> a{q, k, v, la_f, la_b, d_out, dq, dk_out, dla_f, dla_b, L, dk, dv, 0};
     const ScanArgs<T> f{k, q, d_out, la_b, la_f, dv_out, L, dk, dv, 0, -1, 1};   // the adjoint: operands swapped, gates moved by one token
     float2* pairs = static_cast<float2*>(scratch);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const bool many = scan_grad_many(units, dk, dv, sms);
+#define VIG_RPL(CN_, RPL_) \
+    return many ? launch_scan_grad_t<T, CN_, RPL_, kManyWarps>(a, pairs, f, units, stream) : launch_scan_grad_t<T, CN_, RPL_, 8>(a, pairs, f, units, stream);
 #define VIG_CASE(CN_) \
-    if (dv <= 4 * CN_) return dk <= 16 ? launch_scan_grad_t<T, CN_, 4>(a, pairs, f, units, stream) : launch_scan_grad_t<T, CN_, 8>(a, pairs, f, units, stream);
+    if (dv <= 4 * CN_) { \
+        if (dk <= 16) VIG_RPL(CN_, 4) else VIG_RPL(CN_, 8) \
+    }
     VIG_CASE(8) VIG_CASE(12) VIG_CASE(16)
 #undef VIG_CASE
+#undef VIG_RPL
     return cudaErrorInvalidValue;
 }
 template cudaError_t launch_scan_grad<float>(const float*, const float*, const float*, const float*, const float*, const float*, float*, float*, float*,

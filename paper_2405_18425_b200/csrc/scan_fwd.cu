@@ -9,17 +9,17 @@ namespace {
 
 using namespace scan;
 
-template <typename T, int RPL, bool VEC, int CPL>
-__global__ void __launch_bounds__(scan_max_warps(RPL) * 32, RPL <= 8 && CPL == 2 ? 2 : 1) scan_fwd_kernel(const ScanArgs<T> a) {
+template <typename T, int RPL, bool VEC, int CPL, int WARPS>
+__global__ void __launch_bounds__(WARPS * 32, RPL <= 8 && CPL == 2 && WARPS <= 8 ? 2 : 1) scan_fwd_kernel(const ScanArgs<T> a) {
     extern __shared__ __align__(16) float sc_smem[];
     pdl_wait();
     pdl_launch_dependents();
     scan_fwd_slab<T, RPL, VEC, CPL>(a, blockIdx.x, blockIdx.y, threadIdx.x >> 5, blockDim.x >> 5, sc_smem);
 }
 
-template <typename T, int RPL, bool VEC, int CPL>
+template <typename T, int RPL, bool VEC, int CPL, int WARPS = scan_max_warps(RPL)>
 cudaError_t launch_scan_t(ScanArgs<T> a, long long units, cudaStream_t stream) {
-    constexpr int kMaxWarps = scan_max_warps(RPL);
+    constexpr int kMaxWarps = WARPS;
     static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -28,7 +28,7 @@ cudaError_t launch_scan_t(ScanArgs<T> a, long long units, cudaStream_t stream) {
     int sms = sms_of[dev].load(std::memory_order_acquire);
     const size_t per_warp = (scan_stage_floats(RPL, CPL) > scan_fold_floats(RPL, CPL) ? scan_stage_floats(RPL, CPL) : scan_fold_floats(RPL, CPL)) * sizeof(float);
     if (sms == 0) {
-        if ((e = cudaFuncSetAttribute(scan_fwd_kernel<T, RPL, VEC, CPL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxWarps * per_warp))) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(scan_fwd_kernel<T, RPL, VEC, CPL, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxWarps * per_warp))) != cudaSuccess) return e;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
         sms_of[dev].store(sms, std::memory_order_release);
     }
@@ -37,10 +37,11 @@ cudaError_t launch_scan_t(ScanArgs<T> a, long long units, cudaStream_t stream) {
     const int slabs = (a.dv + 8 * CPL - 1) / (8 * CPL);
     const long long n = form_units(units) * slabs;
     long long want = (16LL * sms + n - 1) / n;
-    if (want > kMaxWarps) want = kMaxWarps;
+    const int most = WARPS > 8 ? many_segments(a.L) : kMaxWarps;
+    if (want > most) want = most;
     a.seg_len = (int)(((a.L + want - 1) / want + TG - 1) / TG * TG);
     const int nw = (a.L + a.seg_len - 1) / a.seg_len;
-    const cudaError_t le = launch_pdl(scan_fwd_kernel<T, RPL, VEC, CPL>, dim3((unsigned)units, (unsigned)slabs), dim3(nw * 32), nw * per_warp, stream, a);
+    const cudaError_t le = launch_pdl(scan_fwd_kernel<T, RPL, VEC, CPL, WARPS>, dim3((unsigned)units, (unsigned)slabs), dim3(nw * 32), nw * per_warp, stream, a);
     count_launch();
     return le != cudaSuccess ? le : cudaGetLastError();
 }
@@ -64,6 +65,13 @@ cudaError_t launch_scan_fwd(const T* q, const T* k, const T* v, const T* la_f, c
     if (vec && dk <= 32 && blocks(2) > sms) cpl = blocks(3) <= sms ? 3 : (blocks(4) <= sms ? 4 : 2);
 #define VIG_CASE(RPL_) \
     if (dk <= 4 * RPL_) return vec ? launch_scan_t<T, RPL_, true, 2>(a, units, stream) : launch_scan_t<T, RPL_, false, 2>(a, units, stream);
+    // Few sequences, blocks with an SM each: sixteen warps (training step of 24 units of 196 tokens, 16 x 64, fp32: 42.1 us, 56.3 with eight).
+#define VIG_MANY(RPL_) \
+    if (dk <= 4 * RPL_) return launch_scan_t<T, RPL_, true, 2, kManyWarps>(a, units, stream);
+    if (vec && dk <= 32 && blocks(2) <= sms) {
+        VIG_MANY(4) VIG_MANY(8)
+    }
+#undef VIG_MANY
 #define VIG_WIDE(RPL_) \
     if (cpl > 2 && dk <= 4 * RPL_) return cpl == 3 ? launch_scan_t<T, RPL_, true, 3>(a, units, stream) : launch_scan_t<T, RPL_, true, 4>(a, units, stream);
     VIG_WIDE(4) VIG_WIDE(8)

@@ -30,6 +30,9 @@ struct ScanArgs {
 };
 
 constexpr int scan_max_warps(int rpl) { return rpl <= 16 ? 8 : 1; }   // segments per block (32 rows a lane: no registers for the first pass)
+// Segments of calls whose blocks have an SM each: twice as many, of twelve tokens at least (a segment costs every other one a fold step).
+constexpr int kManyWarps = 16;
+inline int many_segments(int L) { return L / 12 < 8 ? 8 : (L / 12 < kManyWarps ? L / 12 : kManyWarps); }
 constexpr size_t scan_stage_floats(int rpl, int cpl = 2) { return (size_t)TG * (3 * 4 * rpl + 8 * cpl); }
 constexpr size_t scan_fold_floats(int rpl, int cpl = 2) { return (size_t)2 * 4 * rpl * (8 * cpl + 1); }
 

@@ -8,7 +8,7 @@ import torch
 import paper_2405_18425_b200 as vig
 from paper_2405_18425_b200 import synth
 
-from helpers import TOL, device_to_f64, oracle_log_alpha, random_problem, rel_err, to_device, to_stored
+from helpers import TOL, device_to_f64, oracle_log_alpha, oracle_out, random_problem, rel_err, to_device, to_stored
 
 pytestmark = pytest.mark.gpu
 
@@ -277,3 +277,24 @@ def test_pair_whose_exchange_expires_stores_no_gate_gradients():
         assert same(a, b)
     for a, b in zip(got[3:], want[3:]):
         assert bool((a[:, :, :112] == 7.0).all()) and same(a[:, :, 112:].contiguous(), b[:, :, 112:].contiguous())
+
+
+@pytest.mark.parametrize("units,L,dk,dv", [(1, 13, 4, 4), (3, 97, 12, 20), (12, 400, 24, 48), (2, 784, 32, 64), (2, 2047, 16, 32), (47, 61, 32, 64), (60, 30, 32, 32)])
+def test_fp32_walks_of_few_and_of_more_units(oracle, units, L, dk, dv):
+    """Sixteen warps a block where every block has an SM of its own, three and four columns a lane, ragged last segments; forward and
+    gradient, the latter with dv in the same launch."""
+    cfg, x = random_problem(4100 + L, units, 1, L, dk, dv, "f32", gate_mean=1.0)
+    la = [oracle_log_alpha(oracle, x[n], "f32", cfg.tau) for n in ("g_fwd", "g_bwd")]
+    d = {n: to_device(a, "f32") for n, a in dict(q=x["q"], k=x["k"], v=x["v"], f=la[0], b=la[1]).items()}
+    out = torch.empty_like(d["v"])
+    vig.vig_bigla_fwd_f32(d["q"], d["k"], d["v"], d["f"], d["b"], out)
+    assert rel_err(device_to_f64(out, "f32"), oracle_out(oracle, x["q"], x["k"], x["v"], la[0], la[1], "f32")) <= TOL["f32"]
+    g = np.random.default_rng(L).standard_normal(x["v"].shape).astype(np.float32)
+    grads = [torch.empty_like(d[n]) for n in ("q", "k", "v", "q", "q")]
+    before = vig.vig_kernel_launch_count()
+    vig.vig_bigla_bwd(d["q"], d["k"], d["v"], d["f"], d["b"], to_device(g, "f32"), *grads)
+    assert vig.vig_kernel_launch_count() - before == 1
+    f64 = lambda a: a.astype(np.float64)
+    ref = oracle.bigla_bwd(f64(x["q"]), f64(x["k"]), f64(x["v"]), f64(la[0]), f64(la[1]), f64(g))
+    for t, r in zip(grads, ref):
+        assert rel_err(device_to_f64(t, "f32"), r) <= TOL["f32"]
