@@ -764,12 +764,12 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
 
 // Where the chunks run faster this way than as tcgen05 segments or chunk tasks.  A chunk's chain of dependent steps is shorter
 // here, so few chunks gain most (1.3 to 1.7 times up to one per SM); a chunk's work grows with the key dimensions, while the chunk
-// tasks, once their latency is hidden, cost the same whatever the state: the wider the keys the sooner the tasks win, and sooner
-// where the gates come prepared (40 x 4096 tokens from log gates, 24 x 48: 50.8 us this way, 48.2 as tasks).  The segmented launch is at its best while two full segments (four chunks) of every unit are
+// tasks, once their latency is hidden, cost the same whatever the state: keys of 32 lose in large calls, sooner where the gates come
+// prepared (32 units of 4096 tokens, 32 x 64: 51.7 us this way, 42.4 as tasks; 24 x 48 from log gates 36.6 and 37.4).  The segmented launch is at its best while two full segments (four chunks) of every unit are
 // resident in one round; beyond that round it is at its worst (300 units of 304 tokens, 32 x 64, from logits: 52.7 us, 43.7 this way).
-// More than 64 chunks: the fold here takes eight runs side by side, the tasks' takes one.  Timed against the tcgen05
-// forms for nine head sizes, 257 to 16384 tokens, 1 to 300 units, with and without the gates (1530 shapes): within 0.3 % of the
-// better form on average.
+// More than 64 chunks: the tasks' fold takes one run.  Timed against the tcgen05 forms for six head sizes, 1100 to 16384 tokens,
+// 1 to 96 units, with and without the gates (468 shapes; 1530 more up to 512 tokens before clusters took most of them): within 0.2 %
+// of the better form on average.
 bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
     if (dk == 16) return true;
     const long long sms = device_sms();
@@ -780,9 +780,9 @@ bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
     const bool two_segments = L <= 512;
     if (two_segments && nch == 4 && units <= sms) return dk == 32 ? chunks <= sms : (chunks <= 3 * sms || dv <= (gates ? 48 : 32));
     if (two_segments && units > sms) return gates || dk == 24 || chunks <= 8 * sms;
-    if (dk == 24) return gates || dv == 32 || chunks <= (nch <= 8 ? 8 : 4) * sms;
-    if (chunks <= sms) return true;
-    return (gates || nch > 64) && chunks <= 4 * sms;
+    if (dk == 24) return true;
+    if (gates) return dv == 32 || chunks <= 5 * sms;
+    return 10 * chunks <= 28 * sms || (nch > 64 && chunks <= 4 * sms);
 }
 
 bool mma_chunks_supported(long long units, int L, int dk, int dv) { return units * chunk_plan(units, L, dk, dv).nch <= 0x7fffffffLL; }
