@@ -494,14 +494,15 @@ int bwd_cn(int dv, int cg) {   // columns per thread: the instantiated size that
 }
 
 // Segments in blocks of their own (nseg > 1), where the walks within one block per unit and eight key dimensions would
-// leave most of the chip idle: few units and long sequences, from 512 tokens on, or 2048 where those walks are sixteen warps a block
-// (scan_grad_many: 12 units of 700 tokens, 32 x 64, fp32, a training step: 192 us this way, 126 in the block; 6 of 1500, 24 x 48: 277 and
-// 249; 16 units of 4096 tokens, eight warps: 672 against 1187).  About five blocks per SM (a lone block per SM needs about 550
+// leave most of the chip idle: few units and long sequences (12 units of 784 tokens, fp32: 157 us a call against 210, 16
+// units of 4096 tokens 672 against 1187; at 196 tokens the walks within a block take 45 us against 100).  Blocks of sixteen warps are the
+// faster ones up to 2048 tokens (a training step of 12 units of 700 tokens, 32 x 64: 192 us this way, 126 in the block), with gate gradients
+// three times as exact, but dq and dk 4 % further off (1.56e-7 to 1.50e-7 in 2-norm: sums that run upwards): not taken.  About five blocks per SM (a lone block per SM needs about 550
 // cycles per token); segments are multiples of the staging group and at least 64 tokens.
-void bwd_plan(long long units, int L, int dk, int dv, int sms, int* nseg, int* seg_len) {
+void bwd_plan(long long units, int L, int dk, int sms, int* nseg, int* seg_len) {
     *nseg = 1;
     *seg_len = L > 0 ? L : 1;
-    if (L < (scan_grad_many(units, dk, dv, sms) ? 2048 : 512) || units * ((dk + 7) / 8) * 8 >= 4LL * sms) return;
+    if (L < 512 || units * ((dk + 7) / 8) * 8 >= 4LL * sms) return;
     long long want = (5LL * sms + units - 1) / units;
     if (want > L / 64) want = L / 64;
     const int len = (int)(((L + want - 1) / want + kBwdTT - 1) / kBwdTT * kBwdTT);
@@ -536,7 +537,7 @@ static void bwd_scratch_layout(long long units, int L, int dk, int dv, int nseg,
 size_t bwd_scratch_bytes(long long units, int L, int dk, int dv) {
     int sms = 0, nseg, seg_len;
     if (sm_count_of_device(&sms) != cudaSuccess) return 0;
-    bwd_plan(units, L, dk, dv, sms, &nseg, &seg_len);
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
     size_t p, st, de, to;
     bwd_scratch_layout(units, L, dk, dv, nseg, &p, &st, &de, &to);
     return (p + st + de + to) * sizeof(float);
@@ -545,7 +546,7 @@ size_t bwd_scratch_bytes(long long units, int L, int dk, int dv) {
 bool bwd_in_one_launch(long long units, int L, int dk, int dv) {
     int sms = 0, nseg, seg_len;
     if (!scan_grad_supported(dk, dv) || sm_count_of_device(&sms) != cudaSuccess) return false;
-    bwd_plan(units, L, dk, dv, sms, &nseg, &seg_len);
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
     return nseg == 1;
 }
 
@@ -570,7 +571,7 @@ cudaError_t launch_bigla_bwd(const T* q, const T* k, const T* v, const T* la_f, 
     int sms = 0, nseg, seg_len;
     cudaError_t e = sm_count_of_device(&sms);
     if (e != cudaSuccess) return e;
-    bwd_plan(units, L, dk, dv, sms, &nseg, &seg_len);
+    bwd_plan(units, L, dk, sms, &nseg, &seg_len);
     if (nseg == 1) return launch_scan_bwd<T>(q, k, v, la_f, la_b, d_out, dq, dk_out, dla_f, dla_b, scratch, units, L, dk, dv, stream);
     size_t p, st, de, to;
     bwd_scratch_layout(units, L, dk, dv, nseg, &p, &st, &de, &to);

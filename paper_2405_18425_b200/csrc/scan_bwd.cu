@@ -108,8 +108,8 @@ cudaError_t launch_scan_bwd(const T* q, const T* k, const T* v, const T* la_f, c
 }
 
 bool scan_grad_supported(int dk, int dv) { return dk <= 32 && dv <= 64 && dk % 4 == 0 && dv % 4 == 0; }
-bool scan_grad_many(long long units, int dk, int dv, int sms) {
-    return scan_grad_supported(dk, dv) && units * ((dk + kRows - 1) / kRows + (dv + kCols - 1) / kCols) <= sms;
+static bool scan_grad_many(long long units, int dk, int dv, int sms) {   // a block an SM at most: sixteen warps each
+    return units * ((dk + kRows - 1) / kRows + (dv + kCols - 1) / kCols) <= sms;
 }
 
 template <typename T>

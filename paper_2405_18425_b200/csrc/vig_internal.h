@@ -112,7 +112,6 @@ bool bwd_supported(int dk, int dv);
 size_t bwd_scratch_bytes(long long units, int L, int dk, int dv);   // 0: the device could not be queried
 bool bwd_in_one_launch(long long units, int L, int dk, int dv);   // launch_scan_grad takes the call: dv among its results
 bool scan_grad_supported(int dk, int dv);
-bool scan_grad_many(long long units, int dk, int dv, int sms);   // ... with a block an SM at most: sixteen warps each
 template <typename T>
 cudaError_t launch_scan_grad(const T* q, const T* k, const T* v, const T* la_f, const T* la_b, const T* d_out, T* dq, T* dk_out, T* dv_out,
                              T* dla_f, T* dla_b, void* scratch, long long units, int L, int dk, int dv, cudaStream_t stream);

@@ -282,7 +282,7 @@ def test_pair_whose_exchange_expires_stores_no_gate_gradients():
 @pytest.mark.parametrize("units,L,dk,dv", [(1, 13, 4, 4), (3, 97, 12, 20), (12, 400, 24, 48), (2, 784, 32, 64), (2, 2047, 16, 32), (47, 61, 32, 64), (60, 30, 32, 32)])
 def test_fp32_walks_of_few_and_of_more_units(oracle, units, L, dk, dv):
     """Sixteen warps a block where every block has an SM of its own, three and four columns a lane, ragged last segments; forward and
-    gradient, the latter with dv in the same launch."""
+    gradient, the latter with dv in the same launch below 512 tokens."""
     cfg, x = random_problem(4100 + L, units, 1, L, dk, dv, "f32", gate_mean=1.0)
     la = [oracle_log_alpha(oracle, x[n], "f32", cfg.tau) for n in ("g_fwd", "g_bwd")]
     d = {n: to_device(a, "f32") for n, a in dict(q=x["q"], k=x["k"], v=x["v"], f=la[0], b=la[1]).items()}
@@ -293,7 +293,7 @@ def test_fp32_walks_of_few_and_of_more_units(oracle, units, L, dk, dv):
     grads = [torch.empty_like(d[n]) for n in ("q", "k", "v", "q", "q")]
     before = vig.vig_kernel_launch_count()
     vig.vig_bigla_bwd(d["q"], d["k"], d["v"], d["f"], d["b"], to_device(g, "f32"), *grads)
-    assert vig.vig_kernel_launch_count() - before == 1
+    assert (vig.vig_kernel_launch_count() - before == 1) == (L < 512)   # longer ones of few units: segments in blocks of their own
     f64 = lambda a: a.astype(np.float64)
     ref = oracle.bigla_bwd(f64(x["q"]), f64(x["k"]), f64(x["v"]), f64(la[0]), f64(la[1]), f64(g))
     for t, r in zip(grads, ref):
