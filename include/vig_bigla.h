@@ -72,8 +72,8 @@ typedef enum vig_dtype { VIG_DTYPE_F32 = 0, VIG_DTYPE_BF16 = 1 } vig_dtype;
  * boundary states go through scratch), whichever suits the shape.  The library allocates and frees
  * that scratch on `stream` from a stream-ordered memory pool of its own (one per device, which keeps
  * freed memory for later calls instead of returning it to the driver); use the *_ws form to supply it.  The kernels are
- * launched with programmatic stream serialization: each waits for the work before it in `stream`
- * before it reads its inputs.
+ * launched with programmatic stream serialization: none reads anything before the work in front of the call
+ * in `stream` has completed.
  * Errors: NULL_POINTER, BAD_DIM, UNSUPPORTED, MISALIGNED, CUDA. */
 int vig_bigla_fwd_bf16(const void* q, const void* k, const void* v,
                        const void* log_alpha_fwd, const void* log_alpha_bwd, void* out,

@@ -187,7 +187,8 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     // what that launch still writes.
     if (MODE != kMain && tid == 0 && (long long)blockIdx.x < a.ahead) pull(blockIdx.x);
     // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
-    // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
+    // with them all that was launched before.  So inputs and flags are read at once, from L2 (see pdl_wait), and only what the fold
+    // writes is waited for.
     if (MODE != kMain) {
         pdl_wait();
         pdl_launch_dependents();
@@ -374,7 +375,7 @@ bigla_grad_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constan
     }
     if (MODE == kMain) {
         int slow = 0;
-        for (int x = tid; x < nch; x += blockDim.x) slow |= a.flags[unit * nch + x];
+        for (int x = tid; x < nch; x += blockDim.x) slow |= (int)ld_gpu4(a.flags + unit * nch + x);
         const bool missing = __syncthreads_or(slow & 2);
         if (__syncthreads_or(slow)) {
             pdl_wait();

@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     // and L2 stays coherent with what that launch still writes); the blocks after the first round are pulled in by those of it.
     if (MODE != kMain && tid == 32 && (int)blockIdx.x < args.ahead) pull(unit * L + tok0, min(tiles * 16, L - tok0), true, true);
     // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
-    // with them all that was launched before.  So inputs and flags are read at once, and only what the fold writes is waited for.
+    // with them all that was launched before.  So inputs and flags are read at once, from L2 (see pdl_wait), and only what the fold
+    // writes is waited for.
     if (MODE != kMain) {
         pdl_wait();
         pdl_launch_dependents();
@@ -151,10 +152,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         const int row = tok0 + w * 16 + 8 * r + g;
         if (live && row < L) {
             const size_t at = (unit * L + row) * DK;
-            load_pairs<DK>((kTakeKeys ? args.la2_f : args.la_f) + at, c, af[r]);
-            load_pairs<DK>((kTakeKeys ? args.la2_b : args.la_b) + at, c, ab[r]);
-            if (!kTakeKeys) load_pairs<DK>(args.k + at, c, kr[r]);
-            if (MODE != kSummary) load_pairs<DK>(args.q + at, c, qr[r]);
+            load_pairs<DK, MODE == kMain>((kTakeKeys ? args.la2_f : args.la_f) + at, c, af[r]);
+            load_pairs<DK, MODE == kMain>((kTakeKeys ? args.la2_b : args.la_b) + at, c, ab[r]);
+            if (!kTakeKeys) load_pairs<DK, MODE == kMain>(args.k + at, c, kr[r]);
+            if (MODE != kSummary) load_pairs<DK, MODE == kMain>(args.q + at, c, qr[r]);
         } else {
 #pragma unroll
             for (int j = 0; j < NP; ++j) {   // rows past the end: q = k = 0 and no decay (GATES: a logit of 100, log alpha = 0)
@@ -312,7 +313,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     bool redo = MODE == kUnit && *slow;
     if (MODE == kMain) {
         int any = 0;
-        for (int x = tid; x < nch; x += blockDim.x) any |= args.flags[unit * nch + x];
+        for (int x = tid; x < nch; x += blockDim.x) any |= (int)ld_gpu4(args.flags + unit * nch + x);
         const bool missing = __syncthreads_or(any & 2);
         redo = __syncthreads_or(any);
         if (w == 0 || redo) pdl_wait();   // the fold

@@ -175,17 +175,17 @@ __device__ __forceinline__ uint32_t log2_alpha_pair(uint32_t g, float inv_tau) {
 //   DK = 32: dims 8c + 2j, +1;   DK = 24: dims 4c + 2j, +1 (j = 0, 1) and 16 + 2c, +1 (j = 2);   DK = 16: dims 4c + 2j, +1
 // Ordinary loads, not those of the read-only path: this kernel may have started while the one that writes the row still ran
 // (programmatic dependent launch), so the row is not read-only for the kernel's lifetime and the load must stay behind
-// pdl_wait().
-template <int DK>
+// pdl_wait().  AHEAD: loads ahead of it, of rows that are known to be complete, from L2 (see pdl_wait).
+template <int DK, bool AHEAD = false>
 __device__ __forceinline__ void load_pairs(const __nv_bfloat16* row, int c, uint32_t (&r)[DK / 8]) {
     const char* p = reinterpret_cast<const char*>(row);
     if constexpr (DK == 32) {
-        const uint4 x = *reinterpret_cast<const uint4*>(p + 16 * c);
+        const uint4 x = AHEAD ? ld_gpu16(p + 16 * c) : *reinterpret_cast<const uint4*>(p + 16 * c);
         r[0] = x.x; r[1] = x.y; r[2] = x.z; r[3] = x.w;
     } else {
-        const uint2 x = *reinterpret_cast<const uint2*>(p + 8 * c);
+        const uint2 x = AHEAD ? ld_gpu8(p + 8 * c) : *reinterpret_cast<const uint2*>(p + 8 * c);
         r[0] = x.x; r[1] = x.y;
-        if constexpr (DK == 24) r[2] = *reinterpret_cast<const uint32_t*>(p + 32 + 4 * c);
+        if constexpr (DK == 24) r[2] = AHEAD ? ld_gpu4(p + 32 + 4 * c) : *reinterpret_cast<const uint32_t*>(p + 32 + 4 * c);
     }
 }
 

@@ -87,12 +87,33 @@ __device__ __forceinline__ void named_bar(int id, int count) {
 // exited).  `pdl_wait`: blocks until every kernel this grid depends on has completed and its memory operations are
 // visible; a no-op for an ordinary launch.  The kernels here execute it before their first global-memory read into
 // shared memory or registers and before any write; prefetches into L2, which consume nothing, may precede it.  One exception: the last
-// launch of a chunked call reads inputs and flags at once and waits only for what the fold before it writes (see there).
+// launch of a chunked call, which the fold before it lets in behind its own wait.  All earlier work has completed by then and stands in
+// L2, but only the kernel's own wait would make it visible to reads that L1 may answer, and scratch and inputs have the same addresses
+// from call to call: what this launch reads ahead of its wait comes by TMA, by bulk copies or by the loads below, all of them from L2
+// (waiting before any of it: one sequence of 16384 tokens, 24 x 48, 15.0 us instead of 13.2, training step of 4 units of 1200, 32 x 64,
+// 36.6 instead of 33.3; ordinary loads: 13.0 and 33.2).
 // They let the next kernel start behind their own wait: before it, a run of small launches is let in several kernels deep, and the
 // blocks of one kernel, waiting, crowd those of another onto the same SMs (64 units of 196 tokens, 32 x 64, from logits: 11.7 us
 // a call, 7.6 this way; one sequence of 9762 tokens 23.3 and 14.7).
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads at the scope of the GPU, which no L1 answers.
+__device__ __forceinline__ uint4 ld_gpu16(const void* p) {
+    uint4 x;
+    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w) : "l"(p) : "memory");
+    return x;
+}
+__device__ __forceinline__ uint2 ld_gpu8(const void* p) {
+    uint2 x;
+    asm volatile("ld.relaxed.gpu.global.v2.u32 {%0,%1}, [%2];" : "=r"(x.x), "=r"(x.y) : "l"(p) : "memory");
+    return x;
+}
+__device__ __forceinline__ uint32_t ld_gpu4(const void* p) {
+    uint32_t x;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+    return x;
+}
 
 // ---- blocks of a cluster ----
 __device__ __forceinline__ uint32_t cluster_peer(uint32_t addr, uint32_t rank) {

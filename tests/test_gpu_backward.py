@@ -237,6 +237,54 @@ def test_chain_of_dependent_launches_sees_what_the_last_one_wrote(units, L):
             assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
 
 
+@pytest.mark.parametrize("units,L,dk,dv", [(4, 1300, 24, 64), (9, 2100, 24, 32), (2, 4096, 32, 64), (3, 1200, 16, 48)])
+def test_chain_of_chunked_calls_on_reused_buffers_and_scratch(units, L, dk, dv):
+    """Forward from logits, forward from log gates and gradient in three launches each, back to back on the same buffers and the
+    same scratch, the contents changing from pass to pass; in one of the passes a unit's gates are closed, so that its chunks are
+    told to leave it to the walks.  The last of the three launches reads ahead of its own wait: nothing of the pass before may
+    come through."""
+    rng = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda d: torch.randn(1, units, L, d, generator=rng, device="cuda").bfloat16()
+    sets = [dict(q=mk(dk) * dk ** -0.5, k=mk(dk), v=mk(dv), gf=mk(dk), gb=mk(dk), g=mk(dv)) for _ in range(3)]
+    sets[1]["gf"][0, 1, 700:703] = -640.0          # log alpha = -40 a token: outside the range of the factorised tiles
+    now = {n: torch.empty_like(t) for n, t in sets[0].items()}
+    la = [torch.empty_like(now["gf"]) for _ in range(2)]
+    names = ("v", "v", "q", "k", "v", "gf", "gb")
+
+    def counted(call, *a):
+        before = vig.vig_kernel_launch_count()
+        call(*a)
+        assert vig.vig_kernel_launch_count() - before == 3
+
+    def step(out):
+        counted(vig.vig_bigla_fwd_gates_bf16, now["q"], now["k"], now["v"], now["gf"], now["gb"], out[0], 16.0)
+        vig.vig_gate_prep_bf16(now["gf"], now["gb"], la[0], la[1], 16.0)
+        counted(vig.vig_bigla_fwd_bf16, now["q"], now["k"], now["v"], la[0], la[1], out[1])
+        counted(vig.vig_bigla_bwd, now["q"], now["k"], now["v"], la[0], la[1], now["g"], *out[2:])
+        return out
+
+    empty = lambda: [torch.empty_like(now[n]) for n in names]
+    alone = []
+    for s in sets:
+        for n in now:
+            now[n].copy_(s[n])
+        torch.cuda.synchronize()
+        vig.vig_test_take_fallback_count()
+        alone.append(step(empty()))
+        assert vig.vig_test_take_fallback_count() == (3 if s is sets[1] else 0)
+    outs = [[empty() for _ in sets] for _ in range(6)]
+    for rep in outs:
+        for s, keep in zip(sets, rep):
+            for n in now:
+                now[n].copy_(s[n])
+            step(keep)
+    torch.cuda.synchronize()
+    assert vig.vig_last_device_status() == 0
+    for rep in outs:
+        for got, want in zip(rep, alone):
+            assert all(torch.equal(a.view(torch.int16), b.view(torch.int16)) for a, b in zip(got, want))
+
+
 def _gradient_call(L):
     cfg, x = random_problem(4800 + L, 2, 2, L, 24, 48, "bf16", gate_mean=1.0)
     d = {n: to_device(a, "bf16") for n, a in x.items()}
