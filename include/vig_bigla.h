@@ -69,7 +69,8 @@ typedef enum vig_dtype { VIG_DTYPE_F32 = 0, VIG_DTYPE_BF16 = 1 } vig_dtype;
  * Longer ones are cut into chunks of up to 128 tokens that are the blocks of one cluster (one launch, up to 1024 tokens, no scratch),
  * into 256-token segments (one launch; the blocks of a unit exchange segment
  * summaries through scratch) or into 128-token chunk tasks (three launches; chunk summaries and
- * boundary states go through scratch), whichever suits the shape.  The library allocates and frees
+ * boundary states go through scratch, 8 dk dv + 128 dv + 260 bytes a chunk on the warp-level kernels: 122 bytes a token and head at
+ * 24 x 48), whichever suits the shape.  The library allocates and frees
  * that scratch on `stream` from a stream-ordered memory pool of its own (one per device, which keeps
  * freed memory for later calls instead of returning it to the driver); use the *_ws form to supply it.  The kernels are
  * launched with programmatic stream serialization: none reads anything before the work in front of the call
@@ -144,8 +145,10 @@ int vig_gate_prep_f32(const void* g_fwd, const void* g_bwd,
  * Units of at most 256 tokens with dk in {16,24,32}, dv in {32,48,64} run in one kernel that turns each gate
  * tile into log alpha in shared memory (fp32 evaluation with exp and log from the special-function unit,
  * rounded to bf16 as the tensor-core operand of the prefix sums: the same rounding point as the un-fused
- * chain).  Longer sequences and other head sizes run gate preparation into scratch the library allocates and
- * frees on `stream` (its memory pool), then the ordinary forward pass.
+ * chain).  Longer sequences prepare the gates on the way as well where they run as the chunks of a cluster (no scratch) or in
+ * three launches over chunks on the warp-level kernels (scratch as above; calls that fill the GPU at most four times are cut into
+ * chunks of 80 to 128 tokens, so up to 1.6 times that).  Everything else runs gate preparation into scratch the library allocates
+ * and frees on `stream` (its memory pool), then the ordinary forward pass.
  * Errors: NULL_POINTER, BAD_DIM (also tau), UNSUPPORTED, MISALIGNED, CUDA. */
 int vig_bigla_fwd_gates_bf16(const void* q, const void* k, const void* v,
                              const void* g_fwd, const void* g_bwd, void* out,

@@ -46,14 +46,12 @@ struct MArgs {
     const __nv_bfloat16 *q, *k, *v, *la_f, *la_b;   // GATES: la_f / la_b hold the gate logits
     __nv_bfloat16* out;
     int L;
-    long long blocks;  // units (kUnit) or units x chunks
+    long long units, blocks;   // blocks: units (kUnit) or units x chunks
     int nch, tiles;    // chunks per unit, tiles per chunk (long sequences)
     float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
     uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
     float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
     int* flags;        // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
-    uint8_t* keys;     // GATES: [unit][chunk][k~>, k~<][rows][64 B]: the scaled keys of a chunk, as shared-memory tiles
-    __nv_bfloat16 *la2_f, *la2_b;   // GATES: log2 alpha as prepared by the summary launch
     int* dev_status;
     float inv_tau;
     int ahead;         // the block this many further on has its inputs pulled into L2
@@ -94,9 +92,6 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     constexpr int RV = MLayout<DV>::kVRow;
     constexpr uint32_t kState = MLayout<DV>::kState;
     constexpr bool kTwo = MODE == kUnit && MAXT > 8;   // units of two chunks
-    // From logits, the summary launch leaves the prepared gates and the scaled keys behind for the chunks' launch (the keys by one
-    // bulk copy of its tiles), which would spend a third of its instructions on doing both again.
-    constexpr bool kGiveKeys = GATES && MODE == kSummary, kTakeKeys = GATES && MODE == kMain;
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, lane = tid & 31, w = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int g = lane >> 2, c = lane & 3;
@@ -139,8 +134,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         pdl_launch_dependents();
     }
     if (tid == 0) {
-        mbar_expect_tx(bar, (uint32_t)tiles * (16 * RV + (kTakeKeys ? 2048 : 0)));
-        if (kTakeKeys) bulk_load(tkf, args.keys + (size_t)blockIdx.x * tiles * 2048, tiles * 2048, bar);
+        mbar_expect_tx(bar, (uint32_t)tiles * 16 * RV);
         tma_load_3d(tv, &tm_v, 0, tok0, (int)unit, bar);   // rows >= L and columns >= DV arrive as zeros
         if (MODE == kCluster) mbar_expect_tx(bar + 8, (nch - 1) * (DV * DK * 4 + DK * 4 + 4));
     }
@@ -152,15 +146,15 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         const int row = tok0 + w * 16 + 8 * r + g;
         if (live && row < L) {
             const size_t at = (unit * L + row) * DK;
-            load_pairs<DK, MODE == kMain>((kTakeKeys ? args.la2_f : args.la_f) + at, c, af[r]);
-            load_pairs<DK, MODE == kMain>((kTakeKeys ? args.la2_b : args.la_b) + at, c, ab[r]);
-            if (!kTakeKeys) load_pairs<DK, MODE == kMain>(args.k + at, c, kr[r]);
+            load_pairs<DK, MODE == kMain>(args.la_f + at, c, af[r]);
+            load_pairs<DK, MODE == kMain>(args.la_b + at, c, ab[r]);
+            load_pairs<DK, MODE == kMain>(args.k + at, c, kr[r]);
             if (MODE != kSummary) load_pairs<DK, MODE == kMain>(args.q + at, c, qr[r]);
         } else {
 #pragma unroll
             for (int j = 0; j < NP; ++j) {   // rows past the end: q = k = 0 and no decay (GATES: a logit of 100, log alpha = 0)
                 qr[r][j] = kr[r][j] = 0u;
-                af[r][j] = ab[r][j] = GATES && !kTakeKeys ? 0x42C842C8u : 0u;
+                af[r][j] = ab[r][j] = GATES ? 0x42C842C8u : 0u;
             }
         }
     }
@@ -174,20 +168,9 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     for (int j = 0; j < NP; ++j) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-            if (GATES && !kTakeKeys) {
+            if (GATES) {
                 af[r][j] = log2_alpha_pair<MODE != kUnit>(af[r][j], args.inv_tau);
                 ab[r][j] = log2_alpha_pair<MODE != kUnit>(ab[r][j], args.inv_tau);
-            }
-        }
-    }
-    if (kGiveKeys) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int row = tok0 + w * 16 + 8 * r + g;
-            if (live && row < L) {
-                const size_t at = (unit * L + row) * DK;
-                store_pairs<DK>(args.la2_f + at, c, af[r]);
-                store_pairs<DK>(args.la2_b + at, c, ab[r]);
             }
         }
     }
@@ -267,11 +250,9 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                             // Factor and product in fp32, one rounding: what the packed reciprocals are low by on average would
                             // pass into the states and on from chunk to chunk (with them 32 x 4096 tokens, gate logits around 4,
                             // were 4.8e-3 off in 2-norm, the tcgen05 forms 4.5e-3; this way 3.3e-3 in the same time).
-                            if (!kTakeKeys) {
-                                const f32x2 k2 = widen(kr[r][j]);
-                                kfw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(-b0), ex2(-b1))));
-                                kbw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(x0), ex2(x1))));
-                            }
+                            const f32x2 k2 = widen(kr[r][j]);
+                            kfw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(-b0), ex2(-b1))));
+                            kbw[2 * jj + r] = pack_f32x2(fmul2(k2, pack2(ex2(x0), ex2(x1))));
                             if (MODE != kSummary) {
                                 const f32x2 q2 = fmul2(widen(qr[r][j]), pack2(0.5f, 0.5f));   // the 1/2 of the result
                                 qf[m][2 * jj + r] = pack_f32x2(fmul2(q2, pack2(ex2(b0), ex2(b1))));
@@ -284,13 +265,10 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                     for (int r = 0; r < 2; ++r) kfw[2 + r] = kbw[2 + r] = qf[m][2 + r] = qb[m][2 + r] = 0u;
                 }
             }
-            if (!kTakeKeys) {
-                t64.store(tkf, 16 * w, m, kfw[0], kfw[1], kfw[2], kfw[3]);
-                t64.store(tkb, 16 * w, m, kbw[0], kbw[1], kbw[2], kbw[3]);
-            }
+            t64.store(tkf, 16 * w, m, kfw[0], kfw[1], kfw[2], kfw[3]);
+            t64.store(tkb, 16 * w, m, kbw[0], kbw[1], kbw[2], kbw[3]);
         }
     }
-    if (kGiveKeys) fence_async_smem();   // (the tiles, for the bulk copy)
     bool ok = true;
     if (args.expire_wait && tid == 0) ok = mbar_wait_bounded(bar + 16, 0, 64);   // test hook: this wait cannot succeed
     ok = mbar_wait_bounded(bar, 0) && ok;
@@ -303,7 +281,6 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
         return;
     }
-    if (kGiveKeys && tid == 0) bulk_store(args.keys + (size_t)blockIdx.x * tiles * 2048, tkf, tiles * 2048);
     if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
         float s = 0.f;
         for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
@@ -416,10 +393,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
             __syncwarp();
             if (kTwo && lane == 0) mbar_arrive(bar + 8);
         }
-        if (MODE == kSummary) {
-            if (kGiveKeys && tid == 0) bulk_store_wait();   // (the tiles must outlast the copy)
-            return;
-        }
+        if (MODE == kSummary) return;
     }
     if (MODE == kCluster && w == 0) {   // the decay across this chunk, and whether anything is wrong here
         const int word = (*slow ? 1 : 0) | (ok ? 0 : 2);
@@ -642,7 +616,7 @@ template <int DK, int DV, bool GATES>
 cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
     const int T = (a.L + 15) / 16;
     CUtensorMap tv;
-    if (!make_map(&tv, a.v, a.blocks, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
+    if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
     if (T <= 8) return launch_mma_t<DK, DV, GATES, 8, kUnit>(a, tv, T, stream);
     if (T <= 13) return launch_mma_t<DK, DV, GATES, 13, kUnit>(a, tv, T, stream);
     return launch_mma_t<DK, DV, GATES, 16, kUnit>(a, tv, T, stream);
@@ -664,11 +638,12 @@ static int device_sms() {
 // Sequences of any length: chunks of equal numbers of tiles, up to eight.  From logits, beyond eight chunks, the tiles are what makes
 // the rounds of blocks cheapest, a block's time being about that of its loads and hand-overs (eight tiles' worth) and of its tiles, short
 // of the 128 chunks up to which the fold keeps its runs short.  6 x 4 units of 1300 tokens, 24 x 64: 17.8 us a call, 20.6 with
-// eight tiles; 3 x 3 of 5000, 24 x 32: 16.4 and 18.3; 8 x 4 of 4096, 24 x 48: 37.4 and 37.8.  (From log gates the scratch may be the caller's,
-// whose size this keeps.)
+// eight tiles; 3 x 3 of 5000, 24 x 32: 16.4 and 18.3; 8 x 4 of 4096, 24 x 48: 37.4 and 37.8.  Beyond four rounds
+// the last one weighs little, and the scratch, which grows with the number of chunks, stays that of eight tiles (84 units of 4096,
+// 24 x 64: 113.7 us cut by rounds, 110.5 this way).  (From log gates the scratch may be the caller's, whose size this keeps.)
 struct ChunkPlan {
     int nch, tiles;
-    size_t u, img, decay, flags, keys, la2, la2_bytes, total;   // byte offsets in the scratch
+    size_t u, img, decay, flags, total;   // byte offsets in the scratch
 };
 ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false) {
     ChunkPlan p;
@@ -680,7 +655,7 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false)
     };
     cut(kChunkTiles);
     const long long slots = (long long)mma_blocks_per_sm(dk, dv, kChunkTiles, kMain) * device_sms();
-    if (gates && p.nch > kChunkTiles && slots > 0) {
+    if (gates && p.nch > kChunkTiles && form_units(units) * p.nch <= 4 * slots) {
         int best = p.tiles;
         long long best_cost = -1;
         for (int tiles = kChunkTiles; tiles >= 5; --tiles) {
@@ -695,32 +670,27 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false)
     p.img = n * 2 * dk * dv * 4;
     p.decay = p.img + n * 2 * dv * 64;
     p.flags = p.decay + n * 64 * 4;
-    p.keys = p.la2 = p.total = (p.flags + n * 4 + 255) / 256 * 256;
-    p.la2_bytes = ((size_t)units * L * dk * 2 + 255) / 256 * 256;
-    if (gates) {
-        p.la2 = p.keys + n * p.tiles * 2048;
-        p.total = p.la2 + 2 * p.la2_bytes;
-    }
+    p.total = (p.flags + n * 4 + 255) / 256 * 256;
     return p;
 }
 
 // One launch: the chunks of a unit are the blocks of a cluster.
 template <int DK, int DV, bool GATES>
-cudaError_t launch_cluster(MArgs a, long long units, cudaStream_t stream) {
+cudaError_t launch_cluster(MArgs a, cudaStream_t stream) {
     CUtensorMap tv;
-    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
+    if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     return launch_mma_t<DK, DV, GATES, 8, kCluster>(a, tv, a.tiles, stream);
 }
 
 template <int DK, int DV, bool GATES>
-cudaError_t launch_chunks(MArgs a, long long units, cudaStream_t stream) {
+cudaError_t launch_chunks(MArgs a, cudaStream_t stream) {
     CUtensorMap tv;
-    if (!make_map(&tv, a.v, units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
+    if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
     if (e != cudaSuccess) return e;
     e = with_fold_plan(a.nch, [&](auto groups, auto run) {
         constexpr int kGroups = decltype(groups)::value, kItems = kFoldThreads / kGroups;
-        return launch_pdl(mma_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)units, 2, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
+        return launch_pdl(mma_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)a.units, 2, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
     });
     count_launch();
     if (e != cudaSuccess) return e;
@@ -749,7 +719,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
                              int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
     MArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
-    a.L = L; a.blocks = units;
+    a.L = L; a.units = a.blocks = units;
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
@@ -821,21 +791,18 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
     char* b = static_cast<char*>(ws);
     MArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
-    a.L = L; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
+    a.L = L; a.units = units; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
     a.u = reinterpret_cast<float*>(b + p.u);
     a.img = reinterpret_cast<uint8_t*>(b + p.img);
     a.decay = reinterpret_cast<float*>(b + p.decay);
     a.flags = reinterpret_cast<int*>(b + p.flags);
-    a.keys = reinterpret_cast<uint8_t*>(b + p.keys);
-    a.la2_f = reinterpret_cast<__nv_bfloat16*>(b + p.la2);
-    a.la2_b = reinterpret_cast<__nv_bfloat16*>(b + p.la2 + p.la2_bytes);
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_)        \
     if (dk == DK_ && dv == DV_) \
-        return gate_tau > 0.f ? launch_chunks<DK_, DV_, true>(a, units, stream) : launch_chunks<DK_, DV_, false>(a, units, stream);
+        return gate_tau > 0.f ? launch_chunks<DK_, DV_, true>(a, stream) : launch_chunks<DK_, DV_, false>(a, stream);
     VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
     VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
     VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)
@@ -849,14 +816,14 @@ cudaError_t launch_bigla_mma_cluster(const __nv_bfloat16* q, const __nv_bfloat16
     const ChunkPlan p = chunk_plan(units, L, dk, dv);
     MArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
-    a.L = L; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
+    a.L = L; a.units = units; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
     if (!a.dev_status) return cudaErrorUnknown;
 #define VIG_CASE(DK_, DV_)        \
     if (dk == DK_ && dv == DV_) \
-        return gate_tau > 0.f ? launch_cluster<DK_, DV_, true>(a, units, stream) : launch_cluster<DK_, DV_, false>(a, units, stream);
+        return gate_tau > 0.f ? launch_cluster<DK_, DV_, true>(a, stream) : launch_cluster<DK_, DV_, false>(a, stream);
     VIG_CASE(16, 32) VIG_CASE(16, 48) VIG_CASE(16, 64)
     VIG_CASE(24, 32) VIG_CASE(24, 48) VIG_CASE(24, 64)
     VIG_CASE(32, 32) VIG_CASE(32, 48) VIG_CASE(32, 64)

@@ -189,18 +189,6 @@ __device__ __forceinline__ void load_pairs(const __nv_bfloat16* row, int c, uint
     }
 }
 
-// ... and back to a row of the same order
-template <int DK>
-__device__ __forceinline__ void store_pairs(__nv_bfloat16* row, int c, const uint32_t (&r)[DK / 8]) {
-    char* p = reinterpret_cast<char*>(row);
-    if constexpr (DK == 32) {
-        *reinterpret_cast<uint4*>(p + 16 * c) = make_uint4(r[0], r[1], r[2], r[3]);
-    } else {
-        *reinterpret_cast<uint2*>(p + 8 * c) = make_uint2(r[0], r[1]);
-        if constexpr (DK == 24) *reinterpret_cast<uint32_t*>(p + 32 + 4 * c) = r[2];
-    }
-}
-
 // Lane c of a group of four holds words (c, 0 .. 3); afterwards words (0 .. 3, c).
 __device__ __forceinline__ void transpose4(uint32_t (&x)[4], int c) {
 #pragma unroll

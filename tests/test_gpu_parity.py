@@ -4,6 +4,8 @@ for bf16 storage, the maximum taken over the whole output tensor."""
 import ctypes
 import mmap
 import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -630,6 +632,30 @@ def test_host_memory_is_touched_by_kernels_only_where_all_of_it_is_mapped():
     assert not usable(0, 4)
     pinned = torch.empty(1 << 20, dtype=torch.uint8, pin_memory=True)
     assert vig.vig_test_host_copy_usable(pinned.data_ptr(), pinned.numel())
+
+
+def test_scratch_of_a_long_call_from_logits_is_that_from_log_gates():
+    """Scratch of chunk states alone, no copies of gates or keys: what the library's pool takes for a call from logits, in a process
+    of its own (the pool keeps what it has), is what vig_bigla_workspace_bytes gives for the shape, to the pool's granularity."""
+    code = """
+import torch, paper_2405_18425_b200 as vig
+mk = lambda L, u, d: torch.zeros(u, 1, L, d, device="cuda", dtype=torch.bfloat16)
+def call(L, u):
+    q, v, out = mk(L, u, 24), mk(L, u, 48), mk(L, u, 48)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    vig.vig_bigla_fwd_gates_bf16(q, q, v, q, q, out, 16.0)
+    torch.cuda.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+call(300, 1)
+print("TAKEN", call(16384, 64), vig.vig_bigla_workspace_bytes(64, 1, 16384, 24, 48))
+"""
+    p = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert p.returncode == 0, p.stderr[-2000:]
+    taken, stated = (int(x) for x in p.stdout.split("TAKEN")[1].split())
+    assert stated > 100 << 20                      # 8192 chunks
+    assert taken <= stated + (66 << 20), (taken, stated)
 
 
 def test_workspace_variant_and_determinism(oracle):
