@@ -68,7 +68,7 @@ cudaError_t launch_scan_fwd(const T* q, const T* k, const T* v, const T* la_f, c
     // Few sequences, blocks with an SM each: sixteen warps (training step of 24 units of 196 tokens, 16 x 64, fp32: 42.1 us, 56.3 with eight).
 #define VIG_MANY(RPL_) \
     if (dk <= 4 * RPL_) return launch_scan_t<T, RPL_, true, 2, kManyWarps>(a, units, stream);
-    if (vec && dk <= 32 && blocks(2) <= sms) {
+    if (vec && dk <= 32 && blocks(2) <= sms && L <= kManyTokens) {
         VIG_MANY(4) VIG_MANY(8)
     }
 #undef VIG_MANY

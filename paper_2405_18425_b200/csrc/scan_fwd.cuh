@@ -31,7 +31,10 @@ struct ScanArgs {
 
 constexpr int scan_max_warps(int rpl) { return rpl <= 16 ? 8 : 1; }   // segments per block (32 rows a lane: no registers for the first pass)
 // Segments of calls whose blocks have an SM each: twice as many, of twelve tokens at least (a segment costs every other one a fold step).
-constexpr int kManyWarps = 16;
+// Up to 1200 tokens: beyond that they are less exact (error against 64 bits, sixteen to eight, gate logits around -1 / 0 / 2:
+// 1.00 / 1.00 / 0.98 at 1200 tokens, 1.013 / 1.003 / 0.99 at 2048, 1.02 / 1.01 / 0.99 at 3000), if faster (training step of 12 units of
+// 1100, 24 x 48: 258 us, 326 with eight).
+constexpr int kManyWarps = 16, kManyTokens = 1200;
 inline int many_segments(int L) { return L / 12 < 8 ? 8 : (L / 12 < kManyWarps ? L / 12 : kManyWarps); }
 constexpr size_t scan_stage_floats(int rpl, int cpl = 2) { return (size_t)TG * (3 * 4 * rpl + 8 * cpl); }
 constexpr size_t scan_fold_floats(int rpl, int cpl = 2) { return (size_t)2 * 4 * rpl * (8 * cpl + 1); }

@@ -658,6 +658,24 @@ print("TAKEN", call(16384, 64), vig.vig_bigla_workspace_bytes(64, 1, 16384, 24, 
     assert taken <= stated + (66 << 20), (taken, stated)
 
 
+@pytest.mark.parametrize("L", [1201, 1500, 3000])
+def test_long_fp32_walks_of_few_units_have_eight_segments(L):
+    """Beyond 1200 tokens a call of few units cuts its sequences as one of many does (more segments would be less exact): a unit has
+    the same bits in both."""
+    many = torch.cuda.get_device_properties(0).multi_processor_count + 1     # two blocks a unit: eight segments each
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda d: torch.randn(many, 1, L, d, device="cuda", generator=gen)
+    q, k, v = mk(16) * 0.25, mk(16), mk(32)
+    la = [torch.nn.functional.logsigmoid(mk(16)) / 16 for _ in range(2)]
+    outs = []
+    for units in (2, many):
+        a = [t[:units].contiguous() for t in (q, k, v, *la)]
+        outs.append(torch.empty_like(a[2]))
+        vig.vig_bigla_fwd_f32(*a, outs[-1])
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0].view(torch.int32), outs[1][:2].view(torch.int32))
+
+
 def test_workspace_variant_and_determinism(oracle):
     cfg = synth.CONFIGS[4]
     x = synth.make_inputs(cfg, units=slice(0, 6))
