@@ -108,10 +108,11 @@ def test_bf16_random_shapes_repeatable(oracle, case):
     assert rel_err(got, oracle_out(oracle, x["q"], x["k"], x["v"], la_f, la_b, cfg.dtype)) <= TOL["bf16"]
 
 
-@pytest.mark.parametrize("L", [196, 700])
-def test_cuda_graph_replay(L):
-    """Gate preparation + forward captured into a CUDA graph (the programmatic dependent launches included; the long
-    path with caller-owned scratch, so that nothing allocates during capture) and replayed: same bits as the direct calls."""
+@pytest.mark.parametrize("L,launches", [(196, 1), (700, 1), (2100, 3)])
+def test_cuda_graph_replay(L, launches):
+    """Gate preparation + forward captured into a CUDA graph (the programmatic dependent launches included; caller-owned
+    scratch, so that nothing allocates during capture) and replayed: same bits as the direct calls.  A block a unit, the
+    chunks of a unit as a cluster, and chunks in three launches."""
     B, H, dk, dv = 4, 6, 32, 64
     gen = torch.Generator(device="cuda").manual_seed(77 + L)
     def mk(d):
@@ -120,7 +121,9 @@ def test_cuda_graph_replay(L):
     lf, lb, ref = torch.empty_like(gf), torch.empty_like(gb), torch.empty_like(v)
     ws = torch.empty(max(vig.vig_bigla_workspace_bytes(B, H, L, dk, dv), 256), dtype=torch.uint8, device="cuda")
     vig.vig_gate_prep_bf16(gf, gb, lf, lb, 16.0)
+    before = vig.vig_kernel_launch_count()
     vig.vig_bigla_fwd_ws_bf16(q, k, v, lf, lb, ref, ws)     # also the first call per device: one-time set-up before capture
+    assert vig.vig_kernel_launch_count() - before == launches
     torch.cuda.synchronize()
     out = torch.zeros_like(v)
     s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
@@ -137,16 +140,19 @@ def test_cuda_graph_replay(L):
 
 
 def test_two_streams_interleaved(oracle):
-    """Calls of different shapes issued alternately on two streams (the long path allocates its scratch per call
-    on the stream it is given): every result equals, bit for bit, the one the same call gives on its own."""
+    """Calls of different shapes issued alternately on two streams (those of three launches allocate their scratch per call
+    on the stream they are given): every result equals, bit for bit, the one the same call gives on its own."""
     problems = []
-    for i, (B, H, L, dk, dv) in enumerate([(3, 4, 196, 32, 64), (1, 3, 1000, 24, 48), (40, 5, 130, 16, 32), (2, 2, 600, 32, 64)]):
+    for i, (B, H, L, dk, dv, launches) in enumerate([(3, 4, 196, 32, 64, 1), (1, 3, 1000, 24, 48, 1), (40, 5, 130, 16, 32, 1), (2, 2, 600, 32, 64, 1),
+                                                     (1, 4, 1300, 24, 48, 3), (3, 2, 2100, 32, 32, 3), (1, 9, 3000, 24, 32, 3)]):
         cfg, x = random_problem(9500 + i, B, H, L, dk, dv, "bf16", gate_mean=1.0)
         la_f = oracle_log_alpha(oracle, x["g_fwd"], cfg.dtype, cfg.tau)
         la_b = oracle_log_alpha(oracle, x["g_bwd"], cfg.dtype, cfg.tau)
         d = {n: to_device(a, cfg.dtype) for n, a in dict(q=x["q"], k=x["k"], v=x["v"], f=la_f, b=la_b).items()}
         alone = torch.empty_like(d["v"])
+        before = vig.vig_kernel_launch_count()
         vig.vig_bigla_fwd_bf16(d["q"], d["k"], d["v"], d["f"], d["b"], alone)
+        assert vig.vig_kernel_launch_count() - before == launches
         problems.append((d, alone))
     torch.cuda.synchronize()
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
