@@ -203,8 +203,9 @@ def test_f32_walks_in_segments(oracle, units, L, dk, dv):
 
 @pytest.mark.parametrize("units,L", [(3, 100), (200, 196), (4, 700)])
 def test_chain_of_dependent_launches_sees_what_the_last_one_wrote(units, L):
-    """Gate preparation, forward and gradient back to back on the same buffers, the contents changing from pass to pass: each
-    kernel starts while the one before it, which writes its inputs, may still be running."""
+    """Gate preparation, forward (one launch: a block a unit, or a cluster) and gradient (one launch, or three) back to back on the
+    same buffers, the contents changing from pass to pass: each kernel starts while the one before it, which writes its inputs, may
+    still be running.  Forward passes of three launches: the test below."""
     rng = torch.Generator(device="cuda").manual_seed(L)
     mk = lambda d: torch.randn(1, units, L, d, generator=rng, device="cuda").bfloat16()
     sets = [dict(q=mk(24) * 24 ** -0.5, k=mk(24), v=mk(48), gf=mk(24), gb=mk(24), g=mk(48)) for _ in range(3)]
@@ -329,8 +330,8 @@ def test_pair_whose_exchange_expires_stores_no_gate_gradients():
 
 @pytest.mark.parametrize("units,L,dk,dv", [(1, 13, 4, 4), (3, 97, 12, 20), (12, 400, 24, 48), (2, 784, 32, 64), (2, 2047, 16, 32), (47, 61, 32, 64), (60, 30, 32, 32)])
 def test_fp32_walks_of_few_and_of_more_units(oracle, units, L, dk, dv):
-    """Sixteen warps a block where every block has an SM of its own, three and four columns a lane, ragged last segments; forward and
-    gradient, the latter with dv in the same launch below 512 tokens."""
+    """Sixteen warps a block where every block has an SM of its own, blocks with two columns a lane otherwise, ragged last segments;
+    forward and gradient, the latter with dv in the same launch below 512 tokens."""
     cfg, x = random_problem(4100 + L, units, 1, L, dk, dv, "f32", gate_mean=1.0)
     la = [oracle_log_alpha(oracle, x[n], "f32", cfg.tau) for n in ("g_fwd", "g_bwd")]
     d = {n: to_device(a, "f32") for n, a in dict(q=x["q"], k=x["k"], v=x["v"], f=la[0], b=la[1]).items()}
@@ -346,3 +347,23 @@ def test_fp32_walks_of_few_and_of_more_units(oracle, units, L, dk, dv):
     ref = oracle.bigla_bwd(f64(x["q"]), f64(x["k"]), f64(x["v"]), f64(la[0]), f64(la[1]), f64(g))
     for t, r in zip(grads, ref):
         assert rel_err(device_to_f64(t, "f32"), r) <= TOL["f32"]
+
+
+@pytest.mark.parametrize("cpl,L,dk,dv,dtype", [(4, 61, 32, 64, "f32"), (4, 97, 16, 64, "f32"), (4, 30, 32, 32, "f32"), (4, 50, 24, 128, "f32"),
+                                               (4, 45, 8, 64, "bf16"), (4, 33, 20, 28, "bf16"), (3, 61, 32, 64, "f32"), (3, 50, 16, 48, "f32"),
+                                               (3, 41, 12, 20, "f32"), (3, 37, 28, 40, "bf16")])
+def test_forward_walks_of_three_and_four_columns_a_lane(oracle, cpl, L, dk, dv, dtype):
+    """As many units as give every SM one block at this width and more than one at any smaller, widths of whole slabs and ragged ones."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    slabs = lambda x: -(-dv // (8 * x))
+    units = sms // slabs(cpl)
+    assert units * slabs(cpl) <= sms and all(units * slabs(x) > sms for x in range(2, cpl))
+    cfg, x = random_problem(4900 + L, units, 1, L, dk, dv, dtype, gate_mean=1.0)
+    la = [oracle_log_alpha(oracle, x[n], dtype, cfg.tau) for n in ("g_fwd", "g_bwd")]
+    d = [to_device(a, dtype) for a in (x["q"], x["k"], x["v"], *la)]
+    out = torch.full_like(d[2], float("nan"))
+    (vig.vig_bigla_fwd_f32 if dtype == "f32" else vig.vig_bigla_fwd_bf16)(*d, out)
+    torch.cuda.synchronize()
+    got = device_to_f64(out, dtype)
+    assert np.isfinite(got).all()
+    assert rel_err(got, oracle_out(oracle, x["q"], x["k"], x["v"], la[0], la[1], dtype)) <= TOL[dtype]
