@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                 if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
                 return;
             }
-            if (chunk != 0) return;
+            if (chunk != (int)(unit % (unsigned)nch)) return;   // (the first blocks of clusters share SMs)
             if (tid == 0) atomicAdd(args.dev_status + 1, 1);
             __syncthreads();
             const size_t okk = unit * L * DK, ov = unit * L * DV;
