@@ -65,7 +65,7 @@ typedef enum vig_dtype { VIG_DTYPE_F32 = 0, VIG_DTYPE_BF16 = 1 } vig_dtype;
  *       by more than e^-60 inside one chunk of 128 tokens is computed by an in-kernel fp32
  *       recurrence (Eq. 6 step by step) instead of the factorised tiles.
  * f32:  dk <= 128, dv <= 256; fp32 walks on the CUDA cores, a sequence cut into segments that run side by side.
- * Sequences of at most 256 tokens run in one launch with a unit per thread block and use no scratch.
+ * Sequences of at most 256 tokens run in one launch with a unit per thread block (or per cluster of two) and use no scratch.
  * Longer ones are cut into chunks of up to 128 tokens that are the blocks of one cluster (one launch, up to 1024 tokens, no scratch),
  * into 256-token segments (one launch; the blocks of a unit exchange segment
  * summaries through scratch) or into 128-token chunk tasks (three launches; chunk summaries and
@@ -87,8 +87,9 @@ int vig_bigla_fwd(const void* q, const void* k, const void* v,
                   const void* log_alpha_fwd, const void* log_alpha_bwd, void* out,
                   int B, int H, int L, int dk, int dv, void* stream);
 
-/* Bytes of device scratch a vig_bigla_fwd_* call of this shape needs (0 when the whole sequence
- * of a unit is handled by one thread block).  Returns 0 for invalid or unsupported shapes too. */
+/* Bytes of device scratch a vig_bigla_fwd_* call from log gates of this shape asks for (0 up to 256 tokens).  An upper
+ * bound: a call whose chunks run as one cluster asks for the scratch of the other forms and leaves it untouched.
+ * Returns 0 for invalid or unsupported shapes too. */
 size_t vig_bigla_workspace_bytes(int B, int H, int L, int dk, int dv, int dtype);
 /* vig_bigla_fwd_bf16 with caller-owned scratch: `ws` is a 256-byte aligned device buffer of at
  * least vig_bigla_workspace_bytes(...) bytes (may be NULL when that is 0).  Nothing is allocated.

@@ -1,5 +1,6 @@
 // bf16 BiGLA forward on the warp-level tensor-core instructions (mma.sync): one warp per 16 tokens, every product a chain of
-// 16 x 16 tiles whose scores stay in registers.  Units of at most 256 tokens are one block each; longer sequences are cut
+// 16 x 16 tiles whose scores stay in registers.  Units of at most 256 tokens are one block each (a cluster of two, large
+// states of few units); longer sequences are cut
 // into chunks of up to 128 tokens, one block each.  Up to eight chunks (1024 tokens): one launch, a cluster of blocks per unit, each of
 // which gives the others the state it adds through distributed shared memory.  Any length: three launches, the state every chunk adds in
 // either direction, a fold over the chunks, the chunks themselves from the states that enter them.
@@ -80,7 +81,8 @@ constexpr uint32_t slot_bytes(int dk, int dv) { return dv * dk * 4u + 144u; }   
 constexpr uint32_t all_slots(int dk, int dv, int nch) { return (nch - 1) * slot_bytes(dk, dv) + 128u; }
 
 // Blocks per SM the registers are held to (64 registers a thread for four: 19 us against 15 where the state is large, units of one block,
-// 768 of 100 tokens, 32 x 64; chunks of small states gain, 2 x 4 units of 16384 tokens, 24 x 48: 39.8 to 38.5).
+// 768 of 100 tokens, 32 x 64; chunks of small states gain, 2 x 4 units of 16384 tokens, 24 x 48: 39.8 to 38.5, though at 24 x 48 and
+// 32 x 32 some 50 bytes a thread go to the stack; from five chunks on the slots of a cluster leave room for three blocks only).
 constexpr int mma_blocks_per_sm(int dk, int dv, int max_tiles, int mode) {
     return max_tiles > 8 ? 2 : (mode != kUnit && dk * dv <= 1152 ? 4 : 3);
 }
@@ -114,18 +116,16 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         *slow = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    auto pull = [&](size_t at, uint32_t n, bool rest, bool q) {   // n tokens from `at` into L2
-        if (rest) {
-            prefetch_l2(args.la_f + at * DK, n * DK * 2);
-            prefetch_l2(args.la_b + at * DK, n * DK * 2);
-            prefetch_l2(args.k + at * DK, n * DK * 2);
-            prefetch_l2(args.v + at * DV, n * DV * 2);
-        }
-        if (q) prefetch_l2(args.q + at * DK, n * DK * 2);
+    auto pull = [&](size_t at, uint32_t n) {   // n tokens from `at` into L2
+        prefetch_l2(args.la_f + at * DK, n * DK * 2);
+        prefetch_l2(args.la_b + at * DK, n * DK * 2);
+        prefetch_l2(args.k + at * DK, n * DK * 2);
+        prefetch_l2(args.v + at * DV, n * DV * 2);
+        prefetch_l2(args.q + at * DK, n * DK * 2);
     };
     // A block that is let in while the launch before still runs has its tokens brought to L2 meanwhile (a prefetch consumes nothing,
     // and L2 stays coherent with what that launch still writes); the blocks after the first round are pulled in by those of it.
-    if (MODE != kMain && tid == 32 && (int)blockIdx.x < args.ahead) pull(unit * L + tok0, min(tiles * 16, L - tok0), true, true);
+    if (MODE != kMain && tid == 32 && (int)blockIdx.x < args.ahead) pull(unit * L + tok0, min(tiles * 16, L - tok0));
     // The chunks' launch starts under the fold: that one lets it in only behind its own wait, when the summaries are complete, and
     // with them all that was launched before.  So inputs and flags are read at once, from L2 (see pdl_wait), and only what the fold
     // writes is waited for.
@@ -161,7 +161,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
     if (MODE != kMain && tid == 0 && blockIdx.x + (long long)args.ahead < args.blocks) {   // a block that starts when one of these is done finds its inputs in L2
         const size_t next = blockIdx.x + (size_t)args.ahead;
         const int nr = MODE == kUnit ? 0 : (int)(next % (unsigned)nch) * tiles * 16;
-        pull((MODE == kUnit ? next : next / (unsigned)nch) * L + nr, min(tiles * 16, L - nr), true, true);   // (q: of the chunks' launch as well)
+        pull((MODE == kUnit ? next : next / (unsigned)nch) * L + nr, min(tiles * 16, L - nr));   // (q: for the chunks' launch as well)
     }
     // ---- gate totals of the tile; the gates turned, as B operands of products over the tokens ----
 #pragma unroll
@@ -740,7 +740,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
 // resident in one round; beyond that round it is at its worst (300 units of 304 tokens, 32 x 64, from logits: 52.7 us, 43.7 this way).
 // More than 64 chunks: the tasks' fold takes one run.  Timed against the tcgen05 forms for six head sizes, 1100 to 16384 tokens,
 // 1 to 96 units, with and without the gates (468 shapes; 1530 more up to 512 tokens before clusters took most of them): within 0.2 %
-// of the better form on average.
+// of the better form on average.  For the calls that clusters take, this only says what scratch a caller is asked for, as before them.
 bool mma_chunks_preferred(long long units, int L, int dk, int dv, bool gates) {
     if (dk == 16) return true;
     const long long sms = device_sms();

@@ -3,7 +3,8 @@
 //
 // A thread takes four key dimensions of one value column over a run of chunks, GROUPS runs side by side: what a run adds and by how
 // much it decays, then the carry of the runs before it, then the states.  A run of up to RUN chunks is read once and kept in
-// registers, a longer one twice, a batch at a time.  What bounds the launch is how many of its loads are in flight; and until its last
+// registers (but for 20 to 92 bytes that the blocks an SM is to hold leave to the stack, several runs side by side), a longer one twice, a
+// batch at a time.  What bounds the launch is how many of its loads are in flight; and until its last
 // block has started, the launch behind it, which runs under it, does not (8 x 4 units of 4096 tokens, 24 x 48: blocks of 100 registers
 // in two rounds, each run read twice, 39.9 us a call; this way 37.7).
 #pragma once

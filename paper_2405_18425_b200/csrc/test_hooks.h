@@ -7,13 +7,11 @@
  *   VIG_TEST_KERNEL_SIMT   always the fp32 SIMT recurrence kernel
  *   VIG_TEST_KERNEL_CHUNK_TASKS  sequences of more than 256 tokens always take the three chunk-task launches
  *   VIG_TEST_KERNEL_SEGMENTS     sequences of 257 .. 8192 tokens always take the segmented single launch
- *                          (the default chooses between the two by segment count and unit count).
  *   VIG_TEST_KERNEL_TCGEN05      always the tcgen05 kernels: the single-block one up to 256 tokens, chunk tasks or segments beyond
  *   VIG_TEST_KERNEL_WARP_TILES   always the kernels of one warp per 16 tokens, one block per unit or per chunk
  *   VIG_TEST_KERNEL_CLUSTERS     129 .. 1024 tokens: the blocks of up to 128 tokens of a unit always as one cluster
- *                          (the default chooses between these by head size, length and unit count).
- *                          vig_bigla_workspace_bytes follows the setting: query it under the setting the call
- *                          will run with
+ * The default chooses between all of these but SIMT by head size, length and unit count.  vig_bigla_workspace_bytes follows the
+ * setting: query it under the setting the call will run with.
  * Returns VIG_OK, or VIG_ERR_UNSUPPORTED for an unknown value (the setting is then unchanged). */
 #ifndef VIG_TEST_HOOKS_H
 #define VIG_TEST_HOOKS_H

@@ -850,7 +850,7 @@ def cluster_form():
 @pytest.mark.parametrize("L", [129, 200, 256, 257, 289, 400, 513, 1009, 1024])
 def test_chunks_of_a_cluster(oracle, cluster_form, dk, dv, L):
     """Two to eight chunks, a last one of one token, of whole tiles and full; beyond 256 tokens with the bits of the three launches over
-    the same chunks, from log gates (gate logits: there the gates are prepared once and read twice, the same values)."""
+    the same chunks, from log gates and from logits."""
     cfg, x = random_problem(3100 + L, 3, 2, L, dk, dv, "bf16", gate_mean=1.0)
     for run in (_run_unfused, _run_fused):
         before = vig.vig_kernel_launch_count()
