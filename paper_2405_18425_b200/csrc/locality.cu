@@ -67,8 +67,8 @@ __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float
 // shared memory and adds them into the three output rows they touch, which live in rolling accumulators.  Lanes run
 // over channel groups first, so shared-memory reads and the 16-byte output stores are contiguous per warp.
 template <typename T>
-__global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ CUtensorMap tm_x, const T* __restrict__ w,
-                                                        const T* __restrict__ bias, T* __restrict__ out, int Hh, int Ww, int C, int gpb, int tw,
+__global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ CUtensorMap tm_x, const T* w,
+                                                        const T* bias, T* out, int Hh, int Ww, int C, int gpb, int tw,
                                                         int th, int rowsegs, int coltiles, int tasks, int* dev_status) {
     constexpr int V = Vec<T>::N;
     using Raw = typename Vec<T>::Raw;
@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(256) dwconv3x3_kernel(const __grid_constant__ 
         mbar_expect_tx(bar0 + 8 * buf, tile_bytes);
         tma_load_4d(smem_u32(dw_smem) + buf * buf_pitch, &tm_x, c_slab, j0 - 1, i0 - 1, n, bar0 + 8 * buf);
     };
+    // (no __restrict__: filters and bias may be what a kernel still running writes, so they are not read-only for this kernel's lifetime)
     if (threadIdx.x == 0) {   // the first tile and the filters to L2 while the launch before still runs (a prefetch consumes nothing)
         const int task = blockIdx.x, j0 = (task % coltiles) * tw, i0 = ((task / coltiles) % rowsegs) * th, n = task / (coltiles * rowsegs);
         if (task < tasks) tma_prefetch_4d(&tm_x, c_slab, j0 - 1, i0 - 1, n);

@@ -38,3 +38,21 @@ def test_early_rows_are_loaded_at_gpu_scope():
     assert len(loads) == 3 and all(re.search(r"AHEAD \? ld_gpu(16|8|4)\(", line) for line in loads)
     ptx = open(os.path.join(CSRC, "ptx.cuh")).read()
     assert len(re.findall(r"ld\.relaxed\.gpu\.global\.(?:v[24]\.)?u32", ptx)) == 3
+
+
+def test_kernels_that_may_start_early_do_not_take_inputs_for_read_only():
+    """A kernel launched with programmatic serialization may start while the one that writes its inputs still runs: they are not
+    read-only for its lifetime, so nothing may lead the compiler to the loads that assume it."""
+    early = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith(".cu"):
+            continue
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        for m in re.finditer(r"__global__[^{;]*?\b(\w+_kernel)\(([^{;]*?)\) \{", text):
+            if re.search(r"<<<", text) and re.search(m.group(1) + r"(?:<[^<>]*>)?<<<", text):
+                continue   # an ordinary launch
+            early += 1
+            assert "__restrict__" not in m.group(2), m.group(1)
+    assert early >= 10
+    sources = "".join(open(os.path.join(CSRC, n)).read() for n in os.listdir(CSRC) if n.endswith((".cu", ".cuh")))
+    assert "__ldg(" not in sources and "ld.global.nc" not in sources
