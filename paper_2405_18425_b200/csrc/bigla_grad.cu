@@ -897,7 +897,7 @@ cudaError_t launch_grad_t(GArgs a, const GPlan& p, long long units, cudaStream_t
         e = launch_grad(bigla_grad_kernel<DK, DV, kSummary>, grid, three ? 32 * p.tiles : threads(kSummary), GLayout<DV>(p.tiles, kSummary).total, false, stream, tq, tk, tf, tb, tv, tg, a);
         if (e == cudaSuccess) {
             count_launch();
-            e = with_fold_plan(p.nch, [&](auto groups, auto run) {
+            e = with_fold_plan(p.nch, units, 4, DK / 4 * DV, sms, [&](auto groups, auto run) {
                 constexpr int kGroups = decltype(groups)::value, kItems = kFoldThreads / kGroups;
                 return launch_pdl(grad_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)units, 4, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
             });

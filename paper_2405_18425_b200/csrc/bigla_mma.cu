@@ -688,7 +688,7 @@ cudaError_t launch_chunks(MArgs a, cudaStream_t stream) {
     if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
     if (e != cudaSuccess) return e;
-    e = with_fold_plan(a.nch, [&](auto groups, auto run) {
+    e = with_fold_plan(a.nch, a.units, 2, DK / 4 * DV, device_sms(), [&](auto groups, auto run) {
         constexpr int kGroups = decltype(groups)::value, kItems = kFoldThreads / kGroups;
         return launch_pdl(mma_fold_kernel<DK, DV, kGroups, decltype(run)::value>, dim3((unsigned)a.units, 2, (DK / 4 * DV + kItems - 1) / kItems), dim3(kFoldThreads), 0, stream, a);
     });

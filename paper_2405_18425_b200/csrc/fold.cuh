@@ -76,14 +76,20 @@ __device__ __forceinline__ void fold_runs(const float* own0, int own_step, const
 
 // Runs side by side and chunks of a run for a sequence of nch chunks, and the launch: f(groups, run), compile-time numbers.  Few blocks
 // where they do: the launch behind this one shares the chip with it (13 chunks of 16 units, 24 x 48, in four runs of 160 blocks instead
-// of one of 64: 17.2 us a call instead of 14.1).
+// of one of 64: 17.2 us a call instead of 14.1).  So up to 128 chunks in eight longer runs, read twice, where that gives every block of
+// both launches an SM of its own and sixteen do not: the chunks' blocks would come to stand two on an SM beside idle ones.
+// states, pieces: of a unit; a piece is four key dimensions of a value column.
 template <typename F>
-cudaError_t with_fold_plan(int nch, const F& f) {
+cudaError_t with_fold_plan(int nch, long long units, int states, int pieces, int sms, const F& f) {
     using std::integral_constant;
+    auto apart = [&](int groups) {
+        const int items = kFoldThreads / groups;
+        return units * (states * ((pieces + items - 1) / items) + nch) <= sms;
+    };
     if (nch <= 4) return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
     if (nch <= 24) return f(integral_constant<int, 1>{}, integral_constant<int, 8>{});
     if (nch <= 32) return f(integral_constant<int, 8>{}, integral_constant<int, 4>{});
-    if (nch <= 64) return f(integral_constant<int, 8>{}, integral_constant<int, 8>{});
+    if (nch <= 64 || (nch <= 128 && apart(8) && !apart(16))) return f(integral_constant<int, 8>{}, integral_constant<int, 8>{});
     if (nch <= 128) return f(integral_constant<int, 16>{}, integral_constant<int, 8>{});
     return f(integral_constant<int, 32>{}, integral_constant<int, 8>{});
 }

@@ -367,3 +367,28 @@ def test_forward_walks_of_three_and_four_columns_a_lane(oracle, cpl, L, dk, dv, 
     got = device_to_f64(out, dtype)
     assert np.isfinite(got).all()
     assert rel_err(got, oracle_out(oracle, x["q"], x["k"], x["v"], la[0], la[1], dtype)) <= TOL[dtype]
+
+
+@pytest.mark.parametrize("L,dk,dv", [(6200, 32, 64), (6240, 32, 48), (9000, 24, 64), (10300, 24, 32)])
+def test_gradient_fold_over_runs_of_more_chunks_than_it_keeps(oracle, L, dk, dv):
+    """65 to 108 chunks of one unit: eight runs of nine to fourteen chunks, read twice, a last run of fewer, or sixteen runs."""
+    cfg, x = random_problem(5000 + L, 1, 1, L, dk, dv, "bf16", gate_mean=2.0)
+    got, ref = _run(oracle, cfg, x, synth.make_grad_input(cfg))
+    _check(got, ref, "bf16")
+
+
+@pytest.mark.parametrize("L,dk,dv", [(8300, 32, 64), (11600, 32, 64), (13000, 24, 64)])
+def test_forward_fold_over_runs_of_more_chunks_than_it_keeps(oracle, L, dk, dv):
+    """The same of the forward pass, from log gates and from logits: chunks of 128 tokens and fewer."""
+    cfg, x = random_problem(5100 + L, 1, 1, L, dk, dv, "bf16", gate_mean=2.0)
+    la = [oracle_log_alpha(oracle, x[n], "bf16", cfg.tau) for n in ("g_fwd", "g_bwd")]
+    d = {n: to_device(a, "bf16") for n, a in dict(x, f=la[0], b=la[1]).items()}
+    ref = oracle_out(oracle, x["q"], x["k"], x["v"], la[0], la[1], "bf16")
+    for call in (lambda o: vig.vig_bigla_fwd_bf16(d["q"], d["k"], d["v"], d["f"], d["b"], o),
+                 lambda o: vig.vig_bigla_fwd_gates_bf16(d["q"], d["k"], d["v"], d["g_fwd"], d["g_bwd"], o, cfg.tau)):
+        out = torch.full_like(d["v"], float("nan"))
+        before = vig.vig_kernel_launch_count()
+        call(out)
+        assert vig.vig_kernel_launch_count() - before == 3
+        got = device_to_f64(out, "bf16")
+        assert np.isfinite(got).all() and rel_err(got, ref) <= TOL["bf16"]
