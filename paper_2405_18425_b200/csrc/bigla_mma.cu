@@ -25,6 +25,7 @@
 #include <cuda.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "fold.cuh"
 #include "mma.cuh"
@@ -47,17 +48,25 @@ struct MArgs {
     const __nv_bfloat16 *q, *k, *v, *la_f, *la_b;   // GATES: la_f / la_b hold the gate logits
     __nv_bfloat16* out;
     int L;
-    long long units, blocks;   // blocks: units (kUnit) or units x chunks
+    long long blocks;  // units (kUnit) or units x chunks
     int nch, tiles;    // chunks per unit, tiles per chunk (long sequences)
-    float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
-    uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
-    float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
-    int* flags;        // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
     int* dev_status;
     float inv_tau;
     int ahead;         // the block this many further on has its inputs pulled into L2
     int expire_wait;   // test hook: every block lets one bounded wait, on an mbarrier nothing completes, run out
 };
+// What chunks have beside it.  Units of one block do without: with everything in one struct the compiler lets their instances keep fewer of
+// the parameters in registers and put up to 92 bytes a thread on the stack instead of up to 40 (202 units of 187 tokens, 16 x 64: 8.5 us,
+// 7.9 this way); clusters are the faster ones with it (24 x 6 units of 300, 32 x 64: 18.6 us, 20.5 without).
+struct MChunkArgs : MArgs {
+    long long units;
+    float* u;          // [unit][chunk][S>, S<][DV][DK] fp32: what a chunk adds to the states, key dimensions in fragment order
+    uint8_t* img;      // [unit][chunk][S>, S<][DV][64 B]: the states that enter a chunk, as shared-memory tiles
+    float* decay;      // [unit][chunk][2][32]: products of alpha over the chunk
+    int* flags;        // [unit][chunk]: 1: gates out of range, 2: not computed (a wait ran out)
+};
+template <int MODE>
+using ArgsOf = std::conditional_t<MODE == kUnit, MArgs, MChunkArgs>;
 
 // Shared memory: v [rows][RV], k~> and k~< [rows][64 B], the two states [DV][64 B], gate totals [tile][2][32] fp32; chunks of a
 // cluster: a slot for each of the other chunks (the state it adds, [DV][DK] fp32, its decay [DK] and a status word), then the
@@ -88,7 +97,7 @@ constexpr int mma_blocks_per_sm(int dk, int dv, int max_tiles, int mode) {
 }
 
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
-__global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MODE)) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const MArgs args) {
+__global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MODE)) bigla_mma_kernel(const __grid_constant__ CUtensorMap tm_v, const ArgsOf<MODE> args) {
     constexpr int NP = DK / 8, MP = (NP + 1) / 2;   // 8-column tiles of the key dimensions, pairs of them
     constexpr int NV = DV / 8, MV = DV / 16;        // ... of the value dimensions
     constexpr int RV = MLayout<DV>::kVRow;
@@ -277,18 +286,22 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         cluster_wait();
     } else if (!ok) {   // a load that never lands: report it and leave, all threads together, nothing stored
         if (tid == 0) atomicOr(args.dev_status, kDevStatusTimeout);
-        if (MODE == kSummary && tid == 0) args.flags[blockIdx.x] = 2;   // (nor by the launches behind this one)
+        if constexpr (MODE == kSummary) {
+            if (tid == 0) args.flags[blockIdx.x] = 2;   // (nor by the launches behind this one)
+        }
         if (MODE == kMain) pdl_wait();   // (no block ends before the fold: what comes next only waits for this launch)
         return;
     }
-    if (MODE == kSummary && tid < 64 && (tid & 31) < DK) {   // (at least two warps)
-        float s = 0.f;
-        for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
-        args.decay[(size_t)blockIdx.x * 64 + tid] = ex2(GATES ? s : s * kLog2e);
-        if (tid == 0) args.flags[blockIdx.x] = *slow;
+    if constexpr (MODE == kSummary) {
+        if (tid < 64 && (tid & 31) < DK) {   // (at least two warps)
+            float s = 0.f;
+            for (int x = 0; x < T; ++x) s += totals[(x * 2 + (tid >> 5)) * 32 + (tid & 31)];
+            args.decay[(size_t)blockIdx.x * 64 + tid] = ex2(GATES ? s : s * kLog2e);
+            if (tid == 0) args.flags[blockIdx.x] = *slow;
+        }
     }
     bool redo = MODE == kUnit && *slow;
-    if (MODE == kMain) {
+    if constexpr (MODE == kMain) {
         int any = 0;
         for (int x = tid; x < nch; x += blockDim.x) any |= (int)ld_gpu4(args.flags + unit * nch + x);
         const bool missing = __syncthreads_or(any & 2);
@@ -366,7 +379,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
                 for (int r = 0; r < 2; ++r) {
                     const int n = 16 * mt + 8 * r + g;
                     const float u0 = u[j][2 * r] * d0, u1 = u[j][2 * r + 1] * d1;
-                    if (MODE == kSummary)
+                    if constexpr (MODE == kSummary)
                         *reinterpret_cast<float2*>(args.u + (((size_t)blockIdx.x * 2 + dir) * DV + n) * DK + 8 * j + 2 * c) = make_float2(u0, u1);
                     else
                         *reinterpret_cast<uint32_t*>(smem + lay.st + dir * kState + n * 64 + ((j ^ ((n >> 1) & 3)) << 4) + 4 * c) = pack_bf16(u0, u1);
@@ -566,7 +579,7 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
 // Second launch of a long call: the states that enter every chunk from what the chunks add, S> ascending, S< descending, the latter
 // stored times d<(c), the decay from the chunk's end to its start.
 template <int DK, int DV, int GROUPS, int RUN>
-__global__ void __launch_bounds__(kFoldThreads, fold_blocks_per_sm(RUN)) mma_fold_kernel(const MArgs a) {
+__global__ void __launch_bounds__(kFoldThreads, fold_blocks_per_sm(RUN)) mma_fold_kernel(const MChunkArgs a) {
     constexpr int P = DK / 4, kItems = kFoldThreads / GROUPS;
     constexpr int kState = (int)MLayout<DV>::kState;
     const size_t unit = blockIdx.x;
@@ -588,7 +601,7 @@ __global__ void __launch_bounds__(kFoldThreads, fold_blocks_per_sm(RUN)) mma_fol
 }
 
 template <int DK, int DV, bool GATES, int MAXT, int MODE>
-cudaError_t launch_mma_t(MArgs a, const CUtensorMap& tv, int tiles, cudaStream_t stream) {
+cudaError_t launch_mma_t(ArgsOf<MODE> a, const CUtensorMap& tv, int tiles, cudaStream_t stream) {
     const int threads = (tiles < 2 ? 2 : tiles) * 32;
     const size_t smem = MLayout<DV>(tiles, MODE == kMain || MODE == kCluster || (MODE == kUnit && tiles > 8), MODE == kCluster ? all_slots(DK, DV, a.nch) : 0u).total, rec = (size_t)rec_plan(threads < kRecThreads ? threads : kRecThreads, DK, DV).smem_floats * 4;
     static std::atomic<int> sms_of[64];   // 0: this instance is not configured on the device yet
@@ -616,7 +629,7 @@ template <int DK, int DV, bool GATES>
 cudaError_t launch_mma(const MArgs& a, cudaStream_t stream) {
     const int T = (a.L + 15) / 16;
     CUtensorMap tv;
-    if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
+    if (!make_map(&tv, a.v, a.blocks, a.L, DV, DV == 32 ? 32 : 64, T * 16)) return cudaErrorInvalidValue;
     if (T <= 8) return launch_mma_t<DK, DV, GATES, 8, kUnit>(a, tv, T, stream);
     if (T <= 13) return launch_mma_t<DK, DV, GATES, 13, kUnit>(a, tv, T, stream);
     return launch_mma_t<DK, DV, GATES, 16, kUnit>(a, tv, T, stream);
@@ -676,14 +689,14 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false)
 
 // One launch: the chunks of a unit are the blocks of a cluster.
 template <int DK, int DV, bool GATES>
-cudaError_t launch_cluster(MArgs a, cudaStream_t stream) {
+cudaError_t launch_cluster(MChunkArgs a, cudaStream_t stream) {
     CUtensorMap tv;
     if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     return launch_mma_t<DK, DV, GATES, 8, kCluster>(a, tv, a.tiles, stream);
 }
 
 template <int DK, int DV, bool GATES>
-cudaError_t launch_chunks(MArgs a, cudaStream_t stream) {
+cudaError_t launch_chunks(MChunkArgs a, cudaStream_t stream) {
     CUtensorMap tv;
     if (!make_map(&tv, a.v, a.units, a.L, DV, DV == 32 ? 32 : 64, a.tiles * 16)) return cudaErrorInvalidValue;
     cudaError_t e = launch_mma_t<DK, DV, GATES, 8, kSummary>(a, tv, a.tiles, stream);
@@ -719,7 +732,7 @@ cudaError_t launch_bigla_mma(const __nv_bfloat16* q, const __nv_bfloat16* k, con
                              int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
     MArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
-    a.L = L; a.units = a.blocks = units;
+    a.L = L; a.blocks = units;
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
     a.expire_wait = take_expire_next_wait() == 1;
     a.dev_status = device_status_ptr();
@@ -789,7 +802,7 @@ cudaError_t launch_bigla_mma_chunks(const __nv_bfloat16* q, const __nv_bfloat16*
                                     int L, int dk, int dv, float gate_tau, void* ws, cudaStream_t stream) {
     const ChunkPlan p = chunk_plan(units, L, dk, dv, gate_tau > 0.f);
     char* b = static_cast<char*>(ws);
-    MArgs a{};
+    MChunkArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
     a.L = L; a.units = units; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
     a.u = reinterpret_cast<float*>(b + p.u);
@@ -814,7 +827,7 @@ cudaError_t launch_bigla_mma_cluster(const __nv_bfloat16* q, const __nv_bfloat16
                                      const __nv_bfloat16* la_f, const __nv_bfloat16* la_b, __nv_bfloat16* out, long long units,
                                      int L, int dk, int dv, float gate_tau, cudaStream_t stream) {
     const ChunkPlan p = chunk_plan(units, L, dk, dv);
-    MArgs a{};
+    MChunkArgs a{};
     a.q = q; a.k = k; a.v = v; a.la_f = la_f; a.la_b = la_b; a.out = out;
     a.L = L; a.units = units; a.blocks = units * p.nch; a.nch = p.nch; a.tiles = p.tiles;
     a.inv_tau = gate_tau > 0.f ? 1.f / gate_tau : 0.f;
