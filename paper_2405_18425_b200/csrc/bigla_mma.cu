@@ -173,20 +173,23 @@ __global__ void __launch_bounds__(MAXT * 32, mma_blocks_per_sm(DK, DV, MAXT, MOD
         pull((MODE == kUnit ? next : next / (unsigned)nch) * L + nr, min(tiles * 16, L - nr));   // (q: for the chunks' launch as well)
     }
     // ---- gate totals of the tile; the gates turned, as B operands of products over the tokens ----
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            if (GATES) {
-                af[r][j] = log2_alpha_pair<MODE != kUnit>(af[r][j], args.inv_tau);
-                ab[r][j] = log2_alpha_pair<MODE != kUnit>(ab[r][j], args.inv_tau);
-            }
+    auto prepare = [&](int r, int j) {
+        if (GATES) {
+            af[r][j] = log2_alpha_pair<MODE != kUnit>(af[r][j], args.inv_tau);
+            ab[r][j] = log2_alpha_pair<MODE != kUnit>(ab[r][j], args.inv_tau);
         }
+    };
+    if (MODE == kCluster) {   // (all of them first: 12 bytes a thread on the stack at 32 x 64 instead of 52; elsewhere as they are turned: 12 instead of 24 at 24 x 48)
+#pragma unroll
+        for (int j = 0; j < NP; ++j)
+#pragma unroll
+            for (int r = 0; r < 2; ++r) prepare(r, j);
     }
 #pragma unroll
     for (int j = 0; j < NP; ++j) {
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
+            if (MODE != kCluster) prepare(r, j);
             af[r][j] = movmatrix(af[r][j]);
             ab[r][j] = movmatrix(ab[r][j]);
         }
