@@ -147,7 +147,7 @@ int vig_gate_prep_f32(const void* g_fwd, const void* g_bwd,
  * tile into log alpha in shared memory (fp32 evaluation with exp and log from the special-function unit,
  * rounded to bf16 as the tensor-core operand of the prefix sums: the same rounding point as the un-fused
  * chain).  Longer sequences prepare the gates on the way as well where they run as the chunks of a cluster (no scratch) or in
- * three launches over chunks on the warp-level kernels (scratch as above; calls that fill the GPU at most four times are cut into
+ * three launches over chunks on the warp-level kernels (scratch as above; calls that fill the GPU at most 2.25 times, four at 16 x 32, are cut into
  * chunks of 80 to 128 tokens, so up to 1.6 times that).  Everything else runs gate preparation into scratch the library allocates
  * and frees on `stream` (its memory pool), then the ordinary forward pass.
  * Errors: NULL_POINTER, BAD_DIM (also tau), UNSUPPORTED, MISALIGNED, CUDA. */

@@ -654,9 +654,10 @@ static int device_sms() {
 // Sequences of any length: chunks of equal numbers of tiles, up to eight.  From logits, beyond eight chunks, the tiles are what makes
 // the rounds of blocks cheapest, a block's time being about that of its loads and hand-overs (eight tiles' worth) and of its tiles, short
 // of the 128 chunks up to which the fold keeps its runs short.  6 x 4 units of 1300 tokens, 24 x 64: 17.8 us a call, 20.6 with
-// eight tiles; 3 x 3 of 5000, 24 x 32: 16.4 and 18.3; 8 x 4 of 4096, 24 x 48: 37.4 and 37.8.  Beyond four rounds
-// the last one weighs little, and the scratch, which grows with the number of chunks, stays that of eight tiles (84 units of 4096,
-// 24 x 64: 113.7 us cut by rounds, 110.5 this way).  (From log gates the scratch may be the caller's, whose size this keeps.)
+// eight tiles; 3 x 3 of 5000, 24 x 32: 16.4 and 18.3; 8 x 4 of 4096, 24 x 48: 37.4 and 37.8.  Beyond two rounds and
+// a quarter the blocks no longer end together, so that a round saved is none (119 units of 1868, 24 x 48, 3.0 rounds: 67.1 us cut by rounds,
+// 64.1 with eight tiles; 15 of 10813, 2.15 rounds: 46.7 and 48.8), four at 16 x 32, whose blocks are short (129 units of 1300,
+// 2.4 rounds: 28.9 and 31.6), and the scratch, which grows with the number of chunks, stays that of eight tiles.  (From log gates the scratch may be the caller's, whose size this keeps.)
 struct ChunkPlan {
     int nch, tiles;
     size_t u, img, decay, flags, total;   // byte offsets in the scratch
@@ -671,7 +672,7 @@ ChunkPlan chunk_plan(long long units, int L, int dk, int dv, bool gates = false)
     };
     cut(kChunkTiles);
     const long long slots = (long long)mma_blocks_per_sm(dk, dv, kChunkTiles, kMain) * device_sms();
-    if (gates && p.nch > kChunkTiles && form_units(units) * p.nch <= 4 * slots) {
+    if (gates && p.nch > kChunkTiles && 4 * form_units(units) * p.nch <= (dk * dv <= 512 ? 16 : 9) * slots) {
         int best = p.tiles;
         long long best_cost = -1;
         for (int tiles = kChunkTiles; tiles >= 5; --tiles) {

@@ -682,6 +682,23 @@ def test_long_fp32_walks_of_few_units_have_eight_segments(L):
     assert torch.equal(outs[0].view(torch.int32), outs[1][:2].view(torch.int32))
 
 
+def test_calls_of_several_rounds_from_logits_keep_eight_tiles_a_chunk():
+    """Three rounds of blocks are cut as five are, where nothing is gained by shorter chunks: a unit has the same bits in both."""
+    slots = 4 * torch.cuda.get_device_properties(0).multi_processor_count     # four blocks an SM at 24 x 48
+    L, chunks = 1868, 15
+    few, many = 3 * slots // chunks + 1, 5 * slots // chunks
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    mk = lambda d: torch.randn(many, 1, L, d, device="cuda", generator=gen).bfloat16()
+    q, k, v, gf, gb = mk(24) * 24 ** -0.5, mk(24), mk(48), mk(24), mk(24)
+    outs = []
+    for units in (few, many):
+        a = [t[:units] for t in (q, k, v, gf, gb)]
+        outs.append(torch.empty_like(a[2]))
+        vig.vig_bigla_fwd_gates_bf16(*a, outs[-1], 16.0)
+    torch.cuda.synchronize()
+    assert torch.equal(outs[0].view(torch.int16), outs[1][:few].view(torch.int16))
+
+
 def test_workspace_variant_and_determinism(oracle):
     cfg = synth.CONFIGS[4]
     x = synth.make_inputs(cfg, units=slice(0, 6))
